@@ -235,8 +235,10 @@ def _report(r, table, stat="H"):
     if hits.shape[0] == 0:
         return dict(table, n_hits=r["n_hits"])
     order = hits.view(torch.int64)[:, 0].argsort()  # snp << 32 | trait
-    for name, v in (("hits", hits), (stat, torch.as_tensor(r[stat])), ("p", torch.as_tensor(r["p"]))):
-        torch.index_select(v, 0, order, out=table[name][: order.numel()])
+    record = torch.complex128  # a hit record moves as one 16-byte element
+    for v, to in ((hits.view(record)[:, 0], table["hits"].view(record)[:, 0]),
+                  (torch.as_tensor(r[stat]), table[stat]), (torch.as_tensor(r["p"]), table["p"])):
+        torch.index_select(v, 0, order, out=to[: order.numel()])
     return dict(table, n_hits=r["n_hits"])
 
 
