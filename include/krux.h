@@ -188,9 +188,10 @@ krux_status krux_scan_plain(krux_ctx *ctx, const krux_rankset *rs, const int8_t 
  *           that threshold is the mean permuted count over the real count.
  *           fdr_bins >= 1 and fdr_bin_width > 0 when fdr_hist is given.  Row 0 is
  *           complete only when the hits fit the capacity (else KRUX_EOVERFLOW).
- * The unpermuted scan's hits are returned as in krux_scan.  With more than 65,536
- * SNPs a short seed pass over the first 16,384 runs first and primes the minimum-p
- * search with lower bounds; both launches are enqueued back to back on `stream`
+ * The unpermuted scan's hits are returned as in krux_scan.  A seed pass runs
+ * first and primes the minimum-p search with lower bounds (over all SNPs with complete
+ * expression; with NaN expression over the first 16,384, when there are more than
+ * 65,536); both launches are enqueued back to back on `stream`
  * (the rows of perms are checked on the host first, the hit counts read back at
  * the end), and krux_graph_permute captures the same two launches. */
 krux_status krux_permute(krux_ctx *ctx, const krux_rankset *rs, const int8_t *geno, int64_t S,

@@ -271,6 +271,9 @@ struct LaunchShape {
   int ka = 0, nA = 0, b_region = 0, force_nc = 0, no_pair = 0;
 };
 constexpr size_t kSmemLimit = 232448;
+// Shared memory of the plain forms beyond the general one's: the hit-event ring, and
+// outside permutation batches a smaller trait-constant ring.
+constexpr size_t plain_extra(bool perm) { return kEvRegion - (perm ? 0 : kTcSaved); }
 
 size_t shape_overhead(int nA, int codes_k) {
   return scan_smem_bytes2(kTmemSlots, nA, 0, 0, std::max(codes_k, 16));
@@ -337,10 +340,10 @@ bool plain_form_fits(const krux_ctx *ctx, int Np) {
   if (ctx->tune_layout == 0) return false;
   const int kpad = round_up(Np, 16);
   LaunchShape sh;
-  if (!pick_launch_shape(ctx, kpad, 0, sh, kEvRegion)) return false;
+  if (!pick_launch_shape(ctx, kpad, 0, sh, plain_extra(false))) return false;
   const int nc = (int)(sh.b_region / (256 * kpad));
   return sh.ka == kpad && nc >= 2 && nc % 2 == 0 &&
-         shape_overhead(sh.nA, 0) + (size_t)sh.nA * 256 * sh.ka + sh.b_region + kEvRegion <= kSmemLimit;
+         shape_overhead(sh.nA, 0) + (size_t)sh.nA * 256 * sh.ka + sh.b_region + plain_extra(false) <= kSmemLimit;
 }
 
 // Refuses a launch plan whose shared-memory regions or per-group shapes are not
@@ -391,39 +394,92 @@ struct GroupPlan {
   int64_t step_lo = 0;  // first step scanned (a min-p seed pass skips the unpermuted agroup)
 };
 
-std::vector<WorkItem> make_items(const std::vector<GroupPlan> &gp, int nc, int grid) {
-  int64_t nb = 0, maxL = 1;
-  for (auto &g : gp) {
-    nb += g.n_btiles;
-    maxL = std::max(maxL, g.steps - g.step_lo);
+// The work items of a launch: every B tile of every group against its trait steps,
+// the steps cut into ranges.  CTAs take items from a common counter.
+//
+// One group: as many ranges per B tile as fill whole waves of CTAs best, each item
+// costing about two steps on top of its own (the B tile's load).  Where the group's
+// rank matrices together exceed what stays in L2 (permutation batches: 76 MB at P =
+// 16, T = 20,000, against 129 MB of L2 in two halves that both keep what their SMs
+// read), a range holds at most kRangeBytes of them and the ranges come one after the
+// other, each over all B tiles, so that the CTAs running at one time stream the same
+// part; with every range in flight at once the batch of 16 x 20,000 x 200,000 took 2 to
+// 4 % longer (85.3 against 81.5 ms when measured).
+//
+// Several groups (cohorts, missing-value patterns) differ in the cost of a B tile by
+// up to a factor of ten: each is cut into ranges of about the same cost, and the
+// items are taken longest first (5,000 x 100,000 x 102 with 196 missing patterns and
+// 1 % NaN: the scan 1.03 -> 0.58 ms, with two event entries per event warp).
+std::vector<WorkItem> make_items(const std::vector<GroupPlan> &gp, int grid) {
+  constexpr int64_t kRangeBytes = 16 << 20;
+  std::vector<WorkItem> items;
+  auto cut = [&](size_t gi, int64_t b, int64_t k, int64_t s) {
+    const int64_t L = gp[gi].steps - gp[gi].step_lo;
+    WorkItem w;
+    w.group = (int32_t)gi;
+    w.btile = (int32_t)b;
+    w.step_begin = (int32_t)(gp[gi].step_lo + L * k / s);
+    w.step_end = (int32_t)(gp[gi].step_lo + L * (k + 1) / s);
+    if (w.step_end > w.step_begin) items.push_back(w);
+  };
+  if (gp.size() == 1) {
+    const GroupPlan &g = gp[0];
+    const int64_t L = g.steps - g.step_lo;
+    const int64_t min_split =
+        std::max<int64_t>(1, (L * kTileM * g.d.Np * 2 + kRangeBytes - 1) / kRangeBytes);
+    int64_t split = std::max<int64_t>(1, std::min(min_split, L));
+    double best = 1e300;
+    for (int64_t s = split; s <= std::max<int64_t>(32, min_split + 4) && s <= L; ++s) {
+      const int64_t waves = (g.n_btiles * s + grid - 1) / grid;
+      const double cost = (double)waves * ((double)L / s + 2.0);
+      if (cost < best * 0.999) {
+        best = cost;
+        split = s;
+      }
+    }
+    for (int64_t i = 0; i < split * g.n_btiles; ++i) {
+      if (min_split > 1) cut(0, i % g.n_btiles, i / g.n_btiles, split);
+      else cut(0, i / split, i % split, split);
+    }
+    return items;
   }
-  int best_split = 1;
+  // cost of a step: the contraction of its chunk pairs, and a fixed part
+  auto step_cost = [&](const GroupDesc &d, int64_t chunks) {
+    return (double)((chunks + 1) / 2) * (8.0 * d.Np + 300.0);
+  };
+  double total = 0.0;
+  for (auto &g : gp)
+    total += (double)(g.steps - g.step_lo) * g.n_btiles * step_cost(g.d, std::min(g.d.nc, g.d.nchunks));
+  std::vector<int64_t> split(gp.size(), 1), best_split;
   double best = 1e300;
-  for (int s = 1; s <= 32 && s <= maxL; ++s) {
-    const int64_t items = nb * s;
-    const int64_t waves = (items + grid - 1) / grid;
-    const double cost = (double)waves * ((double)maxL / s + 2.0);
-    if (cost < best * 0.999) {
-      best = cost;
-      best_split = s;
+  for (int m = 1; m <= 32; ++m) {
+    const double target = total / ((double)grid * m);
+    double longest = 0.0, extra = 0.0;
+    for (size_t i = 0; i < gp.size(); ++i) {
+      const auto &g = gp[i];
+      const int64_t L = g.steps - g.step_lo;
+      const double c = step_cost(g.d, std::min(g.d.nc, g.d.nchunks));
+      const int64_t s = std::max<int64_t>(1, std::min<int64_t>(L, (int64_t)std::ceil(L * c / target)));
+      split[i] = s;
+      longest = std::max(longest, std::ceil((double)L / s) * c);
+      extra += (double)s * g.n_btiles * 2.0 * c;
+    }
+    const double est = (total + extra) / grid + 0.5 * longest;
+    if (est < best * 0.999) {
+      best = est;
+      best_split = split;
     }
   }
-  std::vector<WorkItem> items;
-  for (size_t gi = 0; gi < gp.size(); ++gi) {
-    const auto &g = gp[gi];
-    const int64_t L = g.steps - g.step_lo;
-    const int s = (int)std::min<int64_t>(best_split, L);
-    for (int64_t b = 0; b < g.n_btiles; ++b)
-      for (int k = 0; k < s; ++k) {
-        WorkItem w;
-        w.group = (int32_t)gi;
-        w.btile = (int32_t)b;
-        w.step_begin = (int32_t)(g.step_lo + L * k / s);
-        w.step_end = (int32_t)(g.step_lo + L * (k + 1) / s);
-        if (w.step_end > w.step_begin) items.push_back(w);
-      }
-  }
-  (void)nc;
+  for (size_t gi = 0; gi < gp.size(); ++gi)
+    for (int64_t b = 0; b < gp[gi].n_btiles; ++b)
+      for (int64_t k = 0; k < best_split[gi]; ++k) cut(gi, b, k, best_split[gi]);
+  auto cost = [&](const WorkItem &w) {
+    const GroupDesc &d = gp[(size_t)w.group].d;
+    return (w.step_end - w.step_begin) *
+           step_cost(d, std::min<int64_t>(d.nc, d.nchunks - (int64_t)w.btile * d.nc));
+  };
+  std::stable_sort(items.begin(), items.end(),
+                   [&](const WorkItem &a, const WorkItem &b) { return cost(a) > cost(b); });
   return items;
 }
 
@@ -920,6 +976,7 @@ struct ScanGroupIn {
   const int64_t *snp_list = nullptr;  // device rows, or nullptr for [snp_begin, +n_snps)
   int64_t list_off = -1;              // offset into the call's list buffer (patched later)
   int64_t snp_begin = 0, n_snps = 0;
+  int64_t row_lo = 0, row_hi = 0;     // genotype rows the call may read (every listed SNP is one)
   int allow_missing = 0;
   int out_slot = 0;
   double *dense_H = nullptr, *dense_p = nullptr;
@@ -956,6 +1013,7 @@ struct CallPlan {
     uint16_t *lists = nullptr;   // [1 + P][T][N] NaN sample lists (rank sets with NaN)
     int32_t *inv = nullptr;      // [P][N] inverse permutations
     bool pre_done = false;       // the stacking was queued already (before a seed pass)
+    bool packed = false;         // and so was the packing (a seed pass over the same SNPs)
     bool seed = false;           // min-p seed pass: permuted agroups only, no hits, no FDR
   } perm;
   bool multi = false;  // markers with codes 0..4 (chunks of kChunkSnpsM SNPs)
@@ -1030,6 +1088,8 @@ krux_status plan_groups(krux_ctx *ctx, CallPlan &cp, const krux_rankset *rs, con
   g0.nan_idx = rs->dev.nan_idx;
   g0.geno = geno;
   g0.ldg = ldg;
+  g0.row_lo = b;
+  g0.row_hi = e;
   g0.out_slot = slot;
   g0.dense_H = dense_H;
   g0.dense_p = dense_p;
@@ -1217,6 +1277,14 @@ std::vector<WorkItem> make_items_cis(const CallPlan &cp, const std::vector<Group
   return items;
 }
 
+// The weights of the plain forms' rows, between sqrt(1 / (512 h)) and sqrt(2 / h)
+// (and the rounding on top), are FP16 normals well inside the range for every P_c
+// but those near 1, where h falls to zero: those calls take the general form.
+bool pq_range_ok(double h1, double h2) {
+  const double lo = std::min(h1, h2), hi = std::max(h1, h2);
+  return lo > 0.0 && std::sqrt(2.0 / lo) < 16384.0 && std::sqrt(1.0 / (kMaxN * hi)) > 1.0 / 4096.0;
+}
+
 // One fused launch, split in three phases so that the middle one can be captured
 // in a CUDA graph: prepare (host planning, buffer sizing, descriptor uploads; no
 // work queued that a replay would need), enqueue (stream work only: packing, the
@@ -1309,7 +1377,8 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     ctx->tune_nc = tnc;
     ctx->tune_nA = tnA;
     ctx->tune_ka = tka;
-    const bool ok = pick_launch_shape(ctx, kpad, codes_k, sh, fast_shape ? kEvRegion : 0);
+    const bool ok = pick_launch_shape(ctx, kpad, codes_k, sh,
+                                      fast_shape ? plain_extra(fl.signed_coef != 0) : 0);
     ctx->tune_nc = s_nc;
     ctx->tune_nA = s_nA;
     ctx->tune_ka = s_ka;
@@ -1426,7 +1495,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     descs[i] = d;
   }
   std::vector<WorkItem> items =
-      cp.cis.on ? make_items_cis(cp, plans) : make_items(plans, nc_max, ctx->sm_count);
+      cp.cis.on ? make_items_cis(cp, plans) : make_items(plans, ctx->sm_count);
   KRUX_CUDA(ctx, t_groups.ensure(sizeof(GroupDesc) * ng));
   KRUX_CUDA(ctx, t_items.ensure(sizeof(WorkItem) * std::max<size_t>(items.size(), 1)));
   // pageable uploads: staged before the calls return, so the host vectors may go
@@ -1435,40 +1504,6 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   if (!items.empty())
     KRUX_CUDA(ctx, cudaMemcpyAsync(t_items.p, items.data(), sizeof(WorkItem) * items.size(),
                                    cudaMemcpyHostToDevice, s));
-  fl.batched_pack = !cp.multi && cp.param.model != 1;
-  if (fl.batched_pack) {
-    std::vector<PackJob> jobs(ng);
-    int64_t slots = 0, halves = 0;
-    for (int i = 0; i < ng; ++i) {
-      const ScanGroupIn &g = cp.groups[i];
-      PackJob &j = jobs[i];
-      std::memset(&j, 0, sizeof j);
-      const int64_t nch = (g.n_snps + kChunkSnps - 1) / kChunkSnps;
-      j.geno = g.geno;
-      j.ldg = g.ldg;
-      j.snp_list = g.snp_list;
-      j.snp_begin = g.snp_begin;
-      j.n_snps = g.n_snps;
-      j.slot0 = slots;
-      j.half0 = halves;
-      j.B = reinterpret_cast<__half *>(ctx->B.as<char>() + fl.boff[i]);
-      j.meta = ctx->meta.as<ChunkMeta>() + fl.moff[i];
-      j.codes = g.nan_cnt ? ctx->codes.as<uint64_t>() + fl.coff[i] : nullptr;
-      j.N = g.rs->N;
-      j.Np = g.rs->Np;
-      j.allow_missing = g.allow_missing;
-      j.coef_nan = j.codes != nullptr && fast_nan ? 1 : 0;
-      slots += nch * kChunkSnps;
-      if (j.codes && !j.coef_nan) halves += nch * 2;
-    }
-    fl.n_pack_jobs = ng;
-    fl.pack_slots = slots;
-    fl.pack_halves = halves;
-    KRUX_CUDA(ctx, t_packjobs.ensure(sizeof(PackJob) * ng));
-    KRUX_CUDA(ctx, cudaMemcpyAsync(t_packjobs.p, jobs.data(), sizeof(PackJob) * ng,
-                                   cudaMemcpyHostToDevice, s));
-    fl.packjobs = t_packjobs.as<PackJob>();
-  }
   std::vector<const double *> cf(ng);
   for (int i = 0; i < ng; ++i) cf[i] = cp.groups[i].cfac;
   KRUX_CUDA(ctx, t_cfacptr.ensure(sizeof(double *) * ng));
@@ -1481,6 +1516,9 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   p.groups = t_groups.as<GroupDesc>();
   p.items = t_items.as<WorkItem>();
   p.n_items = (int32_t)items.size();
+  // the item counters sit behind the status words, one for each launch of a call
+  // (cleared with them before the first)
+  p.next = ctx->status.as<unsigned int>() + (cp.perm.seed ? 9 : 8);
   p.nc = nc_max;
   p.nA = sh.nA;
   p.kpad = std::max(codes_k, 16);
@@ -1521,7 +1559,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     bool fast = layout == 1 && !p.multi && (!p.has_nan || fast_nan) && !p.dense && !p.provisional &&
                 (!p.signed_coef || p.perm) && p.cis_window < 0;
     for (const GroupDesc &d : descs) fast = fast && d.pair == 1 && d.nkb == 1;
-    p.fast = fast ? 1 : 0;
+    p.fast = fast && pq_range_ok(fl.h1, fl.h2) && fast_form_ok() ? 1 : 0;
   }
   fl.grid = (int)std::min<size_t>(items.size(), (size_t)ctx->sm_count);
   // Single hit list: every epilogue warp stages its hits in a segment of its own
@@ -1544,12 +1582,50 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   }
   fl.smem = scan_smem_bytes2(nc_max, sh.nA, (size_t)p.a_tile_bytes, (size_t)p.b_region, p.kpad);
   if (p.fast) {  // the plain scan form also holds its ring of hit-event buffers
-    if (fl.smem + kEvRegion <= kSmemLimit) fl.smem += kEvRegion;
+    const size_t with_ring = fl.smem + plain_extra(p.perm != 0);
+    if (with_ring <= kSmemLimit) fl.smem = with_ring;
     else p.fast = 0;
   }
   if (fast_nan && !p.fast)  // the coefficient sets need the plain form: plan again
     return prepare_fused(ctx, cp, o, fl, s, tables, false);
   p.fast_nan = fast_nan ? 1 : 0;
+  fl.batched_pack = !cp.multi && cp.param.model != 1;
+  if (fl.batched_pack) {
+    std::vector<PackJob> jobs(ng);
+    int64_t slots = 0, halves = 0;
+    for (int i = 0; i < ng; ++i) {
+      const ScanGroupIn &g = cp.groups[i];
+      PackJob &j = jobs[i];
+      std::memset(&j, 0, sizeof j);
+      const int64_t nch = (g.n_snps + kChunkSnps - 1) / kChunkSnps;
+      j.geno = g.geno;
+      j.geno_lo = g.geno + g.row_lo * g.ldg;
+      j.geno_hi = g.geno + (g.row_hi - 1) * g.ldg + g.rs->N;
+      j.ldg = g.ldg;
+      j.snp_list = g.snp_list;
+      j.snp_begin = g.snp_begin;
+      j.n_snps = g.n_snps;
+      j.slot0 = slots;
+      j.half0 = halves;
+      j.B = reinterpret_cast<__half *>(ctx->B.as<char>() + fl.boff[i]);
+      j.meta = ctx->meta.as<ChunkMeta>() + fl.moff[i];
+      j.codes = g.nan_cnt ? ctx->codes.as<uint64_t>() + fl.coff[i] : nullptr;
+      j.N = g.rs->N;
+      j.Np = g.rs->Np;
+      j.allow_missing = g.allow_missing;
+      j.coef_nan = j.codes != nullptr && fast_nan ? 1 : 0;
+      j.pq_bits = p.fast ? pq_bits(g.rs->N) : 0;
+      slots += nch * kChunkSnps;
+      if (j.codes && !j.coef_nan) halves += nch * 2;
+    }
+    fl.n_pack_jobs = ng;
+    fl.pack_slots = slots;
+    fl.pack_halves = halves;
+    KRUX_CUDA(ctx, t_packjobs.ensure(sizeof(PackJob) * ng));
+    KRUX_CUDA(ctx, cudaMemcpyAsync(t_packjobs.p, jobs.data(), sizeof(PackJob) * ng,
+                                   cudaMemcpyHostToDevice, s));
+    fl.packjobs = t_packjobs.as<PackJob>();
+  }
   if (p.fast && p.perm && !cp.perm.seed && fl.grid > 0) {
     // each event warp's list for the deferred FP64 pass: about three times the
     // pairs a 200k-SNP batch passes on, at least 8192 and at most 65536 entries
@@ -1605,7 +1681,7 @@ krux_status enqueue_fused(krux_ctx *ctx, CallPlan &cp, const FusedLaunch &fl, cu
     }
   }
   ev_record(ctx, 2, s);
-  if (fl.batched_pack)
+  if (fl.batched_pack && !cp.perm.packed)
     KRUX_CUDA(ctx, launch_pack_batch(fl.packjobs, fl.n_pack_jobs, fl.pack_slots,
                                      fl.pack_halves, fl.h1, fl.h2, fl.signed_coef, status, s));
   for (int i = 0; i < ng && !fl.batched_pack; ++i) {
@@ -1688,7 +1764,7 @@ krux_status enqueue_fused(krux_ctx *ctx, CallPlan &cp, const FusedLaunch &fl, cu
 int fused_launches(const CallPlan &cp, const FusedLaunch &fl) {
   int n = (fl.grid > 0 ? 1 : 0) + (fl.staged ? 1 : 0);
   if (fl.batched_pack)
-    n += (fl.pack_slots > 0 ? 1 : 0) + (fl.pack_halves > 0 ? 1 : 0);
+    n += cp.perm.packed ? 0 : (fl.pack_slots > 0 ? 1 : 0) + (fl.pack_halves > 0 ? 1 : 0);
   else
     for (auto &g : cp.groups) n += g.nan_cnt ? 2 : 1;
   for (auto &os : cp.slots) n += (os.capacity > 0 && cp.param.model < 0) ? 1 : 0;
@@ -1747,24 +1823,24 @@ krux_status run_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, cudaStrea
 }
 
 // Seed pass of a permutation batch (section "P-value calculation and empirical
-// FDR correction": the minimum p of each permuted trait over all SNPs): the
-// permuted groups against the first kSeedSnps SNPs, so that the main launch
-// starts from running minima over thousands of SNPs instead of none (without it
-// the first wave of CTAs refines nearly every chunk in FP64).  False when the
-// call is too small to gain from one.
+// FDR correction": the minimum p of each permuted trait over all SNPs).  In the plain
+// form it covers every SNP and records, per permutation, trait and class, the 16-SNP
+// block with the largest value; that block is decided exactly, and the main launch
+// then meets only near ties and the pairs of the FDR band.  A shorter seed costs more
+// than it saves: on LD blocks every new maximum comes with its block's neighbours
+// (whole call, 16 x 20,000 x 200,000: 95.5 ms with a third of the SNPs, 71.0 with
+// two thirds, 52.8 with all; independent SNPs, 100,000: 32.4, 31.0, 31.2).  The
+// general form's is over the first kSeedSnps SNPs, so that its main launch starts from
+// running minima over thousands of SNPs instead of none (without it the first wave
+// of CTAs refines nearly every chunk in FP64).  False when the call is too small to
+// gain from one.
 bool make_seed_plan(const CallPlan &cp, CallPlan &seed, bool plain_form) {
   constexpr int64_t kSeedSnps = 16384;
   if (cp.groups.size() != 1) return false;
   const int64_t n = cp.groups[0].n_snps;
-  // the plain form decides every pair past its bounds exactly, so its seed covers a
-  // third of the SNPs (whole chunks; a quarter took 4 % longer over 200,000 SNPs at
-  // P = 16, a sixth 7 %): few later pairs per class then beat the seed's best.  It
-  // needs one at any size: from zero bounds nearly every pair of its first chunks
-  // would go to the event warps (a 20,000-SNP batch took 83 ms without one)
-  if (plain_form ? n < 16 * kChunkSnps : n <= 4 * kSeedSnps) return false;
+  if (!plain_form && n <= 4 * kSeedSnps) return false;
   seed = cp;
-  seed.groups[0].n_snps =
-      plain_form ? std::max<int64_t>(4 * kChunkSnps, n / 3 / kChunkSnps * kChunkSnps) : kSeedSnps;
+  seed.groups[0].n_snps = plain_form ? n : kSeedSnps;
   seed.slots[0].capacity = 0;
   seed.fdr_hist = nullptr;
   seed.perm.seed = true;
@@ -2383,6 +2459,7 @@ extern "C" krux_status krux_permute(krux_ctx *ctx, const krux_rankset *rs, const
     if (st != KRUX_OK) return st;
     if (ctx->profiling) ctx->prof.launches += fused_launches(seed, fs);
     cp.perm.pre_done = true;
+    cp.perm.packed = seed.groups[0].n_snps == cp.groups[0].n_snps;
   }
   st = enqueue_fused(ctx, cp, fm, s);
   if (st != KRUX_OK) return st;
@@ -2468,6 +2545,7 @@ krux_status graph_capture(krux_ctx *ctx, krux_graph *g) {
     if (st != KRUX_OK) return st;
     KRUX_CUDA(w, scan_set_smem(std::max(g->seed_fl.smem, g->fl.smem)));
     g->cp.perm.pre_done = true;
+    g->cp.perm.packed = g->seed_cp.groups[0].n_snps == g->cp.groups[0].n_snps;
   }
   const int nslots = g->fl.nslots;
   KRUX_CUDA(w, cudaHostAlloc(reinterpret_cast<void **>(&g->host), (size_t)(nslots + 1) * 8,
@@ -2767,7 +2845,7 @@ extern "C" krux_status krux_debug_plan(int N, int with_nan, int layout, int nc, 
   if (plain && lay != 1) return KRUX_EUNSUPPORTED;
   const int codes_k = with_nan == 1 ? Np : (with_nan == 3 ? kCoefNanRows : 0);
   LaunchShape sh;
-  if (!pick_launch_shape(&tmp, kpad, codes_k, sh, plain ? kEvRegion : 0)) return KRUX_EUNSUPPORTED;
+  if (!pick_launch_shape(&tmp, kpad, codes_k, sh, plain ? plain_extra(false) : 0)) return KRUX_EUNSUPPORTED;
   GroupDesc d;
   std::memset(&d, 0, sizeof d);
   d.Np = Np;
@@ -2786,7 +2864,7 @@ extern "C" krux_status krux_debug_plan(int N, int with_nan, int layout, int nc, 
   p.b_region = sh.b_region;
   p.layout = lay;
   const size_t smem = scan_smem_bytes2(p.nc, p.nA, (size_t)p.a_tile_bytes, (size_t)p.b_region, p.kpad) +
-                     (plain ? kEvRegion : 0);
+                     (plain ? plain_extra(false) : 0);
   out[0] = sh.ka;
   out[1] = sh.nA;
   out[2] = sh.b_region;

@@ -34,7 +34,7 @@ constexpr int kFastEpiWarps = 4 * (2 * kChunkSnps / kFastSnps);  // 16
 constexpr int kFastThreads = 32 * (kFastEpiWarps + 4);
 // the register file is split among the 4 schedulers: at most 16384 per scheduler
 constexpr int kFastRegsLaunch = (16384 / (32 * (kFastThreads / 128))) / 8 * 8;
-constexpr int kFastRegsLow = 56;
+constexpr int kFastRegsLow = 64;
 constexpr int kFastRegsHigh =
     (kFastRegsLaunch + 4 * (kFastRegsLaunch - kFastRegsLow) / kFastEpiWarps) / 8 * 8;
 static_assert(kFastEpiWarps == 16, "16 epilogue warps in the plain scan form");
@@ -63,7 +63,8 @@ struct MinpPair {
 static_assert(sizeof(MinpPair) == 24, "MinpPair is 24 bytes");
 
 struct EvEntry {
-  float u[kEvSnps], v[kEvSnps];                 // D_0, D_1 of SNP j for this trait
+  float u[kEvSnps], v[kEvSnps];                 // accumulators P, Q of SNP j for this trait
+  uint32_t pq0[kEvSnps], pq1[kEvSnps];          // the SNPs' weights (ChunkMeta), for D_0, D_1
   float alpha[kEvSnps], beta[kEvSnps], gamma[kEvSnps];  // the SNPs' fast-test coefficients
   int32_t snp[kEvSnps];                         // output SNP index
   uint32_t n01[kEvSnps];                        // N_0 | N_1 << 16
@@ -89,13 +90,24 @@ constexpr size_t kEvRegion = 128 + kEvEntries * sizeof(EvEntry) + kEvEntries * 8
 // two-sided plain form stages instead the classes' decided values with their pair
 // identities, u64 [128][2] @1536 (it has no NaN).
 constexpr int kTcDepth = 4;
+constexpr int kItemDepth = 4;  // work items the producer may announce ahead
 constexpr int kTcBytes = 3584;
+// The plain form and its NaN variant have no keys: tau @0, 3/(K(K+1)C) @512, NaN
+// count @1536, in half the bytes (room for the NaN variant's coefficient sets beside
+// four resident chunks at N = 102).  Their launches hold this much less.
+constexpr int kTcLean = 1792;
+constexpr size_t kTcSaved = (size_t)kTcDepth * (kTcBytes - kTcLean);
 
-// ---- per-chunk SNP metadata (one 1536-byte blob per chunk of 64 SNPs) ------
+// ---- per-chunk SNP metadata (one 2304-byte blob per chunk of 64 SNPs) ------
 // Fast-test coefficients: with u = D_0, v = D_1 (D_2 = -u - v) the statistic's
 // quadratic form sum_i D_i^2 / N_i equals alpha (u + beta v)^2 + gamma v^2; alpha
 // and gamma are pre-divided by the chi-square threshold h_df of the SNP's df so
 // that one per-trait bound decides the test.
+//
+// The plain forms contract weighted indicator rows instead of 0/1 ones (PqCoef
+// below), so that the accumulators are the two terms of that form, P and Q, and
+// the test is P^2 + Q^2 >= bound: no coefficient is read and two instead of five
+// FP32 operations are left per pair.
 struct ChunkMeta {
   float alpha[kChunkSnps];      // (r0 + r2) / h_df
   float beta[kChunkSnps];       // r2 / (r0 + r2)
@@ -104,8 +116,31 @@ struct ChunkMeta {
   uint16_t n[3][kChunkSnps];    // genotype group sizes over non-missing samples
   uint8_t df[kChunkSnps];       // non-empty groups - 1
   uint8_t pad_[64];
+  uint32_t pq0[kChunkSnps];     // plain forms: A0 | A1 << 16 (FP16 bits)
+  uint32_t pq1[kChunkSnps];     // G (FP16 bits) | code of group a << 16 | code of group b << 18
+  float sgn[kChunkSnps];        // permutation batches: -1 for a df-1 SNP, else 1
 };
-static_assert(sizeof(ChunkMeta) == 1536, "ChunkMeta must be 1536 bytes");
+static_assert(sizeof(ChunkMeta) == 2304, "ChunkMeta must be 2304 bytes");
+
+// Weighted indicator rows of the plain forms.  With the SNP's largest group L left
+// out (D_L = -D_a - D_b) and b the smaller of the other two,
+//   sum_i D_i^2 / N_i / h_df = alpha (D_a + beta D_b)^2 + gamma D_b^2,
+// and the packed rows hold A0 where the genotype is a and A1 where it is b (row P),
+// G where it is b (row Q), so that the contraction gives P = A0 D_a + A1 D_b and
+// Q = G D_b.  The weights are rounded to `bits` significant bits, A0 and G upwards
+// and with A1 on A0's grid, such that P^2 + Q^2 is never below the form and above
+// it by about 6 * 2^-bits at most (0.3 % at N <= 128): what passes the test is
+// decided on the exact sums afterwards.  `bits` keeps every partial sum of weighted
+// centred ranks an integer multiple, below 2^23, of the weights' last place (at
+// most K^2 / 4 times 2^bits), so the FP32 accumulators are exact and D_a, D_b
+// come back from P and Q without error.
+__host__ __device__ inline int pq_bits(int N) {
+  int64_t m = ((int64_t)N * N + 3) / 4;
+  int b = 0;
+  while (((int64_t)1 << b) < m) ++b;
+  const int bits = 23 - b;
+  return bits > 11 ? 11 : bits;
+}
 
 // ---- markers with up to five genotype groups (section "Input data": values
 // 0..l, any number of alleles, also varying between markers) ------------------
@@ -120,7 +155,7 @@ struct ChunkMetaM {               // the same shared-memory slot as ChunkMeta
   int32_t snp[kChunkSnpsM];                  // output SNP index, -1 = padding / left out
   uint16_t n[kMaxCodeM + 1][kChunkSnpsM];    // group sizes over non-missing samples
   uint8_t df[kChunkSnpsM];                   // non-empty groups - 1
-  uint8_t pad_[1536 - 640 - 128 - 320 - 32];
+  uint8_t pad_[2304 - 640 - 128 - 320 - 32];
 };
 static_assert(sizeof(ChunkMetaM) == sizeof(ChunkMeta), "ChunkMetaM must fill a ChunkMeta slot");
 
@@ -201,6 +236,7 @@ struct RerankJob {
 // halves [half0, half0 + 2 * nchunks) of the flattened launch.
 struct PackJob {
   const int8_t *geno;
+  const int8_t *geno_lo, *geno_hi;  // first byte and end of the rows the call may read
   int64_t ldg;
   const int64_t *snp_list;  // device rows, or null for [snp_begin, snp_begin + n_snps)
   int64_t snp_begin, n_snps;
@@ -211,6 +247,8 @@ struct PackJob {
   int32_t N, Np, allow_missing;
   int32_t coef_nan;         // 1: codes holds the plain form's coefficient blocks (kCoefNanBytes
                             // per chunk) instead of 2-bit codes
+  int32_t pq_bits;          // > 0: weighted rows of the plain forms (their significant bits);
+                            // 0: 0/1 indicators of groups 0 and 1
 };
 
 // ---- one group of a scan launch (a cohort, a missing-pattern bucket, or the
@@ -256,8 +294,8 @@ struct alignas(64) GroupDesc {
 
 // The plain form's hot-test coefficients for traits with NaN samples, one block
 // per chunk (in place of the 2-bit codes): set s serves traits with up to
-// kNanSetC[s] NaN samples, the same alpha (u + beta v)^2 + gamma v^2 form as
-// ChunkMeta's first three arrays, built from group sizes max(N_i - C, 1) and the
+// kNanSetC[s] NaN samples, the same quadratic form as ChunkMeta's first three arrays
+// but on the accumulators, alpha (P + beta Q)^2 + gamma Q^2, built from group sizes max(N_i - C, 1) and the
 // threshold of the smallest df the pair can keep, so that it bounds
 // sum_i D_i^2 / N_i' / h_df' from above whatever genotypes the NaN samples carry
 // (section "Handling missing values": N_i' counts the samples present for both).
@@ -296,6 +334,8 @@ struct WorkItem {
 struct ScanParams {
   const GroupDesc *groups;
   const WorkItem *items;
+  unsigned int *next;       // items taken beyond one per CTA (zero at launch), or null: CTA b
+                            // takes items b, b + grid, b + 2 grid, ...
   int32_t n_items;
   int32_t nc;               // most chunks any group keeps resident (<= kTmemSlots)
   int32_t nA;               // A pipeline stages
@@ -429,6 +469,8 @@ cudaError_t launch_finalize_dev(const krux_hit *hits, const HitAux *aux, const H
                                 int fdr_bins, double fdr_l0, double fdr_w, double pthresh);
 cudaError_t scan_set_smem(size_t smem);
 int scan_form_of(const ScanParams &p);
+// The plain-form kernels were built with the registers their warp split assumes.
+bool fast_form_ok();
 cudaError_t launch_scan_only(const ScanParams &p, int grid, size_t smem, cudaStream_t s);
 cudaError_t launch_finalize(const krux_hit *hits, const HitAux *aux, int64_t n,
                             const double *const *cfac_by_group, double *H, double *p,

@@ -326,32 +326,81 @@ __device__ __forceinline__ void write_meta(ChunkMeta &m, int jj, int n0, int n1,
   m.df[jj] = (uint8_t)df;
 }
 
-// The plain form's coefficient sets of SNP slot jj for traits with NaN samples:
-// set s takes write_meta's alpha, beta, gamma from group sizes max(N_i - C, 1),
-// C = nan_set_c(s) (an empty group stays empty), with the threshold of the
-// smallest df the pair can keep (1/h_1 when some group may vanish).  For a trait
-// with c <= C NaN samples they bound the pair's exact sum_i D_i^2 / N_i' / h_df'
-// from above, whichever groups the NaN samples fall in.
-__device__ __forceinline__ void write_coef_nan(void *block, int jj, int n0, int n1, int n2,
-                                               bool excluded, float rh1, float rh2) {
+// Weights of one SNP's packed rows in the plain forms (see ChunkMeta), and the
+// group order they stand for.
+struct PqCoef {
+  uint32_t w0, w1;          // ChunkMeta's pq0, pq1
+  float a0, a1, g;          // the weights as FP32
+  int na, nb, nl;           // sizes of groups a, b and of the group left out
+};
+// x > 0 rounded up / to nearest at `bits` significant bits (exponent of x)
+__device__ __forceinline__ float round_up_bits(float x, int bits) {
+  const uint32_t m = (1u << (24 - bits)) - 1u;
+  return __uint_as_float((__float_as_uint(x) + m) & ~m);
+}
+__device__ __forceinline__ PqCoef pq_coef(int n0, int n1, int n2, bool excluded, float rh1,
+                                          float rh2, int bits) {
+  PqCoef c;
+  c.w0 = 0u;
+  c.w1 = 1u << 18;  // a = 0, b = 1
+  c.a0 = c.a1 = c.g = 0.f;
+  // L: a largest group; b: a smallest one; a: the third
+  const int n[3] = {n0, n1, n2};
+  const int L = n0 >= n1 && n0 >= n2 ? 0 : (n1 >= n2 ? 1 : 2);
+  const int x = L == 0 ? 1 : 0, y = L == 2 ? 1 : 2;
+  const int nx = x == 0 ? n[0] : n[1], ny = y == 1 ? n[1] : n[2];
+  const int b = nx <= ny ? x : y, a = nx <= ny ? y : x;
+  c.nb = min(nx, ny);
+  c.na = max(nx, ny);
+  c.nl = max(n0, max(n1, n2));
   const int groups = (n0 > 0) + (n1 > 0) + (n2 > 0);
+  if (groups < 2 || excluded) return c;
+  // (a two-group SNP has b empty and D_b = 0: its a and L carry the form)
+  const float rh = groups == 2 ? rh1 : rh2;
+  const float qa = 1.f / (float)c.na, qb = c.nb > 0 ? 1.f / (float)c.nb : 0.f, ql = 1.f / (float)c.nl;
+  const float s = qa + ql;
+  const float alpha = s * rh, beta = ql / s;
+  const float step = exp2f((float)-bits);
+  // A0^2 >= alpha (1 + step), A1 = A0 (beta + d) with |d| <= 2^-bits: the largest of
+  // alpha w^2 - A0^2 (w + d v)^2 over w is alpha d^2 (1 + 1/eta) v^2, eta = A0^2 / alpha
+  // - 1 >= step; G^2 takes that on top of gamma (1e-5: FP32 rounding of all this)
+  c.a0 = round_up_bits(sqrtf(alpha * (1.f + step)) * 1.00001f, bits);
+  const uint32_t e = (__float_as_uint(c.a0) >> 23) & 255u;
+  const float ulp = __uint_as_float((e - (uint32_t)(bits - 1)) << 23);  // A0's last place
+  c.a1 = rintf(c.a0 * beta / ulp) * ulp;
+  const float d = fabsf(c.a1 / c.a0 - beta) + 1e-6f;
+  const float gamma = (qb + ql * qa / s) * rh;
+  c.g = round_up_bits(sqrtf(gamma + alpha * d * d * (1.f + 1.f / step)) * 1.00001f, bits);
+  c.w0 = (uint32_t)__half_as_ushort(__float2half_rn(c.a0)) |
+         ((uint32_t)__half_as_ushort(__float2half_rn(c.a1)) << 16);
+  c.w1 = (uint32_t)__half_as_ushort(__float2half_rn(c.g)) | ((uint32_t)a << 16) | ((uint32_t)b << 18);
+  return c;
+}
+
+// The plain form's coefficient sets of SNP slot jj for traits with NaN samples:
+// set s takes the quadratic form from group sizes max(N_i - C, 1), C = nan_set_c(s)
+// (an empty group stays empty), with the threshold of the smallest df the pair can
+// keep (1/h_1 when some group may vanish).  For a trait with c <= C NaN samples it
+// bounds the pair's exact sum_i D_i^2 / N_i' / h_df' from above, whichever groups the
+// NaN samples fall in.  It is written on the accumulators: D_b = Q / G and D_a =
+// (P - A1 D_b) / A0 turn alpha (D_a + beta D_b)^2 + gamma D_b^2 into
+// alpha / A0^2 (P + (beta A0 - A1) / G Q)^2 + gamma / G^2 Q^2.
+__device__ __forceinline__ void write_coef_nan(void *block, int jj, const PqCoef &w, float rh1,
+                                               float rh2) {
 #pragma unroll
   for (int si = 0; si < kNanSets; ++si) {
     const int c = nan_set_c(si);
     float al = 0.f, be = 0.f, ga = 0.f;
-    if (groups > 1 && !excluded) {
-      const int sure = (n0 > c) + (n1 > c) + (n2 > c);  // groups no c NaN samples can empty
+    if (w.a0 > 0.f) {  // two groups or more: groups a and L are not empty
+      const int sure = (w.na > c) + (w.nb > c) + (w.nl > c);  // groups no c NaN samples can empty
       const float rh = sure >= 3 ? rh2 : rh1;
-      const float q0 = n0 ? 1.f / (float)max(n0 - c, 1) : 0.f, q1 = n1 ? 1.f / (float)max(n1 - c, 1) : 0.f,
-                  q2 = n2 ? 1.f / (float)max(n2 - c, 1) : 0.f;
-      const float a = q0 + q2;
-      if (a > 0.f) {
-        al = a * rh;
-        be = q2 / a;
-        ga = (q1 + q2 * q0 / a) * rh;
-      } else {
-        ga = q1 * rh;  // groups 0 and 2 empty (cannot happen with two groups or more)
-      }
+      const float qa = 1.f / (float)max(w.na - c, 1),
+                  qb = w.nb ? 1.f / (float)max(w.nb - c, 1) : 0.f,
+                  ql = 1.f / (float)max(w.nl - c, 1);
+      const float a = qa + ql;
+      al = a * rh / (w.a0 * w.a0);
+      be = (ql / a * w.a0 - w.a1) / w.g;
+      ga = (qb + ql * qa / a) * rh / (w.g * w.g);
     }
     CoefSet *cs = coef_set(block, si);
     cs->alpha[jj] = al;
@@ -450,192 +499,176 @@ __device__ __forceinline__ int find_job(const PackJob *__restrict__ jobs, int n_
   return lo;
 }
 
-// Staged packing of 32 consecutive genotype rows of at most kStageLd bytes each
-// (no SNP list): the warp copies the rows' byte span into shared memory with
-// 16-byte loads, writes both indicator blocks (32 rows of I_0, then 32 of I_1, each
-// contiguous) with 16-byte stores, and lane i counts the groups of row i.
-constexpr int kStageLd = 128;
-constexpr int kStageBytes = 32 * kStageLd + 32;
-
-// Four codes starting at byte offset o of the staged span (any alignment).
+// Four codes starting at byte offset o of the staged rows (any alignment).
 __device__ __forceinline__ uint32_t stage_word(const uint8_t *st, int o) {
   const uint32_t *w = reinterpret_cast<const uint32_t *>(st + (o & ~3));
   return __funnelshift_r(w[0], w[1], 8 * (o & 3));
 }
-// Bytes 0..3 of a 0x00 / 0xff byte mask as two FP16 pairs (1.0 where 0xff).
-__device__ __forceinline__ uint2 mask_to_halves(uint32_t m) {
-  return make_uint2(__byte_perm(m, 0u, 0x1100) & 0x3c003c00u, __byte_perm(m, 0u, 0x3322) & 0x3c003c00u);
+// Bytes 0..3 of a 0x00 / 0xff byte mask as two FP16 pairs holding the pair v where set.
+__device__ __forceinline__ uint2 mask_to_halves(uint32_t m, uint32_t v) {
+  return make_uint2(__byte_perm(m, 0u, 0x1100) & v, __byte_perm(m, 0u, 0x3322) & v);
 }
 
-__device__ __forceinline__ void pack_staged(const PackJob &J, int64_t j0, uint8_t *st, int lane,
-                                            int &my_n0, int &my_n1, int &my_n2, bool &my_miss,
-                                            bool &any_bad, int64_t &my_s) {
-  const int N = J.N, Np = J.Np;
-  const int64_t ldg = J.ldg;
-  const int64_t left = J.n_snps - j0;
-  const int rows = left < 32 ? (int)left : 32;
-  const uint8_t *src = reinterpret_cast<const uint8_t *>(J.geno + (J.snp_begin + j0) * ldg);
-  // the span [src, src + L) in shared memory at offset pad + b, so that 16-byte
-  // aligned global chunks land on 16-byte aligned shared addresses
-  const int64_t L = (int64_t)(rows - 1) * ldg + N;
-  const int pad = (int)((uintptr_t)src & 15u);
-  const int head = (16 - pad) & 15;
-  const int64_t mid = L > head ? (L - head) / 16 : 0;
-  const int64_t hl = (int64_t)head < L ? (int64_t)head : L;
-  for (int64_t b = lane; b < hl; b += 32) st[pad + b] = src[b];
-  for (int64_t c = lane; c < mid; c += 32)
-    *reinterpret_cast<uint4 *>(st + pad + head + 16 * c) =
-        *reinterpret_cast<const uint4 *>(src + head + 16 * c);
-  for (int64_t b = head + 16 * mid + lane; b < L; b += 32) st[pad + b] = src[b];
-  __syncwarp();
-  // both indicator blocks: item t = row r, samples 8q .. 8q + 7
-  const int c = (int)(j0 / kChunkSnps), jj0 = (int)(j0 % kChunkSnps);
-  const int per_row = Np / 8;
-  uint4 *d0 = reinterpret_cast<uint4 *>(J.B + ((int64_t)c * kChunkRows + jj0) * Np);
-  uint4 *d1 = reinterpret_cast<uint4 *>(J.B + ((int64_t)c * kChunkRows + kChunkSnps + jj0) * Np);
-  for (int t = lane; t < 32 * per_row; t += 32) {
-    const int r = t / per_row, k8 = 8 * (t - r * per_row);
-    uint32_t lo = 0x03030303u, hi = 0x03030303u;  // 3: neither group 0 nor 1
-    if (r < rows) {
-      const int o = pad + (int)(r * ldg) + k8;
-      lo = stage_word(st, o);
-      hi = stage_word(st, o + 4);
-      // samples at or beyond N are padding
-      const int vl = min(max(N - k8, 0), 4), vh = min(max(N - k8 - 4, 0), 4);
-      const uint32_t ml = vl >= 4 ? 0xffffffffu : (1u << (8 * vl)) - 1u;
-      const uint32_t mh = vh >= 4 ? 0xffffffffu : (1u << (8 * vh)) - 1u;
-      lo = (lo & ml) | (0x03030303u & ~ml);
-      hi = (hi & mh) | (0x03030303u & ~mh);
-    }
-    const uint2 a = mask_to_halves(__vcmpeq4(lo, 0u)), b = mask_to_halves(__vcmpeq4(hi, 0u));
-    const uint2 e = mask_to_halves(__vcmpeq4(lo, 0x01010101u)),
-                f = mask_to_halves(__vcmpeq4(hi, 0x01010101u));
-    d0[t] = make_uint4(a.x, a.y, b.x, b.y);
-    d1[t] = make_uint4(e.x, e.y, f.x, f.y);
+// Shared-memory bytes of one warp's staged rows: a row of N codes takes
+// (N + 30) / 16 * 16 bytes (16-byte granules around it, wherever it starts), and a
+// batch holds 32, 16 or 8 rows.
+constexpr int kStageBytes = 8 * ((kMaxN + 30) / 16 * 16);
+static_assert(kStageBytes >= 32 * 128 && kStageBytes >= 16 * 256, "8, 16 and 32 rows fit");
+
+// 16 bytes at p (aligned) into shared memory; only bytes in [lo, hi) may be read.
+__device__ __forceinline__ void stage_granule(uint8_t *d, const int8_t *p, const int8_t *lo,
+                                              const int8_t *hi) {
+  if (p >= lo && p + 16 <= hi) {
+    *reinterpret_cast<uint4 *>(d) = *reinterpret_cast<const uint4 *>(p);
+  } else {  // it crosses the matrix's first or last byte
+    for (int b = 0; b < 16; ++b)
+      if (p + b >= lo && p + b < hi) d[b] = (uint8_t)p[b];
   }
-  // lane i: the group sizes, missing and invalid codes of row i
-  if (lane < rows) {
-    int n0 = 0, n1 = 0, n2 = 0, nm = 0;
-    const int o0 = pad + (int)(lane * ldg);
-    for (int k = 0; k < N; k += 4) {
-      uint32_t w = stage_word(st, o0 + k);
-      const int v = min(N - k, 4);
-      const uint32_t m = v >= 4 ? 0xffffffffu : (1u << (8 * v)) - 1u;
-      w = (w & m) | (0x04040404u & ~m);  // 4: outside every class below
-      n0 += __popc(__vcmpeq4(w, 0u)) >> 3;
-      n1 += __popc(__vcmpeq4(w, 0x01010101u)) >> 3;
-      n2 += __popc(__vcmpeq4(w, 0x02020202u)) >> 3;
-      nm += __popc(__vcmpeq4(w, 0xffffffffu)) >> 3;
-    }
-    my_n0 = n0;
-    my_n1 = n1;
-    my_n2 = n2;
-    my_miss = nm > 0;
-    any_bad = n0 + n1 + n2 + nm != N;
-    my_s = J.snp_begin + j0 + lane;
-  }
-  __syncwarp();
 }
 
 // All SNP sets of a call in one launch (rank-sum form): one warp per 32 flattened
-// slots (half a chunk; every job spans whole chunks).  Lane t writes samples
-// 4t .. 4t + 3 (+ 128 per pass) of both indicator rows of each slot with 8-byte
-// stores, the group sizes come from warp reductions, and lane i then writes the
-// metadata of slot i, so no lane does the per-SNP scalar work alone.
+// slots (half a chunk; every job spans whole chunks).  The warp stages batches of
+// genotype rows in shared memory with 16-byte loads (any row order, alignment and
+// leading dimension), counts the groups of each row (32 / batch lanes per row),
+// derives the rows' weights (ChunkMeta: 0/1 indicators or the plain forms' P and Q
+// rows), and writes both packed rows with 16-byte stores.  Bound by the stores (4 Np
+// bytes per SNP against N read): one pass over the genotypes per SNP, so the group
+// sizes are known before the rows that are scaled by them are written.
 __global__ void __launch_bounds__(kPackWarps * 32)
 pack_batch_kernel(const PackJob *__restrict__ jobs, int n_jobs, int64_t total_slots, float rh1,
                   float rh2, int signed_df1, unsigned int *status) {
-  __shared__ __align__(16) uint8_t stage[kPackWarps][kStageBytes];
+  __shared__ __align__(16) uint8_t stage[kPackWarps][kStageBytes + 32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t x0 = ((int64_t)blockIdx.x * kPackWarps + warp) * 32;
   if (x0 >= total_slots) return;
   const PackJob &J = jobs[find_job(jobs, n_jobs, x0, false)];
   const int64_t j0 = x0 - J.slot0;  // a multiple of 32
-  const int N = J.N, Np = J.Np;
-  if (!J.snp_list && J.ldg <= kStageLd && Np <= kStageLd && j0 < J.n_snps) {
-    int n0 = 0, n1 = 0, n2 = 0;
-    bool miss = false, bad = false;
-    int64_t sn = -1;
-    pack_staged(J, j0, stage[warp], lane, n0, n1, n2, miss, bad, sn);
-    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(status, kDevBadCode);
-    const bool excl = miss && !J.allow_missing;
-    if (__any_sync(0xffffffffu, excl) && lane == 0) atomicOr(status, kDevMissing);
-    ChunkMeta &m = J.meta[j0 / kChunkSnps];
-    const int jj = (int)(j0 % kChunkSnps) + lane;
-    if (sn < 0) write_meta(m, jj, 0, 0, 0, true, 0, rh1, rh2, signed_df1, 0, 0.f);
-    else write_meta(m, jj, n0, n1, n2, excl, sn, rh1, rh2, signed_df1, 0, 0.f);
-    if (J.coef_nan)
-      write_coef_nan(reinterpret_cast<uint8_t *>(J.codes) + (j0 / kChunkSnps) * kCoefNanBytes, jj, sn < 0 ? 0 : n0,
-                     sn < 0 ? 0 : n1, sn < 0 ? 0 : n2, sn < 0 || excl, rh1, rh2);
-    return;
-  }
+  const int N = J.N, Np = J.Np, bits = J.pq_bits;
+  const int64_t ldg = J.ldg;
+  const int8_t *__restrict__ geno = J.geno;
+  const int8_t *lo_end = J.geno_lo, *hi_end = J.geno_hi;
+  uint8_t *st = stage[warp];
+  const int pitch = (N + 30) / 16 * 16, cpr = pitch / 16;
+  const int lgr = pitch <= 128 ? 5 : (pitch <= 256 ? 4 : 3);
+  const int R = 1 << lgr, L = 32 >> lgr;  // rows per batch, lanes per row
+  const int per_row = Np / 8;
+  // t / per_row and t / cpr for t < 1024 as multiplications (divisors up to 66)
+  const uint32_t inv_row = (65536u + (uint32_t)per_row - 1u) / (uint32_t)per_row;
+  const uint32_t inv_cpr = (65536u + (uint32_t)cpr - 1u) / (uint32_t)cpr;
+  // consecutive rows are staged as the one span they form, others row by row
+  const bool span = J.snp_list == nullptr && (int64_t)R * ldg + 32 <= kStageBytes;
   const int64_t c = j0 / kChunkSnps;
   const int jj0 = (int)(j0 % kChunkSnps);
-  const uint32_t one2 = 0x3c003c00u;  // two FP16 ones
-  // the job's arrays through restrict pointers: the genotype reads of a slot may
-  // then be issued before the previous slot's stores
-  const int8_t *__restrict__ geno = J.geno;
-  const int64_t *__restrict__ snp_list = J.snp_list;
-  __half *__restrict__ Bj = J.B;
-  const int64_t ldg = J.ldg, n_snps = J.n_snps, snp_begin = J.snp_begin;
-  int my_n0 = 0, my_n1 = 0, my_n2 = 0;
-  bool my_miss = false, any_bad = false;
-  int64_t my_s = 0;
-#pragma unroll 2
-  for (int i = 0; i < 32; ++i) {
-    const int64_t j = j0 + i;
-    const bool valid = j < n_snps;
-    const int64_t s = valid ? (snp_list ? snp_list[j] : snp_begin + j) : 0;
-    const int8_t *g = geno + s * ldg;
-    __half *r0 = Bj + (c * kChunkRows + jj0 + i) * Np;
-    __half *r1 = Bj + (c * kChunkRows + kChunkSnps + jj0 + i) * Np;
-    int n0 = 0, n1 = 0, n2 = 0;
-    bool miss = false, bad = false;
-    for (int k0 = 4 * lane; k0 < Np; k0 += 128) {
-      uint32_t h0[2] = {0u, 0u}, h1[2] = {0u, 0u};
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int k = k0 + q;
-        const int code = (valid && k < N) ? (int)g[k] : -1;
-        const uint32_t bit = (q & 1) ? 0xffff0000u : 0x0000ffffu;
-        if (code == 0) h0[q >> 1] |= one2 & bit;
-        if (code == 1) h1[q >> 1] |= one2 & bit;
-        n0 += code == 0;
-        n1 += code == 1;
-        n2 += code == 2;
-        if (valid && k < N) {
-          miss |= code == -1;
-          bad |= (code < -1 || code > 2);
+  ChunkMeta &m = J.meta[c];
+  __half *B0 = J.B + (c * kChunkRows + jj0) * Np;
+  bool any_bad = false, any_excl = false;
+  // lane i: the genotype row of slot i (-1: padding of the last chunk)
+  int64_t my_row = -1;
+  if (j0 + lane < J.n_snps) my_row = J.snp_list ? J.snp_list[j0 + lane] : J.snp_begin + j0 + lane;
+  for (int r0 = 0; r0 < 32; r0 += R) {
+    const int64_t row0 = __shfl_sync(0xffffffffu, my_row, r0);
+    if (span) {
+      if (row0 >= 0) {
+        const int64_t last = min((int64_t)R, J.n_snps - j0 - r0) - 1;
+        const int8_t *src = geno + row0 * ldg;
+        const int pad = (int)((uintptr_t)src & 15u);
+        const int len = pad + (int)(last * ldg) + N;
+        for (int o = 16 * lane; o < len; o += 512) stage_granule(st + o, src - pad + o, lo_end, hi_end);
+      }
+    } else {
+      for (int t0 = 0; t0 < R * cpr; t0 += 32) {
+        const int t = t0 + lane;
+        const int r = (int)(((uint32_t)t * inv_cpr) >> 16), q = t - r * cpr;
+        const int64_t row = __shfl_sync(0xffffffffu, my_row, (r0 + r) & 31);
+        if (t < R * cpr && row >= 0) {
+          const int8_t *src = geno + row * ldg;
+          const int pad = (int)((uintptr_t)src & 15u);
+          if (16 * q < pad + N)
+            stage_granule(st + r * pitch + 16 * q, src - pad + 16 * q, lo_end, hi_end);
         }
       }
-      *reinterpret_cast<uint2 *>(r0 + k0) = make_uint2(h0[0], h0[1]);
-      *reinterpret_cast<uint2 *>(r1 + k0) = make_uint2(h1[0], h1[1]);
     }
-    n0 = (int)__reduce_add_sync(0xffffffffu, (unsigned)n0);
-    n1 = (int)__reduce_add_sync(0xffffffffu, (unsigned)n1);
-    n2 = (int)__reduce_add_sync(0xffffffffu, (unsigned)n2);
-    miss = __any_sync(0xffffffffu, miss);
-    any_bad |= bad;
-    if (lane == i) {
-      my_n0 = valid ? n0 : 0;
-      my_n1 = valid ? n1 : 0;
-      my_n2 = valid ? n2 : 0;
-      my_miss = miss;
-      my_s = valid ? s : -1;
+    __syncwarp();
+    // lanes L r .. L r + L - 1: the group sizes, missing and invalid codes of row r
+    const int mr = lane >> (5 - lgr), sub = lane & (L - 1);
+    const int64_t row = __shfl_sync(0xffffffffu, my_row, r0 + mr);
+    int n0 = 0, n1 = 0, n2 = 0, nm = 0;
+    const int o0 = row < 0 ? 0
+                   : span  ? (int)((uintptr_t)(geno + row0 * ldg) & 15u) + mr * (int)ldg
+                           : mr * pitch + (int)((uintptr_t)(geno + row * ldg) & 15u);
+    if (row >= 0) {
+      for (int k = 4 * sub; k < N; k += 4 * L) {
+        uint32_t w = stage_word(st, o0 + k);
+        const int v = min(N - k, 4);
+        const uint32_t vm = v >= 4 ? 0xffffffffu : (1u << (8 * v)) - 1u;
+        w = (w & vm) | (0x04040404u & ~vm);  // 4: outside every class below
+        n0 += __popc(__vcmpeq4(w, 0u)) >> 3;
+        n1 += __popc(__vcmpeq4(w, 0x01010101u)) >> 3;
+        n2 += __popc(__vcmpeq4(w, 0x02020202u)) >> 3;
+        nm += __popc(__vcmpeq4(w, 0xffffffffu)) >> 3;
+      }
     }
+    for (int o = 1; o < L; o <<= 1) {
+      n0 += __shfl_xor_sync(0xffffffffu, n0, o);
+      n1 += __shfl_xor_sync(0xffffffffu, n1, o);
+      n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+      nm += __shfl_xor_sync(0xffffffffu, nm, o);
+    }
+    const bool excl = row >= 0 && nm > 0 && !J.allow_missing;
+    any_bad |= row >= 0 && n0 + n1 + n2 + nm != N;
+    any_excl |= excl;
+    PqCoef w;
+    w.w0 = 0x3c00u;  // 0/1 indicators of groups 0 and 1
+    w.w1 = 0x3c00u | (1u << 18);
+    if (bits > 0) w = pq_coef(n0, n1, n2, row < 0 || excl, rh1, rh2, bits);
+    if (sub == 0) {
+      const int jj = jj0 + r0 + mr;
+      write_meta(m, jj, n0, n1, n2, row < 0 || excl, row < 0 ? 0 : row, rh1, rh2, signed_df1, 0,
+                 0.f);
+      if (bits > 0) {
+        m.pq0[jj] = w.w0;
+        m.pq1[jj] = w.w1;
+        m.sgn[jj] = signed_df1 && (n0 > 0) + (n1 > 0) + (n2 > 0) == 2 ? -1.f : 1.f;
+        if (J.coef_nan)
+          write_coef_nan(reinterpret_cast<uint8_t *>(J.codes) + c * kCoefNanBytes, jj, w, rh1, rh2);
+      }
+    }
+    // both packed rows: item t = row r, samples 8q .. 8q + 7
+    uint4 *d0 = reinterpret_cast<uint4 *>(B0 + (int64_t)r0 * Np);
+    uint4 *d1 = reinterpret_cast<uint4 *>(B0 + (int64_t)(kChunkSnps + r0) * Np);
+    for (int t0 = 0; t0 < R * per_row; t0 += 32) {
+      const int t = t0 + lane;
+      const int r = (int)(((uint32_t)t * inv_row) >> 16), k8 = 8 * (t - r * per_row);
+      const int ln = (r << (5 - lgr)) & 31;
+      const uint32_t w0 = __shfl_sync(0xffffffffu, w.w0, ln), w1 = __shfl_sync(0xffffffffu, w.w1, ln);
+      const int ob = __shfl_sync(0xffffffffu, row >= 0 ? o0 : -1, ln);
+      if (t >= R * per_row) continue;
+      uint32_t lo = 0x03030303u, hi = 0x03030303u;  // 3: in no group
+      if (ob >= 0) {
+        lo = stage_word(st, ob + k8);
+        hi = stage_word(st, ob + k8 + 4);
+        // samples at or beyond N are padding
+        const int vl = min(max(N - k8, 0), 4), vh = min(max(N - k8 - 4, 0), 4);
+        const uint32_t ml = vl >= 4 ? 0xffffffffu : (1u << (8 * vl)) - 1u;
+        const uint32_t mh = vh >= 4 ? 0xffffffffu : (1u << (8 * vh)) - 1u;
+        lo = (lo & ml) | (0x03030303u & ~ml);
+        hi = (hi & mh) | (0x03030303u & ~mh);
+      }
+      const uint32_t ca = ((w1 >> 16) & 3u) * 0x01010101u, cb = ((w1 >> 18) & 3u) * 0x01010101u;
+      const uint32_t va = __byte_perm(w0, 0u, 0x1010), vb = __byte_perm(w0, 0u, 0x3232),
+                     vg = __byte_perm(w1, 0u, 0x1010);
+      const uint32_t la = __vcmpeq4(lo, ca), ha = __vcmpeq4(hi, ca);
+      const uint32_t lb = __vcmpeq4(lo, cb), hb = __vcmpeq4(hi, cb);
+      const uint2 p0 = mask_to_halves(la, va), p1 = mask_to_halves(lb, vb);
+      const uint2 p2 = mask_to_halves(ha, va), p3 = mask_to_halves(hb, vb);
+      const uint2 q0 = mask_to_halves(lb, vg), q1 = mask_to_halves(hb, vg);
+      d0[t] = make_uint4(p0.x | p1.x, p0.y | p1.y, p2.x | p3.x, p2.y | p3.y);
+      d1[t] = make_uint4(q0.x, q0.y, q1.x, q1.y);
+    }
+    __syncwarp();
   }
   if (__any_sync(0xffffffffu, any_bad) && lane == 0) atomicOr(status, kDevBadCode);
-  const bool excl = my_miss && !J.allow_missing;
-  if (__any_sync(0xffffffffu, excl) && lane == 0) atomicOr(status, kDevMissing);
-  ChunkMeta &m = J.meta[c];
-  if (my_s < 0) {  // padding slot of the last chunk
-    write_meta(m, jj0 + lane, 0, 0, 0, true, 0, rh1, rh2, signed_df1, 0, 0.f);
-  } else {
-    write_meta(m, jj0 + lane, my_n0, my_n1, my_n2, excl, my_s, rh1, rh2, signed_df1, 0, 0.f);
-  }
-  if (J.coef_nan)
-    write_coef_nan(reinterpret_cast<uint8_t *>(J.codes) + c * kCoefNanBytes, jj0 + lane, my_s < 0 ? 0 : my_n0,
-                   my_s < 0 ? 0 : my_n1, my_s < 0 ? 0 : my_n2, my_s < 0 || excl, rh1, rh2);
+  if (__any_sync(0xffffffffu, any_excl) && lane == 0) atomicOr(status, kDevMissing);
 }
 
 __device__ __forceinline__ uint64_t spread_bits(uint32_t v) {

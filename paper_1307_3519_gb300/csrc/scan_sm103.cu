@@ -82,6 +82,17 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0u;
 }
+// Whether the phase of parity `parity` is complete, without waiting.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      " selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0u;
+}
 // The same with a suspend-time hint: a thread whose phase is not complete sleeps
 // (issuing nothing) until the phase completes or about `ns` nanoseconds pass.
 __device__ __forceinline__ bool mbar_try_wait_sleep(uint32_t bar, uint32_t parity, uint32_t ns) {
@@ -831,11 +842,11 @@ __device__ __forceinline__ void tmem_ld_half(uint32_t taddr, uint32_t (&u)[kFast
   tmem_ld16p(taddr + 64u, v);
 }
 
-// Hot test of kFastSnps SNPs of a chunk (from SNP `off`) for this lane's trait:
-// true when some pair may lie at or above the lower edge of the band (q >= 0),
-// two SNPs per packed instruction, w = u + beta v, q = alpha w^2 + gamma v^2 -
+// Hot test of the plain form's traits with NaN samples on NS SNPs of a chunk (from SNP
+// `off`): true when some pair may lie at or above the lower edge of the band (q >= 0),
+// two SNPs per packed instruction, w = P + beta Q, q = alpha w^2 + gamma Q^2 -
 // tau (1 - margin).  Blocks of 16 SNPs; two sign accumulators.
-// The coefficients come from three arrays of a chunk (ChunkMeta's, or a CoefSet).
+// The coefficients come from the three arrays of a CoefSet.
 template <int NS>
 __device__ __forceinline__ bool hit_fast_wc(const uint32_t (&d0)[NS], const uint32_t (&d1)[NS],
                                             const float *alpha, const float *beta,
@@ -874,86 +885,93 @@ __device__ __forceinline__ bool hit_fast_wc(const uint32_t (&d0)[NS], const uint
   }
   return (int)(acc0 & acc1) >= 0;
 }
+// Hot test of the plain forms on the accumulators P and Q of NS SNPs (weighted rows,
+// ChunkMeta): true when some P^2 + Q^2 reaches -ntlo.  Two SNPs per packed
+// instruction, two FP32 operations and half a sign accumulation per pair; no
+// coefficient is read.  With indicator rows and the coefficients of ChunkMeta the
+// same test took five operations and three shared-memory words per SNP: 3.9 ms for
+// 20,000 x 500,000 x 102 without planted effects against 2.64 ms with this one
+// (1.55 PFLOP/s of 4 N flop per pair, 1.70 with the padding of N to 112).
 template <int NS>
-__device__ __forceinline__ bool hit_fast_w(const uint32_t (&d0)[NS], const uint32_t (&d1)[NS],
-                                           const ChunkMeta &m, int off, float ntlo) {
-  return hit_fast_wc<NS>(d0, d1, m.alpha, m.beta, m.gamma, off, ntlo);
+__device__ __forceinline__ bool hit_pq(const uint32_t (&P)[NS], const uint32_t (&Q)[NS], float ntlo) {
+  const uint64_t nt2 = pk2(__float_as_uint(ntlo), __float_as_uint(ntlo));
+  uint32_t acc0 = 0xffffffffu, acc1 = 0xffffffffu;  // AND of the sign bits (two chains)
+#pragma unroll
+  for (int j = 0; j < NS; j += 4) {
+    const uint64_t q0 = pk2(Q[j], Q[j + 1]), q1 = pk2(Q[j + 2], Q[j + 3]);
+    const uint64_t p0 = pk2(P[j], P[j + 1]), p1 = pk2(P[j + 2], P[j + 3]);
+    const uint64_t s0 = ffma2(p0, p0, ffma2(q0, q0, nt2));
+    const uint64_t s1 = ffma2(p1, p1, ffma2(q1, q1, nt2));
+    uint32_t x, y;
+    upk2(s0, x, y);
+    acc0 &= x & y;
+    upk2(s1, x, y);
+    acc1 &= x & y;
+  }
+  return (int)(acc0 & acc1) >= 0;
 }
 
-// Two-sided hot test of a permutation batch, whose df-1 SNPs carry a negated form
-// value s (signed coefficients): true when some pair has s >= b2 (df 2) or
-// s <= -b1 (df 1), with nb2 = -b2 and sb = b1 + b2 (both finite); two SNPs per
-// packed instruction, as hit_fast_w.
+// The same in a permutation batch, where the two classes of SNPs have bounds of their
+// own (b1 for df 1, b2 for df 2): the bound of each SNP is selected by its sign
+// (ChunkMeta's sgn, +1 for df 2) as -(b1 + b2) / 2 + sgn (b1 - b2) / 2.
 template <int NS>
-__device__ __forceinline__ bool hit_fast_w2(const uint32_t (&d0)[NS], const uint32_t (&d1)[NS],
-                                            const ChunkMeta &m, int off, float nb2, float sb) {
-  const uint64_t nt2 = pk2(__float_as_uint(nb2), __float_as_uint(nb2));
-  const uint64_t sb2 = pk2(__float_as_uint(sb), __float_as_uint(sb));
-  uint32_t hi = 0xffffffffu, lo = 0u;  // AND of the signs of s - b2, OR of those of s + b1
+__device__ __forceinline__ bool hit_pq2(const uint32_t (&P)[NS], const uint32_t (&Q)[NS],
+                                        const float *sgn, float b1, float b2) {
+  const float mid = -0.5f * (b1 + b2), dif = 0.5f * (b1 - b2);
+  const uint64_t m2 = pk2(__float_as_uint(mid), __float_as_uint(mid));
+  const uint64_t f2 = pk2(__float_as_uint(dif), __float_as_uint(dif));
+  uint32_t acc0 = 0xffffffffu, acc1 = 0xffffffffu;
 #pragma unroll
-  for (int b = 0; b < NS / 16; ++b) {
-    const uint64_t *al = reinterpret_cast<const uint64_t *>(m.alpha + off + 16 * b);
-    const uint64_t *be = reinterpret_cast<const uint64_t *>(m.beta + off + 16 * b);
-    const uint64_t *ga = reinterpret_cast<const uint64_t *>(m.gamma + off + 16 * b);
-#pragma unroll
-    for (int j = 0; j < 8; j += 2) {
-      const ulonglong2 A = *reinterpret_cast<const ulonglong2 *>(al + j);
-      const ulonglong2 B = *reinterpret_cast<const ulonglong2 *>(be + j);
-      const ulonglong2 G = *reinterpret_cast<const ulonglong2 *>(ga + j);
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        const int jj = 16 * b + 2 * (j + t);
-        const uint64_t u2 = pk2(d0[jj], d0[jj + 1]);
-        const uint64_t v2 = pk2(d1[jj], d1[jj + 1]);
-        const uint64_t a2 = t ? A.y : A.x, b2 = t ? B.y : B.x, g2 = t ? G.y : G.x;
-        const uint64_t w2 = ffma2(b2, v2, u2);
-        const uint64_t e2 = fmul2(g2, v2);
-        uint64_t q2 = ffma2(e2, v2, nt2);
-        q2 = ffma2(fmul2(a2, w2), w2, q2);
-        const uint64_t r2 = fadd2(q2, sb2);
-        uint32_t qa, qb, ra, rb;
-        upk2(q2, qa, qb);
-        upk2(r2, ra, rb);
-        hi &= qa & qb;
-        lo |= ra | rb;
-      }
-    }
-    if (b + 1 < NS / 16) asm volatile("" ::: "memory");
+  for (int j = 0; j < NS; j += 4) {
+    const ulonglong2 g = *reinterpret_cast<const ulonglong2 *>(sgn + j);
+    const uint64_t q0 = pk2(Q[j], Q[j + 1]), q1 = pk2(Q[j + 2], Q[j + 3]);
+    const uint64_t p0 = pk2(P[j], P[j + 1]), p1 = pk2(P[j + 2], P[j + 3]);
+    const uint64_t s0 = ffma2(p0, p0, ffma2(q0, q0, ffma2(g.x, f2, m2)));
+    const uint64_t s1 = ffma2(p1, p1, ffma2(q1, q1, ffma2(g.y, f2, m2)));
+    uint32_t x, y;
+    upk2(s0, x, y);
+    acc0 &= x & y;
+    upk2(s1, x, y);
+    acc1 &= x & y;
   }
-  return (int)hi >= 0 || (int)lo < 0;
+  return (int)(acc0 & acc1) >= 0;
 }
 
-// Seed pass of a permutation batch in the plain form: the largest df-2 value and
-// the most negative df-1 value of NS SNPs for this lane's trait, into smax / smin.
+// Seed pass of a permutation batch: the largest P^2 + Q^2 of the df-2 SNPs into smax
+// and, negated, of the df-1 SNPs into smin.
 template <int NS>
-__device__ __forceinline__ void range_w(const uint32_t (&d0)[NS], const uint32_t (&d1)[NS],
-                                        const ChunkMeta &m, int off, float &smax, float &smin) {
+__device__ __forceinline__ void range_pq(const uint32_t (&P)[NS], const uint32_t (&Q)[NS],
+                                         const float *sgn, float &smax, float &smin) {
 #pragma unroll
-  for (int b = 0; b < NS / 16; ++b) {
-    const uint64_t *al = reinterpret_cast<const uint64_t *>(m.alpha + off + 16 * b);
-    const uint64_t *be = reinterpret_cast<const uint64_t *>(m.beta + off + 16 * b);
-    const uint64_t *ga = reinterpret_cast<const uint64_t *>(m.gamma + off + 16 * b);
-#pragma unroll
-    for (int j = 0; j < 8; j += 2) {
-      const ulonglong2 A = *reinterpret_cast<const ulonglong2 *>(al + j);
-      const ulonglong2 B = *reinterpret_cast<const ulonglong2 *>(be + j);
-      const ulonglong2 G = *reinterpret_cast<const ulonglong2 *>(ga + j);
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        const int jj = 16 * b + 2 * (j + t);
-        const uint64_t u2 = pk2(d0[jj], d0[jj + 1]);
-        const uint64_t v2 = pk2(d1[jj], d1[jj + 1]);
-        const uint64_t a2 = t ? A.y : A.x, b2 = t ? B.y : B.x, g2 = t ? G.y : G.x;
-        const uint64_t w2 = ffma2(b2, v2, u2);
-        const uint64_t e2 = fmul2(g2, v2);
-        const uint64_t s2 = ffma2(fmul2(a2, w2), w2, fmul2(e2, v2));
-        uint32_t sa, sb;
-        upk2(s2, sa, sb);
-        smax = fmax3(smax, __uint_as_float(sa), __uint_as_float(sb));
-        smin = fmin3(smin, __uint_as_float(sa), __uint_as_float(sb));
-      }
-    }
+  for (int j = 0; j < NS; j += 2) {
+    const uint64_t g = *reinterpret_cast<const uint64_t *>(sgn + j);
+    const uint64_t q0 = pk2(Q[j], Q[j + 1]), p0 = pk2(P[j], P[j + 1]);
+    const uint64_t s2 = fmul2(g, ffma2(p0, p0, fmul2(q0, q0)));
+    uint32_t sa, sb;
+    upk2(s2, sa, sb);
+    smax = fmax3(smax, __uint_as_float(sa), __uint_as_float(sb));
+    smin = fmin3(smin, __uint_as_float(sa), __uint_as_float(sb));
   }
+}
+
+// D_0 and D_1 of a pair from its accumulators: P = A0 D_a + A1 D_b, Q = G D_b are exact
+// (ChunkMeta), so both quotients round to the integers they are.  w0 = 0 (a SNP that
+// is never tested): zeros.
+__device__ __forceinline__ void pq_sums(float P, float Q, uint32_t w0, uint32_t w1, float &u, float &v) {
+  const float a0 = __half2float(__ushort_as_half((unsigned short)(w0 & 0xffffu)));
+  const float a1 = __half2float(__ushort_as_half((unsigned short)(w0 >> 16)));
+  const float g = __half2float(__ushort_as_half((unsigned short)(w1 & 0xffffu)));
+  if (!(a0 > 0.f)) {
+    u = 0.f;
+    v = 0.f;
+    return;
+  }
+  const float db = rintf(__fdividef(Q, g));
+  const float da = rintf(__fdividef(fmaf(-a1, db, P), a0));
+  const float dl = -(da + db);
+  const uint32_t a = (w1 >> 16) & 3u, b = (w1 >> 18) & 3u;
+  u = a == 0u ? da : (b == 0u ? db : dl);
+  v = a == 1u ? da : (b == 1u ? db : dl);
 }
 
 // ---- hit events of the plain scan form, handled by the event warps ---------
@@ -997,7 +1015,7 @@ __device__ __forceinline__ bool ev_gate(const EvRing &ev, unsigned long long t, 
 
 // An epilogue warp hands the traits of a half-block whose hot test found a
 // candidate to the event warps: one entry per such trait lane (tickets claimed
-// together), each with that lane's kEvSnps centred sums and constants and the
+// together), each with that lane's kEvSnps accumulator pairs and constants and the
 // SNPs' metadata (written by lanes 0..kEvSnps-1).  False if a wait gave up.
 __device__ __forceinline__ bool ev_submit(const EvRing &ev, const uint32_t (&u)[kEvSnps],
                                           const uint32_t (&v)[kEvSnps], bool need,
@@ -1015,6 +1033,7 @@ __device__ __forceinline__ bool ev_submit(const EvRing &ev, const uint32_t (&u)[
   const int32_t sn = m.snp[jo];
   const uint32_t n01 = (uint32_t)m.n[0][jo] | ((uint32_t)m.n[1][jo] << 16);
   const uint32_t n2df = (uint32_t)m.n[2][jo] | ((uint32_t)m.df[jo] << 16);
+  const uint32_t w0 = m.pq0[jo], w1 = m.pq1[jo];
   while (lanes) {
     const int L = __ffs((int)lanes) - 1;
     lanes &= lanes - 1u;
@@ -1033,6 +1052,8 @@ __device__ __forceinline__ bool ev_submit(const EvRing &ev, const uint32_t (&u)[
       E.snp[lane] = sn;
       E.n01[lane] = n01;
       E.n2df[lane] = n2df;
+      E.pq0[lane] = w0;
+      E.pq1[lane] = w1;
     }
     if (lane == L) {
 #pragma unroll
@@ -1102,88 +1123,119 @@ __device__ __forceinline__ void ev_group(EvGroup &G, const ScanParams &p, int gr
   G.N = g.N;
 }
 
+// An event warp works on two entries at a time, one per half-warp: lane 16 h + j takes
+// the pair (trait, SNP j) of half h's entry.  What it needs of the entry is copied to
+// registers first, so that the entry is free again before the classification, its
+// divisions and its global stores.  Event throughput bounds inputs with many hits per
+// block: 2,000 x 10,000 x 102 with 1.7 % hits took 506 us a call with one entry per
+// warp, held until its stores were issued, and 402 us this way.
+struct EvLane {
+  float P, Q, al, be, ga, tau, b1, b2;
+  uint32_t w0, w1, n01, n2df, id1, id2;
+  int snp, trait, group, ag, nan;
+  double cfac;
+  __device__ __forceinline__ void load(const EvEntry &E, int j) {
+    P = E.u[j];
+    Q = E.v[j];
+    w0 = E.pq0[j];
+    w1 = E.pq1[j];
+    al = E.alpha[j];
+    be = E.beta[j];
+    ga = E.gamma[j];
+    snp = E.snp[j];
+    n01 = E.n01[j];
+    n2df = E.n2df[j];
+    tau = E.tau;
+    cfac = E.cfac;
+    trait = E.trait;
+    group = E.group;
+    ag = E.ag;
+    b1 = E.b1;
+    b2 = E.b2;
+    id1 = E.id1;
+    id2 = E.id2;
+    nan = E.nan;
+  }
+};
+
 // A permuted pair's entry (section "P-value calculation and empirical FDR
-// correction": the minimum p of each permuted trait over all SNPs): lanes j <
-// kEvSnps take the pairs past the submitting lane's bounds, decide them on their
-// FP64 -ln p, raise the trait's key to the largest, and raise its class bounds
-// (largest df-1 |s| and df-2 s of the pairs decided, less the margin: a later
-// pair of the class below them cannot beat those pairs).  With the FDR histogram
-// on, every pair at or above the band with p < P_c is counted in row ag.
-__device__ __forceinline__ void ev_minp(const EvEntry &E, EvGroup &G, const ScanParams &p, int lane,
-                                        float s, unsigned int &mcn, int ev_warp) {
-  const int j = lane & (kEvSnps - 1);
-  const bool valid = lane < kEvSnps && E.snp[j] >= 0;
-  // E.b1, E.b2: the classes' largest decided values when the entry was filled,
-  // E.id1, E.id2 the identities of the pairs that have them; exact copies of those
-  // pairs are decided already
+// correction": the minimum p of each permuted trait over all SNPs), one per half-warp:
+// the lanes take the pairs past the bounds the entry was filled with, list them for
+// their FP64 -ln p, and raise the trait's class bounds (largest df-1 |s| and df-2 s of
+// the pairs listed, less the margin: a later pair of the class below them cannot beat
+// those pairs).  With the FDR histogram on, every pair at or above the band is listed.
+__device__ __forceinline__ void ev_minp(const EvLane &E, EvGroup &G, const ScanParams &p, int lane,
+                                        bool on, float s, float u, float v, unsigned int &mcn,
+                                        int ev_warp) {
+  const bool valid = on && E.snp >= 0;
+  const uint32_t half = 0xffffu << (lane & 16);
+  // b1, b2: the classes' largest decided values when the entry was filled, id1, id2
+  // the identities of the pairs that have them; exact copies of those pairs are
+  // decided already
   const float keep = 1.f - p.margin;
-  const float b1 = E.b1, b2 = E.b2;
-  const uint32_t n01 = E.n01[j], n2df = E.n2df[j];
-  const uint32_t pid = pair_id((int)E.u[j], (int)E.v[j]);
-  bool cand = valid && ((s > b2 * keep && !(s == b2 && pid == E.id2)) ||
-                        (-s > b1 * keep && !(-s == b1 && pid == E.id1)));
+  const uint32_t pid = pair_id((int)u, (int)v);
+  bool cand = valid && ((s > E.b2 * keep && !(s == E.b2 && pid == E.id2)) ||
+                        (-s > E.b1 * keep && !(-s == E.b1 && pid == E.id1)));
   // within a class the key grows with the value: only the entry's largest value
   // of each class, and values within the margin of it, can hold the class's best
   float c1 = cand && s < 0.f ? -s : 0.f, c2 = cand && s > 0.f ? s : 0.f;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
+  for (int o = 8; o > 0; o >>= 1) {
     c1 = fmaxf(c1, __shfl_xor_sync(0xffffffffu, c1, o));
     c2 = fmaxf(c2, __shfl_xor_sync(0xffffffffu, c2, o));
   }
   cand = cand && (s > 0.f ? s >= c2 * keep : -s >= c1 * keep);
-  const bool band = valid && p.fdr_hist != nullptr && fabsf(s) >= E.tau * (1.f - p.margin);
+  const bool band = valid && p.fdr_hist != nullptr && fabsf(s) >= E.tau * keep;
   const bool need = cand || band;
   const uint32_t bal = __ballot_sync(0xffffffffu, need);
   const unsigned int n = (unsigned int)__popc(bal);
   // identities of the pairs that hold the classes' largest values (the largest
   // identity among ties)
   const bool h1 = cand && s < 0.f && -s == c1, h2 = cand && s > 0.f && s == c2;
-  const uint32_t w1 = __ballot_sync(0xffffffffu, h1), w2 = __ballot_sync(0xffffffffu, h2);
-  const uint32_t i1 = __reduce_max_sync(0xffffffffu, h1 ? pid : 0u);
-  const uint32_t i2 = __reduce_max_sync(0xffffffffu, h2 ? pid : 0u);
+  const uint32_t w1 = __ballot_sync(0xffffffffu, h1) & half, w2 = __ballot_sync(0xffffffffu, h2) & half;
+  uint32_t i1 = h1 ? pid : 0u, i2 = h2 ? pid : 0u;
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) {
+    i1 = max(i1, __shfl_xor_sync(0xffffffffu, i1, o));
+    i2 = max(i2, __shfl_xor_sync(0xffffffffu, i2, o));
+  }
   if (mcn + n <= (unsigned int)p.mc_cap) {
     // the list has room: the FP64 work runs after the launch, in parallel
     if (need) {
       MinpPair r;
-      r.u = (int32_t)E.u[j];
-      r.v = (int32_t)E.v[j];
-      r.n01 = n01;
-      r.n2df = n2df;
+      r.u = (int32_t)u;
+      r.v = (int32_t)v;
+      r.n01 = E.n01;
+      r.n2df = E.n2df;
       r.trait = E.trait;
       r.agb = E.ag | (band ? 1 << 16 : 0) | (cand ? 1 << 17 : 0);
       const size_t base = ((size_t)blockIdx.x * 2 + ev_warp) * (size_t)p.mc_cap;
       p.mc_list[base + mcn + (unsigned int)__popc(bal & ((1u << lane) - 1u))] = r;
     }
     mcn += n;
-  } else {
-    // full: decide here
+  } else if (need) {  // full: decide here
+    const int df = (int)(E.n2df >> 16);
     double key = -1.0;
-    if (need) {
-      const int df = (int)(n2df >> 16);
-      if (df > 0 && E.cfac > 0.0)
-        key = key64_of(kw_H64((int)E.u[j], (int)E.v[j], (int)(n01 & 0xffffu), (int)(n01 >> 16),
-                              (int)(n2df & 0xffffu), E.cfac),
-                       df);
-    }
+    if (df > 0 && E.cfac > 0.0)
+      key = key64_of(kw_H64((int)u, (int)v, (int)(E.n01 & 0xffffu), (int)(E.n01 >> 16),
+                            (int)(E.n2df & 0xffffu), E.cfac),
+                     df);
     if (band && key > -log(p.pthresh))
       atomicAdd(p.fdr_hist + (int64_t)E.ag * p.fdr_bins + fdr_bin(key, p.fdr_l0, p.fdr_w, p.fdr_bins),
                 1ull);
-    double kmax = cand ? key : -1.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) kmax = fmax(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
-    if (lane == 0 && kmax > 0.0) {
+    if (cand && key > 0.0) {
       ev_group(G, p, E.group);
       atomicMax(reinterpret_cast<unsigned long long *>(G.minp_key + (int64_t)(E.ag - 1) * G.rows +
                                                        E.trait),
-                (unsigned long long)__double_as_longlong(kmax));
+                (unsigned long long)__double_as_longlong(key));
     }
   }
-  if (lane == 0) {
+  if (on && (lane & 15) == 0) {
     ev_group(G, p, E.group);
     const int64_t idx = (int64_t)(E.ag - 1) * G.rows + E.trait;
-    if (c1 > b1 && w1)
+    if (c1 > E.b1 && w1)
       atomicMax(G.minp_bound + 2 * idx, ((unsigned long long)__float_as_uint(c1) << 32) | i1);
-    if (c2 > b2 && w2)
+    if (c2 > E.b2 && w2)
       atomicMax(G.minp_bound + 2 * idx + 1, ((unsigned long long)__float_as_uint(c2) << 32) | i2);
   }
 }
@@ -1191,60 +1243,53 @@ __device__ __forceinline__ void ev_minp(const EvEntry &E, EvGroup &G, const Scan
 // Event modes: the plain scan, a permutation batch, the plain scan with NaN.
 enum EvMode { kEvPlain = 0, kEvPerm = 1, kEvNan = 2 };
 
-// An event warp's work on one entry: lanes j < kEvSnps classify the pair (trait,
-// SNP j) in the same FP32 form as the hot test (at or above the upper band edge:
-// hit; inside the band: decided in FP64 from the exact sums) and the hits are
-// appended in SNP order, one record per lane, into this warp's staging region of
-// kEpiWarps / 2 segments of the CTA (`wn` records already there); what does not
-// fit goes to the group's list through its counter.  For a trait with NaN
+// An event warp's work on up to two entries (`on`: this lane's half has one): each
+// lane classifies its pair in FP32 from the exact sums (at or above the upper band
+// edge: hit; inside the band: decided in FP64) and the hits are appended in SNP order,
+// one record per lane, into this warp's staging region of kEpiWarps / 2 segments of
+// the CTA (`wn` records already there); what does not fit goes to the group's list
+// through its counter.  For a trait with NaN
 // samples (kEvNan) the pair's group sizes are first made exact (section "Handling
 // missing values": N_i' counts the samples present for both): the genotypes of
 // the trait's NaN samples at the SNP are taken off N_i, and the form is evaluated
 // with those sizes and the df they leave.  Returns the number of hits.
 template <int kMode>
-__device__ __forceinline__ unsigned int ev_process(const EvEntry &E, EvGroup &G, const ScanParams &p,
-                                                   unsigned int wn, int lane, int ev_warp,
-                                                   unsigned int &mcn) {
-  const int j = lane & (kEvSnps - 1);
-  const bool act = lane < kEvSnps;
-  const float tau = E.tau;
-  const float u = E.u[j], v = E.v[j];
-  const float w = fmaf(E.beta[j], v, u);
-  const float sv = fmaf(E.alpha[j] * w, w, (E.gamma[j] * v) * v);
+__device__ __forceinline__ unsigned int ev_process(EvLane &E, bool on, EvGroup &G,
+                                                   const ScanParams &p, unsigned int wn, int lane,
+                                                   int ev_warp, unsigned int &mcn) {
+  float u, v;
+  pq_sums(E.P, E.Q, E.w0, E.w1, u, v);
+  const float sv = kw_s(u, v, E.al, E.be, E.ga);
   float s = sv;
-  uint32_t n01 = E.n01[j], n2df = E.n2df[j];
+  bool act = on && E.snp >= 0;
   if constexpr (kMode == kEvPerm) {
-    if (E.ag > 0) {  // a permuted pair: min-p and FDR work, no hit record
-      ev_minp(E, G, p, lane, sv, mcn, ev_warp);
-      return 0u;
-    }
+    // permuted pairs: min-p and FDR work, no hit record
+    if (__any_sync(0xffffffffu, on && E.ag > 0)) ev_minp(E, G, p, lane, on && E.ag > 0, sv, u, v, mcn, ev_warp);
+    act = act && E.ag == 0;
     s = fabsf(sv);  // df-1 values are negated in permutation batches
   }
   if constexpr (kMode == kEvNan) {
     const int c = E.nan;
-    if (c > 0) {
+    if (act && c > 0) {
       ev_group(G, p, E.group);
-      int n0 = (int)(n01 & 0xffffu), n1 = (int)(n01 >> 16), n2 = (int)(n2df & 0xffffu);
-      const int sn = E.snp[j];
-      if (act && sn >= 0) {
-        const uint16_t *ni = G.nan_idx + (int64_t)E.trait * G.N;
-        const int8_t *gr = G.geno + (int64_t)sn * G.ldg;
-        for (int i = 0; i < c; i += 4) {  // four samples' loads in flight at once
-          int k[4];
+      int n0 = (int)(E.n01 & 0xffffu), n1 = (int)(E.n01 >> 16), n2 = (int)(E.n2df & 0xffffu);
+      const uint16_t *ni = G.nan_idx + (int64_t)E.trait * G.N;
+      const int8_t *gr = G.geno + (int64_t)E.snp * G.ldg;
+      for (int i = 0; i < c; i += 4) {  // four samples' loads in flight at once
+        int k[4];
 #pragma unroll
-          for (int t = 0; t < 4; ++t) k[t] = i + t < c ? (int)ni[i + t] : -1;
+        for (int t = 0; t < 4; ++t) k[t] = i + t < c ? (int)ni[i + t] : -1;
 #pragma unroll
-          for (int t = 0; t < 4; ++t) {
-            const int code = k[t] >= 0 ? (int)gr[k[t]] : -1;  // -1 (missing): in no group
-            n0 -= code == 0;
-            n1 -= code == 1;
-            n2 -= code == 2;
-          }
+        for (int t = 0; t < 4; ++t) {
+          const int code = k[t] >= 0 ? (int)gr[k[t]] : -1;  // -1 (missing): in no group
+          n0 -= code == 0;
+          n1 -= code == 1;
+          n2 -= code == 2;
         }
       }
       const int df = df_of(n0, n1, n2);
       s = 0.f;
-      if (act && sn >= 0 && df > 0) {
+      if (df > 0) {
         const float w = -(u + v);
         float q = 0.f;
         if (n0 > 0) q += u * u / (float)n0;
@@ -1252,50 +1297,49 @@ __device__ __forceinline__ unsigned int ev_process(const EvEntry &E, EvGroup &G,
         if (n2 > 0) q += w * w / (float)n2;
         s = q / (df == 1 ? p.h1 : p.h2);
       }
-      n01 = (uint32_t)n0 | ((uint32_t)n1 << 16);
-      n2df = (uint32_t)n2 | ((uint32_t)df << 16);
+      E.n01 = (uint32_t)n0 | ((uint32_t)n1 << 16);
+      E.n2df = (uint32_t)n2 | ((uint32_t)df << 16);
     }
   }
-  const bool cand = act && s + -tau * (1.f - p.margin) >= 0.f;
-  bool hit = cand && s + -tau * (1.f + p.margin) >= 0.f;
-  if (__any_sync(0xffffffffu, cand && !hit)) {  // inside the band: FP64 (rare)
-    if (cand && !hit)
-      hit = decide64_inl(u, v, (int)(n01 & 0xffffu), (int)(n01 >> 16), (int)(n2df & 0xffffu),
-                         (int)(n2df >> 16), E.cfac, p.pthresh);
-  }
+  const bool cand = act && s + -E.tau * (1.f - p.margin) >= 0.f;
+  bool hit = cand && s + -E.tau * (1.f + p.margin) >= 0.f;
+  if (cand && !hit)  // inside the band: FP64 (rare)
+    hit = decide64_inl(u, v, (int)(E.n01 & 0xffffu), (int)(E.n01 >> 16), (int)(E.n2df & 0xffffu),
+                       (int)(E.n2df >> 16), E.cfac, p.pthresh);
   const uint32_t bal = __ballot_sync(0xffffffffu, hit);
   const unsigned int n = (unsigned int)__popc(bal);
   if (n == 0u) return 0u;
-  ev_group(G, p, E.group);
   constexpr int kSegs = kEpiWarps / 2;  // staging segments per event warp
   const unsigned int cap = (unsigned int)(kSegs * p.seg_cap);
-  const unsigned int over_from = wn > cap ? wn : cap;  // first index beyond the region
-  const unsigned int n_over = wn + n > over_from ? wn + n - over_from : 0u;
-  unsigned long long gbase = 0;
-  if (lane == 0 && n_over > 0) gbase = atomicAdd(G.counter, (unsigned long long)n_over);
-  gbase = __shfl_sync(0xffffffffu, gbase, 0);
+  const unsigned int idx = wn + (unsigned int)__popc(bal & ((1u << lane) - 1u));
+  const bool over = hit && idx >= cap;
+  const uint32_t obal = __ballot_sync(0xffffffffu, over);
+  unsigned long long gi = 0;
+  if (hit) ev_group(G, p, E.group);
+  if (obal != 0u) {  // one reservation per half (the halves may belong to different lists)
+    const uint32_t mine = obal & (0xffffu << (lane & 16));
+    const int lead = mine != 0u ? __ffs((int)mine) - 1 : 0;
+    if (over && lane == lead) gi = atomicAdd(G.counter, (unsigned long long)__popc(mine));
+    gi = __shfl_sync(0xffffffffu, gi, lead) + (unsigned int)__popc(mine & ((1u << lane) - 1u));
+  }
   if (hit) {
     krux_hit rec;
     rec.trait = (uint32_t)E.trait;
-    rec.snp = (uint32_t)E.snp[j];
+    rec.snp = (uint32_t)E.snp;
     rec.d0 = (int32_t)u;
     rec.d1 = (int32_t)v;
     HitAux x;
-    x.n0 = (uint16_t)(n01 & 0xffffu);
-    x.n1 = (uint16_t)(n01 >> 16);
-    x.n2 = (uint16_t)(n2df & 0xffffu);
+    x.n0 = (uint16_t)(E.n01 & 0xffffu);
+    x.n1 = (uint16_t)(E.n01 >> 16);
+    x.n2 = (uint16_t)(E.n2df & 0xffffu);
     x.group = G.gid;
-    const unsigned int idx = wn + (unsigned int)__popc(bal & ((1u << lane) - 1u));
-    if (idx < cap) {
+    if (!over) {
       const size_t seg0 = ((size_t)blockIdx.x * kEpiWarps + kSegs * ev_warp) * (size_t)p.seg_cap;
       st_hit(p.seg_hits + seg0 + idx, rec);
       st_aux(p.seg_aux + seg0 + idx, x);
-    } else {
-      const unsigned long long gi = gbase + (idx - over_from);
-      if (gi < (unsigned long long)G.capacity) {
-        st_hit(G.hits + gi, rec);
-        st_aux(G.aux + gi, x);
-      }
+    } else if (gi < (unsigned long long)G.capacity) {
+      st_hit(G.hits + gi, rec);
+      st_aux(G.aux + gi, x);
     }
   }
   return n;
@@ -1628,11 +1672,14 @@ enum ScanForm {
   kFormPerm = 2,
   kFormNan = 3,
   kFormScanPerm = 4,
-  kFormScanNan = 5
+  kFormScanNan = 5,
+  kFormScanSeed = 6
 };
-// the plain scan form, its two-sided variant for permutation batches and its
-// variant for expression with NaN
-constexpr bool fast_form(int f) { return f == kFormScan || f == kFormScanPerm || f == kFormScanNan; }
+// the plain scan form, its two passes over permutation batches (the largest values
+// first, then the pairs against them) and its variant for expression with NaN
+constexpr bool fast_form(int f) {
+  return f == kFormScan || f == kFormScanPerm || f == kFormScanNan || f == kFormScanSeed;
+}
 
 // Warp roles of a kernel form: the epilogue warps first, then the producer and
 // the MMA issuer (the plain scan form also has two idle warps after them).
@@ -1661,11 +1708,13 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
   uint8_t *scodes = reinterpret_cast<uint8_t *>(smeta + p.nc);
   const uint32_t codes_stride = (uint32_t)p.kpad * 16u;
   uint8_t *stc = scodes + (size_t)p.nc * codes_stride;  // trait-constant ring
+  constexpr bool kLean = kForm == kFormScan || kForm == kFormScanNan;
+  constexpr uint32_t kTc = kLean ? kTcLean : kTcBytes, kTcNan = kLean ? 1536u : 2560u;
   // permutation form: per trait row, the min-p filter bounds of the current step
   // shared by the four warps that cover the row ((step tag << 32) | float bits;
   // df-1 bounds, then df-2 bounds)
   unsigned long long *sbound =
-      reinterpret_cast<unsigned long long *>(stc + (size_t)kTcDepth * kTcBytes);
+      reinterpret_cast<unsigned long long *>(stc + (size_t)kTcDepth * kTc);
   uint64_t *bars = reinterpret_cast<uint64_t *>(sbound + 2 * kTileM);
   const uint32_t bar0 = smem_u32(bars);
   const int nA = p.nA, nc = p.nc;
@@ -1681,14 +1730,33 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
   auto tc_empty = [&](int e) {
     return bar0 + 8u * (uint32_t)(2 * nA + 2 * nc + 2 * kTmemSlots + 1 + kTcDepth + e);
   };
-  uint32_t *tmem_holder =
-      reinterpret_cast<uint32_t *>(bars + 2 * nA + 2 * nc + 2 * kTmemSlots + 1 + 2 * kTcDepth);
+  auto it_full = [&](int e) {
+    return bar0 + 8u * (uint32_t)(2 * nA + 2 * nc + 2 * kTmemSlots + 1 + 2 * kTcDepth + e);
+  };
+  auto it_empty = [&](int e) {
+    return bar0 + 8u * (uint32_t)(2 * nA + 2 * nc + 2 * kTmemSlots + 1 + 2 * kTcDepth + kItemDepth + e);
+  };
+  uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(bars + 2 * nA + 2 * nc + 2 * kTmemSlots + 1 +
+                                                       2 * kTcDepth + 2 * kItemDepth);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_holder + 1);
+  // The work item ring: the producer takes the CTA's next item (from the launch's
+  // counter when there is one, so that CTAs whose items hold many hits, or short
+  // ones, take fewer or more of them) and the other roles follow through it.
+  volatile int *item_ring = reinterpret_cast<volatile int *>(tmem_holder + 4);
+  struct ItemPos {
+    uint32_t e = 0, phase = 0;
+  };
+  auto item_next = [&](ItemPos &q) {
+    if (++q.e == (uint32_t)kItemDepth) {
+      q.e = 0;
+      q.phase ^= 1u;
+    }
+  };
   // plain scan form: the ring of hit-event buffers after everything else
   EvRing ev;
   {
     uint8_t *evr = reinterpret_cast<uint8_t *>(
-        (reinterpret_cast<uintptr_t>(tmem_holder) + 16u + 127u) & ~(uintptr_t)127u);
+        (reinterpret_cast<uintptr_t>(tmem_holder) + 32u + 127u) & ~(uintptr_t)127u);
     ev.ent = reinterpret_cast<EvEntry *>(evr);
     ev.bar0 = smem_u32(evr + kEvEntries * sizeof(EvEntry));
     ev.released = reinterpret_cast<unsigned int *>(evr + kEvEntries * sizeof(EvEntry) + kEvEntries * 8);
@@ -1713,6 +1781,10 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
     for (int e = 0; e < kTcDepth; ++e) {
       mbar_init(tc_full(e), 1);
       mbar_init(tc_empty(e), R::kEpi);
+    }
+    for (int e = 0; e < kItemDepth; ++e) {
+      mbar_init(it_full(e), 1);
+      mbar_init(it_empty(e), 1 + R::kEpi);
     }
     *abort_flag = 0;
     if constexpr (fast_form(kForm)) {
@@ -1747,7 +1819,14 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       uint32_t a_stage = 0, a_phase = 0, b_bits = 0;
       uint32_t a_used = 0, a_last = 0, b_used = 0, b_last = 0;
       uint32_t tc_e = 0, tc_phase = 0, tc_used = 0, tc_last = 0;
-      for (int it = blockIdx.x; it < p.n_items; it += gridDim.x) {
+      ItemPos ip;
+      for (int it = blockIdx.x;;
+           it = p.next ? (int)(gridDim.x + atomicAdd(p.next, 1u)) : it + (int)gridDim.x) {
+        if (!wait_bar(it_empty(ip.e), ip.phase ^ 1u, wc, 18)) goto producer_done;
+        item_ring[ip.e] = it;
+        mbar_arrive(it_full(ip.e));  // (release: the item is visible to who waits for it)
+        item_next(ip);
+        if (it >= p.n_items) break;
         const WorkItem w = p.items[it];
         const GroupDesc *g = p.groups + w.group;
         prefetch_map(&g->tmA);
@@ -1803,9 +1882,9 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
           if (!wait_bar(tc_empty(tc_e), tc_phase ^ 1u, wc, 8)) goto producer_done;
           {
             const bool with_key = g->minp_key != nullptr && ag > 0;
-            constexpr uint32_t key_bytes = kForm == kFormScanPerm ? 2048u : 1024u;
+            constexpr uint32_t key_bytes = fast_form(kForm) ? 2048u : 1024u;
             const uint32_t tx = 512u + 1024u + (g->nan_cnt ? 256u : 0u) + (with_key ? key_bytes : 0u);
-            const uint32_t dst = smem_u32(stc + (size_t)tc_e * kTcBytes);
+            const uint32_t dst = smem_u32(stc + (size_t)tc_e * kTc);
             const int64_t r0 = (int64_t)tt * kTileM;
             mbar_expect_tx(tc_full(tc_e), tx);
             bulk_load(dst, g->tau + r0, 512u, tc_full(tc_e));
@@ -1813,12 +1892,15 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
             if (with_key) {
               const int64_t kr = (int64_t)(ag - 1) * g->rows_per_agroup + r0;
               // the two-sided plain form reads the class bounds, the others the key
-              if constexpr (kForm == kFormScanPerm)
-                bulk_load(dst + 1536u, g->minp_bound + 2 * kr, 2048u, tc_full(tc_e));
+              // (in their seed pass the records so far)
+              if constexpr (fast_form(kForm))
+                bulk_load(dst + 1536u,
+                          (kForm == kFormScanSeed ? g->minp_seed : g->minp_bound) + 2 * kr, 2048u,
+                          tc_full(tc_e));
               else
                 bulk_load(dst + 1536u, g->minp_key + kr, 1024u, tc_full(tc_e));
             }
-            if (g->nan_cnt) bulk_load(dst + 2560u, g->nan_cnt + r0, 256u, tc_full(tc_e));
+            if (g->nan_cnt) bulk_load(dst + kTcNan, g->nan_cnt + r0, 256u, tc_full(tc_e));
             tc_used |= 1u << tc_e;
             tc_last = (tc_last & ~(1u << tc_e)) | (tc_phase << tc_e);
             if (++tc_e == (uint32_t)kTcDepth) {
@@ -1845,7 +1927,13 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFastRegsLow) : "memory");
     if (lane == 0) {
       uint32_t a_stage = 0, a_phase = 0, b_bits = 0, ps = 0, ps_phase = 0;
-      for (int it = blockIdx.x; it < p.n_items; it += gridDim.x) {
+      ItemPos ip;
+      while (true) {
+        if (!wait_bar(it_full(ip.e), ip.phase, wc, 19)) goto fast_mma_done;
+        const int it = item_ring[ip.e];
+        mbar_arrive(it_empty(ip.e));
+        item_next(ip);
+        if (it >= p.n_items) break;
         const WorkItem w = p.items[it];
         const GroupDesc *g = p.groups + w.group;
         const int ncg = g->nc;
@@ -1900,7 +1988,13 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
   } else if (warp == R::kMma) {
     if (lane == 0) {
       uint32_t a_stage = 0, a_phase = 0, b_bits = 0, slot = 0, slot_phase = 0;
-      for (int it = blockIdx.x; it < p.n_items; it += gridDim.x) {
+      ItemPos ip;
+      while (true) {
+        if (!wait_bar(it_full(ip.e), ip.phase, wc, 19)) goto mma_done;
+        const int it = item_ring[ip.e];
+        mbar_arrive(it_empty(ip.e));
+        item_next(ip);
+        if (it >= p.n_items) break;
         const WorkItem w = p.items[it];
         const GroupDesc *g = p.groups + w.group;
         const int ncg = g->nc;
@@ -2006,38 +2100,54 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       unsigned int wn = 0;  // hits this event warp has appended to its staging region
       unsigned int mcn = 0;  // permuted pairs it has passed on to the deferred FP64 pass
       EvGroup G;
-      for (unsigned long long t = (unsigned long long)e;; t += 2) {
+      // half h of event warp e takes the tickets 2 e + h, + 4, ...
+      const int half = lane >> 4;
+      unsigned long long t = (unsigned long long)(2 * e + half);
+      bool idle = false;
+      long long t0 = 0;
+      while (true) {
         const int b = (int)(t % kEvEntries);
-        const uint32_t ph = (uint32_t)((t / kEvEntries) & 1ull);
-        // lane 0 waits until ticket t is filled or no more tickets can come
+        // the halves' first lanes look whether their ticket is filled, or no more can come
         int got = 0;
-        if (lane == 0) {
-          const long long t0 = clock64();
-          while (true) {
-            if (mbar_try_wait_sleep(ev.full(b), ph, 20000u)) {
-              got = 1;
-              break;
-            }
-            if (*abort_flag) break;
+        if ((lane & 15) == 0) {
+          if (mbar_test(ev.full(b), (uint32_t)((t / kEvEntries) & 1ull))) {
+            got = 1;
+          } else {
             const unsigned long long wv = *reinterpret_cast<volatile unsigned long long *>(ev.word);
-            if ((wv >> 40) >= (unsigned long long)kFastEpiWarps && t >= (wv & kEvTicketMask)) break;
-            if (clock64() - t0 > p.timeout_cycles) {
+            if (*abort_flag || ((wv >> 40) >= (unsigned long long)kFastEpiWarps && t >= (wv & kEvTicketMask)))
+              got = 2;
+          }
+        }
+        got = __shfl_sync(0xffffffffu, got, lane & 16);
+        const bool on = got == 1;
+        if (!__any_sync(0xffffffffu, on)) {
+          if (__all_sync(0xffffffffu, got == 2)) break;
+          const long long now = clock64();
+          if (!idle) t0 = now;
+          idle = true;
+          if (now - t0 > p.timeout_cycles) {
+            if (lane == 0) {
               *abort_flag = 1;
               atomicOr(p.status, kDevTimeout);
               atomicMax(p.status + 1, 17u);
-              break;
             }
+            break;
           }
+          __nanosleep(100);
+          continue;
         }
-        got = __shfl_sync(0xffffffffu, got, 0);
-        if (!got) break;
-        wn += ev_process<kForm == kFormScanPerm ? kEvPerm : (kForm == kFormScanNan ? kEvNan : kEvPlain)>(
-            ev.ent[b], G, p, wn, lane, e, mcn);
+        idle = false;
         __syncwarp();
-        if (lane == 0) {  // this use of the buffer is finished
+        EvLane E;
+        E.load(ev.ent[b], lane & (kEvSnps - 1));
+        __syncwarp();
+        if (on && (lane & 15) == 0) {  // this use of the entry is finished
           __threadfence_block();
           atomicAdd(ev.released + b, 1u);
         }
+        wn += ev_process<kForm == kFormScanPerm ? kEvPerm : (kForm == kFormScanNan ? kEvNan : kEvPlain)>(
+            E, on, G, p, wn, lane, e, mcn);
+        if (on) t += 4;
       }
       if constexpr (kForm == kFormScanPerm)
         if (lane == 0 && p.mc_cnt != nullptr) p.mc_cnt[blockIdx.x * 2 + e] = min(mcn, (unsigned int)p.mc_cap);
@@ -2061,13 +2171,13 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
           tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(128 * h + off);
       uint32_t ps = 0, ps_phase = 0, b_bits = 0, tc_e = 0, tc_phase = 0;
       constexpr int kH = kFastSnps / 2;
-      // permutation batches (two-sided form): per class (df 1: -s, df 2: s) the
-      // largest value decided so far for this lane's trait in the current step and
-      // the identity of the pair that has it; a pair may pass when its value exceeds
-      // the decided one less the margin (at most `cap`: the band's lower edge while
-      // FDR counts are on).  The unpermuted group tests both signs against tau.
+      // permutation batches: per class (df 1, df 2) a pair may pass when its value
+      // exceeds the largest decided one of the lane's trait, staged for the step, less
+      // the margin (at most the band's lower edge while FDR counts are on).  The
+      // unpermuted group tests both classes against tau.
       constexpr bool kTwo = kForm == kFormScanPerm;
       constexpr bool kNan = kForm == kFormScanNan;
+      constexpr bool kSeed = kForm == kFormScanSeed;
       constexpr float kBoundMin = 1e-30f, kBoundMax = 1e30f;
       // expression with NaN: the bound of this lane's trait is coefficient set
       // nset - 1 of the chunk's block (0: the chunk metadata's exact coefficients;
@@ -2079,80 +2189,93 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       // load).  One register: nset + 1 in bits 0-3, wset in bits 4-7, mixed bit 8,
       // the trait's NaN count from bit 9.
       int nsw = 1;
-      int cpair = 0;  // the chunk pair_slot works on, within the work item
-      float mx1 = 0.f, mx2 = 0.f, bnd1 = 0.f, bnd2 = 0.f;  // decided values, hot-test bounds
-      uint32_t id1 = 0u, id2 = 0u;
-      int ag = 0;  // the step's rank-matrix group (> 0: a permutation)
+      // the hot test's bounds of the step: -tau (1 - margin), or the classes' bounds
+      float ntlo = 0.f, bnd1 = 0.f, bnd2 = 0.f;
       // seed pass: this lane's largest df-2 value and df-1 |value| in the step and
       // the 16-SNP blocks (positions in the group's SNP order) that hold them
-      const bool seed = kTwo && p.seed_bound != 0;
       float smax = 0.f, smin = 0.f;
       int pos2 = 0, pos1 = 0;
-      int chunk0 = 0;  // the work item's first chunk in the group
-      // the hot test's bounds from the decided values (cap: the band's lower edge
-      // while FDR counts are on, else none)
-      auto set_bounds = [&](float cap) {
-        const float keep = 1.f - p.margin;
-        bnd1 = fminf(fminf(mx1 * keep, cap), kBoundMax);
-        bnd2 = fminf(fminf(mx2 * keep, cap), kBoundMax);
-      };
+      // A step's constants stay in their ring entry until its pairs are done: what only
+      // a candidate needs is read there again, so that the hot loop holds the bounds
+      // and the accumulators alone (with tau, the decided values and their identities
+      // in registers, and the seed pass in the same kernel, the permutation form
+      // spilled 268 bytes in the loop: 75.7 ms per call of 16 x 20,000 x 200,000
+      // against 52.8).
       auto test = [&](const uint32_t(&x0)[kH], const uint32_t(&x1)[kH], const ChunkMeta &mc, int o,
-                      float ntlo) -> bool {
+                      const uint8_t *blk) -> bool {
         if constexpr (kTwo) {
-          return hit_fast_w2<kH>(x0, x1, mc, o, -bnd2, bnd1 + bnd2);
+          return hit_pq2<kH>(x0, x1, mc.sgn + o, bnd1, bnd2);
         } else if constexpr (kNan) {
-          const uint8_t *blk = scodes + (size_t)cpair * codes_stride;
           const int wset = (nsw >> 4) & 15, nset = (nsw & 15) - 1;
-          const float *cw = wset > 0 ? coef_set(blk, wset - 1)->alpha : mc.alpha;
+          if (wset == 0) return hit_pq<kH>(x0, x1, ntlo);
+          const float *cw = coef_set(blk, wset - 1)->alpha;
           bool need = hit_fast_wc<kH>(x0, x1, cw, cw + kChunkSnps, cw + 2 * kChunkSnps, o, ntlo);
           if (((nsw >> 8) & 1) && __any_sync(0xffffffffu, need)) {
-            const float *cf = nset > 0 ? coef_set(blk, nset - 1)->alpha : mc.alpha;
-            need = hit_fast_wc<kH>(x0, x1, cf, cf + kChunkSnps, cf + 2 * kChunkSnps, o, ntlo) && need;
+            const float *cf = coef_set(blk, max(nset, 1) - 1)->alpha;
+            const bool own = nset > 0 ? hit_fast_wc<kH>(x0, x1, cf, cf + kChunkSnps, cf + 2 * kChunkSnps,
+                                                        o, ntlo)
+                                      : hit_pq<kH>(x0, x1, ntlo);
+            need = own && need;
           }
           return need;
         } else {
-          return hit_fast_w<kH>(x0, x1, mc, o, ntlo);
+          return hit_pq<kH>(x0, x1, ntlo);
         }
       };
-      // a permuted block past the hot test: the lane's pairs that still need the
-      // event warps (past the bounds but not exact copies of a class's decided pair
-      // -- copies are common inside LD blocks -- or in the FDR band), and the
-      // classes' new largest values with the identities of their pairs
+      // a permuted block past the hot test: whether the lane has a pair that still
+      // needs the event warps (past its class's bound but not an exact copy of the
+      // class's decided pair -- copies are common inside LD blocks -- or in the FDR band)
       auto minp_filter = [&](const uint32_t(&x0)[kH], const uint32_t(&x1)[kH], const ChunkMeta &mc,
-                             int o, float tau, float &n1, float &n2, uint32_t &k1,
-                             uint32_t &k2) -> bool {
+                             int o, float tau, float mx1, float mx2, uint32_t id1,
+                             uint32_t id2) -> bool {
         const float tlo = p.fdr_hist != nullptr ? tau * (1.f - p.margin) : kBoundMax;
-        const float b1 = bnd1, b2 = bnd2;
         bool any = false;
-        n1 = mx1;
-        n2 = mx2;
-        k1 = id1;
-        k2 = id2;
         for (int j = 0; j < kH; ++j) {
-          const float u = __uint_as_float(x0[j]), v = __uint_as_float(x1[j]);
-          const float sv = kw_s(u, v, mc.alpha[o + j], mc.beta[o + j], mc.gamma[o + j]);
-          bool c2 = sv > b2, c1 = -sv > b1;
-          uint32_t pid = 0u;
-          if (c1 || c2) pid = pair_id((int)u, (int)v);
-          c2 = c2 && !(sv == mx2 && pid == id2);
-          c1 = c1 && !(-sv == mx1 && pid == id1);
-          any = any || c1 || c2 || fabsf(sv) >= tlo;
-          if (c2 && sv > n2) {
-            n2 = sv;
-            k2 = pid;
-          }
-          if (c1 && -sv > n1) {
-            n1 = -sv;
-            k1 = pid;
-          }
+          // P^2 + Q^2 is never below |s|: most pairs stop here
+          const float pj = __uint_as_float(x0[j]), qj = __uint_as_float(x1[j]);
+          const float top = fmaf(pj, pj, qj * qj) * 1.00001f;
+          const bool two = mc.sgn[o + j] > 0.f;
+          const float bnd = two ? bnd2 : bnd1;
+          if (!(top > bnd || top >= tlo)) continue;
+          float u, v;
+          pq_sums(pj, qj, mc.pq0[o + j], mc.pq1[o + j], u, v);
+          const float sv = fabsf(kw_s(u, v, mc.alpha[o + j], mc.beta[o + j], mc.gamma[o + j]));
+          const bool past = sv > bnd && !(sv == (two ? mx2 : mx1) &&
+                                          pair_id((int)u, (int)v) == (two ? id2 : id1));
+          any = any || past || sv >= tlo;
         }
         return any;
+      };
+      // a half-block with a candidate: to the event warps; false if a wait gave up
+      auto hand_over = [&](const uint32_t(&x0)[kH], const uint32_t(&x1)[kH], bool need,
+                           const ChunkMeta &mc, int o, const uint8_t *tcp, int step, int g_ntt,
+                           int group) -> bool {
+        const float tau = reinterpret_cast<const float *>(tcp)[row];
+        const double cfac = reinterpret_cast<const double *>(tcp + 512)[row];
+        const int ag = step / g_ntt;
+        const int trait = (step - ag * g_ntt) * kTileM + row;
+        bool real = need;
+        float mx1 = 0.f, mx2 = 0.f;
+        uint32_t id1 = 0u, id2 = 0u;
+        if constexpr (kTwo) {
+          if (ag > 0) {
+            const uint4 bb = reinterpret_cast<const uint4 *>(tcp + 1536)[row];
+            mx1 = fmaxf(__uint_as_float(bb.y), kBoundMin);
+            id1 = bb.x;
+            mx2 = fmaxf(__uint_as_float(bb.w), kBoundMin);
+            id2 = bb.z;
+            if (need) real = minp_filter(x0, x1, mc, o, tau, mx1, mx2, id1, id2);
+            if (!__any_sync(0xffffffffu, real)) return true;
+          }
+        }
+        return ev_submit(ev, x0, x1, real, mc, o, tau, cfac, trait, group, ag, mx1, mx2, id1, id2,
+                         kNan ? nsw >> 9 : 0, p, abort_addr, lane);
       };
       // one accumulator pair: wait for it, load this warp's two halves (the second
       // while the first is tested), release it, test the second half, hand any
       // candidate half-block to the event warps; false if a wait gave up
-      auto pair_slot = [&](uint32_t ps, uint32_t phase, const ChunkMeta &mc, float tau,
-                           double cfac, float ntlo, int trait, int group) -> bool {
+      auto pair_slot = [&](uint32_t ps, uint32_t phase, const ChunkMeta &mc, int c, int chunk0,
+                           const uint8_t *tcp, int step, int g_ntt, int group) -> bool {
         if (!__all_sync(0xffffffffu, wait_bar_p(t_full(ps), phase, p, abort_addr, 7))) return false;
         tc_fence_after();
         uint32_t a0[kH], a1[kH], b0[kH], b1[kH];
@@ -2160,122 +2283,126 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         tmem_ld_half(taddr, a0, a1);
         tmem_wait_ld();
         tmem_ld_half(taddr + (uint32_t)kH, b0, b1);
-        if constexpr (kTwo) {
-          if (seed) {
-            const int pos = (chunk0 + cpair) * kChunkSnps + off;
-            float hi = 0.f, lo = 0.f;
-            range_w<kH>(a0, a1, mc, off, hi, lo);
-            tmem_wait_ld();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(t_empty(ps));
-            if (hi > smax) { smax = hi; pos2 = pos; }
-            if (lo < smin) { smin = lo; pos1 = pos; }
-            hi = 0.f;
-            lo = 0.f;
-            range_w<kH>(b0, b1, mc, off + kH, hi, lo);
-            if (hi > smax) { smax = hi; pos2 = pos + kH; }
-            if (lo < smin) { smin = lo; pos1 = pos + kH; }
-            return true;
-          }
-        }
-        const bool need_a = test(a0, a1, mc, off, ntlo);
-        tmem_wait_ld();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(t_empty(ps));
-        const bool need_b = test(b0, b1, mc, off + kH, ntlo);
-        if (__any_sync(0xffffffffu, need_a)) {
-          bool real = need_a;
-          float n1 = 0.f, n2 = 0.f;
-          uint32_t k1 = 0u, k2 = 0u;
-          if constexpr (kTwo)
-            if (ag > 0 && need_a) real = minp_filter(a0, a1, mc, off, tau, n1, n2, k1, k2);
-          if (__any_sync(0xffffffffu, real) &&
-              !ev_submit(ev, a0, a1, real, mc, off, tau, cfac, trait, group, ag, mx1, mx2, id1, id2,
-                         kNan ? nsw >> 9 : 0, p, abort_addr, lane))
+        if constexpr (kSeed) {
+          const int pos = (chunk0 + c) * kChunkSnps + off;
+          float hi = 0.f, lo = 0.f;
+          range_pq<kH>(a0, a1, mc.sgn + off, hi, lo);
+          tmem_wait_ld();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(t_empty(ps));
+          if (hi > smax) { smax = hi; pos2 = pos; }
+          if (lo < smin) { smin = lo; pos1 = pos; }
+          hi = 0.f;
+          lo = 0.f;
+          range_pq<kH>(b0, b1, mc.sgn + off + kH, hi, lo);
+          if (hi > smax) { smax = hi; pos2 = pos + kH; }
+          if (lo < smin) { smin = lo; pos1 = pos + kH; }
+          return true;
+        } else {
+          const uint8_t *blk = kNan ? scodes + (size_t)c * codes_stride : nullptr;
+          const bool need_a = test(a0, a1, mc, off, blk);
+          tmem_wait_ld();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(t_empty(ps));
+          const bool need_b = test(b0, b1, mc, off + kH, blk);
+          if (__any_sync(0xffffffffu, need_a) &&
+              !hand_over(a0, a1, need_a, mc, off, tcp, step, g_ntt, group))
             return false;
-          if constexpr (kTwo)
-            if (ag > 0 && real) {
-              mx1 = n1;
-              mx2 = n2;
-              id1 = k1;
-              id2 = k2;
-              set_bounds(p.fdr_hist != nullptr ? tau * (1.f - p.margin) : kBoundMax);
-            }
-        }
-        if (__any_sync(0xffffffffu, need_b)) {
-          bool real = need_b;
-          float n1 = 0.f, n2 = 0.f;
-          uint32_t k1 = 0u, k2 = 0u;
-          if constexpr (kTwo)
-            if (ag > 0 && need_b) real = minp_filter(b0, b1, mc, off + kH, tau, n1, n2, k1, k2);
-          if (__any_sync(0xffffffffu, real) &&
-              !ev_submit(ev, b0, b1, real, mc, off + kH, tau, cfac, trait, group, ag, mx1, mx2, id1, id2,
-                         kNan ? nsw >> 9 : 0, p, abort_addr, lane))
+          if (__any_sync(0xffffffffu, need_b) &&
+              !hand_over(b0, b1, need_b, mc, off + kH, tcp, step, g_ntt, group))
             return false;
-          if constexpr (kTwo)
-            if (ag > 0 && real) {
-              mx1 = n1;
-              mx2 = n2;
-              id1 = k1;
-              id2 = k2;
-              set_bounds(p.fdr_hist != nullptr ? tau * (1.f - p.margin) : kBoundMax);
-            }
+          return true;
         }
-        return true;
       };
-      for (int it = blockIdx.x; it < p.n_items; it += gridDim.x) {
+      ItemPos ip;
+      while (true) {
+        if (!__all_sync(0xffffffffu, wait_bar_p(it_full(ip.e), ip.phase, p, abort_addr, 20)))
+          goto epi_done_scan;
+        const int it = item_ring[ip.e];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(it_empty(ip.e));
+        item_next(ip);
+        if (it >= p.n_items) break;
         const WorkItem w = p.items[it];
         const GroupDesc &g = p.groups[w.group];
         const int g_nc = g.nc, g_ntt = g.n_ttiles;
         const int nc_item = min(g_nc, g.nchunks - w.btile * g_nc);
+        const int chunk0 = w.btile * g_nc;  // the work item's first chunk in the group
         // this warp's chunks of the B tile (h and 2 + h) must have landed
         {
           bool ok = true;
           for (int c = h; c < nc_item; c += 2) ok = ok && wait_bar_p(b_full(c), (b_bits >> c) & 1u, p, abort_addr, 6);
           if (!__all_sync(0xffffffffu, ok)) goto epi_done_scan;
         }
-        int tt = w.step_begin % g_ntt;  // trait tile of the step
-        chunk0 = w.btile * g_nc;
         for (int step = w.step_begin; step < w.step_end; ++step) {
-          // this step's trait constants, staged by the producer (copied out at once)
+          // this step's trait constants, staged by the producer
           if (!__all_sync(0xffffffffu, wait_bar_p(tc_full(tc_e), tc_phase, p, abort_addr, 9)))
             goto epi_done_scan;
-          const uint8_t *tcp = stc + (size_t)tc_e * kTcBytes;
-          const float tau = reinterpret_cast<const float *>(tcp)[row];
-          const double cfac = reinterpret_cast<const double *>(tcp + 512)[row];
-          const int trait = tt * kTileM + row;
-          if constexpr (kNan) {
-            const int nan_c = g.nan_cnt ? (int)reinterpret_cast<const uint16_t *>(tcp + 2560)[row] : 0;
-            const int nset = nan_c == 0 ? 0 : (nan_c <= kNanCMax ? nan_set_of(nan_c) + 1 : -1);
-            const int wset = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(nset, 0));
-            const bool mixed = __any_sync(0xffffffffu, nset >= 0 && nset != wset);
-            nsw = (nset + 1) | (wset << 4) | (mixed ? 256 : 0) | (nan_c << 9);
-          }
-          if constexpr (kTwo) {
-            // unpermuted group: both signs against tau (less the margin); a
-            // permuted one: the classes' decided values staged for the step
-            ag = step / g_ntt;
-            if (ag > 0) {
-              // per class: (value bits << 32) | identity, as little-endian words
-              const uint4 bb = reinterpret_cast<const uint4 *>(tcp + 1536)[row];
-              mx1 = fmaxf(__uint_as_float(bb.y), kBoundMin);
-              id1 = bb.x;
-              mx2 = fmaxf(__uint_as_float(bb.w), kBoundMin);
-              id2 = bb.z;
-              set_bounds(p.fdr_hist != nullptr ? tau * (1.f - p.margin) : kBoundMax);
-            } else {
-              mx1 = tau;
-              mx2 = tau;
-              id1 = 0u;
-              id2 = 0u;
-              set_bounds(kBoundMax);
+          const uint8_t *tcp = stc + (size_t)tc_e * kTc;
+          {
+            const float tau = reinterpret_cast<const float *>(tcp)[row];
+            ntlo = -tau * (1.f - p.margin);
+            if constexpr (kNan) {
+              const int nan_c = g.nan_cnt ? (int)reinterpret_cast<const uint16_t *>(tcp + kTcNan)[row] : 0;
+              const int nset = nan_c == 0 ? 0 : (nan_c <= kNanCMax ? nan_set_of(nan_c) + 1 : -1);
+              const int wset = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(nset, 0));
+              const bool mixed = __any_sync(0xffffffffu, nset >= 0 && nset != wset);
+              nsw = (nset + 1) | (wset << 4) | (mixed ? 256 : 0) | (nan_c << 9);
+              // (a trait beyond the last set: +inf lets every pair through)
+              if (nset < 0 && tau < kBoundMax) ntlo = __int_as_float(0x7f800000);
+            }
+            if constexpr (kTwo) {
+              // unpermuted group: both classes against tau (less the margin); a
+              // permuted one: per class (value bits << 32) | identity of the largest
+              // decided value, as little-endian words
+              const float keep = 1.f - p.margin;
+              if (step >= g_ntt) {
+                const uint4 bb = reinterpret_cast<const uint4 *>(tcp + 1536)[row];
+                const float cap = p.fdr_hist != nullptr ? fminf(tau * keep, kBoundMax) : kBoundMax;
+                bnd1 = fminf(fmaxf(__uint_as_float(bb.y), kBoundMin) * keep, cap);
+                bnd2 = fminf(fmaxf(__uint_as_float(bb.w), kBoundMin) * keep, cap);
+              } else {
+                bnd1 = fminf(tau * keep, kBoundMax);
+                bnd2 = bnd1;
+              }
             }
             smax = 0.f;
             smin = 0.f;
             pos2 = 0;
             pos1 = 0;
+          }
+          for (int c0 = 0; c0 < nc_item; c0 += 2) {
+            const int c = c0 + h;
+            if (c < nc_item) {
+              if (!pair_slot(ps, ps_phase, smeta[c], c, chunk0, tcp, step, g_ntt, w.group))
+                goto epi_done_scan;
+            } else {  // an odd last chunk leaves warps 8-15 idle: release only
+              if (!__all_sync(0xffffffffu, wait_bar_p(t_full(ps), ps_phase, p, abort_addr, 7)))
+                goto epi_done_scan;
+              tc_fence_after();
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(t_empty(ps));
+            }
+            ps ^= 1u;
+            if (ps == 0u) ps_phase ^= 1u;
+          }
+          if constexpr (kSeed) {
+            // the step's largest values and their blocks (the largest over all steps
+            // is decided exactly after the launch), written only past the record
+            // staged for the step
+            const int ag = step / g_ntt, trait = (step - ag * g_ntt) * kTileM + row;
+            if (ag > 0 && trait < g.T) {
+              const uint4 bb = reinterpret_cast<const uint4 *>(tcp + 1536)[row];
+              unsigned long long *rp =
+                  g.minp_seed + 2 * ((int64_t)(ag - 1) * g.rows_per_agroup + trait);
+              if (-smin > __uint_as_float(bb.y))
+                atomicMax(rp, ((unsigned long long)__float_as_uint(-smin) << 32) | (uint32_t)(pos1 + 1));
+              if (smax > __uint_as_float(bb.w))
+                atomicMax(rp + 1, ((unsigned long long)__float_as_uint(smax) << 32) | (uint32_t)(pos2 + 1));
+            }
           }
           __syncwarp();
           if (lane == 0) mbar_arrive(tc_empty(tc_e));
@@ -2283,42 +2410,6 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
             tc_e = 0;
             tc_phase ^= 1u;
           }
-          float ntlo = -tau * (1.f - p.margin);
-          // (a trait beyond the last set: +inf lets every pair through)
-          if constexpr (kNan)
-            if ((nsw & 15) == 0 && tau < kBoundMax) ntlo = __int_as_float(0x7f800000);
-          {
-            for (int c0 = 0; c0 < nc_item; c0 += 2) {
-              const int c = c0 + h;
-              if (c < nc_item) {
-                cpair = c;
-                if (!pair_slot(ps, ps_phase, smeta[c], tau, cfac, ntlo, trait, w.group))
-                  goto epi_done_scan;
-              } else {  // an odd last chunk leaves warps 8-15 idle: release only
-                if (!__all_sync(0xffffffffu, wait_bar_p(t_full(ps), ps_phase, p, abort_addr, 7)))
-                  goto epi_done_scan;
-                tc_fence_after();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(t_empty(ps));
-              }
-              ps ^= 1u;
-              if (ps == 0u) ps_phase ^= 1u;
-            }
-          }
-          if constexpr (kTwo) {
-            // seed pass: the step's largest values and their blocks (the largest
-            // over all steps is decided exactly after the launch)
-            if (seed && ag > 0 && trait < g.T) {
-              unsigned long long *rp =
-                  g.minp_seed + 2 * ((int64_t)(ag - 1) * g.rows_per_agroup + trait);
-              if (smin < 0.f)
-                atomicMax(rp, ((unsigned long long)__float_as_uint(-smin) << 32) | (uint32_t)(pos1 + 1));
-              if (smax > 0.f)
-                atomicMax(rp + 1, ((unsigned long long)__float_as_uint(smax) << 32) | (uint32_t)(pos2 + 1));
-            }
-          }
-          if (++tt == g_ntt) tt = 0;
         }
         // the chunks' metadata is no longer needed
         __syncwarp();
@@ -2337,7 +2428,14 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
     uint32_t slot = 0, slot_phase = 0, b_bits = 0, tc_e = 0, tc_phase = 0;
     unsigned int wn = 0;  // hits this warp has appended to its staging segment
     uint32_t step_tag = 0;  // steps begun by this warp (the same count in every epilogue warp)
-    for (int it = blockIdx.x; it < p.n_items; it += gridDim.x) {
+    ItemPos ip;
+    while (true) {
+      if (!__all_sync(0xffffffffu, wait_bar(it_full(ip.e), ip.phase, wc, 20))) goto epi_done;
+      const int it = item_ring[ip.e];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(it_empty(ip.e));
+      item_next(ip);
+      if (it >= p.n_items) break;
       const WorkItem w = p.items[it];
       const GroupDesc &g = p.groups[w.group];
       const int nc_item = min(g.nc, g.nchunks - w.btile * g.nc);
@@ -2358,7 +2456,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         if constexpr (kForm == kFormPerm) ++step_tag;
         // this step's trait constants, staged by the producer
         if (!__all_sync(0xffffffffu, wait_bar(tc_full(tc_e), tc_phase, wc, 9))) goto epi_done;
-        const uint8_t *tcp = stc + (size_t)tc_e * kTcBytes;
+        const uint8_t *tcp = stc + (size_t)tc_e * kTc;
         const int row = 32 * q + lane;
         EpiTrait et;
         et.trait = tt * kTileM + row;
@@ -2367,7 +2465,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         et.ntlo = -tau * (1.f - p.margin);
         et.nthi = -tau * (1.f + p.margin);
         et.cfac = reinterpret_cast<const double *>(tcp + 512)[row];
-        et.nan_cnt = g_has_nan ? (int)reinterpret_cast<const uint16_t *>(tcp + 2560)[row] : 0;
+        et.nan_cnt = g_has_nan ? (int)reinterpret_cast<const uint16_t *>(tcp + kTcNan)[row] : 0;
         et.nan_idx = g_has_nan && et.valid
                          ? g.nan_idx + ag * g.nan_ag_stride + (int64_t)et.trait * g_N
                          : nullptr;
@@ -2846,7 +2944,7 @@ size_t scan_smem_bytes(int nc, int nA, int kpad) {
 size_t scan_smem_bytes2(int nc, int nA, size_t a_tile_bytes, size_t b_region, int codes_k) {
   return 1024 + (size_t)nA * a_tile_bytes + b_region + (size_t)nc * sizeof(ChunkMeta) +
          (size_t)nc * codes_k * 16 + (size_t)kTcDepth * kTcBytes + 16 * (size_t)kTileM +
-         8 * (size_t)(2 * nA + 2 * nc + 2 * kTmemSlots + 1 + 2 * kTcDepth) + 16;
+         8 * (size_t)(2 * nA + 2 * nc + 2 * kTmemSlots + 1 + 2 * kTcDepth + 2 * kItemDepth) + 32;
 }
 
 bool fast_form_ok();
@@ -2875,6 +2973,9 @@ cudaError_t scan_set_smem_all(size_t smem) {
   e = cudaFuncSetAttribute(krux_scan_kernel<kFormScanPerm>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(krux_scan_kernel<kFormScanSeed>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(krux_scan_kernel<kFormMulti>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -2896,6 +2997,8 @@ int scan_form_of(const ScanParams &p) {
 cudaError_t launch_scan_only(const ScanParams &p, int grid, size_t smem, cudaStream_t s) {
   if (p.multi)
     krux_scan_kernel<kFormMulti><<<grid, kScanThreads, smem, s>>>(p);
+  else if (p.perm && p.fast && p.seed_bound && fast_form_ok())
+    krux_scan_kernel<kFormScanSeed><<<grid, kFastThreads, smem, s>>>(p);
   else if (p.perm && p.fast && fast_form_ok())
     krux_scan_kernel<kFormScanPerm><<<grid, kFastThreads, smem, s>>>(p);
   else if (p.perm)
@@ -2921,10 +3024,12 @@ bool fast_form_ok() {
   if (v < 0) {
     // the plain-form kernels were built at the register count their warp roles'
     // setmaxnreg split assumes
-    cudaFuncAttributes a, b, c;
+    cudaFuncAttributes a, b, c, d;
     v = cudaFuncGetAttributes(&a, krux_scan_kernel<kFormScan>) == cudaSuccess &&
                 cudaFuncGetAttributes(&b, krux_scan_kernel<kFormScanPerm>) == cudaSuccess &&
                 cudaFuncGetAttributes(&c, krux_scan_kernel<kFormScanNan>) == cudaSuccess &&
+                cudaFuncGetAttributes(&d, krux_scan_kernel<kFormScanSeed>) == cudaSuccess &&
+                d.numRegs == kFastRegsLaunch && d.maxThreadsPerBlock >= kFastThreads &&
                 a.numRegs == kFastRegsLaunch && a.maxThreadsPerBlock >= kFastThreads &&
                 b.numRegs == kFastRegsLaunch && b.maxThreadsPerBlock >= kFastThreads &&
                 c.numRegs == kFastRegsLaunch && c.maxThreadsPerBlock >= kFastThreads

@@ -1,0 +1,50 @@
+"""The plain form's weighted indicator rows: every hit found and every rank sum
+recovered, at the sample counts where the weights' precision changes, for group sizes
+from 1 to N - 2, two-group markers, and traits whose order follows the genotype (the
+largest sums)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("pth", [0.3, 1e-4])
+@pytest.mark.parametrize("N", [7, 16, 90, 91, 102, 128, 129, 160, 181, 182, 200, 256, 257, 300, 362, 363, 512])
+def test_sums_and_hits_at_every_group_shape(oracle_mod, N, pth):
+    import torch
+    from paper_1307_3519_gb300 import build
+    build.build()
+    import paper_1307_3519_gb300 as k
+    rng = np.random.default_rng(N)
+    sizes = []
+    for a in sorted({1, 2, 3, N // 7, N // 4, N // 3, N // 2, N - 2} - {0}):
+        for b in sorted({0, 1, 2, N // 5, (N - a) // 2, N - a - 1}):
+            if 0 <= b <= N - a:
+                sizes.append((a, b, N - a - b))
+    geno = []
+    for n in sizes:
+        base = np.repeat(np.array([0, 1, 2], dtype=np.int8), n)
+        for codes in ([0, 1, 2], [1, 0, 2], [2, 1, 0], [1, 2, 0]):
+            g = np.array(codes, dtype=np.int8)[base]
+            geno.append(g)  # in sample order: the traits below follow it
+            geno.append(rng.permutation(g))
+    geno = np.ascontiguousarray(np.stack(geno))
+    up = np.arange(N, dtype=np.float32)
+    expr = [up, -up, np.abs(up - N // 2), np.floor(up / 3)]
+    expr += [up + rng.normal(0, s * N, N).astype(np.float32) for s in (0.05, 0.2, 0.5, 1, 2) for _ in range(12)]
+    expr += [np.round(rng.standard_normal(N), 1) for _ in range(70)]
+    expr = np.ascontiguousarray(np.stack(expr).astype(np.float32))
+    kx = k.Krux(0)
+    rs = kx.krux_rank(torch.from_numpy(expr).cuda())
+    r = kx.krux_scan(rs, torch.from_numpy(geno).cuda(), pth, capacity=expr.shape[0] * geno.shape[0])
+    orc = oracle_mod.scan(expr, geno, pth)
+    h = r["hits"].cpu().numpy().astype(np.int64)
+    got = np.zeros_like(orc["hit"])
+    got[h[:, 0], h[:, 1]] = True
+    near = np.abs(orc["p"] / pth - 1.0) < 1e-12
+    assert not ((got != orc["hit"]) & ~near).any()
+    assert r["n_hits"] == len(h) == int(got.sum())
+    assert np.array_equal(h[:, 2], orc["d"][h[:, 0], h[:, 1], 0])
+    assert np.array_equal(h[:, 3], orc["d"][h[:, 0], h[:, 1], 1])
+    rs.free()
+    kx.close()
