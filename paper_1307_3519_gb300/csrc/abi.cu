@@ -271,9 +271,9 @@ struct LaunchShape {
   int ka = 0, nA = 0, b_region = 0, force_nc = 0, no_pair = 0;
 };
 constexpr size_t kSmemLimit = 232448;
-// Shared memory of the plain forms beyond the general one's: the hit-event ring, and
-// outside permutation batches a smaller trait-constant ring.
-constexpr size_t plain_extra(bool perm) { return kEvRegion - (perm ? 0 : kTcSaved); }
+// Shared memory of the plain forms beyond the general one's: the hit-event ring, less
+// what they do without.
+constexpr size_t kPlainExtra = kEvRegion - kFastSaved;
 
 size_t shape_overhead(int nA, int codes_k) {
   return scan_smem_bytes2(kTmemSlots, nA, 0, 0, std::max(codes_k, 16));
@@ -340,10 +340,10 @@ bool plain_form_fits(const krux_ctx *ctx, int Np) {
   if (ctx->tune_layout == 0) return false;
   const int kpad = round_up(Np, 16);
   LaunchShape sh;
-  if (!pick_launch_shape(ctx, kpad, 0, sh, plain_extra(false))) return false;
+  if (!pick_launch_shape(ctx, kpad, 0, sh, kPlainExtra)) return false;
   const int nc = (int)(sh.b_region / (256 * kpad));
   return sh.ka == kpad && nc >= 2 && nc % 2 == 0 &&
-         shape_overhead(sh.nA, 0) + (size_t)sh.nA * 256 * sh.ka + sh.b_region + plain_extra(false) <= kSmemLimit;
+         shape_overhead(sh.nA, 0) + (size_t)sh.nA * 256 * sh.ka + sh.b_region + kPlainExtra <= kSmemLimit;
 }
 
 // Refuses a launch plan whose shared-memory regions or per-group shapes are not
@@ -1378,7 +1378,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     ctx->tune_nA = tnA;
     ctx->tune_ka = tka;
     const bool ok = pick_launch_shape(ctx, kpad, codes_k, sh,
-                                      fast_shape ? plain_extra(fl.signed_coef != 0) : 0);
+                                      fast_shape ? kPlainExtra : 0);
     ctx->tune_nc = s_nc;
     ctx->tune_nA = s_nA;
     ctx->tune_ka = s_ka;
@@ -1582,7 +1582,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   }
   fl.smem = scan_smem_bytes2(nc_max, sh.nA, (size_t)p.a_tile_bytes, (size_t)p.b_region, p.kpad);
   if (p.fast) {  // the plain scan form also holds its ring of hit-event buffers
-    const size_t with_ring = fl.smem + plain_extra(p.perm != 0);
+    const size_t with_ring = fl.smem + kPlainExtra;
     if (with_ring <= kSmemLimit) fl.smem = with_ring;
     else p.fast = 0;
   }
@@ -2845,7 +2845,7 @@ extern "C" krux_status krux_debug_plan(int N, int with_nan, int layout, int nc, 
   if (plain && lay != 1) return KRUX_EUNSUPPORTED;
   const int codes_k = with_nan == 1 ? Np : (with_nan == 3 ? kCoefNanRows : 0);
   LaunchShape sh;
-  if (!pick_launch_shape(&tmp, kpad, codes_k, sh, plain ? plain_extra(false) : 0)) return KRUX_EUNSUPPORTED;
+  if (!pick_launch_shape(&tmp, kpad, codes_k, sh, plain ? kPlainExtra : 0)) return KRUX_EUNSUPPORTED;
   GroupDesc d;
   std::memset(&d, 0, sizeof d);
   d.Np = Np;
@@ -2864,7 +2864,7 @@ extern "C" krux_status krux_debug_plan(int N, int with_nan, int layout, int nc, 
   p.b_region = sh.b_region;
   p.layout = lay;
   const size_t smem = scan_smem_bytes2(p.nc, p.nA, (size_t)p.a_tile_bytes, (size_t)p.b_region, p.kpad) +
-                     (plain ? plain_extra(false) : 0);
+                     (plain ? kPlainExtra : 0);
   out[0] = sh.ka;
   out[1] = sh.nA;
   out[2] = sh.b_region;

@@ -92,11 +92,14 @@ constexpr size_t kEvRegion = 128 + kEvEntries * sizeof(EvEntry) + kEvEntries * 8
 constexpr int kTcDepth = 4;
 constexpr int kItemDepth = 4;  // work items the producer may announce ahead
 constexpr int kTcBytes = 3584;
-// The plain form and its NaN variant have no keys: tau @0, 3/(K(K+1)C) @512, NaN
-// count @1536, in half the bytes (room for the NaN variant's coefficient sets beside
-// four resident chunks at N = 102).  Their launches hold this much less.
-constexpr int kTcLean = 1792;
-constexpr size_t kTcSaved = (size_t)kTcDepth * (kTcBytes - kTcLean);
+// The plain forms have neither this ring nor the bounds shared by a row's warps: their
+// lanes read the constants of the next step from global memory while they work on the
+// current one, without a barrier wait and arrival per step (189 -> 156 warp
+// instructions per warp and pair of chunks, with the branches of the waits; 0.80 ->
+// 0.69 ms for 15,000 x 200,000 x 48), and four chunks stay resident up to N = 128
+// instead of 112 (1.49 -> 0.90 ms at N = 128).  Their launches hold this much less
+// shared memory.
+constexpr size_t kFastSaved = (size_t)kTcDepth * kTcBytes + 16 * (size_t)kTileM;
 
 // ---- per-chunk SNP metadata (one 2304-byte blob per chunk of 64 SNPs) ------
 // Fast-test coefficients: with u = D_0, v = D_1 (D_2 = -u - v) the statistic's

@@ -72,6 +72,14 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+// One arrival by lane 0 of a converged warp, predicated (no branch).
+__device__ __forceinline__ void mbar_arrive_lane0(uint32_t bar, int lane) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.eq.s32 p, %1, 0;\n"
+      " @p mbarrier.arrive.shared::cta.b64 _, [%0];\n}" ::"r"(bar),
+      "r"(lane)
+      : "memory");
+}
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -152,6 +160,14 @@ __device__ __forceinline__ bool wait_bar_p(uint32_t bar, uint32_t parity, const 
       return false;
     }
   }
+}
+
+// A warp's wait: one look and one vote when the phase is complete already, else the
+// bounded wait; false (in every lane) when some lane's wait gave up.
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, const ScanParams &p,
+                                          uint32_t abort_addr, unsigned int where) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  return __all_sync(0xffffffffu, wait_bar_p(bar, parity, p, abort_addr, where));
 }
 
 // Wait used while shutting down: ignores the abort flag (copies and MMAs already
@@ -890,8 +906,7 @@ __device__ __forceinline__ bool hit_fast_wc(const uint32_t (&d0)[NS], const uint
 // instruction, two FP32 operations and half a sign accumulation per pair; no
 // coefficient is read.  With indicator rows and the coefficients of ChunkMeta the
 // same test took five operations and three shared-memory words per SNP: 3.9 ms for
-// 20,000 x 500,000 x 102 without planted effects against 2.64 ms with this one
-// (1.55 PFLOP/s of 4 N flop per pair, 1.70 with the padding of N to 112).
+// 20,000 x 500,000 x 102 without planted effects against 2.6 ms with this one.
 template <int NS>
 __device__ __forceinline__ bool hit_pq(const uint32_t (&P)[NS], const uint32_t (&Q)[NS], float ntlo) {
   const uint64_t nt2 = pk2(__float_as_uint(ntlo), __float_as_uint(ntlo));
@@ -1708,14 +1723,14 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
   uint8_t *scodes = reinterpret_cast<uint8_t *>(smeta + p.nc);
   const uint32_t codes_stride = (uint32_t)p.kpad * 16u;
   uint8_t *stc = scodes + (size_t)p.nc * codes_stride;  // trait-constant ring
-  constexpr bool kLean = kForm == kFormScan || kForm == kFormScanNan;
-  constexpr uint32_t kTc = kLean ? kTcLean : kTcBytes, kTcNan = kLean ? 1536u : 2560u;
   // permutation form: per trait row, the min-p filter bounds of the current step
   // shared by the four warps that cover the row ((step tag << 32) | float bits;
   // df-1 bounds, then df-2 bounds)
   unsigned long long *sbound =
-      reinterpret_cast<unsigned long long *>(stc + (size_t)kTcDepth * kTc);
-  uint64_t *bars = reinterpret_cast<uint64_t *>(sbound + 2 * kTileM);
+      reinterpret_cast<unsigned long long *>(stc + (size_t)kTcDepth * kTcBytes);
+  // (the plain forms have neither the ring nor these bounds)
+  uint64_t *bars = fast_form(kForm) ? reinterpret_cast<uint64_t *>(stc)
+                                    : reinterpret_cast<uint64_t *>(sbound + 2 * kTileM);
   const uint32_t bar0 = smem_u32(bars);
   const int nA = p.nA, nc = p.nc;
   // barrier addresses
@@ -1803,7 +1818,8 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  for (int i = threadIdx.x; i < 2 * kTileM; i += blockDim.x) sbound[i] = 0ull;
+  if constexpr (!fast_form(kForm))
+    for (int i = threadIdx.x; i < 2 * kTileM; i += blockDim.x) sbound[i] = 0ull;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1879,28 +1895,20 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
             }
           }
           // this step's per-trait constants into the ring (padded to whole tiles)
-          if (!wait_bar(tc_empty(tc_e), tc_phase ^ 1u, wc, 8)) goto producer_done;
-          {
+          if constexpr (!fast_form(kForm)) {
+            if (!wait_bar(tc_empty(tc_e), tc_phase ^ 1u, wc, 8)) goto producer_done;
             const bool with_key = g->minp_key != nullptr && ag > 0;
-            constexpr uint32_t key_bytes = fast_form(kForm) ? 2048u : 1024u;
-            const uint32_t tx = 512u + 1024u + (g->nan_cnt ? 256u : 0u) + (with_key ? key_bytes : 0u);
-            const uint32_t dst = smem_u32(stc + (size_t)tc_e * kTc);
+            const uint32_t tx = 512u + 1024u + (g->nan_cnt ? 256u : 0u) + (with_key ? 1024u : 0u);
+            const uint32_t dst = smem_u32(stc + (size_t)tc_e * kTcBytes);
             const int64_t r0 = (int64_t)tt * kTileM;
             mbar_expect_tx(tc_full(tc_e), tx);
             bulk_load(dst, g->tau + r0, 512u, tc_full(tc_e));
             bulk_load(dst + 512u, g->cfac + r0, 1024u, tc_full(tc_e));
             if (with_key) {
               const int64_t kr = (int64_t)(ag - 1) * g->rows_per_agroup + r0;
-              // the two-sided plain form reads the class bounds, the others the key
-              // (in their seed pass the records so far)
-              if constexpr (fast_form(kForm))
-                bulk_load(dst + 1536u,
-                          (kForm == kFormScanSeed ? g->minp_seed : g->minp_bound) + 2 * kr, 2048u,
-                          tc_full(tc_e));
-              else
-                bulk_load(dst + 1536u, g->minp_key + kr, 1024u, tc_full(tc_e));
+              bulk_load(dst + 1536u, g->minp_key + kr, 1024u, tc_full(tc_e));
             }
-            if (g->nan_cnt) bulk_load(dst + kTcNan, g->nan_cnt + r0, 256u, tc_full(tc_e));
+            if (g->nan_cnt) bulk_load(dst + 2560u, g->nan_cnt + r0, 256u, tc_full(tc_e));
             tc_used |= 1u << tc_e;
             tc_last = (tc_last & ~(1u << tc_e)) | (tc_phase << tc_e);
             if (++tc_e == (uint32_t)kTcDepth) {
@@ -2133,7 +2141,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
             }
             break;
           }
-          __nanosleep(100);
+          __nanosleep(400);
           continue;
         }
         idle = false;
@@ -2195,11 +2203,11 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       // the 16-SNP blocks (positions in the group's SNP order) that hold them
       float smax = 0.f, smin = 0.f;
       int pos2 = 0, pos1 = 0;
-      // A step's constants stay in their ring entry until its pairs are done: what only
-      // a candidate needs is read there again, so that the hot loop holds the bounds
-      // and the accumulators alone (with tau, the decided values and their identities
-      // in registers, and the seed pass in the same kernel, the permutation form
-      // spilled 268 bytes in the loop: 75.7 ms per call of 16 x 20,000 x 200,000
+      // What only a candidate needs (tau, the factor of H, decided values and their
+      // identities) is read from global memory when there is one: the hot loop holds
+      // the bounds and the accumulators alone (with tau, the decided values and their
+      // identities in registers, and the seed pass in the same kernel, the permutation
+      // form spilled 268 bytes in the loop: 75.7 ms per call of 16 x 20,000 x 200,000
       // against 52.8).
       auto test = [&](const uint32_t(&x0)[kH], const uint32_t(&x1)[kH], const ChunkMeta &mc, int o,
                       const uint8_t *blk) -> bool {
@@ -2221,6 +2229,19 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         } else {
           return hit_pq<kH>(x0, x1, ntlo);
         }
+      };
+      // a permuted trait's two class words, (value bits << 32) | identity (seed pass:
+      // position) of the largest value so far, and the values alone; other CTAs raise
+      // them during the launch
+      auto class_words = [&](const GroupDesc &g, int ag, int trait) -> uint4 {
+        const unsigned long long *b = kSeed ? g.minp_seed : g.minp_bound;
+        return __ldcg(reinterpret_cast<const uint4 *>(b) + (int64_t)(ag - 1) * g.rows_per_agroup + trait);
+      };
+      auto class_values = [&](const GroupDesc &g, int ag, int trait, float &v1, float &v2) {
+        if (ag == 0) return;
+        const uint4 bb = class_words(g, ag, trait);
+        v1 = __uint_as_float(bb.y);
+        v2 = __uint_as_float(bb.w);
       };
       // a permuted block past the hot test: whether the lane has a pair that still
       // needs the event warps (past its class's bound but not an exact copy of the
@@ -2248,18 +2269,17 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       };
       // a half-block with a candidate: to the event warps; false if a wait gave up
       auto hand_over = [&](const uint32_t(&x0)[kH], const uint32_t(&x1)[kH], bool need,
-                           const ChunkMeta &mc, int o, const uint8_t *tcp, int step, int g_ntt,
+                           const ChunkMeta &mc, int o, const GroupDesc &g, int ag, int tt,
                            int group) -> bool {
-        const float tau = reinterpret_cast<const float *>(tcp)[row];
-        const double cfac = reinterpret_cast<const double *>(tcp + 512)[row];
-        const int ag = step / g_ntt;
-        const int trait = (step - ag * g_ntt) * kTileM + row;
+        const int trait = tt * kTileM + row;
+        const float tau = g.tau[trait];
+        const double cfac = g.cfac[trait];
         bool real = need;
         float mx1 = 0.f, mx2 = 0.f;
         uint32_t id1 = 0u, id2 = 0u;
         if constexpr (kTwo) {
           if (ag > 0) {
-            const uint4 bb = reinterpret_cast<const uint4 *>(tcp + 1536)[row];
+            const uint4 bb = class_words(g, ag, trait);
             mx1 = fmaxf(__uint_as_float(bb.y), kBoundMin);
             id1 = bb.x;
             mx2 = fmaxf(__uint_as_float(bb.w), kBoundMin);
@@ -2271,58 +2291,51 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         return ev_submit(ev, x0, x1, real, mc, o, tau, cfac, trait, group, ag, mx1, mx2, id1, id2,
                          kNan ? nsw >> 9 : 0, p, abort_addr, lane);
       };
-      // one accumulator pair: wait for it, load this warp's two halves (the second
-      // while the first is tested), release it, test the second half, hand any
-      // candidate half-block to the event warps; false if a wait gave up
+      // one accumulator pair: wait for it, load and test this warp's two halves one
+      // after the other (release after the second load) and hand any candidate
+      // half-block to the event warps; false if a wait gave up.  Only one half's
+      // accumulators are live: with the second half's load overlapping the first
+      // half's test the loop held 64 of them and spilled (N = 128, 15,000 x 200,000:
+      // 0.898 against 0.875 ms; the permutation form's main launch of 16 x 20,000 x
+      // 200,000: 30.9 against 25.1 ms); the four warps of a scheduler cover each
+      // other's loads.
       auto pair_slot = [&](uint32_t ps, uint32_t phase, const ChunkMeta &mc, int c, int chunk0,
-                           const uint8_t *tcp, int step, int g_ntt, int group) -> bool {
-        if (!__all_sync(0xffffffffu, wait_bar_p(t_full(ps), phase, p, abort_addr, 7))) return false;
+                           const GroupDesc &g, int ag, int tt, int group) -> bool {
+        if (!wait_warp(t_full(ps), phase, p, abort_addr, 7)) return false;
         tc_fence_after();
-        uint32_t a0[kH], a1[kH], b0[kH], b1[kH];
+        uint32_t x0[kH], x1[kH];
         const uint32_t taddr = lane_cols + ps * 256u;
-        tmem_ld_half(taddr, a0, a1);
-        tmem_wait_ld();
-        tmem_ld_half(taddr + (uint32_t)kH, b0, b1);
-        if constexpr (kSeed) {
-          const int pos = (chunk0 + c) * kChunkSnps + off;
-          float hi = 0.f, lo = 0.f;
-          range_pq<kH>(a0, a1, mc.sgn + off, hi, lo);
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+          tmem_ld_half(taddr + (uint32_t)(kH * half), x0, x1);
           tmem_wait_ld();
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(t_empty(ps));
-          if (hi > smax) { smax = hi; pos2 = pos; }
-          if (lo < smin) { smin = lo; pos1 = pos; }
-          hi = 0.f;
-          lo = 0.f;
-          range_pq<kH>(b0, b1, mc.sgn + off + kH, hi, lo);
-          if (hi > smax) { smax = hi; pos2 = pos + kH; }
-          if (lo < smin) { smin = lo; pos1 = pos + kH; }
-          return true;
-        } else {
-          const uint8_t *blk = kNan ? scodes + (size_t)c * codes_stride : nullptr;
-          const bool need_a = test(a0, a1, mc, off, blk);
-          tmem_wait_ld();
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(t_empty(ps));
-          const bool need_b = test(b0, b1, mc, off + kH, blk);
-          if (__any_sync(0xffffffffu, need_a) &&
-              !hand_over(a0, a1, need_a, mc, off, tcp, step, g_ntt, group))
-            return false;
-          if (__any_sync(0xffffffffu, need_b) &&
-              !hand_over(b0, b1, need_b, mc, off + kH, tcp, step, g_ntt, group))
-            return false;
-          return true;
+          if (half) {
+            tc_fence_before();
+            __syncwarp();
+            mbar_arrive_lane0(t_empty(ps), lane);
+          }
+          const int o = off + kH * half;
+          if constexpr (kSeed) {
+            const int pos = (chunk0 + c) * kChunkSnps + o;
+            float hi = 0.f, lo = 0.f;
+            range_pq<kH>(x0, x1, mc.sgn + o, hi, lo);
+            if (hi > smax) { smax = hi; pos2 = pos; }
+            if (lo < smin) { smin = lo; pos1 = pos; }
+          } else {
+            const uint8_t *blk = kNan ? scodes + (size_t)c * codes_stride : nullptr;
+            const bool need = test(x0, x1, mc, o, blk);
+            if (__any_sync(0xffffffffu, need) && !hand_over(x0, x1, need, mc, o, g, ag, tt, group))
+              return false;
+          }
         }
+        return true;
       };
       ItemPos ip;
       while (true) {
-        if (!__all_sync(0xffffffffu, wait_bar_p(it_full(ip.e), ip.phase, p, abort_addr, 20)))
-          goto epi_done_scan;
+        if (!wait_warp(it_full(ip.e), ip.phase, p, abort_addr, 20)) goto epi_done_scan;
         const int it = item_ring[ip.e];
         __syncwarp();
-        if (lane == 0) mbar_arrive(it_empty(ip.e));
+        mbar_arrive_lane0(it_empty(ip.e), lane);
         item_next(ip);
         if (it >= p.n_items) break;
         const WorkItem w = p.items[it];
@@ -2330,85 +2343,88 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         const int g_nc = g.nc, g_ntt = g.n_ttiles;
         const int nc_item = min(g_nc, g.nchunks - w.btile * g_nc);
         const int chunk0 = w.btile * g_nc;  // the work item's first chunk in the group
+        const float *g_tau = g.tau + row;
+        const uint16_t *g_nan = kNan ? g.nan_cnt : nullptr;
+        int ag = w.step_begin / g_ntt;            // the step's rank-matrix group (> 0: a permutation)
+        int tt = w.step_begin - ag * g_ntt;       // and its trait tile
         // this warp's chunks of the B tile (h and 2 + h) must have landed
         {
           bool ok = true;
           for (int c = h; c < nc_item; c += 2) ok = ok && wait_bar_p(b_full(c), (b_bits >> c) & 1u, p, abort_addr, 6);
           if (!__all_sync(0xffffffffu, ok)) goto epi_done_scan;
         }
+        // the constants of the lane's trait, one step ahead
+        float tau_n = g_tau[tt * kTileM];
+        uint32_t nan_n = 0u;
+        float v1_n = 0.f, v2_n = 0.f;
+        if constexpr (kNan)
+          if (g_nan) nan_n = g_nan[tt * kTileM + row];
+        if constexpr (kTwo || kSeed) class_values(g, ag, tt * kTileM + row, v1_n, v2_n);
         for (int step = w.step_begin; step < w.step_end; ++step) {
-          // this step's trait constants, staged by the producer
-          if (!__all_sync(0xffffffffu, wait_bar_p(tc_full(tc_e), tc_phase, p, abort_addr, 9)))
-            goto epi_done_scan;
-          const uint8_t *tcp = stc + (size_t)tc_e * kTc;
-          {
-            const float tau = reinterpret_cast<const float *>(tcp)[row];
-            ntlo = -tau * (1.f - p.margin);
-            if constexpr (kNan) {
-              const int nan_c = g.nan_cnt ? (int)reinterpret_cast<const uint16_t *>(tcp + kTcNan)[row] : 0;
-              const int nset = nan_c == 0 ? 0 : (nan_c <= kNanCMax ? nan_set_of(nan_c) + 1 : -1);
-              const int wset = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(nset, 0));
-              const bool mixed = __any_sync(0xffffffffu, nset >= 0 && nset != wset);
-              nsw = (nset + 1) | (wset << 4) | (mixed ? 256 : 0) | (nan_c << 9);
-              // (a trait beyond the last set: +inf lets every pair through)
-              if (nset < 0 && tau < kBoundMax) ntlo = __int_as_float(0x7f800000);
-            }
-            if constexpr (kTwo) {
-              // unpermuted group: both classes against tau (less the margin); a
-              // permuted one: per class (value bits << 32) | identity of the largest
-              // decided value, as little-endian words
-              const float keep = 1.f - p.margin;
-              if (step >= g_ntt) {
-                const uint4 bb = reinterpret_cast<const uint4 *>(tcp + 1536)[row];
-                const float cap = p.fdr_hist != nullptr ? fminf(tau * keep, kBoundMax) : kBoundMax;
-                bnd1 = fminf(fmaxf(__uint_as_float(bb.y), kBoundMin) * keep, cap);
-                bnd2 = fminf(fmaxf(__uint_as_float(bb.w), kBoundMin) * keep, cap);
-              } else {
-                bnd1 = fminf(tau * keep, kBoundMax);
-                bnd2 = bnd1;
-              }
-            }
-            smax = 0.f;
-            smin = 0.f;
-            pos2 = 0;
-            pos1 = 0;
+          const float tau = tau_n, v1 = v1_n, v2 = v2_n;
+          const int ag0 = ag, tt0 = tt;
+          if (++tt == g_ntt) {
+            tt = 0;
+            ++ag;
           }
-          for (int c0 = 0; c0 < nc_item; c0 += 2) {
-            const int c = c0 + h;
+          tau_n = g_tau[tt * kTileM];  // (past the last step: a row that exists, unused)
+          ntlo = -tau * (1.f - p.margin);
+          if constexpr (kNan) {
+            const int nan_c = (int)nan_n;
+            if (g_nan) nan_n = g_nan[tt * kTileM + row];
+            const int nset = nan_c == 0 ? 0 : (nan_c <= kNanCMax ? nan_set_of(nan_c) + 1 : -1);
+            const int wset = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(nset, 0));
+            const bool mixed = __any_sync(0xffffffffu, nset >= 0 && nset != wset);
+            nsw = (nset + 1) | (wset << 4) | (mixed ? 256 : 0) | (nan_c << 9);
+            // (a trait beyond the last set: +inf lets every pair through)
+            if (nset < 0 && tau < kBoundMax) ntlo = __int_as_float(0x7f800000);
+          }
+          if constexpr (kTwo || kSeed)
+            if (step + 1 < w.step_end) class_values(g, ag, tt * kTileM + row, v1_n, v2_n);
+          if constexpr (kTwo) {
+            // unpermuted group: both classes against tau (less the margin); a
+            // permuted one: the classes' largest decided values
+            const float keep = 1.f - p.margin;
+            if (ag0 > 0) {
+              const float cap = p.fdr_hist != nullptr ? fminf(tau * keep, kBoundMax) : kBoundMax;
+              bnd1 = fminf(fmaxf(v1, kBoundMin) * keep, cap);
+              bnd2 = fminf(fmaxf(v2, kBoundMin) * keep, cap);
+            } else {
+              bnd1 = fminf(tau * keep, kBoundMax);
+              bnd2 = bnd1;
+            }
+          }
+          smax = 0.f;
+          smin = 0.f;
+          pos2 = 0;
+          pos1 = 0;
+          for (int c = h; c - h < nc_item; c += 2) {
             if (c < nc_item) {
-              if (!pair_slot(ps, ps_phase, smeta[c], c, chunk0, tcp, step, g_ntt, w.group))
+              if (!pair_slot(ps, ps_phase, smeta[c], c, chunk0, g, ag0, tt0, w.group))
                 goto epi_done_scan;
             } else {  // an odd last chunk leaves warps 8-15 idle: release only
-              if (!__all_sync(0xffffffffu, wait_bar_p(t_full(ps), ps_phase, p, abort_addr, 7)))
-                goto epi_done_scan;
+              if (!wait_warp(t_full(ps), ps_phase, p, abort_addr, 7)) goto epi_done_scan;
               tc_fence_after();
               tc_fence_before();
               __syncwarp();
-              if (lane == 0) mbar_arrive(t_empty(ps));
+              mbar_arrive_lane0(t_empty(ps), lane);
             }
             ps ^= 1u;
             if (ps == 0u) ps_phase ^= 1u;
           }
           if constexpr (kSeed) {
             // the step's largest values and their blocks (the largest over all steps
-            // is decided exactly after the launch), written only past the record
-            // staged for the step
-            const int ag = step / g_ntt, trait = (step - ag * g_ntt) * kTileM + row;
-            if (ag > 0 && trait < g.T) {
-              const uint4 bb = reinterpret_cast<const uint4 *>(tcp + 1536)[row];
+            // is decided exactly after the launch), written only past the record read
+            // before the step
+            const int trait = tt0 * kTileM + row;
+            if (ag0 > 0 && trait < g.T) {
               unsigned long long *rp =
-                  g.minp_seed + 2 * ((int64_t)(ag - 1) * g.rows_per_agroup + trait);
-              if (-smin > __uint_as_float(bb.y))
+                  g.minp_seed + 2 * ((int64_t)(ag0 - 1) * g.rows_per_agroup + trait);
+              if (-smin > v1)
                 atomicMax(rp, ((unsigned long long)__float_as_uint(-smin) << 32) | (uint32_t)(pos1 + 1));
-              if (smax > __uint_as_float(bb.w))
+              if (smax > v2)
                 atomicMax(rp + 1, ((unsigned long long)__float_as_uint(smax) << 32) | (uint32_t)(pos2 + 1));
             }
-          }
-          __syncwarp();
-          if (lane == 0) mbar_arrive(tc_empty(tc_e));
-          if (++tc_e == (uint32_t)kTcDepth) {
-            tc_e = 0;
-            tc_phase ^= 1u;
           }
         }
         // the chunks' metadata is no longer needed
@@ -2456,7 +2472,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         if constexpr (kForm == kFormPerm) ++step_tag;
         // this step's trait constants, staged by the producer
         if (!__all_sync(0xffffffffu, wait_bar(tc_full(tc_e), tc_phase, wc, 9))) goto epi_done;
-        const uint8_t *tcp = stc + (size_t)tc_e * kTc;
+        const uint8_t *tcp = stc + (size_t)tc_e * kTcBytes;
         const int row = 32 * q + lane;
         EpiTrait et;
         et.trait = tt * kTileM + row;
@@ -2465,7 +2481,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         et.ntlo = -tau * (1.f - p.margin);
         et.nthi = -tau * (1.f + p.margin);
         et.cfac = reinterpret_cast<const double *>(tcp + 512)[row];
-        et.nan_cnt = g_has_nan ? (int)reinterpret_cast<const uint16_t *>(tcp + kTcNan)[row] : 0;
+        et.nan_cnt = g_has_nan ? (int)reinterpret_cast<const uint16_t *>(tcp + 2560u)[row] : 0;
         et.nan_idx = g_has_nan && et.valid
                          ? g.nan_idx + ag * g.nan_ag_stride + (int64_t)et.trait * g_N
                          : nullptr;
