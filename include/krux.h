@@ -92,7 +92,8 @@ typedef struct {
   int32_t scan_form;    /* kernel form of the fused scan launch: 0 plain, 1 markers with up to
                            five groups, 2 permutation batch, 3 general (dense, cis, NaN
                            beyond the plain form's coefficient sets), 4 plain permutation
-                           batch, 5 plain with NaN expression */
+                           batch, 5 plain with NaN expression, 7 plain over pairs of CTAs
+                           (large sample counts) */
   int32_t reserved_;
 } krux_profile;
 

@@ -56,7 +56,7 @@ cudaError_t launch_pack_batch(const PackJob *jobs, int n_jobs, int64_t total_slo
                               int64_t total_halves, double h1, double h2, int signed_df1,
                               unsigned int *status, cudaStream_t s);
 cudaError_t launch_rerank_buckets(const RerankJob *djobs, const RerankJob *hjobs,
-                                  const int32_t *drops, int n_jobs, cudaStream_t s);
+                                  const int32_t *drops, int n_jobs, bool tiled, cudaStream_t s);
 cudaError_t launch_plain_epilogue2(const float *C, int64_t ldc, int T, int n_slots,
                                    const ChunkMeta *meta, const float *tau, const double *cfac,
                                    const uint16_t *nan_cnt, const uint16_t *nan_idx, int N,
@@ -269,20 +269,30 @@ krux_status encode_map(krux_ctx *ctx, CUtensorMap *map, const void *base, int Np
 // split into blocks, so that its accumulators stay double-buffered).
 struct LaunchShape {
   int ka = 0, nA = 0, b_region = 0, force_nc = 0, no_pair = 0;
+  bool plain = false;  // picked for the plain forms: chunk pairs only
+  bool pair_cta = false;  // for the plain form over pairs of CTAs: one chunk in each
 };
 constexpr size_t kSmemLimit = 232448;
 // Shared memory of the plain forms beyond the general one's: the hit-event ring, less
 // what they do without.
-constexpr size_t kPlainExtra = kEvRegion - kFastSaved;
+constexpr size_t kPlainExtra = ev_region(kEvEntries) - kFastSaved;
+constexpr size_t kPairSaved = ev_region(kEvEntries) - ev_region(kEvEntriesPair);
 
 size_t shape_overhead(int nA, int codes_k) {
   return scan_smem_bytes2(kTmemSlots, nA, 0, 0, std::max(codes_k, 16));
 }
 
+// Whether complete data of this width go to pairs of CTAs where the whole K does not
+// fit a rank stage beside a chunk pair (up to 192 samples it does).  Below 240 a single
+// CTA with K blocks still has room for three long stages (15,000 x 200,000: N = 200 1.49
+// against 1.61 ms, N = 224 1.54 against 1.67); from there it has not (N = 240 1.78
+// against 1.68, N = 256 2.00 against 1.75, N = 320 3.10 against 2.07).
+bool pair_cta_wanted(int kpad) { return kpad >= 240 && pair_clusters() > 0; }
+
 // reserve: shared memory kept free for the plain form's hit-event ring (0 when
 // the call cannot take that form).
 bool pick_launch_shape(const krux_ctx *ctx, int kpad, int codes_k, LaunchShape &sh,
-                       size_t reserve = 0) {
+                       size_t reserve = 0, bool pair_cta = false) {
   const size_t chunk = (size_t)256 * kpad;
   if (ctx->tune_nc > 0) {  // explicit shape (tests, autotuner)
     sh.ka = ctx->tune_ka > 0 ? ctx->tune_ka : kpad;
@@ -292,8 +302,10 @@ bool pick_launch_shape(const krux_ctx *ctx, int kpad, int codes_k, LaunchShape &
     if (sh.ka % 64 != 0 && sh.ka != kpad) return false;
     return shape_overhead(sh.nA, codes_k) + (size_t)sh.nA * 256 * sh.ka + sh.b_region <= kSmemLimit;
   }
-  if (reserve > 0) {  // the plain form: whole K per stage and an even number of chunks
+  if (reserve > 0) {
+    // the plain form: whole K per stage and an even number of chunks
     int best = 0;
+    sh.plain = true;
     for (int a = 3; a >= 2; --a) {
       const size_t used = shape_overhead(a, codes_k) + (size_t)a * chunk + reserve;
       if (used >= kSmemLimit) continue;
@@ -306,6 +318,24 @@ bool pick_launch_shape(const krux_ctx *ctx, int kpad, int codes_k, LaunchShape &
       }
     }
     if (best >= 2) return true;
+    // or one resident pair (in one CTA, or a chunk in each of two) and K in the fewest
+    // equal blocks that leave three stages, four in a pair of CTAs, whose second CTA's
+    // operands are announced a little later
+    const int held = pair_cta ? 1 : 2;
+    const size_t fixed = scan_smem_bytes2(2, 8, 0, 0, std::max(codes_k, 16)) + held * chunk + reserve -
+                         (pair_cta ? kPairSaved : 0);
+    const int atoms = kpad / 16;
+    for (int blocks = pair_cta ? 1 : 2; fixed < kSmemLimit && blocks <= atoms; ++blocks) {
+      const int ka = 16 * ((atoms + blocks - 1) / blocks);
+      const int a = (int)std::min<size_t>(8, (kSmemLimit - fixed) / (256 * (size_t)ka));
+      if (a < (pair_cta ? 4 : 3) || (pair_cta && ka > 128)) continue;  // (a box: 8 atoms at most)
+      sh.ka = ka;
+      sh.nA = a;
+      sh.b_region = (int)(held * chunk);
+      sh.pair_cta = pair_cta;
+      return true;
+    }
+    sh.plain = false;
   }
   for (int a = 3; a >= 2; --a) {  // whole K per stage
     const size_t used = shape_overhead(a, codes_k) + (size_t)a * chunk;
@@ -333,17 +363,28 @@ bool pick_launch_shape(const krux_ctx *ctx, int kpad, int codes_k, LaunchShape &
   return best_nc >= 1;
 }
 
-// True when a group of this width can take the plain scan form: a launch shape
-// with the whole K per rank stage, an even number of resident chunks and room for
-// the hit-event ring (the 32-byte swizzle layout).
-bool plain_form_fits(const krux_ctx *ctx, int Np) {
-  if (ctx->tune_layout == 0) return false;
+// Whether a group of this width can take the plain scan form (the 32-byte swizzle
+// layout, an even number of resident chunks, room for the hit-event ring): 2 with the
+// whole K per rank stage, 1 with K blocks, 0 not.
+int plain_form_fits(const krux_ctx *ctx, int Np) {
+  if (ctx->tune_layout == 0) return 0;
   const int kpad = round_up(Np, 16);
   LaunchShape sh;
-  if (!pick_launch_shape(ctx, kpad, 0, sh, kPlainExtra)) return false;
+  if (!pick_launch_shape(ctx, kpad, 0, sh, kPlainExtra, pair_cta_wanted(kpad))) return 0;
+  if (sh.pair_cta) return 1;
   const int nc = (int)(sh.b_region / (256 * kpad));
-  return sh.ka == kpad && nc >= 2 && nc % 2 == 0 &&
-         shape_overhead(sh.nA, 0) + (size_t)sh.nA * 256 * sh.ka + sh.b_region + kPlainExtra <= kSmemLimit;
+  if (nc < 2 || nc % 2 != 0 ||
+      shape_overhead(sh.nA, 0) + (size_t)sh.nA * 256 * sh.ka + sh.b_region + kPlainExtra > kSmemLimit)
+    return 0;
+  return sh.ka == kpad ? 2 : (sh.plain ? 1 : 0);
+}
+
+// The weights of the plain forms' rows, between sqrt(1 / (512 h)) and sqrt(2 / h)
+// (and the rounding on top), are FP16 normals well inside the range for every P_c
+// but those near 1, where h falls to zero: those calls take the general form.
+bool pq_range_ok(double h1, double h2) {
+  const double lo = std::min(h1, h2), hi = std::max(h1, h2);
+  return lo > 0.0 && std::sqrt(2.0 / lo) < 16384.0 && std::sqrt(1.0 / (kMaxN * hi)) > 1.0 / 4096.0;
 }
 
 // Refuses a launch plan whose shared-memory regions or per-group shapes are not
@@ -363,7 +404,9 @@ std::string validate_plan(const ScanParams &p, const std::vector<GroupDesc> &g, 
   if ((size_t)p.nA * p.a_tile_bytes + (size_t)p.b_region + 1024 > smem) return bad("regions exceed the allocation");
   for (const GroupDesc &d : g) {
     if (d.nc < 1 || d.nc > p.nc) return bad("group chunk count");
-    if (d.b_stride % 4096 || (int64_t)d.nc * d.b_stride > p.b_region) return bad("group B chunks");
+    if (d.b_stride % 4096 || (int64_t)(p.pair_cta ? 1 : d.nc) * d.b_stride > p.b_region)
+      return bad("group B chunks");
+    if (p.pair_cta && (d.nc != 2 || d.n_agroups > 1 || p.next != nullptr)) return bad("pairs of CTAs");
     if (d.b_stride < 256 * d.n_atoms * atom) return bad("group B stride");
     if ((int64_t)d.nkb * p.ka < (int64_t)d.n_atoms * atom || d.nkb < 1) return bad("group K blocks");
     if (d.nkb > 1 && d.nc * 2 > kTmemSlots) return bad("TMEM slots for K blocks");
@@ -380,8 +423,14 @@ void group_shape(const LaunchShape &sh, int kpad_g, int atom, GroupDesc &d) {
   const int atoms_per_block = sh.ka / atom;
   d.nkb = (d.n_atoms + atoms_per_block - 1) / atoms_per_block;
   int nc = (int)std::min<int64_t>(kTmemSlots, sh.b_region / d.b_stride);
+  if (sh.pair_cta) {
+    d.nc = 2;
+    d.pair = 1;
+    return;
+  }
   if (d.nkb > 1) nc = std::min(nc, 2);
   if (sh.force_nc > 0) nc = std::min(nc, sh.force_nc);
+  if (sh.plain && nc >= 2) nc &= ~1;
   d.nc = std::max(nc, 1);
   // N = 256 MMAs over chunk pairs (32-byte swizzle layout, even chunk count)
   d.pair = (atom == 16 && d.nc >= 2 && d.nc % 2 == 0 && !sh.no_pair) ? 1 : 0;
@@ -507,6 +556,7 @@ krux_status alloc_rankset(krux_ctx *ctx, krux_rankset *rs, int T, int N, bool wi
     return o;
   };
   const size_t oA = take((size_t)rs->rows_pad * rs->Np * 2);
+  const size_t oAt = take((size_t)rs->rows_pad * rs->Np * 2);
   const size_t olo = with_lists ? take((size_t)T * N * 2) : 0;
   const size_t oeq = with_lists ? take((size_t)T * N * 2) : 0;
   const size_t otie = take((size_t)T * 8);
@@ -528,6 +578,7 @@ krux_status alloc_rankset(krux_ctx *ctx, krux_rankset *rs, int T, int N, bool wi
   rs->bytes = off;
   char *b = (char *)rs->mem;
   rs->dev.A = (__half *)(b + oA);
+  rs->dev.At = (__half *)(b + oAt);
   rs->dev.lo = with_lists ? (uint16_t *)(b + olo) : nullptr;
   rs->dev.eq = with_lists ? (uint16_t *)(b + oeq) : nullptr;
   rs->dev.tie = (int64_t *)(b + otie);
@@ -687,7 +738,10 @@ krux_status krux_rank(krux_ctx *ctx, const float *expr, int T, int N, int64_t ld
     return st;
   }
   ev_record(ctx, 0, s);
-  cudaError_t e = cudaMemsetAsync(rs->dev.A, 0, (size_t)rs->rows_pad * rs->Np * 2, s);
+  // (the rows past T of the last tile stay zero in both layouts)
+  const size_t tile0 = (size_t)(T / kTileM) * kTileM * rs->Np, tail = (size_t)rs->rows_pad * rs->Np - tile0;
+  cudaError_t e = tail ? cudaMemsetAsync(rs->dev.A + tile0, 0, tail * 2, s) : cudaSuccess;
+  if (e == cudaSuccess && tail) e = cudaMemsetAsync(rs->dev.At + tile0, 0, tail * 2, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(rs->dev.tile_nan, 0, (size_t)rs->n_ttiles * 4, s);
   if (e == cudaSuccess) e = launch_rank(expr, T, N, ld, rs->Np, rs->rows_pad, rs->dev, s);
   ev_record(ctx, 1, s);
@@ -964,6 +1018,7 @@ struct OutSlot {
 struct ScanGroupIn {
   const krux_rankset *rs = nullptr;  // geometry (T, N, Np, rows_pad)
   const __half *A = nullptr;         // n_agroups stacked rank matrices of rows_pad rows
+  const __half *At = nullptr;        // the same in the plain forms' layout
   int n_agroups = 1;
   const float *tau = nullptr;
   const double *cfac = nullptr;
@@ -1003,6 +1058,10 @@ struct CallPlan {
   std::vector<int64_t> lists;         // host copy of all SNP lists
   std::vector<BucketJob> bucket_jobs;
   std::vector<krux_rankset> bucket_sets;  // host shells of the re-ranked sets
+  std::vector<RerankJob> rerank_hjobs;    // their job table, on the host and the device
+  const RerankJob *rerank_djobs = nullptr;
+  const int32_t *rerank_drops = nullptr;
+  bool rerank_tiled = false;              // the layout the matrices were last written in
   struct PermJob {  // permutation batch: the stacked, permuted rank matrices
     bool on = false;
     const krux_rankset *rs = nullptr;
@@ -1080,6 +1139,7 @@ krux_status plan_groups(krux_ctx *ctx, CallPlan &cp, const krux_rankset *rs, con
   ScanGroupIn g0;
   g0.rs = rs;
   g0.A = A ? A : rs->dev.A;
+  g0.At = A ? A : rs->dev.At;  // (a stack or a bucket's matrix is written in the form's layout)
   g0.n_agroups = n_agroups;
   g0.tau = rs->dev.tau;
   g0.cfac = rs->dev.cfac;
@@ -1217,7 +1277,14 @@ krux_status materialise(krux_ctx *ctx, CallPlan &cp, cudaStream_t s) {
   int32_t *ddrop = reinterpret_cast<int32_t *>(base + drop_off);
   KRUX_CUDA(ctx, cudaMemcpyAsync(djobs, jobs.data(), nb * sizeof(RerankJob), cudaMemcpyHostToDevice, s));
   KRUX_CUDA(ctx, cudaMemcpyAsync(ddrop, drops.data(), drops.size() * 4, cudaMemcpyHostToDevice, s));
-  KRUX_CUDA(ctx, launch_rerank_buckets(djobs, jobs.data(), ddrop, (int)nb, s));
+  // most calls with buckets take the plain form: their matrices are written in its
+  // layout now, beside the host's planning, and again (enqueue_fused) if not
+  cp.rerank_hjobs = jobs;
+  cp.rerank_djobs = djobs;
+  cp.rerank_drops = ddrop;
+  cp.rerank_tiled = !cp.multi && !cp.cis.on && cp.slots.size() == 1 && ctx->tune_layout != 0 &&
+                    cp.groups[0].dense_H == nullptr;
+  KRUX_CUDA(ctx, launch_rerank_buckets(djobs, jobs.data(), ddrop, (int)nb, cp.rerank_tiled, s));
   if (ctx->profiling) ctx->prof.launches += 1;
   // runs of buckets of the same rank set: one A map each
   std::vector<size_t> run(nb);
@@ -1233,6 +1300,7 @@ krux_status materialise(krux_ctx *ctx, CallPlan &cp, cudaStream_t s) {
     g.a_map_rows = run_rows[r];
     g.a_row0 = (int64_t)((aoff[(size_t)g.bucket] - aoff[r]) / ((size_t)bs.Np * 2));
     g.A = bs.dev.A;
+    g.At = bs.dev.A;
     g.tau = bs.dev.tau;
     g.cfac = bs.dev.cfac;
     g.tile_nan = bs.dev.tile_nan;
@@ -1275,14 +1343,6 @@ std::vector<WorkItem> make_items_cis(const CallPlan &cp, const std::vector<Group
     }
   }
   return items;
-}
-
-// The weights of the plain forms' rows, between sqrt(1 / (512 h)) and sqrt(2 / h)
-// (and the rounding on top), are FP16 normals well inside the range for every P_c
-// but those near 1, where h falls to zero: those calls take the general form.
-bool pq_range_ok(double h1, double h2) {
-  const double lo = std::min(h1, h2), hi = std::max(h1, h2);
-  return lo > 0.0 && std::sqrt(2.0 / lo) < 16384.0 && std::sqrt(1.0 / (kMaxN * hi)) > 1.0 / 4096.0;
 }
 
 // One fused launch, split in three phases so that the middle one can be captured
@@ -1356,7 +1416,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   // than the last set covers (each such trait sends all its pairs to the exact
   // test; beyond that share the general form is faster)
   bool fast_shape = layout == 1 && !cp.multi && cp.param.model < 0 && o->dense_H == nullptr &&
-                    !cp.cis.on;
+                    !cp.cis.on && pq_range_ok(fl.h1, fl.h2) && fast_form_ok();
   bool any_nan = false, fast_nan = allow_fast_nan && fast_shape;
   for (auto &g : cp.groups) {
     fast_nan = fast_nan && g.minp_key == nullptr &&
@@ -1377,8 +1437,10 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     ctx->tune_nc = tnc;
     ctx->tune_nA = tnA;
     ctx->tune_ka = tka;
-    const bool ok = pick_launch_shape(ctx, kpad, codes_k, sh,
-                                      fast_shape ? kPlainExtra : 0);
+    // pairs of CTAs take complete data without permutations
+    const bool pairs = fast_shape && !fast_nan && fl.signed_coef == 0 && tnc == 0 && tnA == 0 &&
+                       pair_cta_wanted(kpad);
+    const bool ok = pick_launch_shape(ctx, kpad, codes_k, sh, fast_shape ? kPlainExtra : 0, pairs);
     ctx->tune_nc = s_nc;
     ctx->tune_nA = s_nA;
     ctx->tune_ka = s_ka;
@@ -1430,6 +1492,20 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     *out = it->second;
     return KRUX_OK;
   };
+  // pairs of CTAs: a rank matrix in the plain forms' layout as rows of 128 bytes, 32 per
+  // atom, in boxes of `atoms` atoms
+  auto tile_map = [&](CUtensorMap *map, const __half *At, int Np, int n_tiles, int atoms) -> krux_status {
+    cuuint64_t dims[2] = {64, (cuuint64_t)n_tiles * Np * 2};
+    cuuint64_t strides[1] = {128};
+    cuuint32_t box[2] = {64, (cuuint32_t)(32 * atoms)};
+    cuuint32_t estr[2] = {1, 1};
+    CUresult r = ctx->encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<__half *>(At), dims,
+                             strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(ctx, KRUX_ECUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
+    return KRUX_OK;
+  };
   for (int i = 0; i < ng; ++i) {
     ScanGroupIn &g = cp.groups[i];
     const krux_rankset *rs = g.rs;
@@ -1440,7 +1516,11 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     const int64_t csn = cp.multi ? kChunkSnpsM : kChunkSnps;
     const int64_t nch = (g.n_snps + csn - 1) / csn;
     krux_status st;
-    if (g.a_map) {
+    if (sh.pair_cta) {  // (tmB: the last, shorter K block)
+      const int atoms = rs->Np / 16, block = std::min(sh.ka / 16, atoms), tail = atoms % block;
+      st = tile_map(&d.tmA, g.At, rs->Np, rs->n_ttiles, block);
+      if (st == KRUX_OK) st = tile_map(&d.tmB, g.At, rs->Np, rs->n_ttiles, tail ? tail : block);
+    } else if (g.a_map) {
       st = map_of(&d.tmA, g.a_map, rs->Np, g.a_map_rows);
       d.a_row0 = (int32_t)g.a_row0;
     } else {
@@ -1448,7 +1528,9 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     }
     if (st != KRUX_OK) return st;
     const int64_t pitch = (int64_t)rs->Np * 2;  // bytes per B row
-    if (fl.boff[i] % pitch == 0) {  // the whole B buffer as rows of this width
+    if (sh.pair_cta) {
+      // (the genotypes are copied as they lie)
+    } else if (fl.boff[i] % pitch == 0) {  // the whole B buffer as rows of this width
       st = map_of(&d.tmB, ctx->B.p, rs->Np, std::max<int64_t>(btot / pitch, 1));
       d.b_row0 = (int32_t)(fl.boff[i] / pitch);
     } else {
@@ -1457,6 +1539,8 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     if (st != KRUX_OK) return st;
     d.meta = ctx->meta.as<ChunkMeta>() + fl.moff[i];
     d.codes = g.nan_cnt ? ctx->codes.as<uint64_t>() + fl.coff[i] : nullptr;
+    d.At = g.At;
+    d.Bt = B;
     d.codes_k = g.nan_cnt ? (fast_nan ? kCoefNanRows : rs->Np) : 0;
     d.geno = g.geno;
     d.ldg = g.ldg;
@@ -1490,12 +1574,12 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     group_shape(sh, round_up(rs->Np, atom), atom, d);
     nc_max = std::max(nc_max, d.nc);
     plans[i].n_btiles = (nch + d.nc - 1) / d.nc;
-    plans[i].steps = (int64_t)g.n_agroups * rs->n_ttiles;
+    plans[i].steps = sh.pair_cta ? (rs->n_ttiles + 1) / 2 : (int64_t)g.n_agroups * rs->n_ttiles;
     if (cp.perm.seed) plans[i].step_lo = rs->n_ttiles;
     descs[i] = d;
   }
-  std::vector<WorkItem> items =
-      cp.cis.on ? make_items_cis(cp, plans) : make_items(plans, ctx->sm_count);
+  const int workers = sh.pair_cta ? std::min(pair_clusters(), ctx->sm_count / 2) : ctx->sm_count;
+  std::vector<WorkItem> items = cp.cis.on ? make_items_cis(cp, plans) : make_items(plans, workers);
   KRUX_CUDA(ctx, t_groups.ensure(sizeof(GroupDesc) * ng));
   KRUX_CUDA(ctx, t_items.ensure(sizeof(WorkItem) * std::max<size_t>(items.size(), 1)));
   // pageable uploads: staged before the calls return, so the host vectors may go
@@ -1518,7 +1602,8 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   p.n_items = (int32_t)items.size();
   // the item counters sit behind the status words, one for each launch of a call
   // (cleared with them before the first)
-  p.next = ctx->status.as<unsigned int>() + (cp.perm.seed ? 9 : 8);
+  p.pair_cta = sh.pair_cta ? 1 : 0;
+  p.next = sh.pair_cta ? nullptr : ctx->status.as<unsigned int>() + (cp.perm.seed ? 9 : 8);
   p.nc = nc_max;
   p.nA = sh.nA;
   p.kpad = std::max(codes_k, 16);
@@ -1553,15 +1638,15 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     p.cis_window = cp.cis.window;
   }
   // the plain scan form: 32-byte swizzle, every group's chunks paired and its K
-  // in one rank stage, complete data, no dense output, cis window, provisional
+  // in one rank stage (or one pair resident and its K in blocks), complete data, no dense output, cis window, provisional
   // hits, permutations or markers with more than three groups
   {
     bool fast = layout == 1 && !p.multi && (!p.has_nan || fast_nan) && !p.dense && !p.provisional &&
                 (!p.signed_coef || p.perm) && p.cis_window < 0;
-    for (const GroupDesc &d : descs) fast = fast && d.pair == 1 && d.nkb == 1;
-    p.fast = fast && pq_range_ok(fl.h1, fl.h2) && fast_form_ok() ? 1 : 0;
+    for (const GroupDesc &d : descs) fast = fast && d.pair == 1 && (d.nkb == 1 || d.nc == 2);
+    p.fast = fast && fast_shape ? 1 : 0;
   }
-  fl.grid = (int)std::min<size_t>(items.size(), (size_t)ctx->sm_count);
+  fl.grid = (int)std::min<size_t>(items.size(), (size_t)workers) * (sh.pair_cta ? 2 : 1);
   // Single hit list: every epilogue warp stages its hits in a segment of its own
   // (no atomic per hit event) and the segments are appended after the launch.
   fl.staged = fl.nslots == 1 && cp.slots[0].capacity > 0 && fl.grid > 0;
@@ -1582,10 +1667,11 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   }
   fl.smem = scan_smem_bytes2(nc_max, sh.nA, (size_t)p.a_tile_bytes, (size_t)p.b_region, p.kpad);
   if (p.fast) {  // the plain scan form also holds its ring of hit-event buffers
-    const size_t with_ring = fl.smem + kPlainExtra;
+    const size_t with_ring = fl.smem + kPlainExtra - (sh.pair_cta ? kPairSaved : 0);
     if (with_ring <= kSmemLimit) fl.smem = with_ring;
     else p.fast = 0;
   }
+  if (sh.pair_cta && !p.fast) return fail(ctx, KRUX_EUNSUPPORTED, "internal launch plan: pairs of CTAs");
   if (fast_nan && !p.fast)  // the coefficient sets need the plain form: plan again
     return prepare_fused(ctx, cp, o, fl, s, tables, false);
   p.fast_nan = fast_nan ? 1 : 0;
@@ -1665,9 +1751,10 @@ krux_status enqueue_fused(krux_ctx *ctx, CallPlan &cp, const FusedLaunch &fl, cu
     const CallPlan::PermJob &pj = cp.perm;
     const krux_rankset *rs = pj.rs;
     const size_t one = (size_t)rs->rows_pad * rs->Np;
-    KRUX_CUDA(ctx, cudaMemcpyAsync(pj.stack, rs->dev.A, one * 2, cudaMemcpyDeviceToDevice, s));
+    KRUX_CUDA(ctx, cudaMemcpyAsync(pj.stack, fl.p.fast ? rs->dev.At : rs->dev.A, one * 2,
+                                   cudaMemcpyDeviceToDevice, s));
     KRUX_CUDA(ctx, launch_permute_rows(rs->dev.A, pj.stack + one, rs->rows_pad, rs->Np, rs->N,
-                                       pj.perms, pj.P, status, s));
+                                       pj.perms, pj.P, fl.p.fast != 0, status, s));
     KRUX_CUDA(ctx, cudaMemsetAsync(ctx->minpkey.p, 0, (size_t)pj.P * rs->rows_pad * 40, s));
     if (pj.lists) {
       // NaN samples of permutation q sit at inv_q(original position)
@@ -1679,6 +1766,14 @@ krux_status enqueue_fused(krux_ctx *ctx, CallPlan &cp, const FusedLaunch &fl, cu
       KRUX_CUDA(ctx, launch_permute_nan_idx(rs->dev.nan_cnt, rs->dev.nan_idx, rs->T, rs->N, pj.inv,
                                             pj.P, pj.lists + lst, s));
     }
+  }
+  bool buckets = false;
+  for (auto &g : cp.groups) buckets = buckets || g.bucket >= 0;
+  if (buckets && cp.rerank_tiled != (fl.p.fast != 0)) {
+    cp.rerank_tiled = fl.p.fast != 0;
+    KRUX_CUDA(ctx, launch_rerank_buckets(cp.rerank_djobs, cp.rerank_hjobs.data(), cp.rerank_drops,
+                                         (int)cp.rerank_hjobs.size(), cp.rerank_tiled, s));
+    if (ctx->profiling) ctx->prof.launches += 1;
   }
   ev_record(ctx, 2, s);
   if (fl.batched_pack && !cp.perm.packed)
@@ -2225,21 +2320,25 @@ extern "C" krux_status krux_scan_grouped(krux_ctx *ctx, krux_cohort *cohorts, in
   st = materialise(ctx, cp, s);
   if (st != KRUX_OK) return st;
   // Cohorts whose every group can take the plain scan form run in one launch of
-  // that form, the others in one launch of the general form (one launch holds one
-  // form); each cohort's groups stay in one launch, so its hit list has one writer.
-  std::vector<char> plain(n_cohorts, cp.multi ? 0 : 1);
+  // that form for each of its shapes (one launch has one shape), the others in one
+  // launch of the general form; each cohort's groups stay in one launch, so its hit
+  // list has one writer.
+  constexpr int kParts = 3;
+  std::vector<int> plain(n_cohorts, cp.multi ? 0 : 2);
   for (const ScanGroupIn &g : cp.groups)
-    if (g.nan_cnt || g.bucket >= 0 || !plain_form_fits(ctx, g.rs->Np)) plain[g.out_slot] = 0;
-  CallPlan parts[2];
-  for (int k = 0; k < 2; ++k) {
+    plain[g.out_slot] = g.nan_cnt || g.bucket >= 0
+                            ? 0
+                            : std::min(plain[g.out_slot], plain_form_fits(ctx, g.rs->Np));
+  CallPlan parts[kParts];
+  for (int k = 0; k < kParts; ++k) {
     parts[k] = cp;
     parts[k].groups.clear();
   }
-  for (const ScanGroupIn &g : cp.groups) parts[plain[g.out_slot] ? 0 : 1].groups.push_back(g);
+  for (const ScanGroupIn &g : cp.groups) parts[kParts - 1 - plain[g.out_slot]].groups.push_back(g);
   std::vector<unsigned long long> total(n_cohorts, 0ull);
   float ms_scan = 0.f;
   int launches = 0;
-  for (int k = 0; k < 2; ++k) {
+  for (int k = 0; k < kParts; ++k) {
     if (parts[k].groups.empty()) continue;
     std::vector<unsigned long long> counts;
     st = run_fused(ctx, parts[k], opts, s, counts);

@@ -51,6 +51,7 @@ static_assert(4 * (kFastRegsLaunch - kFastRegsLow) >= kFastEpiWarps * (kFastRegs
 // entry's pairs (FP64 inside the band) and appends the hit records.
 constexpr int kEvSnps = kFastSnps / 2;  // 16
 constexpr int kEvEntries = 32;
+constexpr int kEvEntriesPair = 16;  // in the form over pairs of CTAs (room for rank tiles)
 // A permuted pair the event warps passed on for its FP64 -ln p, decided after the
 // launch: exact centred sums, group sizes, trait, and rank-matrix group | FDR-band
 // flag << 16.
@@ -83,7 +84,7 @@ static_assert(sizeof(EvEntry) % 16 == 0, "event entries keep 16-byte alignment")
 // shared memory of the ring: alignment slack, entries, a full barrier and a
 // release count per entry, one 64-bit word (tickets claimed in the low 40 bits,
 // epilogue warps done above)
-constexpr size_t kEvRegion = 128 + kEvEntries * sizeof(EvEntry) + kEvEntries * 8 + kEvEntries * 4 + 8;
+constexpr size_t ev_region(int entries) { return 128 + entries * (sizeof(EvEntry) + 8 + 4) + 8; }
 // Per-step trait constants staged in shared memory by the producer (one entry per
 // 128-trait tile step): tau f32 [128] @0, 3/(K(K+1)C) f64 [128] @512, starting
 // -ln p key f64 [128] @1536 (permutation batches), NaN count u16 [128] @2560; the
@@ -205,9 +206,24 @@ __device__ __forceinline__ HitAux ld_aux(const HitAux *src) {
   return a;
 }
 
+// ---- the plain forms' operand layout ---------------------------------------
+// Their rank and genotype operands lie in global memory as the tiles that the tensor
+// cores read: per 128 rows, atoms of 16 samples, each [128 rows][32 bytes] with the
+// 32-byte swizzle (the two 16-byte halves of a row exchanged where bit 2 of the row is
+// set).  A tile, or a K block of it, is one contiguous bulk copy; as boxes of a
+// row-major matrix the same tile is a request of 32 bytes per row and atom (15,000 x
+// 200,000: N = 150 1.35 -> 1.07 ms, N = 176 1.44 -> 1.25; N = 192 in this form 1.21 ms, 99 %
+// of the measured bf16 rate).
+__host__ __device__ inline int64_t tiled_index(int64_t row, int k, int Np) {
+  const int r = (int)(row & 127);
+  return (row >> 7) * (int64_t)(kTileM * Np) + (k >> 4) * 2048 + r * 16 +
+         ((((k >> 3) ^ (r >> 2)) & 1) << 3) + (k & 7);
+}
+
 // ---- rank set: everything the scan needs about one expression matrix ------
 struct RankDev {
   __half *A;            // [rows_pad][Np] centred 2*rank (0 at NaN and padding)
+  __half *At;           // the same in the plain forms' layout, or null
   uint16_t *lo;         // [T][N] #present values strictly below (for bucket re-ranks)
   uint16_t *eq;         // [T][N] #present values equal (itself included), 0 at NaN
   int64_t *tie;         // [T] sum over present samples of eq^2 - 1 = sum (t^3 - t)
@@ -225,7 +241,7 @@ struct RankDev {
 // and tile flags are the base set's own).
 struct RerankJob {
   RankDev base;             // lo, eq, K and nan_cnt are read
-  __half *A;                // [rows_pad][Np] (padding rows written as 0)
+  __half *A;                // [rows_pad][Np] (padding rows written as 0), in either layout
   int64_t *tie;             // [T]
   int32_t *K;               // [T]
   float *tau;               // [rows_pad]
@@ -259,6 +275,8 @@ struct PackJob {
 struct alignas(64) GroupDesc {
   CUtensorMap tmA;          // 2D fp16 [rowsA][Np], box {atom K, 128}, swizzled
   CUtensorMap tmB;          // 2D fp16 [nchunks*128][Np], box {atom K, 128}, swizzled
+  const __half *At;         // plain forms: the rank operand and the packed genotypes in
+  const __half *Bt;         // their layout (tiled_index), from the group's first row / chunk
   const ChunkMeta *meta;    // [nchunks]
   const uint64_t *codes;    // [nchunks][Np][2] 2-bit genotype codes (3 = missing), or null
   const float *tau;         // [T]
@@ -392,6 +410,8 @@ struct ScanParams {
   // fast_nan = 1, when at most one trait in 128 has more than kNanCMax NaN samples)
   int32_t fast = 0;
   int32_t fast_nan = 0;
+  // 1: over pairs of CTAs (steps are pairs of trait tiles, each CTA holds one chunk)
+  int32_t pair_cta = 0;
 };
 
 enum : unsigned int {
@@ -412,8 +432,10 @@ cudaError_t launch_permute_nan_idx(const uint16_t *nan_cnt, const uint16_t *nan_
 // inv[q][perms[q][k]] = k for every in-range entry.
 cudaError_t launch_invert_perms(const int32_t *perms, int P, int N, int32_t *inv, cudaStream_t s);
 // status (may be null) gets kDevBadPerm for an entry outside 0..N-1.
+// tiled: out in the plain forms' layout, else row-major as A.
 cudaError_t launch_permute_rows(const __half *A, __half *out, int rows_pad, int Np, int N,
-                                const int32_t *perms, int P, unsigned int *status, cudaStream_t s);
+                                const int32_t *perms, int P, bool tiled, unsigned int *status,
+                                cudaStream_t s);
 cudaError_t launch_scan(const ScanParams &p, int grid, size_t smem, cudaStream_t s);
 size_t scan_smem_bytes(int nc, int nA, int kpad);
 size_t scan_smem_bytes2(int nc, int nA, size_t a_tile_bytes, size_t b_region, int codes_k);
@@ -474,6 +496,8 @@ cudaError_t scan_set_smem(size_t smem);
 int scan_form_of(const ScanParams &p);
 // The plain-form kernels were built with the registers their warp split assumes.
 bool fast_form_ok();
+// Pairs of CTAs the pair form can run at one time (0: not at all).
+int pair_clusters();
 cudaError_t launch_scan_only(const ScanParams &p, int grid, size_t smem, cudaStream_t s);
 cudaError_t launch_finalize(const krux_hit *hits, const HitAux *aux, int64_t n,
                             const double *const *cfac_by_group, double *H, double *p,

@@ -560,7 +560,7 @@ pack_batch_kernel(const PackJob *__restrict__ jobs, int n_jobs, int64_t total_sl
   const int64_t c = j0 / kChunkSnps;
   const int jj0 = (int)(j0 % kChunkSnps);
   ChunkMeta &m = J.meta[c];
-  __half *B0 = J.B + (c * kChunkRows + jj0) * Np;
+  __half *Bc = J.B + c * kChunkRows * Np;
   bool any_bad = false, any_excl = false;
   // lane i: the genotype row of slot i (-1: padding of the last chunk)
   int64_t my_row = -1;
@@ -633,12 +633,12 @@ pack_batch_kernel(const PackJob *__restrict__ jobs, int n_jobs, int64_t total_sl
           write_coef_nan(reinterpret_cast<uint8_t *>(J.codes) + c * kCoefNanBytes, jj, w, rh1, rh2);
       }
     }
-    // both packed rows: item t = row r, samples 8q .. 8q + 7
-    uint4 *d0 = reinterpret_cast<uint4 *>(B0 + (int64_t)r0 * Np);
-    uint4 *d1 = reinterpret_cast<uint4 *>(B0 + (int64_t)(kChunkSnps + r0) * Np);
+    // both packed rows: item t = row r, samples 8q .. 8q + 7; the plain forms' layout
+    // is walked atom by atom, so that consecutive lanes fill consecutive rows' bytes
     for (int t0 = 0; t0 < R * per_row; t0 += 32) {
       const int t = t0 + lane;
-      const int r = (int)(((uint32_t)t * inv_row) >> 16), k8 = 8 * (t - r * per_row);
+      const int r = bits > 0 ? (t >> 1) & (R - 1) : (int)(((uint32_t)t * inv_row) >> 16);
+      const int k8 = bits > 0 ? 16 * (t >> (lgr + 1)) + 8 * (t & 1) : 8 * (t - r * per_row);
       const int ln = (r << (5 - lgr)) & 31;
       const uint32_t w0 = __shfl_sync(0xffffffffu, w.w0, ln), w1 = __shfl_sync(0xffffffffu, w.w1, ln);
       const int ob = __shfl_sync(0xffffffffu, row >= 0 ? o0 : -1, ln);
@@ -662,8 +662,11 @@ pack_batch_kernel(const PackJob *__restrict__ jobs, int n_jobs, int64_t total_sl
       const uint2 p0 = mask_to_halves(la, va), p1 = mask_to_halves(lb, vb);
       const uint2 p2 = mask_to_halves(ha, va), p3 = mask_to_halves(hb, vb);
       const uint2 q0 = mask_to_halves(lb, vg), q1 = mask_to_halves(hb, vg);
-      d0[t] = make_uint4(p0.x | p1.x, p0.y | p1.y, p2.x | p3.x, p2.y | p3.y);
-      d1[t] = make_uint4(q0.x, q0.y, q1.x, q1.y);
+      const int rp = jj0 + r0 + r, rq = kChunkSnps + rp;  // rows of the chunk
+      const int64_t ap = bits > 0 ? tiled_index(rp, k8, Np) : (int64_t)rp * Np + k8;
+      const int64_t aq = bits > 0 ? tiled_index(rq, k8, Np) : (int64_t)rq * Np + k8;
+      *reinterpret_cast<uint4 *>(Bc + ap) = make_uint4(p0.x | p1.x, p0.y | p1.y, p2.x | p3.x, p2.y | p3.y);
+      *reinterpret_cast<uint4 *>(Bc + aq) = make_uint4(q0.x, q0.y, q1.x, q1.y);
     }
     __syncwarp();
   }

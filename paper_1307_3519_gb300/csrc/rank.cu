@@ -81,6 +81,7 @@ rank_kernel(const float *__restrict__ expr, int T, int N, int64_t ld, int Np, Ra
       r.eq[(int64_t)t * N + k] = eq16;
     }
     r.A[(int64_t)t * Np + k] = __int2half_rn(a);
+    if (r.At) r.At[tiled_index(t, k, Np)] = __int2half_rn(a);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) tie += __shfl_xor_sync(0xffffffffu, tie, o);
@@ -96,26 +97,49 @@ rank_kernel(const float *__restrict__ expr, int T, int N, int64_t ld, int Np, Ra
 
 // out[p][row][k] = A[row][perm_p[k]] for k < N (padding columns stay 0): the
 // rank matrix of the expression with its sample columns permuted (ranks, tie
-// sums and K are invariant under a column permutation).
-__global__ void permute_rows_kernel(const __half *__restrict__ A, __half *__restrict__ out,
-                                    int rows_pad, int Np, int N, const int32_t *__restrict__ perms,
-                                    int P, unsigned int *status) {
-  const int64_t total = (int64_t)P * rows_pad * Np;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int k = (int)(i % Np);
-    const int64_t pr = i / Np;
-    const int row = (int)(pr % rows_pad);
-    const int p = (int)(pr / rows_pad);
-    __half v = __int2half_rn(0);
-    if (k < N) {
-      const int32_t src = perms[(int64_t)p * N + k];
-      if (src >= 0 && src < N)
-        v = A[(int64_t)row * Np + src];
-      else if (status != nullptr)
-        atomicOr(status, kDevBadPerm);
+// sums and K are invariant under a column permutation).  One block per 32 rows, its
+// rows staged in shared memory once for all permutations; a thread gathers 8
+// consecutive samples and stores 16 bytes, in either layout.  Bound by the stores
+// (72 MB for 16 x 20,000 x 102: 110 us with one 2-byte element per thread).
+constexpr int kPermRows = 32;
+template <bool kTiled>
+__global__ void __launch_bounds__(256)
+permute_rows_kernel(const __half *__restrict__ A, __half *__restrict__ out, int rows_pad, int Np,
+                    int N, const int32_t *__restrict__ perms, int P, unsigned int *status) {
+  __shared__ __align__(16) __half rows[kPermRows * kMaxN];
+  __shared__ __align__(16) int32_t perm[kMaxN];
+  const int row0 = blockIdx.x * kPermRows;  // (rows_pad is a multiple of 128)
+  const int per_row = Np / 8;
+  for (int i = threadIdx.x; i < kPermRows * per_row; i += blockDim.x)
+    reinterpret_cast<uint4 *>(rows)[i] = reinterpret_cast<const uint4 *>(A + (int64_t)row0 * Np)[i];
+  for (int p = blockIdx.y; p < P; p += gridDim.y) {
+    __syncthreads();
+    for (int k = threadIdx.x; k < Np; k += blockDim.x) {
+      int32_t src = -1;
+      if (k < N) {
+        src = perms[(int64_t)p * N + k];
+        if (src < 0 || src >= N) {
+          if (status != nullptr) atomicOr(status, kDevBadPerm);
+          src = -1;
+        }
+      }
+      perm[k] = src;
     }
-    out[i] = v;
+    __syncthreads();
+    __half *o = out + (int64_t)p * rows_pad * Np;
+    for (int i = threadIdx.x; i < kPermRows * per_row; i += blockDim.x) {
+      // tiled: consecutive threads take the halves and rows of one atom
+      const int r = kTiled ? (i >> 1) % kPermRows : i / per_row;
+      const int q = kTiled ? 2 * (i / (2 * kPermRows)) + (i & 1) : i - r * per_row;
+      __align__(16) __half v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int32_t src = perm[8 * q + j];
+        v[j] = src >= 0 ? rows[r * Np + src] : __int2half_rn(0);
+      }
+      const int64_t at = kTiled ? tiled_index(row0 + r, 8 * q, Np) : (int64_t)(row0 + r) * Np + 8 * q;
+      *reinterpret_cast<uint4 *>(o + at) = *reinterpret_cast<const uint4 *>(v);
+    }
   }
 }
 // inv[q][perms[q][k]] = k (entries outside 0..N-1 are skipped; the row gather
@@ -209,11 +233,12 @@ cudaError_t launch_permute_nan_idx(const uint16_t *nan_cnt, const uint16_t *nan_
 }
 
 cudaError_t launch_permute_rows(const __half *A, __half *out, int rows_pad, int Np, int N,
-                                const int32_t *perms, int P, unsigned int *status, cudaStream_t s) {
-  const int64_t total = (int64_t)P * rows_pad * Np;
-  int grid = (int)((total + 255) / 256);
-  if (grid > 152 * 16) grid = 152 * 16;
-  permute_rows_kernel<<<grid, 256, 0, s>>>(A, out, rows_pad, Np, N, perms, P, status);
+                                const int32_t *perms, int P, bool tiled, unsigned int *status,
+                                cudaStream_t s) {
+  if (P <= 0 || rows_pad <= 0) return cudaSuccess;
+  const dim3 grid((unsigned)(rows_pad / kPermRows), (unsigned)(P < 8 ? P : 8));
+  if (tiled) permute_rows_kernel<true><<<grid, 256, 0, s>>>(A, out, rows_pad, Np, N, perms, P, status);
+  else permute_rows_kernel<false><<<grid, 256, 0, s>>>(A, out, rows_pad, Np, N, perms, P, status);
   return cudaGetLastError();
 }
 
@@ -253,7 +278,8 @@ struct RerankOut {  // a bucket's outputs and drop list, staged per block
 // kPasses = ceil(Np / 128) passes of 4 samples per lane (the row in registers).
 template <int kPasses>
 __global__ void __launch_bounds__(kRerankWarps * 32, kPasses == 1 ? 5 : (kPasses == 2 ? 2 : 1))
-rerank_kernel(const RerankJob *__restrict__ jobs, int n_jobs_all, const int32_t *__restrict__ drops) {
+rerank_kernel(const RerankJob *__restrict__ jobs, int n_jobs_all, const int32_t *__restrict__ drops,
+              int tiled) {
   __shared__ uint32_t srow[kRerankWarps][kMaxN];  // lo | eq << 16 of the warp's row
   __shared__ RerankOut sj[kRerankChunk];
   __shared__ int32_t sdrop[kRerankDrops];          // the chunk's drop lists, when they fit
@@ -279,7 +305,8 @@ rerank_kernel(const RerankJob *__restrict__ jobs, int n_jobs_all, const int32_t 
   if (t >= T) {  // padding row: zeros, never a hit
     for (int j = 0; j < n_jobs; ++j) {
       const RerankOut &J = sj[j];
-      for (int k = lane; k < Np; k += 32) J.A[(int64_t)t * Np + k] = __int2half_rn(0);
+      for (int k = lane; k < Np; k += 32)
+        J.A[tiled ? tiled_index(t, k, Np) : (int64_t)t * Np + k] = __int2half_rn(0);
       if (lane == 0) {
         J.tau[t] = __int_as_float(0x7f800000);
         J.cfac[t] = 0.0;
@@ -348,7 +375,7 @@ rerank_kernel(const RerankJob *__restrict__ jobs, int n_jobs_all, const int32_t 
         uint2 v;
         v.x = *reinterpret_cast<const uint32_t *>(&h01);
         v.y = *reinterpret_cast<const uint32_t *>(&h23);
-        *reinterpret_cast<uint2 *>(J.A + (int64_t)t * Np + k0) = v;
+        *reinterpret_cast<uint2 *>(J.A + (tiled ? tiled_index(t, k0, Np) : (int64_t)t * Np + k0)) = v;
       }
     }
     tie = (int)__reduce_add_sync(0xffffffffu, (unsigned)tie);
@@ -372,9 +399,9 @@ rerank_kernel(const RerankJob *__restrict__ jobs, int n_jobs_all, const int32_t 
 }  // namespace
 
 // One launch per run of buckets with the same base rank set (hjobs: the host copy
-// of the device table djobs).
+// of the device table djobs).  tiled: the matrices in the plain forms' layout.
 cudaError_t launch_rerank_buckets(const RerankJob *djobs, const RerankJob *hjobs,
-                                  const int32_t *drops, int n_jobs, cudaStream_t s) {
+                                  const int32_t *drops, int n_jobs, bool tiled, cudaStream_t s) {
   for (int j0 = 0; j0 < n_jobs;) {
     int j1 = j0 + 1;
     while (j1 < n_jobs && hjobs[j1].base.lo == hjobs[j0].base.lo) ++j1;
@@ -383,11 +410,11 @@ cudaError_t launch_rerank_buckets(const RerankJob *djobs, const RerankJob *hjobs
                     (unsigned)((j1 - j0 + kRerankChunk - 1) / kRerankChunk));
     const int Np = hjobs[j0].Np;
     if (Np <= 128)
-      rerank_kernel<1><<<grid, kRerankWarps * 32, 0, s>>>(djobs + j0, j1 - j0, drops);
+      rerank_kernel<1><<<grid, kRerankWarps * 32, 0, s>>>(djobs + j0, j1 - j0, drops, tiled);
     else if (Np <= 256)
-      rerank_kernel<2><<<grid, kRerankWarps * 32, 0, s>>>(djobs + j0, j1 - j0, drops);
+      rerank_kernel<2><<<grid, kRerankWarps * 32, 0, s>>>(djobs + j0, j1 - j0, drops, tiled);
     else
-      rerank_kernel<4><<<grid, kRerankWarps * 32, 0, s>>>(djobs + j0, j1 - j0, drops);
+      rerank_kernel<4><<<grid, kRerankWarps * 32, 0, s>>>(djobs + j0, j1 - j0, drops, tiled);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     j0 = j1;

@@ -34,6 +34,9 @@ constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(128 >> 3) << 17) | ((uint32_
 // Same with N = 256: one MMA over a pair of chunks whose B rows are interleaved
 // per K atom (256 rows of 32 B), writing two adjacent 128-column accumulators.
 constexpr uint32_t kIdesc256 = (1u << 4) | ((uint32_t)(256 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+// Over a pair of CTAs (cta_group::2): M = 256 traits, 128 in each CTA, N = 256, the
+// rows of one chunk in each CTA.
+constexpr uint32_t kIdescPair = (1u << 4) | ((uint32_t)(256 >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
 // Two K-major shared-memory layouts: 128-byte swizzle with 64-element K atoms
 // (K padded to a multiple of 64, zero-filled by TMA), or 32-byte swizzle with
 // 16-element atoms (K padded to a multiple of 16 only).  An atom block holds 128
@@ -221,6 +224,90 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t da, uint64_t db
       "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// ---- the same over the two CTAs of a cluster --------------------------------
+__device__ __forceinline__ void tc_mma_pair(uint32_t d_tmem, uint64_t da, uint64_t db,
+                                            uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
+      "l"(da), "l"(db), "r"(kIdescPair), "r"(accumulate)
+      : "memory");
+}
+// a box of a tensor map into this CTA, its bytes counted on a barrier (shared::cluster
+// address) that may be the other CTA's
+__device__ __forceinline__ void tma_load_pair(uint32_t dst, const CUtensorMap *map, int x, int y,
+                                              uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2 [%0], "
+      "[%1, {%2, %3}], [%4];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
+      : "memory");
+}
+// arrives on the barrier at this offset in both CTAs
+__device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], "
+      "%1;" ::"r"(bar),
+      "h"((uint16_t)3)
+      : "memory");
+}
+// arrives on this CTA's barrier only
+__device__ __forceinline__ void tc_commit_own(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// shared::cluster address of CTA `rank`'s copy of a shared-memory address
+__device__ __forceinline__ uint32_t peer_addr(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr)
+               : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster_lane0(uint32_t cluster_addr, int lane) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.eq.s32 p, %1, 0;\n"
+      " @p mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n}" ::"r"(cluster_addr),
+      "r"(lane)
+      : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+      " selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0u;
+}
+// Bounded wait for arrivals of both CTAs.
+__device__ __forceinline__ bool wait_bar_cluster(uint32_t bar, uint32_t parity, const WaitCtl &w,
+                                                 unsigned int where) {
+  if (mbar_try_wait_cluster(bar, parity)) return true;
+  const long long t0 = clock64();
+  while (!mbar_try_wait_cluster(bar, parity)) {
+    if (*w.abort_flag) return false;
+    if (clock64() - t0 > w.limit) {
+      *w.abort_flag = 1;
+      atomicOr(w.status, kDevTimeout);
+      atomicMax(w.status + 1, where);
+      return false;
+    }
+  }
+  return true;
+}
+
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                : "memory");
@@ -996,21 +1083,23 @@ __device__ __forceinline__ void pq_sums(float P, float Q, uint32_t w0, uint32_t 
 // (uses the event warp has finished) reaching k; the uses of an entry are then
 // filled in order, and its single consumer can wait on the full barrier by phase
 // parity.
+template <int kEntries>
 struct EvRing {
   EvEntry *ent;
   uint32_t bar0;                // ev_full[e] at bar0 + 8 e
-  unsigned int *released;       // [kEvEntries] uses of each entry the event warps have finished
+  unsigned int *released;       // [kEntries] uses of each entry the event warps have finished
   unsigned long long *word;     // tickets claimed (low 40 bits), epilogue warps done (above)
   __device__ __forceinline__ uint32_t full(int e) const { return bar0 + 8u * (uint32_t)e; }
 };
 constexpr unsigned long long kEvTicketMask = (1ull << 40) - 1ull;
 
 // Bounded wait of lane 0 until the entry of ticket t is free for its use t /
-// kEvEntries; false on timeout or abort.
-__device__ __forceinline__ bool ev_gate(const EvRing &ev, unsigned long long t, const ScanParams &p,
-                                        uint32_t abort_addr) {
-  const unsigned int k = (unsigned int)(t / kEvEntries);
-  const volatile unsigned int *rel = ev.released + (t % kEvEntries);
+// kEntries; false on timeout or abort.
+template <int kEntries>
+__device__ __forceinline__ bool ev_gate(const EvRing<kEntries> &ev, unsigned long long t,
+                                        const ScanParams &p, uint32_t abort_addr) {
+  const unsigned int k = (unsigned int)(t / kEntries);
+  const volatile unsigned int *rel = ev.released + (t % kEntries);
   if (*rel >= k) return true;
   const long long t0 = clock64();
   while (*rel < k) {
@@ -1032,7 +1121,8 @@ __device__ __forceinline__ bool ev_gate(const EvRing &ev, unsigned long long t, 
 // candidate to the event warps: one entry per such trait lane (tickets claimed
 // together), each with that lane's kEvSnps accumulator pairs and constants and the
 // SNPs' metadata (written by lanes 0..kEvSnps-1).  False if a wait gave up.
-__device__ __forceinline__ bool ev_submit(const EvRing &ev, const uint32_t (&u)[kEvSnps],
+template <int kEntries>
+__device__ __forceinline__ bool ev_submit(const EvRing<kEntries> &ev, const uint32_t (&u)[kEvSnps],
                                           const uint32_t (&v)[kEvSnps], bool need,
                                           const ChunkMeta &m, int off, float tau, double cfac,
                                           int trait, int group, int ag, float b1, float b2,
@@ -1058,7 +1148,7 @@ __device__ __forceinline__ bool ev_submit(const EvRing &ev, const uint32_t (&u)[
       __threadfence_block();  // the event warp's reads of the old contents come first
     }
     if (!__shfl_sync(0xffffffffu, ok, 0)) return false;
-    const int e = (int)(t % kEvEntries);
+    const int e = (int)(t % kEntries);
     EvEntry &E = ev.ent[e];
     if (lane < kEvSnps) {
       E.alpha[lane] = al;
@@ -1688,13 +1778,28 @@ enum ScanForm {
   kFormNan = 3,
   kFormScanPerm = 4,
   kFormScanNan = 5,
-  kFormScanSeed = 6
+  kFormScanSeed = 6,
+  kFormScanPair = 7
 };
 // the plain scan form, its two passes over permutation batches (the largest values
-// first, then the pairs against them) and its variant for expression with NaN
+// first, then the pairs against them), its variant for expression with NaN, and the
+// one over pairs of CTAs
 constexpr bool fast_form(int f) {
-  return f == kFormScan || f == kFormScanPerm || f == kFormScanNan || f == kFormScanSeed;
+  return f == kFormScan || f == kFormScanPerm || f == kFormScanNan || f == kFormScanSeed ||
+         f == kFormScanPair;
 }
+// The plain form over clusters of two CTAs, for sample counts whose chunk pair leaves
+// one CTA's shared memory too little room for rank tiles in flight: the pair's tensor
+// cores contract 256 traits with a chunk pair, each CTA holding 128 traits' rank tiles
+// and one chunk, so a rank tile is still read once per 128 SNPs.  An MMA is issued by
+// the first CTA (cta_group::2) and fills both CTAs' accumulators, 128 traits x 128 SNPs
+// in each, which the epilogue reads as in the plain form.  The second CTA's chunk is
+// announced by its otherwise idle MMA warp; its rank tiles count on the first CTA's
+// barriers themselves.  15,000 x 200,000: N = 256
+// 2.00 ms with a pair in one CTA -> 1.75, N = 300 3.06 -> 2.01; N = 400 and 500, which do
+// not fit one CTA, 9.02 -> 2.66 and 10.35 -> 3.42 ms (93 % of the measured bf16 rate)
+// against the general form.
+constexpr bool pair_form(int f) { return f == kFormScanPair; }
 
 // Warp roles of a kernel form: the epilogue warps first, then the producer and
 // the MMA issuer (the plain scan form also has two idle warps after them).
@@ -1768,29 +1873,33 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
     }
   };
   // plain scan form: the ring of hit-event buffers after everything else
-  EvRing ev;
+  constexpr int kEv = pair_form(kForm) ? kEvEntriesPair : kEvEntries;
+  EvRing<kEv> ev;
   {
     uint8_t *evr = reinterpret_cast<uint8_t *>(
         (reinterpret_cast<uintptr_t>(tmem_holder) + 32u + 127u) & ~(uintptr_t)127u);
     ev.ent = reinterpret_cast<EvEntry *>(evr);
-    ev.bar0 = smem_u32(evr + kEvEntries * sizeof(EvEntry));
-    ev.released = reinterpret_cast<unsigned int *>(evr + kEvEntries * sizeof(EvEntry) + kEvEntries * 8);
-    ev.word = reinterpret_cast<unsigned long long *>(evr + kEvEntries * sizeof(EvEntry) +
-                                                     kEvEntries * 8 + kEvEntries * 4);
+    ev.bar0 = smem_u32(evr + kEv * sizeof(EvEntry));
+    ev.released = reinterpret_cast<unsigned int *>(evr + kEv * sizeof(EvEntry) + kEv * 8);
+    ev.word = reinterpret_cast<unsigned long long *>(evr + kEv * sizeof(EvEntry) +
+                                                     kEv * 8 + kEv * 4);
   }
 
+  constexpr bool kPair = pair_form(kForm);
+  const uint32_t rank = kPair ? cluster_rank() : 0u;  // 0: issues the MMAs
   if (threadIdx.x == 0) {
     for (int s = 0; s < nA; ++s) {
       mbar_init(a_full(s), 1);
       mbar_init(a_empty(s), 1);
     }
     for (int c = 0; c < nc; ++c) {
-      mbar_init(b_full(c), 1);
+      // (a pair's first CTA also counts the second's word that its chunk is there)
+      mbar_init(b_full(c), kPair && rank == 0u ? 2 : 1);
       mbar_init(b_empty(c), 1 + R::kEpi);
     }
     for (int s = 0; s < kTmemSlots; ++s) {
       mbar_init(t_full(s), 1);
-      mbar_init(t_empty(s), R::kEpi);
+      mbar_init(t_empty(s), kPair ? 2 * R::kEpi : R::kEpi);
     }
     mbar_init(drain, 1);
     for (int e = 0; e < kTcDepth; ++e) {
@@ -1803,7 +1912,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
     }
     *abort_flag = 0;
     if constexpr (fast_form(kForm)) {
-      for (int e = 0; e < kEvEntries; ++e) {
+      for (int e = 0; e < kEv; ++e) {
         mbar_init(ev.full(e), 1);
         ev.released[e] = 0u;
       }
@@ -1812,16 +1921,25 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  if constexpr (kPair) cluster_sync();  // both CTAs run and their barriers exist
   if (warp == R::kMma) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
-                     smem_u32(tmem_holder))
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (kPair) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
+                       smem_u32(tmem_holder))
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
+                       smem_u32(tmem_holder))
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   if constexpr (!fast_form(kForm))
     for (int i = threadIdx.x; i < 2 * kTileM; i += blockDim.x) sbound[i] = 0ull;
   tc_fence_before();
   __syncthreads();
+  if constexpr (kPair) cluster_sync();  // both allocations stand before the first MMA
   tc_fence_after();
   const uint32_t tmem_base = *tmem_holder;
   const WaitCtl wc{abort_flag, p.status, p.timeout_cycles};
@@ -1836,8 +1954,11 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       uint32_t a_used = 0, a_last = 0, b_used = 0, b_last = 0;
       uint32_t tc_e = 0, tc_phase = 0, tc_used = 0, tc_last = 0;
       ItemPos ip;
-      for (int it = blockIdx.x;;
-           it = p.next ? (int)(gridDim.x + atomicAdd(p.next, 1u)) : it + (int)gridDim.x) {
+      // (the two CTAs of a pair take the same items, in fixed turns)
+      for (int it = kPair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;;
+           it = kPair    ? it + (int)(gridDim.x >> 1)
+                : p.next ? (int)(gridDim.x + atomicAdd(p.next, 1u))
+                         : it + (int)gridDim.x) {
         if (!wait_bar(it_empty(ip.e), ip.phase ^ 1u, wc, 18)) goto producer_done;
         item_ring[ip.e] = it;
         mbar_arrive(it_full(ip.e));  // (release: the item is visible to who waits for it)
@@ -1845,8 +1966,10 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         if (it >= p.n_items) break;
         const WorkItem w = p.items[it];
         const GroupDesc *g = p.groups + w.group;
-        prefetch_map(&g->tmA);
-        prefetch_map(&g->tmB);
+        if constexpr (!fast_form(kForm) || kPair) {
+          prefetch_map(&g->tmA);
+          prefetch_map(&g->tmB);
+        }
         const int ncg = g->nc;
         const int nc_item = min(ncg, g->nchunks - w.btile * ncg);
         const uint32_t b_stride = (uint32_t)g->b_stride;
@@ -1854,7 +1977,22 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         const int ak = (int)atom_k(p.layout);
         const uint32_t b_tx = (uint32_t)g->n_atoms * abytes;
         const uint32_t codes_bytes = g->codes ? (uint32_t)g->codes_k * 16u : 0u;
-        for (int c = 0; c < nc_item; ++c) {
+        if constexpr (kPair) {
+          // this CTA's chunk of the pair, and both chunks' metadata
+          const uint32_t ph = b_bits & 1u;
+          if (!wait_bar(b_empty(0), ph ^ 1u, wc, 1)) goto producer_done;
+          const int chunk = w.btile * 2;
+          const bool own = (int)rank < nc_item;
+          mbar_expect_tx(b_full(0), (own ? b_tx : 0u) + (uint32_t)nc_item * (uint32_t)sizeof(ChunkMeta));
+          if (own)
+            bulk_load(sB, g->Bt + (int64_t)(chunk + (int)rank) * kChunkRows * g->Np, b_tx, b_full(0));
+          bulk_load(smem_u32(smeta), g->meta + chunk, (uint32_t)nc_item * (uint32_t)sizeof(ChunkMeta),
+                    b_full(0));
+          b_used |= 1u;
+          b_last = ph;
+          b_bits ^= 1u;
+        }
+        for (int c = 0; c < nc_item && !kPair; ++c) {
           const uint32_t ph = (b_bits >> c) & 1u;
           if (!wait_bar(b_empty(c), ph ^ 1u, wc, 1)) goto producer_done;
           const int chunk = w.btile * ncg + c;
@@ -1863,9 +2001,15 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
           const uint32_t bbase = g->pair ? sB + (uint32_t)(c >> 1) * 2u * b_stride + (uint32_t)(c & 1) * abytes
                                          : sB + (uint32_t)c * b_stride;
           const uint32_t astep = g->pair ? 2u * abytes : abytes;
-          for (int a = 0; a < g->n_atoms; ++a)
-            tma_load_2d(bbase + (uint32_t)a * astep, &g->tmB, a * ak, g->b_row0 + chunk * kChunkRows,
-                        b_full(c));
+          if constexpr (fast_form(kForm)) {
+            const __half *src = g->Bt + (int64_t)chunk * kChunkRows * g->Np;
+            for (int a = 0; a < g->n_atoms; ++a)
+              bulk_load(bbase + (uint32_t)a * astep, src + a * 2048, abytes, b_full(c));
+          } else {
+            for (int a = 0; a < g->n_atoms; ++a)
+              tma_load_2d(bbase + (uint32_t)a * astep, &g->tmB, a * ak, g->b_row0 + chunk * kChunkRows,
+                          b_full(c));
+          }
           bulk_load(smem_u32(smeta + c), g->meta + chunk, (uint32_t)sizeof(ChunkMeta), b_full(c));
           if (codes_bytes)
             bulk_load(smem_u32(scodes + (size_t)c * codes_stride), g->codes + (size_t)chunk * g->codes_k * 2,
@@ -1875,6 +2019,54 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
           b_bits ^= 1u << c;
         }
         const int atoms_per_block = p.ka / ak;
+        if constexpr (fast_form(kForm)) {
+          // the rank tiles lie in step order; the descriptor's fields stay in registers
+          // (every barrier operation and copy would have them read again)
+          const int n_atoms = g->n_atoms;
+          const __half *tile = g->At + (int64_t)w.step_begin * (kTileM * g->Np);
+          if constexpr (kPair) {
+            // a pair's step is two tiles, one per CTA (an odd last one: the same twice);
+            // both CTAs' copies count on the first CTA's barrier, where the MMAs wait
+            const int last_tile = g->n_ttiles - 1, tile_rows = 32 * n_atoms;
+            for (int step = w.step_begin; step < w.step_end; ++step) {
+              const int y = min(2 * step + (int)rank, last_tile) * tile_rows;
+              for (int a0 = 0; a0 < n_atoms; a0 += atoms_per_block) {
+                if (!wait_bar(a_empty(a_stage), a_phase ^ 1u, wc, 2)) goto producer_done;
+                const int na = min(atoms_per_block, n_atoms - a0);
+                if (rank == 0u) {
+                  mbar_expect_tx(a_full(a_stage), (uint32_t)na * 8192u);
+                  a_used |= 1u << a_stage;
+                  a_last = (a_last & ~(1u << a_stage)) | (a_phase << a_stage);
+                }
+                tma_load_pair(sA + (uint32_t)a_stage * a_tile_bytes,
+                              na == atoms_per_block ? &g->tmA : &g->tmB, 0, y + 32 * a0,
+                              peer_addr(a_full(a_stage), 0u));
+                if (++a_stage == (uint32_t)nA) {
+                  a_stage = 0;
+                  a_phase ^= 1u;
+                }
+              }
+            }
+            continue;
+          }
+          for (int step = w.step_begin; step < w.step_end; ++step) {
+            for (int a0 = 0; a0 < n_atoms; a0 += atoms_per_block) {
+              if (!wait_bar(a_empty(a_stage), a_phase ^ 1u, wc, 2)) goto producer_done;
+              const int na = min(atoms_per_block, n_atoms - a0);
+              mbar_expect_tx(a_full(a_stage), (uint32_t)na * 4096u);
+              bulk_load(sA + (uint32_t)a_stage * a_tile_bytes, tile + a0 * 2048, (uint32_t)na * 4096u,
+                        a_full(a_stage));
+              a_used |= 1u << a_stage;
+              a_last = (a_last & ~(1u << a_stage)) | (a_phase << a_stage);
+              if (++a_stage == (uint32_t)nA) {
+                a_stage = 0;
+                a_phase ^= 1u;
+              }
+            }
+            tile += n_atoms * 2048;
+          }
+          continue;
+        }
         for (int step = w.step_begin; step < w.step_end; ++step) {
           const int ag = step / g->n_ttiles, tt = step - ag * g->n_ttiles;
           const int row0 = g->a_row0 + ag * g->rows_per_agroup + tt * kTileM;
@@ -1919,13 +2111,71 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         }
       }
     producer_done:
-      // let every copy this thread issued land before the CTA can exit
+      // let every copy this thread issued land before the CTA can exit (a pair of CTAs
+      // counts them together: without a timeout every copy was waited for by the MMAs,
+      // after one the pause before the exit stands in)
+      if (kPair && *abort_flag) a_used = b_used = 0u;
       for (int s = 0; s < nA; ++s)
         if ((a_used >> s) & 1u) wait_drain(a_full(s), (a_last >> s) & 1u, p.status, 10);
       for (int c = 0; c < nc; ++c)
         if ((b_used >> c) & 1u) wait_drain(b_full(c), (b_last >> c) & 1u, p.status, 11);
       for (int e = 0; e < kTcDepth; ++e)
         if ((tc_used >> e) & 1u) wait_drain(tc_full(e), (tc_last >> e) & 1u, p.status, 13);
+    }
+    __syncwarp();
+  } else if (warp == R::kMma && kPair) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFastRegsLow) : "memory");
+    if (lane == 0) {
+      uint32_t a_stage = 0, a_phase = 0, b_bits = 0, ps = 0, ps_phase = 0;
+      ItemPos ip;
+      while (true) {
+        if (!wait_bar(it_full(ip.e), ip.phase, wc, 19)) goto pair_done;
+        const int it = item_ring[ip.e];
+        mbar_arrive(it_empty(ip.e));
+        item_next(ip);
+        if (it >= p.n_items) break;
+        const WorkItem w = p.items[it];
+        const GroupDesc *g = p.groups + w.group;
+        const int ksteps = g->Np / 16;
+        const int kpb = p.ka / 16;
+        if (rank != 0u) {
+          // announce this CTA's chunk to the issuing one
+          if (!wait_bar(b_full(0), b_bits, wc, 4)) goto pair_done;
+          mbar_arrive_cluster(peer_addr(b_full(0), 0u));
+        } else {
+          if (!wait_bar_cluster(b_full(0), b_bits, wc, 4)) goto pair_done;
+          for (int step = w.step_begin; step < w.step_end; ++step) {
+            if (!wait_bar_cluster(t_empty(ps), ps_phase ^ 1u, wc, 5)) goto pair_done;
+            const uint32_t d_tmem = tmem_base + ps * 256u;
+            uint64_t db = umma_desc(sB, 1);
+            for (int k = 0; k < ksteps;) {
+              if (!wait_bar_cluster(a_full(a_stage), a_phase, wc, 3)) goto pair_done;
+              tc_fence_after();
+              uint64_t da = umma_desc(sA + a_stage * a_tile_bytes, 1);
+              for (const int k1 = min(k + kpb, ksteps); k < k1; ++k) {
+                tc_mma_pair(d_tmem, da, db, k > 0 ? 1u : 0u);
+                da += 4096u >> 4;
+                db += 4096u >> 4;
+              }
+              tc_commit_pair(a_empty(a_stage));
+              if (++a_stage == (uint32_t)nA) {
+                a_stage = 0;
+                a_phase ^= 1u;
+              }
+            }
+            tc_commit_pair(t_full(ps));
+            ps ^= 1u;
+            if (ps == 0u) ps_phase ^= 1u;
+          }
+          tc_commit_pair(b_empty(0));
+        }
+        b_bits ^= 1u;
+      }
+    pair_done:
+      if (rank == 0u) {  // all issued MMAs must finish before TMEM is released
+        tc_commit_own(drain);
+        wait_drain(drain, 0, p.status, 12);
+      }
     }
     __syncwarp();
   } else if (warp == R::kMma && fast_form(kForm)) {
@@ -1948,6 +2198,42 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         const int nc_item = min(ncg, g->nchunks - w.btile * ncg);
         const uint32_t b_stride = (uint32_t)g->b_stride;
         const int ksteps = g->Np / 16;
+        if (g->nkb > 1) {
+          // one resident pair, its K in blocks of p.ka samples per rank stage
+          const bool two = nc_item > 1;
+          const uint32_t idesc = two ? kIdesc256 : kIdesc;
+          const int kpb = p.ka / 16;
+          if (!wait_bar(b_full(0), b_bits & 1u, wc, 4)) goto fast_mma_done;
+          if (two && !wait_bar(b_full(1), (b_bits >> 1) & 1u, wc, 4)) goto fast_mma_done;
+          for (int step = w.step_begin; step < w.step_end; ++step) {
+            if (!wait_bar(t_empty(ps), ps_phase ^ 1u, wc, 5)) goto fast_mma_done;
+            const uint32_t d_tmem = tmem_base + ps * 256u;
+            uint64_t db = umma_desc(sB, 1);
+            for (int k = 0; k < ksteps;) {
+              if (!wait_bar(a_full(a_stage), a_phase, wc, 3)) goto fast_mma_done;
+              tc_fence_after();
+              uint64_t da = umma_desc(sA + a_stage * a_tile_bytes, 1);
+              for (const int k1 = min(k + kpb, ksteps); k < k1; ++k) {
+                tc_mma(d_tmem, da, db, idesc, k > 0 ? 1u : 0u);
+                da += 4096u >> 4;
+                db += 8192u >> 4;
+              }
+              tc_commit(a_empty(a_stage));
+              if (++a_stage == (uint32_t)nA) {
+                a_stage = 0;
+                a_phase ^= 1u;
+              }
+            }
+            tc_commit(t_full(ps));
+            ps ^= 1u;
+            if (ps == 0u) ps_phase ^= 1u;
+          }
+          for (int c = 0; c < nc_item; ++c) {
+            tc_commit(b_empty(c));
+            b_bits ^= 1u << c;
+          }
+          continue;
+        }
         for (int step = w.step_begin; step < w.step_end; ++step) {
           if (!wait_bar(a_full(a_stage), a_phase, wc, 3)) goto fast_mma_done;
           tc_fence_after();
@@ -2114,11 +2400,11 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       bool idle = false;
       long long t0 = 0;
       while (true) {
-        const int b = (int)(t % kEvEntries);
+        const int b = (int)(t % kEv);
         // the halves' first lanes look whether their ticket is filled, or no more can come
         int got = 0;
         if ((lane & 15) == 0) {
-          if (mbar_test(ev.full(b), (uint32_t)((t / kEvEntries) & 1ull))) {
+          if (mbar_test(ev.full(b), (uint32_t)((t / kEv) & 1ull))) {
             got = 1;
           } else {
             const unsigned long long wv = *reinterpret_cast<volatile unsigned long long *>(ev.word);
@@ -2312,7 +2598,8 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
           if (half) {
             tc_fence_before();
             __syncwarp();
-            mbar_arrive_lane0(t_empty(ps), lane);
+            if constexpr (kPair) mbar_arrive_cluster_lane0(peer_addr(t_empty(ps), 0u), lane);
+            else mbar_arrive_lane0(t_empty(ps), lane);
           }
           const int o = off + kH * half;
           if constexpr (kSeed) {
@@ -2345,16 +2632,21 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         const int chunk0 = w.btile * g_nc;  // the work item's first chunk in the group
         const float *g_tau = g.tau + row;
         const uint16_t *g_nan = kNan ? g.nan_cnt : nullptr;
-        int ag = w.step_begin / g_ntt;            // the step's rank-matrix group (> 0: a permutation)
-        int tt = w.step_begin - ag * g_ntt;       // and its trait tile
+        // the step's rank-matrix group (> 0: a permutation) and its trait tile (of a
+        // pair's two tiles, this CTA's)
+        int ag = kPair ? 0 : w.step_begin / g_ntt;
+        int tt = kPair ? 2 * w.step_begin + (int)rank : w.step_begin - ag * g_ntt;
         // this warp's chunks of the B tile (h and 2 + h) must have landed
-        {
+        if constexpr (kPair) {
+          if (!wait_warp(b_full(0), b_bits & 1u, p, abort_addr, 6)) goto epi_done_scan;
+        } else {
           bool ok = true;
           for (int c = h; c < nc_item; c += 2) ok = ok && wait_bar_p(b_full(c), (b_bits >> c) & 1u, p, abort_addr, 6);
           if (!__all_sync(0xffffffffu, ok)) goto epi_done_scan;
         }
         // the constants of the lane's trait, one step ahead
-        float tau_n = g_tau[tt * kTileM];
+        const float kNever = __int_as_float(0x7f800000);
+        float tau_n = kPair && tt >= g_ntt ? kNever : g_tau[tt * kTileM];
         uint32_t nan_n = 0u;
         float v1_n = 0.f, v2_n = 0.f;
         if constexpr (kNan)
@@ -2363,11 +2655,16 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         for (int step = w.step_begin; step < w.step_end; ++step) {
           const float tau = tau_n, v1 = v1_n, v2 = v2_n;
           const int ag0 = ag, tt0 = tt;
-          if (++tt == g_ntt) {
-            tt = 0;
-            ++ag;
+          if constexpr (kPair) {
+            tt += 2;  // (past the last tile, an odd one's second half: never a candidate)
+            tau_n = tt < g_ntt ? g_tau[tt * kTileM] : kNever;
+          } else {
+            if (++tt == g_ntt) {
+              tt = 0;
+              ++ag;
+            }
+            tau_n = g_tau[tt * kTileM];  // (past the last step: a row that exists, unused)
           }
-          tau_n = g_tau[tt * kTileM];  // (past the last step: a row that exists, unused)
           ntlo = -tau * (1.f - p.margin);
           if constexpr (kNan) {
             const int nan_c = (int)nan_n;
@@ -2407,7 +2704,8 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
               tc_fence_after();
               tc_fence_before();
               __syncwarp();
-              mbar_arrive_lane0(t_empty(ps), lane);
+              if constexpr (kPair) mbar_arrive_cluster_lane0(peer_addr(t_empty(ps), 0u), lane);
+              else mbar_arrive_lane0(t_empty(ps), lane);
             }
             ps ^= 1u;
             if (ps == 0u) ps_phase ^= 1u;
@@ -2430,8 +2728,8 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         // the chunks' metadata is no longer needed
         __syncwarp();
         if (lane == 0)
-          for (int c = 0; c < nc_item; ++c) mbar_arrive(b_empty(c));
-        for (int c = 0; c < nc_item; ++c) b_bits ^= 1u << c;
+          for (int c = 0; c < (kPair ? 1 : nc_item); ++c) mbar_arrive(b_empty(c));
+        for (int c = 0; c < (kPair ? 1 : nc_item); ++c) b_bits ^= 1u << c;
       }
     epi_done_scan:
       tc_fence_before();
@@ -2668,7 +2966,22 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
   }
 
   __syncthreads();
-  if (warp == R::kMma) {
+  if constexpr (kPair) {
+    // The other CTA may still read this one's shared memory.  After a wait that gave up
+    // (a launch that ends in KRUX_ETIMEOUT) rank tiles of the second CTA may be under
+    // way that nothing counts any more: they land well within this pause.
+    if (*abort_flag) {
+      const long long t0 = clock64();
+      while (clock64() - t0 < 400000) __nanosleep(1000);
+    }
+    cluster_sync();
+    if (warp == R::kMma) {
+      tc_fence_after();
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
+    }
+    return;
+  }
+  if (warp == R::kMma && !kPair) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
   }
@@ -2851,7 +3164,7 @@ __global__ void seed_decide_kernel(const unsigned long long *__restrict__ rec,
     const unsigned long long v = rec[2 * idx + cls];
     if (v == 0ull) continue;
     const int64_t pos0 = (int64_t)(uint32_t)(v & 0xffffffffull) - 1;
-    const __half *a = stack + ((int64_t)(1 + q) * rows_pad + trait) * Np;
+    const int64_t arow = (int64_t)(1 + q) * rows_pad + trait;  // (the plain forms' layout)
     float best = 0.f;
     int bj = -1, bu = 0, bv = 0;
     for (int j = 0; j < 16 && pos0 + j < n_snps; ++j) {
@@ -2859,7 +3172,7 @@ __global__ void seed_decide_kernel(const unsigned long long *__restrict__ rec,
       const int8_t *g = geno + (snp_begin + pos) * ldg;
       int d0 = 0, d1 = 0;
       for (int k = lane; k < N; k += 32) {
-        const int ak = (int)__half2float(a[k]);
+        const int ak = (int)__half2float(stack[tiled_index(arow, k, Np)]);
         const int8_t gk = g[k];
         d0 += gk == 0 ? ak : 0;
         d1 += gk == 1 ? ak : 0;
@@ -2989,6 +3302,9 @@ cudaError_t scan_set_smem_all(size_t smem) {
   e = cudaFuncSetAttribute(krux_scan_kernel<kFormScanPerm>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(krux_scan_kernel<kFormScanPair>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(krux_scan_kernel<kFormScanSeed>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -3006,8 +3322,49 @@ cudaError_t scan_set_smem_all(size_t smem) {
 int scan_form_of(const ScanParams &p) {
   if (p.multi) return kFormMulti;
   if (p.perm) return p.fast && fast_form_ok() ? kFormScanPerm : kFormPerm;
-  if (p.fast && fast_form_ok()) return p.fast_nan ? kFormScanNan : kFormScan;
+  if (p.fast && fast_form_ok()) return p.fast_nan ? kFormScanNan : (p.pair_cta ? kFormScanPair : kFormScan);
   return kFormNan;
+}
+
+// Launch of the pair form: clusters of two CTAs.
+static void pair_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr, int grid, size_t smem,
+                        cudaStream_t s) {
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kFastThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = 2;
+  attr.val.clusterDim.y = 1;
+  attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+}
+
+// Pairs of CTAs that run at one time (its items are taken in fixed turns, so a grid
+// must not exceed them), 0 where the pair form cannot run; looked up once per device.
+int pair_clusters() {
+  static std::atomic<int> known[64];
+  int dev = 0;
+  if (!fast_form_ok() || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  int v = known[dev].load(std::memory_order_acquire);
+  if (v == 0) {
+    constexpr size_t kSmem = 232448;
+    cudaFuncAttributes a;
+    int n = 0;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr{};
+    pair_config(cfg, attr, 2, kSmem, nullptr);
+    const bool ok = cudaFuncGetAttributes(&a, krux_scan_kernel<kFormScanPair>) == cudaSuccess &&
+                    a.numRegs == kFastRegsLaunch && a.maxThreadsPerBlock >= kFastThreads &&
+                    cudaFuncSetAttribute(krux_scan_kernel<kFormScanPair>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kSmem) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&n, krux_scan_kernel<kFormScanPair>, &cfg) == cudaSuccess;
+    v = 1 + (ok ? n : 0);
+    known[dev].store(v, std::memory_order_release);
+  }
+  return v - 1;
 }
 
 cudaError_t launch_scan_only(const ScanParams &p, int grid, size_t smem, cudaStream_t s) {
@@ -3021,7 +3378,12 @@ cudaError_t launch_scan_only(const ScanParams &p, int grid, size_t smem, cudaStr
     krux_scan_kernel<kFormPerm><<<grid, kScanThreads, smem, s>>>(p);
   else if (p.fast && p.fast_nan && fast_form_ok())
     krux_scan_kernel<kFormScanNan><<<grid, kFastThreads, smem, s>>>(p);
-  else if (p.fast && fast_form_ok())
+  else if (p.fast && p.pair_cta && fast_form_ok()) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr{};
+    pair_config(cfg, attr, grid, smem, s);
+    return cudaLaunchKernelEx(&cfg, krux_scan_kernel<kFormScanPair>, p);
+  } else if (p.fast && fast_form_ok())
     krux_scan_kernel<kFormScan><<<grid, kFastThreads, smem, s>>>(p);
   else
     // the general form: traits with NaN, dense output, cis window, provisional

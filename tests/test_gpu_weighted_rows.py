@@ -48,3 +48,54 @@ def test_sums_and_hits_at_every_group_shape(oracle_mod, N, pth):
     assert np.array_equal(h[:, 3], orc["d"][h[:, 0], h[:, 1], 1])
     rs.free()
     kx.close()
+
+
+@pytest.mark.parametrize("T", [100, 129, 300])  # one trait tile, an odd and an even last step
+@pytest.mark.parametrize("S", [40, 64, 65, 700])  # one chunk, a whole one, an odd last chunk
+@pytest.mark.parametrize("N", [193, 224, 240, 257, 336, 352, 512])
+def test_wide_shapes_at_the_edges_of_their_tiles(oracle_mod, N, S, T):
+    """K blocks (up to 224 samples) and pairs of CTAs (from 240): every number of K
+    blocks, a last shorter one, odd numbers of trait tiles and of chunks."""
+    import torch
+    from paper_1307_3519_gb300 import build
+    build.build()
+    import paper_1307_3519_gb300 as k
+    rng = np.random.default_rng(N + S + T)
+    geno = rng.binomial(2, rng.uniform(0.02, 0.5, S)[:, None], (S, N)).astype(np.int8)
+    expr = rng.standard_normal((T, N)).astype(np.float32)
+    kx = k.Krux(0)
+    rs = kx.krux_rank(torch.from_numpy(expr).cuda())
+    r = kx.krux_scan(rs, torch.from_numpy(geno).cuda(), 0.02, capacity=T * S)
+    orc = oracle_mod.scan(expr, geno, 0.02)
+    h = r["hits"].cpu().numpy().astype(np.int64)
+    got = np.zeros_like(orc["hit"])
+    got[h[:, 0], h[:, 1]] = True
+    near = np.abs(orc["p"] / 0.02 - 1.0) < 1e-12
+    assert not ((got != orc["hit"]) & ~near).any()
+    assert r["n_hits"] == len(h) == int(got.sum())
+    assert np.array_equal(h[:, 2], orc["d"][h[:, 0], h[:, 1], 0])
+    rs.free()
+    kx.close()
+
+
+def test_pairs_of_ctas_report_a_wait_that_ran_out():
+    """A one-cycle wait limit ends a launch over pairs of CTAs with KRUX_ETIMEOUT; the
+    next call on the context is right again."""
+    import torch
+    from paper_1307_3519_gb300 import build
+    build.build()
+    import paper_1307_3519_gb300 as k
+    rng = np.random.default_rng(5)
+    geno = torch.from_numpy(rng.integers(0, 3, (9000, 300)).astype(np.int8)).cuda()
+    expr = torch.from_numpy(rng.standard_normal((2000, 300)).astype(np.float32)).cuda()
+    kx = k.Krux(0)
+    rs = kx.krux_rank(expr)
+    want = kx.krux_scan(rs, geno, 1e-3, capacity=200_000)["n_hits"]
+    kx.set_wait_limit(1)
+    with pytest.raises(k.KruxError) as e:
+        kx.krux_scan(rs, geno, 1e-3, capacity=200_000)
+    assert e.value.status == k.KRUX_ETIMEOUT
+    kx.set_wait_limit(0)
+    assert kx.krux_scan(rs, geno, 1e-3, capacity=200_000)["n_hits"] == want
+    rs.free()
+    kx.close()
