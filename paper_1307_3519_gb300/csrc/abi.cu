@@ -29,19 +29,19 @@ cudaError_t launch_missing_scan(const int8_t *geno, int64_t ldg, int N, int64_t 
 cudaError_t launch_pack_linear(const int8_t *geno, int64_t ldg, int N, int Np, int64_t snp_begin,
                                int64_t n_snps, double rl, __half *B, ChunkMeta *meta,
                                unsigned int *status, cudaStream_t s);
+size_t param_table_bytes();
 cudaError_t launch_standardize(const float *expr, int T, int N, int64_t ld, int Np, __half *A,
-                               double *mean, double *sd, float *tau, double *cfac,
-                               uint16_t *nan_cnt, unsigned int *status, cudaStream_t s);
-cudaError_t launch_finalize_param(const krux_hit *hits, const unsigned long long *count,
-                                  int64_t capacity, const float *expr, int64_t ld,
-                                  const int8_t *geno, int64_t ldg, int N, const double *mean,
-                                  int model, double *stat, double *P, int sm_count,
+                               __half *At, long long *fixed, double *squares, float *tau,
+                               double *cfac, uint16_t *nan_cnt, double *table,
+                               unsigned int *status, cudaStream_t s);
+cudaError_t launch_finalize_param(const krux_hit *hits, const HitAux *aux,
+                                  const unsigned long long *count, int64_t capacity,
+                                  const long long *fixed, const double *squares,
+                                  const int8_t *geno, int64_t ldg, const int8_t *lo,
+                                  const int8_t *hi, int N, int model, const double *table,
+                                  double pthresh, krux_hit *out, double *out_stat, double *out_p,
+                                  int64_t out_capacity, unsigned long long *n_out, int sm_count,
                                   cudaStream_t s);
-cudaError_t launch_filter_param(const krux_hit *hits, const unsigned long long *count,
-                                int64_t capacity, const double *stat, const double *P,
-                                double pthresh, krux_hit *out, double *out_stat, double *out_p,
-                                int64_t out_capacity, unsigned long long *n_out, int sm_count,
-                                cudaStream_t s);
 double param_f_crit(double pthresh, double d1, double d2);
 double param_t_crit(double pthresh, double nu);
 cudaError_t launch_pack_multi(const int8_t *geno, int64_t ldg, int N, int Np,
@@ -204,6 +204,7 @@ struct krux_ctx {
       list, gemm_out, bucket_ranks, permA, minpkey, seg, permNan, aux2, param, paramOut, packjobs,
       host_in, host_out,  // krux_scan_host: device copies of the inputs, device hit list
       groups2, items2, packjobs2, cfacptr2,  // launch tables of a second launch in the same call
+      cistab,  // cis scans: their groups, for the planning on the device
       mcand,  // plain-form permutation batches: pairs for the deferred FP64 pass
       pattern, dlist;  // device-side missing-pattern grouping: scratch, SNP lists
   HostBuf list_host;  // staging of the SNP lists
@@ -385,6 +386,11 @@ int plain_form_fits(const krux_ctx *ctx, int Np) {
 bool pq_range_ok(double h1, double h2) {
   const double lo = std::min(h1, h2), hi = std::max(h1, h2);
   return lo > 0.0 && std::sqrt(2.0 / lo) < 16384.0 && std::sqrt(1.0 / (kMaxN * hi)) > 1.0 / 4096.0;
+}
+
+// The same for the regression's weights, sqrt(4 rl / S_gg) with 1/2 < S_gg <= N.
+bool pq_range_linear(double rl) {
+  return std::sqrt(8.0 * rl) < 16384.0 && std::sqrt(4.0 * rl / kMaxN) > 1.0 / 4096.0;
 }
 
 // Refuses a launch plan whose shared-memory regions or per-group shapes are not
@@ -663,7 +669,7 @@ void krux_destroy(krux_ctx *ctx) {
                     &ctx->list, &ctx->gemm_out, &ctx->bucket_ranks, &ctx->permA, &ctx->minpkey, &ctx->seg,
                     &ctx->permNan, &ctx->aux2, &ctx->param, &ctx->paramOut, &ctx->packjobs,
                     &ctx->host_in, &ctx->host_out, &ctx->groups2, &ctx->items2, &ctx->packjobs2,
-                    &ctx->cfacptr2, &ctx->mcand, &ctx->pattern, &ctx->dlist};
+                    &ctx->cfacptr2, &ctx->mcand, &ctx->cistab, &ctx->pattern, &ctx->dlist};
   for (DevBuf *b : bufs) b->release();
   ctx->list_host.release();
   for (auto &pb : ctx->pool) cudaFree(pb.second);
@@ -1080,18 +1086,18 @@ struct CallPlan {
     int model = -1;                 // -1 off, 0 ANOVA, 1 dosage regression
     double h1 = 0.0, h2 = 0.0;      // ANOVA bounds tau_1, tau_2 on sum_i S_i^2 / N_i
     double rl = 0.0;                // regression: 1 / ((K - 1) r_c^2)
-    const float *expr = nullptr;    // the caller's values, for the FP64 recomputation
-    int64_t ld = 0;
-    const double *mean = nullptr;   // per-trait mean the recomputation centres on
+    const long long *fixed = nullptr;  // the centred values in fixed point, for the recomputation
+    const double *squares = nullptr;   // and their sums of squares
+    const double *table = nullptr;     // continued fraction of the tail
     krux_hit *out = nullptr;        // the caller's lists
     double *out_stat = nullptr, *out_p = nullptr;
     int64_t out_capacity = 0;
   } param;
-  struct Cis {  // cis scans: SNP and trait coordinates (host copies) and the window
+  struct Cis {  // cis scans: SNP and trait coordinates and the window
     bool on = false;
     const int64_t *snp_pos = nullptr, *trait_pos = nullptr;  // device
-    std::vector<int64_t> h_snp, h_trait;                      // host copies
-    int64_t window = -1;
+    int64_t S = 0, window = -1;
+    int T = 0;
   } cis;
   int64_t dlist_used = 0;  // entries of ctx->dlist this call's device groupings use
   unsigned long long *fdr_hist = nullptr;  // permutation calls: [fdr_rows = 1 + P][fdr_bins] or null
@@ -1282,7 +1288,7 @@ krux_status materialise(krux_ctx *ctx, CallPlan &cp, cudaStream_t s) {
   cp.rerank_hjobs = jobs;
   cp.rerank_djobs = djobs;
   cp.rerank_drops = ddrop;
-  cp.rerank_tiled = !cp.multi && !cp.cis.on && cp.slots.size() == 1 && ctx->tune_layout != 0 &&
+  cp.rerank_tiled = !cp.multi && cp.slots.size() == 1 && ctx->tune_layout != 0 &&
                     cp.groups[0].dense_H == nullptr;
   KRUX_CUDA(ctx, launch_rerank_buckets(djobs, jobs.data(), ddrop, (int)nb, cp.rerank_tiled, s));
   if (ctx->profiling) ctx->prof.launches += 1;
@@ -1310,41 +1316,6 @@ krux_status materialise(krux_ctx *ctx, CallPlan &cp, cudaStream_t s) {
   return KRUX_OK;
 }
 
-// cis scans: for every B tile, only the trait tiles whose traits can lie within
-// the window of one of the tile's SNPs (SNP and trait coordinates are
-// nondecreasing, so that is one contiguous range of trait tiles); B tiles with
-// none are skipped.
-std::vector<WorkItem> make_items_cis(const CallPlan &cp, const std::vector<GroupPlan> &gp) {
-  std::vector<WorkItem> items;
-  const std::vector<int64_t> &tp = cp.cis.h_trait;
-  const int64_t W = cp.cis.window;
-  for (size_t gi = 0; gi < gp.size(); ++gi) {
-    const ScanGroupIn &g = cp.groups[gi];
-    const GroupDesc &d = gp[gi].d;
-    auto snp_at = [&](int64_t i) {
-      return g.list_off >= 0 ? cp.lists[(size_t)(g.list_off + i)] : g.snp_begin + i;
-    };
-    for (int64_t b = 0; b < gp[gi].n_btiles; ++b) {
-      const int64_t csn = cp.multi ? kChunkSnpsM : kChunkSnps;
-      const int64_t first = b * d.nc * csn;
-      const int64_t last = std::min<int64_t>((b + 1) * d.nc * csn, g.n_snps) - 1;
-      if (first > last) continue;
-      const int64_t lo = cp.cis.h_snp[(size_t)snp_at(first)] - W;
-      const int64_t hi = cp.cis.h_snp[(size_t)snp_at(last)] + W;
-      const int64_t t0 = std::lower_bound(tp.begin(), tp.end(), lo) - tp.begin();
-      const int64_t t1 = std::upper_bound(tp.begin(), tp.end(), hi) - tp.begin();
-      if (t0 >= t1) continue;
-      WorkItem w;
-      w.group = (int32_t)gi;
-      w.btile = (int32_t)b;
-      w.step_begin = (int32_t)(t0 / kTileM);
-      w.step_end = (int32_t)((t1 - 1) / kTileM + 1);
-      items.push_back(w);
-    }
-  }
-  return items;
-}
-
 // One fused launch, split in three phases so that the middle one can be captured
 // in a CUDA graph: prepare (host planning, buffer sizing, descriptor uploads; no
 // work queued that a replay would need), enqueue (stream work only: packing, the
@@ -1360,6 +1331,7 @@ struct FusedLaunch {
   double h1 = 0.0, h2 = 0.0;
   int signed_coef = 0;
   bool fast_nan = false;  // the plain form's NaN variant (coefficient sets in the codes)
+  int64_t cis_tiles = 0;  // cis scans: B tiles of all groups
   std::vector<int64_t> boff, moff, coff;
   int layout = 1;
   double hm[4] = {0.0, 0.0, 0.0, 0.0};  // markers with codes 0..4: h_d for d = 1..4
@@ -1415,8 +1387,9 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   // place of the 2-bit codes) when at most one trait in 128 has more NaN samples
   // than the last set covers (each such trait sends all its pairs to the exact
   // test; beyond that share the general form is faster)
-  bool fast_shape = layout == 1 && !cp.multi && cp.param.model < 0 && o->dense_H == nullptr &&
-                    !cp.cis.on && pq_range_ok(fl.h1, fl.h2) && fast_form_ok();
+  bool fast_shape = layout == 1 && !cp.multi && o->dense_H == nullptr &&
+                    (cp.param.model == 1 ? pq_range_linear(cp.param.rl) : pq_range_ok(fl.h1, fl.h2)) &&
+                    fast_form_ok();
   bool any_nan = false, fast_nan = allow_fast_nan && fast_shape;
   for (auto &g : cp.groups) {
     fast_nan = fast_nan && g.minp_key == nullptr &&
@@ -1438,7 +1411,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     ctx->tune_nA = tnA;
     ctx->tune_ka = tka;
     // pairs of CTAs take complete data without permutations
-    const bool pairs = fast_shape && !fast_nan && fl.signed_coef == 0 && tnc == 0 && tnA == 0 &&
+    const bool pairs = fast_shape && !fast_nan && fl.signed_coef == 0 && !cp.cis.on && tnc == 0 && tnA == 0 &&
                        pair_cta_wanted(kpad);
     const bool ok = pick_launch_shape(ctx, kpad, codes_k, sh, fast_shape ? kPlainExtra : 0, pairs);
     ctx->tune_nc = s_nc;
@@ -1579,9 +1552,28 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     descs[i] = d;
   }
   const int workers = sh.pair_cta ? std::min(pair_clusters(), ctx->sm_count / 2) : ctx->sm_count;
-  std::vector<WorkItem> items = cp.cis.on ? make_items_cis(cp, plans) : make_items(plans, workers);
+  // cis scans: the items are made on the device from the coordinates (enqueue_fused),
+  // at most one per B tile
+  std::vector<WorkItem> items;
+  std::vector<CisGroup> cis;
+  size_t n_items = 0;
+  if (cp.cis.on) {
+    for (int i = 0; i < ng; ++i) {
+      const ScanGroupIn &g = cp.groups[i];
+      cis.push_back(CisGroup{g.snp_list, g.snp_begin, g.n_snps, (int64_t)n_items,
+                             descs[i].nc * (cp.multi ? kChunkSnpsM : kChunkSnps), i});
+      n_items += (size_t)plans[i].n_btiles;
+    }
+    fl.cis_tiles = (int64_t)n_items;
+    KRUX_CUDA(ctx, ctx->cistab.ensure(sizeof(CisGroup) * ng));
+    KRUX_CUDA(ctx, cudaMemcpyAsync(ctx->cistab.p, cis.data(), sizeof(CisGroup) * ng,
+                                   cudaMemcpyHostToDevice, s));
+  } else {
+    items = make_items(plans, workers);
+    n_items = items.size();
+  }
   KRUX_CUDA(ctx, t_groups.ensure(sizeof(GroupDesc) * ng));
-  KRUX_CUDA(ctx, t_items.ensure(sizeof(WorkItem) * std::max<size_t>(items.size(), 1)));
+  KRUX_CUDA(ctx, t_items.ensure(sizeof(WorkItem) * std::max<size_t>(n_items, 1)));
   // pageable uploads: staged before the calls return, so the host vectors may go
   KRUX_CUDA(ctx, cudaMemcpyAsync(t_groups.p, descs.data(), sizeof(GroupDesc) * ng,
                                  cudaMemcpyHostToDevice, s));
@@ -1599,7 +1591,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   p = ScanParams{};
   p.groups = t_groups.as<GroupDesc>();
   p.items = t_items.as<WorkItem>();
-  p.n_items = (int32_t)items.size();
+  p.n_items = (int32_t)n_items;
   // the item counters sit behind the status words, one for each launch of a call
   // (cleared with them before the first)
   p.pair_cta = sh.pair_cta ? 1 : 0;
@@ -1636,17 +1628,18 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     p.cis_snp_pos = cp.cis.snp_pos;
     p.cis_trait_pos = cp.cis.trait_pos;
     p.cis_window = cp.cis.window;
+    p.n_items_dev = ctx->status.as<int32_t>() + 10;  // (cleared with the status words)
   }
   // the plain scan form: 32-byte swizzle, every group's chunks paired and its K
-  // in one rank stage (or one pair resident and its K in blocks), complete data, no dense output, cis window, provisional
-  // hits, permutations or markers with more than three groups
+  // in one rank stage (or one pair resident and its K in blocks), no dense output, at
+  // most three groups per marker
   {
-    bool fast = layout == 1 && !p.multi && (!p.has_nan || fast_nan) && !p.dense && !p.provisional &&
-                (!p.signed_coef || p.perm) && p.cis_window < 0;
+    bool fast = layout == 1 && !p.multi && (!p.has_nan || fast_nan) && !p.dense &&
+                (!p.signed_coef || p.perm);
     for (const GroupDesc &d : descs) fast = fast && d.pair == 1 && (d.nkb == 1 || d.nc == 2);
     p.fast = fast && fast_shape ? 1 : 0;
   }
-  fl.grid = (int)std::min<size_t>(items.size(), (size_t)workers) * (sh.pair_cta ? 2 : 1);
+  fl.grid = (int)std::min<size_t>(n_items, (size_t)workers) * (sh.pair_cta ? 2 : 1);
   // Single hit list: every epilogue warp stages its hits in a segment of its own
   // (no atomic per hit event) and the segments are appended after the launch.
   fl.staged = fl.nslots == 1 && cp.slots[0].capacity > 0 && fl.grid > 0;
@@ -1675,7 +1668,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   if (fast_nan && !p.fast)  // the coefficient sets need the plain form: plan again
     return prepare_fused(ctx, cp, o, fl, s, tables, false);
   p.fast_nan = fast_nan ? 1 : 0;
-  fl.batched_pack = !cp.multi && cp.param.model != 1;
+  fl.batched_pack = !cp.multi && (cp.param.model != 1 || p.fast);
   if (fl.batched_pack) {
     std::vector<PackJob> jobs(ng);
     int64_t slots = 0, halves = 0;
@@ -1701,6 +1694,8 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
       j.allow_missing = g.allow_missing;
       j.coef_nan = j.codes != nullptr && fast_nan ? 1 : 0;
       j.pq_bits = p.fast ? pq_bits(g.rs->N) : 0;
+      j.linear = cp.param.model == 1 ? 1 : 0;
+      j.rl = (float)cp.param.rl;
       slots += nch * kChunkSnps;
       if (j.codes && !j.coef_nan) halves += nch * 2;
     }
@@ -1737,6 +1732,11 @@ krux_status enqueue_fused(krux_ctx *ctx, CallPlan &cp, const FusedLaunch &fl, cu
     KRUX_CUDA(ctx, cudaMemsetAsync(ctx->status.p, 0, 64, s));
   if (cp.fdr_hist)
     KRUX_CUDA(ctx, cudaMemsetAsync(cp.fdr_hist, 0, (size_t)cp.fdr_rows * cp.fdr_bins * 8, s));
+  if (cp.cis.on)
+    KRUX_CUDA(ctx, launch_cis_items(ng ? ctx->cistab.as<CisGroup>() : nullptr, ng, fl.cis_tiles,
+                                    cp.cis.snp_pos, cp.cis.S, cp.cis.trait_pos, cp.cis.T,
+                                    cp.cis.window, const_cast<WorkItem *>(fl.p.items),
+                                    ctx->status.as<int32_t>() + 10, ctx->status.as<unsigned int>(), s));
   if (ng == 0) {  // nothing to scan: a permutation batch still reports min p = 1
     if (cp.perm.on) {
       KRUX_CUDA(ctx, cudaMemsetAsync(ctx->minpkey.p, 0,
@@ -1816,17 +1816,15 @@ krux_status enqueue_fused(krux_ctx *ctx, CallPlan &cp, const FusedLaunch &fl, cu
   }
   // FP64 H and p of the stored hits: each slot's count is read on the device
   ev_record(ctx, 5, s);
-  if (cp.param.model >= 0) {  // FP64 decision of the provisional hits, then the filter
+  if (cp.param.model >= 0) {  // the exact decision of the provisional hits
     const OutSlot &os = cp.slots[0];
     const ScanGroupIn &g = cp.groups[0];
-    KRUX_CUDA(ctx, launch_finalize_param(os.hits, totals, os.capacity, cp.param.expr, cp.param.ld,
-                                         g.geno, g.ldg, g.rs->N, cp.param.mean, cp.param.model,
-                                         os.H, os.P, ctx->sm_count, s));
-    KRUX_CUDA(ctx, launch_filter_param(os.hits, totals, os.capacity, os.H, os.P, fl.p.pthresh,
-                                       cp.param.out, cp.param.out_stat, cp.param.out_p,
-                                       cp.param.out_capacity,
-                                       ctx->counters.as<unsigned long long>() + 2 * nslots,
-                                       ctx->sm_count, s));
+    KRUX_CUDA(ctx, launch_finalize_param(
+                       os.hits, os.aux, totals, os.capacity, cp.param.fixed, cp.param.squares, g.geno,
+                       g.ldg, g.geno + g.row_lo * g.ldg, g.geno + (g.row_hi - 1) * g.ldg + g.rs->N,
+                       g.rs->N, cp.param.model, cp.param.table, fl.p.pthresh, cp.param.out,
+                       cp.param.out_stat, cp.param.out_p, cp.param.out_capacity,
+                       ctx->counters.as<unsigned long long>() + 2 * nslots, ctx->sm_count, s));
   }
   for (int k = 0; k < nslots && cp.param.model < 0; ++k) {
     const OutSlot &os = cp.slots[k];
@@ -1863,7 +1861,8 @@ int fused_launches(const CallPlan &cp, const FusedLaunch &fl) {
   else
     for (auto &g : cp.groups) n += g.nan_cnt ? 2 : 1;
   for (auto &os : cp.slots) n += (os.capacity > 0 && cp.param.model < 0) ? 1 : 0;
-  if (cp.param.model >= 0) n += 2;
+  if (cp.param.model >= 0) n += 1;
+  if (cp.cis.on) n += 2;
   if (cp.perm.on) {
     // the permuted stack (and NaN lists) unless a seed pass built them; then the
     // minimum-p read-out, or after a plain-form seed pass its exact decisions
@@ -1877,6 +1876,7 @@ int fused_launches(const CallPlan &cp, const FusedLaunch &fl) {
 // Reads the status word back; KRUX_OK, or the device-side error.
 krux_status device_status(krux_ctx *ctx, const unsigned int *hst) {
   if (hst[0] & kDevBadCode) return fail(ctx, KRUX_EINVAL, "genotype code outside {-1,0,1,2}");
+  if (hst[0] & kDevUnsorted) return fail(ctx, KRUX_EINVAL, "cis coordinates must be nondecreasing");
   if (hst[0] & kDevBadPerm) return fail(ctx, KRUX_EINVAL, "a permutation entry is outside 0..N-1");
   if (hst[0] & kDevTimeout)
     return fail(ctx, KRUX_ETIMEOUT, "device wait timed out (site %u)", hst[1]);
@@ -1888,7 +1888,7 @@ krux_status finish_fused(krux_ctx *ctx, CallPlan &cp, const FusedLaunch &fl, cud
   const int nslots = fl.nslots;
   counts.assign(nslots, 0);
   unsigned int hst[2] = {0, 0};
-  if (!cp.groups.empty()) {
+  if (!cp.groups.empty() || cp.cis.on) {
     KRUX_CUDA(ctx, cudaMemcpyAsync(counts.data(), ctx->counters.as<unsigned long long>() + nslots,
                                    (size_t)nslots * 8, cudaMemcpyDeviceToHost, s));
     KRUX_CUDA(ctx, cudaMemcpyAsync(hst, ctx->status.p, 8, cudaMemcpyDeviceToHost, s));
@@ -2120,17 +2120,8 @@ extern "C" krux_status krux_scan_cis(krux_ctx *ctx, const krux_rankset *rs, cons
   cp.cis.snp_pos = snp_pos;
   cp.cis.trait_pos = trait_pos;
   cp.cis.window = window;
-  cp.cis.h_snp.resize((size_t)S);
-  cp.cis.h_trait.resize((size_t)rs->T);
-  if (S > 0)
-    KRUX_CUDA(ctx, cudaMemcpyAsync(cp.cis.h_snp.data(), snp_pos, (size_t)S * 8,
-                                   cudaMemcpyDeviceToHost, s));
-  KRUX_CUDA(ctx, cudaMemcpyAsync(cp.cis.h_trait.data(), trait_pos, (size_t)rs->T * 8,
-                                 cudaMemcpyDeviceToHost, s));
-  KRUX_CUDA(ctx, cudaStreamSynchronize(s));
-  if (!std::is_sorted(cp.cis.h_snp.begin(), cp.cis.h_snp.end()) ||
-      !std::is_sorted(cp.cis.h_trait.begin(), cp.cis.h_trait.end()))
-    return fail(ctx, KRUX_EINVAL, "cis coordinates must be nondecreasing");
+  cp.cis.S = S;
+  cp.cis.T = rs->T;
   const int64_t b = opts->snp_begin, e = opts->snp_end > 0 ? opts->snp_end : S;
   if (ctx->profiling) {
     ctx->prof = krux_profile{};
@@ -2198,10 +2189,12 @@ extern "C" krux_status krux_scan_parametric(krux_ctx *ctx, const float *expr, in
   const size_t oA = take((size_t)rs.rows_pad * rs.Np * 2), oTau = take((size_t)rs.rows_pad * 4),
                oCf = take((size_t)rs.rows_pad * 8), oNc = take((size_t)rs.rows_pad * 2),
                oNi = take((size_t)T * N * 2), oTile = take((size_t)rs.n_ttiles * 4),
-               oMean = take((size_t)T * 8), oSd = take((size_t)T * 8);
+               oAt = take((size_t)rs.rows_pad * rs.Np * 2);
+  const size_t zeroed = off;
+  const size_t oFix = take((size_t)T * N * 8), oSq = take((size_t)T * 8), oTab = take(param_table_bytes());
   KRUX_CUDA(ctx, ctx->param.ensure(off));
   char *pb = ctx->param.as<char>();
-  KRUX_CUDA(ctx, cudaMemsetAsync(pb, 0, off, s));
+  KRUX_CUDA(ctx, cudaMemsetAsync(pb, 0, zeroed, s));
   rs.dev = RankDev{};
   rs.dev.A = reinterpret_cast<__half *>(pb + oA);
   rs.dev.tau = reinterpret_cast<float *>(pb + oTau);
@@ -2209,13 +2202,15 @@ extern "C" krux_status krux_scan_parametric(krux_ctx *ctx, const float *expr, in
   rs.dev.nan_cnt = reinterpret_cast<uint16_t *>(pb + oNc);
   rs.dev.nan_idx = reinterpret_cast<uint16_t *>(pb + oNi);
   rs.dev.tile_nan = reinterpret_cast<uint32_t *>(pb + oTile);
-  double *mean = reinterpret_cast<double *>(pb + oMean);
-  double *sd = reinterpret_cast<double *>(pb + oSd);
+  rs.dev.At = reinterpret_cast<__half *>(pb + oAt);
+  long long *fixed = reinterpret_cast<long long *>(pb + oFix);
+  double *squares = reinterpret_cast<double *>(pb + oSq), *table = reinterpret_cast<double *>(pb + oTab);
   KRUX_CUDA(ctx, ctx->status.ensure(64));
   KRUX_CUDA(ctx, cudaMemsetAsync(ctx->status.p, 0, 64, s));
   ev_record(ctx, 0, s);
-  KRUX_CUDA(ctx, launch_standardize(expr, T, N, ld, rs.Np, rs.dev.A, mean, sd, rs.dev.tau,
-                                    rs.dev.cfac, rs.dev.nan_cnt, ctx->status.as<unsigned int>(), s));
+  KRUX_CUDA(ctx, launch_standardize(expr, T, N, ld, rs.Np, rs.dev.A, rs.dev.At, fixed, squares,
+                                    rs.dev.tau, rs.dev.cfac, rs.dev.nan_cnt, table,
+                                    ctx->status.as<unsigned int>(), s));
   KRUX_CUDA(ctx, launch_pad_traits(T, rs.rows_pad, rs.dev.tau, rs.dev.cfac, rs.dev.nan_cnt, s));
   ev_record(ctx, 1, s);
   unsigned int hst = 0;
@@ -2237,9 +2232,9 @@ extern "C" krux_status krux_scan_parametric(krux_ctx *ctx, const float *expr, in
     const double rc2 = tc * tc / (K - 2.0 + tc * tc);
     cp.param.rl = 1.0 / ((K - 1.0) * rc2);
   }
-  cp.param.expr = expr;
-  cp.param.ld = ld;
-  cp.param.mean = mean;
+  cp.param.fixed = fixed;
+  cp.param.squares = squares;
+  cp.param.table = table;
   cp.param.out = hits;
   cp.param.out_stat = hit_stat;
   cp.param.out_p = hit_p;

@@ -268,6 +268,8 @@ struct PackJob {
                             // per chunk) instead of 2-bit codes
   int32_t pq_bits;          // > 0: weighted rows of the plain forms (their significant bits);
                             // 0: 0/1 indicators of groups 0 and 1
+  int32_t linear;           // dosage regression (parametric comparison): its coefficients,
+  float rl;                 // rl (2 S_0 + S_1)^2 / S_gg
 };
 
 // ---- one group of a scan launch (a cohort, a missing-pattern bucket, or the
@@ -358,6 +360,7 @@ struct ScanParams {
   unsigned int *next;       // items taken beyond one per CTA (zero at launch), or null: CTA b
                             // takes items b, b + grid, b + 2 grid, ...
   int32_t n_items;
+  const int32_t *n_items_dev = nullptr;  // cis: their number, decided on the device
   int32_t nc;               // most chunks any group keeps resident (<= kTmemSlots)
   int32_t nA;               // A pipeline stages
   int32_t kpad;             // widest K of the groups (codes rows are kpad * 16 bytes)
@@ -420,9 +423,26 @@ enum : unsigned int {
   kDevBadPerm = 4u,     // a permutation entry outside 0..N-1 (its row is gathered as zeros)
   kDevMissing = 8u,     // a -1 code in a group packed as complete (graph replays)
   kDevHashCollision = 16u,  // two missing-sample patterns with one 64-bit hash
+  kDevUnsorted = 32u,       // cis coordinates that are not nondecreasing
+};
+
+// One group of a cis scan: where its B tiles' SNPs are (rows of the genotype matrix).
+struct CisGroup {
+  const int64_t *snp_list;  // device rows, or null for [snp_begin, snp_begin + n_snps)
+  int64_t snp_begin, n_snps;
+  int64_t tile0;            // its first B tile in the flattened launch
+  int32_t tile_snps;        // SNPs of one B tile
+  int32_t group;
 };
 
 // ---- launch wrappers (defined in the .cu files) -----------------------------
+// Work items of a cis scan: every B tile of the groups (n_tiles in all) against the
+// trait tiles its window reaches, appended to items / n_items (zero at launch); tiles
+// that reach no trait get none.  Coordinates out of order set kDevUnsorted.
+cudaError_t launch_cis_items(const CisGroup *groups, int n_groups, int64_t n_tiles,
+                             const int64_t *snp_pos, int64_t S, const int64_t *trait_pos, int T,
+                             int64_t window, WorkItem *items, int32_t *n_items,
+                             unsigned int *status, cudaStream_t s);
 cudaError_t launch_rank(const float *expr, int T, int N, int64_t ld, int Np, int rows_pad,
                         const RankDev &r, cudaStream_t s);
 // NaN sample lists of the permuted rank matrices: out[q][t][j] = inv[q][nan_idx[t][j]]

@@ -6,6 +6,8 @@
 // satisfy D_0 + D_1 + D_2 = 0, so D_2 follows from the other two.  The packed
 // operand is FP16 0/1 in chunks of 64 SNPs: chunk c holds rows [0,64) = I_0 and
 // rows [64,128) = I_1 of SNPs 64c .. 64c+63, each row Np samples long.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace krux {
@@ -377,6 +379,20 @@ __device__ __forceinline__ PqCoef pq_coef(int n0, int n1, int n2, bool excluded,
   return c;
 }
 
+// The regression's only row: sqrt(alpha) (D_0 + D_1 / 2), Q = 0 (see write_meta).
+__device__ __forceinline__ PqCoef pq_coef_linear(int n0, int n1, int n2, bool excluded, float rl) {
+  PqCoef c{};
+  c.w1 = 1u << 18;
+  const int K = n0 + n1 + n2;
+  const float gs = (float)n1 + 2.f * (float)n2;
+  const float sgg = K > 0 ? (float)n1 + 4.f * (float)n2 - gs * gs / (float)K : 0.f;
+  if (excluded || !(sgg > 0.5f / (float)(K > 0 ? K : 1))) return c;
+  c.a0 = round_up_bits(sqrtf(4.f * rl / sgg) * 1.00001f, 10);
+  c.w0 = (uint32_t)__half_as_ushort(__float2half_rn(c.a0)) |
+         ((uint32_t)__half_as_ushort(__float2half_rn(0.5f * c.a0)) << 16);
+  return c;
+}
+
 // The plain form's coefficient sets of SNP slot jj for traits with NaN samples:
 // set s takes the quadratic form from group sizes max(N_i - C, 1), C = nan_set_c(s)
 // (an empty group stays empty), with the threshold of the smallest df the pair can
@@ -620,11 +636,13 @@ pack_batch_kernel(const PackJob *__restrict__ jobs, int n_jobs, int64_t total_sl
     PqCoef w;
     w.w0 = 0x3c00u;  // 0/1 indicators of groups 0 and 1
     w.w1 = 0x3c00u | (1u << 18);
-    if (bits > 0) w = pq_coef(n0, n1, n2, row < 0 || excl, rh1, rh2, bits);
+    if (bits > 0)
+      w = J.linear ? pq_coef_linear(n0, n1, n2, row < 0 || excl, J.rl)
+                   : pq_coef(n0, n1, n2, row < 0 || excl, rh1, rh2, bits);
     if (sub == 0) {
       const int jj = jj0 + r0 + mr;
-      write_meta(m, jj, n0, n1, n2, row < 0 || excl, row < 0 ? 0 : row, rh1, rh2, signed_df1, 0,
-                 0.f);
+      write_meta(m, jj, n0, n1, n2, row < 0 || excl, row < 0 ? 0 : row, rh1, rh2, signed_df1,
+                 J.linear, J.rl);
       if (bits > 0) {
         m.pq0[jj] = w.w0;
         m.pq1[jj] = w.w1;
@@ -926,6 +944,94 @@ cudaError_t launch_pattern_lists(const unsigned int *n_missing, const int64_t *m
   complete_offsets_kernel<<<1, 1024, 0, s>>>(flags, n_snps, w.woff);
   complete_scatter_kernel<<<(unsigned)std::min<int64_t>((nw + 255) / 256, 152 * 8), 256, 0, s>>>(
       flags, w.woff, snp_begin, n_snps, complete_list);
+  return cudaGetLastError();
+}
+
+namespace {
+// One thread per neighbouring pair of coordinates.
+__global__ void order_kernel(const int64_t *__restrict__ a, int64_t n, const int64_t *__restrict__ b,
+                             int64_t m, unsigned int *status) {
+  bool bad = false;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i + 1 < n || i + 1 < m;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    if (i + 1 < n) bad |= a[i] > a[i + 1];
+    if (i + 1 < m) bad |= b[i] > b[i + 1];
+  }
+  if (bad) atomicOr(status, kDevUnsorted);
+}
+
+// First index of the nondecreasing a[0..n) with a[i] >= x (or > x).
+template <bool kAfter>
+__device__ __forceinline__ int bound_of(const int64_t *__restrict__ a, int n, int64_t x) {
+  int lo = 0, hi = n;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (kAfter ? a[mid] <= x : a[mid] < x) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+
+// One warp per B tile: the range of its SNP rows (lists need not be in order), whose
+// ends carry its smallest and largest coordinate, and the trait tiles within the
+// window of that range.
+__global__ void cis_items_kernel(const CisGroup *__restrict__ groups, int n_groups, int64_t n_tiles,
+                                 const int64_t *__restrict__ snp_pos,
+                                 const int64_t *__restrict__ trait_pos, int T, int64_t window,
+                                 WorkItem *__restrict__ items, int32_t *__restrict__ n_items) {
+  const int lane = threadIdx.x & 31;
+  const int64_t x = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (x >= n_tiles) return;
+  int gi = 0;
+  for (int lo = 0, hi = n_groups - 1; lo < hi;) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (groups[mid].tile0 <= x) lo = mid; else hi = mid - 1;
+    gi = lo;
+  }
+  const CisGroup g = groups[gi];
+  const int64_t b = x - g.tile0, j0 = b * g.tile_snps;
+  const int64_t j1 = j0 + g.tile_snps < g.n_snps ? j0 + g.tile_snps : g.n_snps;
+  int64_t first = INT64_MAX, last = -1;
+  if (g.snp_list) {
+    for (int64_t j = j0 + lane; j < j1; j += 32) {
+      const int64_t r = g.snp_list[j];
+      first = r < first ? r : first;
+      last = r > last ? r : last;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const int64_t f = __shfl_xor_sync(0xffffffffu, first, o), l = __shfl_xor_sync(0xffffffffu, last, o);
+      first = f < first ? f : first;
+      last = l > last ? l : last;
+    }
+  } else if (j0 < j1) {
+    first = g.snp_begin + j0;
+    last = g.snp_begin + j1 - 1;
+  }
+  if (lane != 0 || last < 0) return;
+  const int64_t lo = snp_pos[first], hi = snp_pos[last];
+  // (a window that leaves the integers' range reaches to the end)
+  const int t0 = lo < INT64_MIN + window ? 0 : bound_of<false>(trait_pos, T, lo - window);
+  const int t1 = hi > INT64_MAX - window ? T : bound_of<true>(trait_pos, T, hi + window);
+  if (t0 >= t1) return;
+  WorkItem w;
+  w.group = g.group;
+  w.btile = (int32_t)b;
+  w.step_begin = t0 / kTileM;
+  w.step_end = (t1 - 1) / kTileM + 1;
+  items[atomicAdd(n_items, 1)] = w;
+}
+}  // namespace
+
+cudaError_t launch_cis_items(const CisGroup *groups, int n_groups, int64_t n_tiles,
+                             const int64_t *snp_pos, int64_t S, const int64_t *trait_pos, int T,
+                             int64_t window, WorkItem *items, int32_t *n_items,
+                             unsigned int *status, cudaStream_t s) {
+  const int64_t most = S > T ? S : T;
+  if (most > 1)
+    order_kernel<<<(unsigned)std::min<int64_t>((most + 255) / 256, 152 * 8), 256, 0, s>>>(
+        snp_pos, S, trait_pos, T, status);
+  if (n_tiles > 0)
+    cis_items_kernel<<<(unsigned)((n_tiles + 7) / 8), 256, 0, s>>>(groups, n_groups, n_tiles, snp_pos,
+                                                                   trait_pos, T, window, items, n_items);
   return cudaGetLastError();
 }
 

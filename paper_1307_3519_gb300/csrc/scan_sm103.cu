@@ -1058,7 +1058,10 @@ __device__ __forceinline__ void range_pq(const uint32_t (&P)[NS], const uint32_t
 
 // D_0 and D_1 of a pair from its accumulators: P = A0 D_a + A1 D_b, Q = G D_b are exact
 // (ChunkMeta), so both quotients round to the integers they are.  w0 = 0 (a SNP that
-// is never tested): zeros.
+// is never tested): zeros.  kWhole off: standardised values instead of ranks, whose
+// sums are not whole numbers (a regression's SNP has no Q row: D_1 = 0, D_0 = P / A0
+// stands for both).
+template <bool kWhole = true>
 __device__ __forceinline__ void pq_sums(float P, float Q, uint32_t w0, uint32_t w1, float &u, float &v) {
   const float a0 = __half2float(__ushort_as_half((unsigned short)(w0 & 0xffffu)));
   const float a1 = __half2float(__ushort_as_half((unsigned short)(w0 >> 16)));
@@ -1068,8 +1071,10 @@ __device__ __forceinline__ void pq_sums(float P, float Q, uint32_t w0, uint32_t 
     v = 0.f;
     return;
   }
-  const float db = rintf(__fdividef(Q, g));
-  const float da = rintf(__fdividef(fmaf(-a1, db, P), a0));
+  float db = kWhole || g > 0.f ? __fdividef(Q, g) : 0.f;
+  if (kWhole) db = rintf(db);
+  float da = __fdividef(fmaf(-a1, db, P), a0);
+  if (kWhole) da = rintf(da);
   const float dl = -(da + db);
   const uint32_t a = (w1 >> 16) & 3u, b = (w1 >> 18) & 3u;
   u = a == 0u ? da : (b == 0u ? db : dl);
@@ -1363,7 +1368,9 @@ __device__ __forceinline__ unsigned int ev_process(EvLane &E, bool on, EvGroup &
                                                    const ScanParams &p, unsigned int wn, int lane,
                                                    int ev_warp, unsigned int &mcn) {
   float u, v;
-  pq_sums(E.P, E.Q, E.w0, E.w1, u, v);
+  const bool param = kMode == kEvPlain && p.provisional != 0;
+  if (param) pq_sums<false>(E.P, E.Q, E.w0, E.w1, u, v);
+  else pq_sums(E.P, E.Q, E.w0, E.w1, u, v);
   const float sv = kw_s(u, v, E.al, E.be, E.ga);
   float s = sv;
   bool act = on && E.snp >= 0;
@@ -1406,8 +1413,10 @@ __device__ __forceinline__ unsigned int ev_process(EvLane &E, bool on, EvGroup &
       E.n2df = (uint32_t)n2 | ((uint32_t)df << 16);
     }
   }
-  const bool cand = act && s + -E.tau * (1.f - p.margin) >= 0.f;
-  bool hit = cand && s + -E.tau * (1.f + p.margin) >= 0.f;
+  bool cand = act && s + -E.tau * (1.f - p.margin) >= 0.f;
+  if (kMode != kEvPerm && cand) cand = in_cis_window(p, E.snp, E.trait);
+  // (the parametric comparison keeps its whole band: it is decided after the launch)
+  bool hit = cand && (param || s + -E.tau * (1.f + p.margin) >= 0.f);
   if (cand && !hit)  // inside the band: FP64 (rare)
     hit = decide64_inl(u, v, (int)(E.n01 & 0xffffu), (int)(E.n01 >> 16), (int)(E.n2df & 0xffffu),
                        (int)(E.n2df >> 16), E.cfac, p.pthresh);
@@ -1838,6 +1847,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
                                     : reinterpret_cast<uint64_t *>(sbound + 2 * kTileM);
   const uint32_t bar0 = smem_u32(bars);
   const int nA = p.nA, nc = p.nc;
+  const int n_items = p.n_items_dev ? *p.n_items_dev : p.n_items;
   // barrier addresses
   auto a_full = [&](int s) { return bar0 + 8u * (uint32_t)s; };
   auto a_empty = [&](int s) { return bar0 + 8u * (uint32_t)(nA + s); };
@@ -1963,7 +1973,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         item_ring[ip.e] = it;
         mbar_arrive(it_full(ip.e));  // (release: the item is visible to who waits for it)
         item_next(ip);
-        if (it >= p.n_items) break;
+        if (it >= n_items) break;
         const WorkItem w = p.items[it];
         const GroupDesc *g = p.groups + w.group;
         if constexpr (!fast_form(kForm) || kPair) {
@@ -2133,7 +2143,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         const int it = item_ring[ip.e];
         mbar_arrive(it_empty(ip.e));
         item_next(ip);
-        if (it >= p.n_items) break;
+        if (it >= n_items) break;
         const WorkItem w = p.items[it];
         const GroupDesc *g = p.groups + w.group;
         const int ksteps = g->Np / 16;
@@ -2191,7 +2201,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         const int it = item_ring[ip.e];
         mbar_arrive(it_empty(ip.e));
         item_next(ip);
-        if (it >= p.n_items) break;
+        if (it >= n_items) break;
         const WorkItem w = p.items[it];
         const GroupDesc *g = p.groups + w.group;
         const int ncg = g->nc;
@@ -2288,7 +2298,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         const int it = item_ring[ip.e];
         mbar_arrive(it_empty(ip.e));
         item_next(ip);
-        if (it >= p.n_items) break;
+        if (it >= n_items) break;
         const WorkItem w = p.items[it];
         const GroupDesc *g = p.groups + w.group;
         const int ncg = g->nc;
@@ -2624,7 +2634,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         __syncwarp();
         mbar_arrive_lane0(it_empty(ip.e), lane);
         item_next(ip);
-        if (it >= p.n_items) break;
+        if (it >= n_items) break;
         const WorkItem w = p.items[it];
         const GroupDesc &g = p.groups[w.group];
         const int g_nc = g.nc, g_ntt = g.n_ttiles;
@@ -2749,7 +2759,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(it_empty(ip.e));
       item_next(ip);
-      if (it >= p.n_items) break;
+      if (it >= n_items) break;
       const WorkItem w = p.items[it];
       const GroupDesc &g = p.groups[w.group];
       const int nc_item = min(g.nc, g.nchunks - w.btile * g.nc);
