@@ -53,7 +53,7 @@ cudaError_t launch_pack2(const int8_t *geno, int64_t ldg, int N, int Np, const i
                          double h2, int allow_missing, int signed_df1, __half *B,
                          ChunkMeta *meta, uint64_t *codes, unsigned int *status, cudaStream_t s);
 cudaError_t launch_pack_batch(const PackJob *jobs, int n_jobs, int64_t total_slots,
-                              int64_t total_halves, double h1, double h2, int signed_df1,
+                              int64_t total_halves, const double *h, bool multi, int signed_df1,
                               unsigned int *status, cudaStream_t s);
 cudaError_t launch_rerank_buckets(const RerankJob *djobs, const RerankJob *hjobs,
                                   const int32_t *drops, int n_jobs, bool tiled, cudaStream_t s);
@@ -367,11 +367,11 @@ bool pick_launch_shape(const krux_ctx *ctx, int kpad, int codes_k, LaunchShape &
 // Whether a group of this width can take the plain scan form (the 32-byte swizzle
 // layout, an even number of resident chunks, room for the hit-event ring): 2 with the
 // whole K per rank stage, 1 with K blocks, 0 not.
-int plain_form_fits(const krux_ctx *ctx, int Np) {
+int plain_form_fits(const krux_ctx *ctx, int Np, bool pairs) {
   if (ctx->tune_layout == 0) return 0;
   const int kpad = round_up(Np, 16);
   LaunchShape sh;
-  if (!pick_launch_shape(ctx, kpad, 0, sh, kPlainExtra, pair_cta_wanted(kpad))) return 0;
+  if (!pick_launch_shape(ctx, kpad, 0, sh, kPlainExtra, pairs && pair_cta_wanted(kpad))) return 0;
   if (sh.pair_cta) return 1;
   const int nc = (int)(sh.b_region / (256 * kpad));
   if (nc < 2 || nc % 2 != 0 ||
@@ -1288,7 +1288,7 @@ krux_status materialise(krux_ctx *ctx, CallPlan &cp, cudaStream_t s) {
   cp.rerank_hjobs = jobs;
   cp.rerank_djobs = djobs;
   cp.rerank_drops = ddrop;
-  cp.rerank_tiled = !cp.multi && cp.slots.size() == 1 && ctx->tune_layout != 0 &&
+  cp.rerank_tiled = cp.slots.size() == 1 && ctx->tune_layout != 0 &&
                     cp.groups[0].dense_H == nullptr;
   KRUX_CUDA(ctx, launch_rerank_buckets(djobs, jobs.data(), ddrop, (int)nb, cp.rerank_tiled, s));
   if (ctx->profiling) ctx->prof.launches += 1;
@@ -1387,8 +1387,13 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   // place of the 2-bit codes) when at most one trait in 128 has more NaN samples
   // than the last set covers (each such trait sends all its pairs to the exact
   // test; beyond that share the general form is faster)
-  bool fast_shape = layout == 1 && !cp.multi && o->dense_H == nullptr &&
-                    (cp.param.model == 1 ? pq_range_linear(cp.param.rl) : pq_range_ok(fl.h1, fl.h2)) &&
+  if (cp.multi)
+    for (int d = 1; d <= 4; ++d) fl.hm[d - 1] = h_dfk(o->pthresh, d);
+  else
+    fl.hm[0] = fl.h1, fl.hm[1] = fl.h2;
+  bool fast_shape = layout == 1 && o->dense_H == nullptr &&
+                    (cp.param.model == 1 ? pq_range_linear(cp.param.rl)
+                                         : pq_range_ok(fl.h1, cp.multi ? fl.hm[3] : fl.h2)) &&
                     fast_form_ok();
   bool any_nan = false, fast_nan = allow_fast_nan && fast_shape;
   for (auto &g : cp.groups) {
@@ -1411,7 +1416,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     ctx->tune_nA = tnA;
     ctx->tune_ka = tka;
     // pairs of CTAs take complete data without permutations
-    const bool pairs = fast_shape && !fast_nan && fl.signed_coef == 0 && !cp.cis.on && tnc == 0 && tnA == 0 &&
+    const bool pairs = fast_shape && !fast_nan && fl.signed_coef == 0 && !cp.cis.on && !cp.multi && tnc == 0 && tnA == 0 &&
                        pair_cta_wanted(kpad);
     const bool ok = pick_launch_shape(ctx, kpad, codes_k, sh, fast_shape ? kPlainExtra : 0, pairs);
     ctx->tune_nc = s_nc;
@@ -1444,7 +1449,6 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
       total = std::max<int64_t>(total, (int64_t)(os.aux - base) + std::max<int64_t>(os.capacity, 1));
     KRUX_CUDA(ctx, ctx->aux2.ensure((size_t)total * sizeof(HitAux2)));
     for (auto &os : cp.slots) os.aux2 = ctx->aux2.as<HitAux2>() + (os.aux - base);
-    for (int d = 1; d <= 4; ++d) fl.hm[d - 1] = h_dfk(o->pthresh, d);
   }
   KRUX_CUDA(ctx, ctx->meta.ensure(std::max<int64_t>(mtot, 1) * sizeof(ChunkMeta)));
   KRUX_CUDA(ctx, ctx->codes.ensure(std::max<int64_t>(ctot, 1) * 8));
@@ -1634,7 +1638,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   // in one rank stage (or one pair resident and its K in blocks), no dense output, at
   // most three groups per marker
   {
-    bool fast = layout == 1 && !p.multi && (!p.has_nan || fast_nan) && !p.dense &&
+    bool fast = layout == 1 && (!p.has_nan || fast_nan) && !p.dense &&
                 (!p.signed_coef || p.perm);
     for (const GroupDesc &d : descs) fast = fast && d.pair == 1 && (d.nkb == 1 || d.nc == 2);
     p.fast = fast && fast_shape ? 1 : 0;
@@ -1668,7 +1672,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   if (fast_nan && !p.fast)  // the coefficient sets need the plain form: plan again
     return prepare_fused(ctx, cp, o, fl, s, tables, false);
   p.fast_nan = fast_nan ? 1 : 0;
-  fl.batched_pack = !cp.multi && (cp.param.model != 1 || p.fast);
+  fl.batched_pack = p.fast || (!cp.multi && cp.param.model != 1);
   if (fl.batched_pack) {
     std::vector<PackJob> jobs(ng);
     int64_t slots = 0, halves = 0;
@@ -1676,7 +1680,8 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
       const ScanGroupIn &g = cp.groups[i];
       PackJob &j = jobs[i];
       std::memset(&j, 0, sizeof j);
-      const int64_t nch = (g.n_snps + kChunkSnps - 1) / kChunkSnps;
+      const int64_t csn = cp.multi ? kChunkSnpsM : kChunkSnps;
+      const int64_t nch = (g.n_snps + csn - 1) / csn;
       j.geno = g.geno;
       j.geno_lo = g.geno + g.row_lo * g.ldg;
       j.geno_hi = g.geno + (g.row_hi - 1) * g.ldg + g.rs->N;
@@ -1696,7 +1701,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
       j.pq_bits = p.fast ? pq_bits(g.rs->N) : 0;
       j.linear = cp.param.model == 1 ? 1 : 0;
       j.rl = (float)cp.param.rl;
-      slots += nch * kChunkSnps;
+      slots += nch * csn;
       if (j.codes && !j.coef_nan) halves += nch * 2;
     }
     fl.n_pack_jobs = ng;
@@ -1777,8 +1782,8 @@ krux_status enqueue_fused(krux_ctx *ctx, CallPlan &cp, const FusedLaunch &fl, cu
   }
   ev_record(ctx, 2, s);
   if (fl.batched_pack && !cp.perm.packed)
-    KRUX_CUDA(ctx, launch_pack_batch(fl.packjobs, fl.n_pack_jobs, fl.pack_slots,
-                                     fl.pack_halves, fl.h1, fl.h2, fl.signed_coef, status, s));
+    KRUX_CUDA(ctx, launch_pack_batch(fl.packjobs, fl.n_pack_jobs, fl.pack_slots, fl.pack_halves,
+                                     fl.hm, cp.multi, fl.signed_coef, status, s));
   for (int i = 0; i < ng && !fl.batched_pack; ++i) {
     const ScanGroupIn &g = cp.groups[i];
     const krux_rankset *rs = g.rs;
@@ -2319,11 +2324,11 @@ extern "C" krux_status krux_scan_grouped(krux_ctx *ctx, krux_cohort *cohorts, in
   // launch of the general form; each cohort's groups stay in one launch, so its hit
   // list has one writer.
   constexpr int kParts = 3;
-  std::vector<int> plain(n_cohorts, cp.multi ? 0 : 2);
+  std::vector<int> plain(n_cohorts, 2);
   for (const ScanGroupIn &g : cp.groups)
     plain[g.out_slot] = g.nan_cnt || g.bucket >= 0
                             ? 0
-                            : std::min(plain[g.out_slot], plain_form_fits(ctx, g.rs->Np));
+                            : std::min(plain[g.out_slot], plain_form_fits(ctx, g.rs->Np, !cp.multi));
   CallPlan parts[kParts];
   for (int k = 0; k < kParts; ++k) {
     parts[k] = cp;

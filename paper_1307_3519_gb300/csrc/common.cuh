@@ -6,6 +6,7 @@
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include "../../include/krux.h"
@@ -159,7 +160,11 @@ struct ChunkMetaM {               // the same shared-memory slot as ChunkMeta
   int32_t snp[kChunkSnpsM];                  // output SNP index, -1 = padding / left out
   uint16_t n[kMaxCodeM + 1][kChunkSnpsM];    // group sizes over non-missing samples
   uint8_t df[kChunkSnpsM];                   // non-empty groups - 1
-  uint8_t pad_[2304 - 640 - 128 - 320 - 32];
+  // plain form: weights of the SNP's packed rows and the codes of its groups by size
+  // (PqCoefM), 3 bits each, the largest group's last
+  uint32_t pq[kMaxCodeM][kChunkSnpsM];       // A_i | C_i << 16 (FP16 bits)
+  uint32_t order[kChunkSnpsM];
+  uint8_t pad_[2304 - 640 - 128 - 320 - 32 - 512 - 128];
 };
 static_assert(sizeof(ChunkMetaM) == sizeof(ChunkMeta), "ChunkMetaM must fill a ChunkMeta slot");
 
@@ -219,6 +224,24 @@ __host__ __device__ inline int64_t tiled_index(int64_t row, int k, int Np) {
   return (row >> 7) * (int64_t)(kTileM * Np) + (k >> 4) * 2048 + r * 16 +
          ((((k >> 3) ^ (r >> 2)) & 1) << 3) + (k & 7);
 }
+
+// An event entry of the plain form for markers with up to five groups: 8 SNPs' four
+// accumulators, in the same slots and with the same tail as EvEntry.
+struct EvEntryM {
+  float P[kMaxCodeM][kEpiSnpsM];
+  uint32_t pq[kMaxCodeM][kEpiSnpsM], order[kEpiSnpsM];
+  float coef[kMaxCodeM + 1][kEpiSnpsM];
+  int32_t snp[kEpiSnpsM];
+  uint32_t n01[kEpiSnpsM], n23[kEpiSnpsM], n4df[kEpiSnpsM];
+  uint32_t pad_[2 * kEpiSnpsM];
+  double cfac;
+  float tau;
+  int32_t trait, group;
+};
+static_assert(offsetof(EvEntryM, cfac) == offsetof(EvEntry, cfac) &&
+                  offsetof(EvEntryM, group) == offsetof(EvEntry, group) &&
+                  sizeof(EvEntryM) <= sizeof(EvEntry),
+              "event entries share their slots");
 
 // ---- rank set: everything the scan needs about one expression matrix ------
 struct RankDev {

@@ -393,6 +393,66 @@ __device__ __forceinline__ PqCoef pq_coef_linear(int n0, int n1, int n2, bool ex
   return c;
 }
 
+// Weights of one marker's four packed rows in the plain form (up to five groups).  With
+// the groups by size, the largest left out and g_0 >= g_1 >= .. the others, the
+// quadratic form sum_i D_i^2 / N_i / h_df has the Cholesky factor
+//   P_i = l_i D_{g_i} + c_i sum_{k > i} D_{g_k},
+//   l_i = sqrt(r_i + rho_i), c_i = rho_i / l_i, rho_0 = r_largest, rho_{i+1} = rho_i r_i / l_i^2
+// (r = 1 / (N h_df)); empty groups have no row.  Rows are scaled by 1 + 4 * 2^-bits and
+// rounded as PqCoef's: A_i upwards, C_i on A_i's grid.  The grid error of row i is at
+// most 2^-bits l_i |sum_{k > i} D| <= 2^-bits sqrt(2 (3 - i)) times the form's root (l_i^2
+// <= 2 r_i <= 2 r_k), 3.5 * 2^-bits over the rows, so sum P_i^2 never falls below the
+// form (and exceeds it by about 20 * 2^-bits at most).
+struct PqCoefM {
+  uint32_t w[kMaxCodeM], order;
+};
+__device__ __forceinline__ PqCoefM pq_coef_multi(const int (&n)[kMaxCodeM + 1], bool excluded,
+                                                 const float *rh, int bits) {
+  PqCoefM c{};
+  // codes by size, largest first (selection: five entries)
+  int ord[kMaxCodeM + 1], sz[kMaxCodeM + 1];
+#pragma unroll
+  for (int i = 0; i <= kMaxCodeM; ++i) {
+    ord[i] = i;
+    sz[i] = n[i];
+  }
+#pragma unroll
+  for (int i = 0; i < kMaxCodeM; ++i)
+#pragma unroll
+    for (int k = i + 1; k <= kMaxCodeM; ++k)
+      if (sz[k] > sz[i]) {
+        const int a = sz[i], b = ord[i];
+        sz[i] = sz[k];
+        ord[i] = ord[k];
+        sz[k] = a;
+        ord[k] = b;
+      }
+  int groups = 0;
+#pragma unroll
+  for (int i = 0; i <= kMaxCodeM; ++i) groups += n[i] > 0;
+#pragma unroll
+  for (int i = 0; i < kMaxCodeM; ++i) c.order |= (uint32_t)ord[i + 1] << (3 * i);
+  c.order |= (uint32_t)ord[0] << 12;
+  if (groups < 2 || excluded) return c;
+  const float h = rh[groups - 2];
+  float rho = h / (float)sz[0];
+  const float up = (1.f + 4.f * exp2f((float)-bits)) * 1.00001f;
+#pragma unroll
+  for (int i = 0; i < kMaxCodeM; ++i) {
+    if (sz[i + 1] == 0) break;
+    const float r = h / (float)sz[i + 1];
+    const float l2 = r + rho;
+    const float a = round_up_bits(sqrtf(l2) * up, bits);
+    const uint32_t e = (__float_as_uint(a) >> 23) & 255u;
+    const float ulp = __uint_as_float((e - (uint32_t)(bits - 1)) << 23);
+    const float cc = rintf(a * (rho / l2) / ulp) * ulp;
+    c.w[i] = (uint32_t)__half_as_ushort(__float2half_rn(a)) |
+             ((uint32_t)__half_as_ushort(__float2half_rn(cc)) << 16);
+    rho = rho * r / l2;
+  }
+  return c;
+}
+
 // The plain form's coefficient sets of SNP slot jj for traits with NaN samples:
 // set s takes the quadratic form from group sizes max(N_i - C, 1), C = nan_set_c(s)
 // (an empty group stays empty), with the threshold of the smallest df the pair can
@@ -550,9 +610,16 @@ __device__ __forceinline__ void stage_granule(uint8_t *d, const int8_t *p, const
 // rows), and writes both packed rows with 16-byte stores.  Bound by the stores (4 Np
 // bytes per SNP against N read): one pass over the genotypes per SNP, so the group
 // sizes are known before the rows that are scaled by them are written.
+// kMulti: markers with up to five groups in the plain form's layout (chunks of 32 SNPs,
+// four rows each).
+struct RecipH {
+  float r[4];  // 1 / h_df
+};
+template <bool kMulti>
 __global__ void __launch_bounds__(kPackWarps * 32)
-pack_batch_kernel(const PackJob *__restrict__ jobs, int n_jobs, int64_t total_slots, float rh1,
-                  float rh2, int signed_df1, unsigned int *status) {
+pack_batch_kernel(const PackJob *__restrict__ jobs, int n_jobs, int64_t total_slots, RecipH rh,
+                  int signed_df1, unsigned int *status) {
+  const float rh1 = rh.r[0], rh2 = rh.r[1];
   __shared__ __align__(16) uint8_t stage[kPackWarps][kStageBytes + 32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t x0 = ((int64_t)blockIdx.x * kPackWarps + warp) * 32;
@@ -573,8 +640,9 @@ pack_batch_kernel(const PackJob *__restrict__ jobs, int n_jobs, int64_t total_sl
   const uint32_t inv_cpr = (65536u + (uint32_t)cpr - 1u) / (uint32_t)cpr;
   // consecutive rows are staged as the one span they form, others row by row
   const bool span = J.snp_list == nullptr && (int64_t)R * ldg + 32 <= kStageBytes;
-  const int64_t c = j0 / kChunkSnps;
-  const int jj0 = (int)(j0 % kChunkSnps);
+  constexpr int kSnps = kMulti ? kChunkSnpsM : kChunkSnps;
+  const int64_t c = j0 / kSnps;
+  const int jj0 = (int)(j0 % kSnps);
   ChunkMeta &m = J.meta[c];
   __half *Bc = J.B + c * kChunkRows * Np;
   bool any_bad = false, any_excl = false;
@@ -608,7 +676,7 @@ pack_batch_kernel(const PackJob *__restrict__ jobs, int n_jobs, int64_t total_sl
     // lanes L r .. L r + L - 1: the group sizes, missing and invalid codes of row r
     const int mr = lane >> (5 - lgr), sub = lane & (L - 1);
     const int64_t row = __shfl_sync(0xffffffffu, my_row, r0 + mr);
-    int n0 = 0, n1 = 0, n2 = 0, nm = 0;
+    int n0 = 0, n1 = 0, n2 = 0, n3 = 0, n4 = 0, nm = 0;
     const int o0 = row < 0 ? 0
                    : span  ? (int)((uintptr_t)(geno + row0 * ldg) & 15u) + mr * (int)ldg
                            : mr * pitch + (int)((uintptr_t)(geno + row * ldg) & 15u);
@@ -617,11 +685,15 @@ pack_batch_kernel(const PackJob *__restrict__ jobs, int n_jobs, int64_t total_sl
         uint32_t w = stage_word(st, o0 + k);
         const int v = min(N - k, 4);
         const uint32_t vm = v >= 4 ? 0xffffffffu : (1u << (8 * v)) - 1u;
-        w = (w & vm) | (0x04040404u & ~vm);  // 4: outside every class below
+        w = (w & vm) | (0x07070707u & ~vm);  // 7: outside every class below
         n0 += __popc(__vcmpeq4(w, 0u)) >> 3;
         n1 += __popc(__vcmpeq4(w, 0x01010101u)) >> 3;
         n2 += __popc(__vcmpeq4(w, 0x02020202u)) >> 3;
         nm += __popc(__vcmpeq4(w, 0xffffffffu)) >> 3;
+        if (kMulti) {
+          n3 += __popc(__vcmpeq4(w, 0x03030303u)) >> 3;
+          n4 += __popc(__vcmpeq4(w, 0x04040404u)) >> 3;
+        }
       }
     }
     for (int o = 1; o < L; o <<= 1) {
@@ -629,10 +701,73 @@ pack_batch_kernel(const PackJob *__restrict__ jobs, int n_jobs, int64_t total_sl
       n1 += __shfl_xor_sync(0xffffffffu, n1, o);
       n2 += __shfl_xor_sync(0xffffffffu, n2, o);
       nm += __shfl_xor_sync(0xffffffffu, nm, o);
+      if (kMulti) {
+        n3 += __shfl_xor_sync(0xffffffffu, n3, o);
+        n4 += __shfl_xor_sync(0xffffffffu, n4, o);
+      }
     }
     const bool excl = row >= 0 && nm > 0 && !J.allow_missing;
-    any_bad |= row >= 0 && n0 + n1 + n2 + nm != N;
+    any_bad |= row >= 0 && n0 + n1 + n2 + n3 + n4 + nm != N;
     any_excl |= excl;
+    if constexpr (kMulti) {
+      const int n[kMaxCodeM + 1] = {n0, n1, n2, n3, n4};
+      const PqCoefM w = pq_coef_multi(n, row < 0 || excl, rh.r, bits);
+      if (sub == 0) {
+        ChunkMetaM &mm = reinterpret_cast<ChunkMetaM &>(m);
+        const int jj = jj0 + r0 + mr;
+        const int groups = (n0 > 0) + (n1 > 0) + (n2 > 0) + (n3 > 0) + (n4 > 0);
+        const float h = groups > 1 && row >= 0 && !excl ? rh.r[groups - 2] : 0.f;
+#pragma unroll
+        for (int i = 0; i <= kMaxCodeM; ++i) {
+          mm.coef[i][jj] = n[i] > 0 ? h / (float)n[i] : 0.f;
+          mm.n[i][jj] = (uint16_t)n[i];
+        }
+        mm.snp[jj] = row < 0 || excl ? -1 : (int32_t)row;
+        mm.df[jj] = (uint8_t)(groups > 0 ? groups - 1 : 0);
+#pragma unroll
+        for (int i = 0; i < kMaxCodeM; ++i) mm.pq[i][jj] = w.w[i];
+        mm.order[jj] = w.order;
+      }
+      for (int t0 = 0; t0 < R * per_row; t0 += 32) {
+        const int t = t0 + lane;
+        const int r = (t >> 1) & (R - 1), k8 = 16 * (t >> (lgr + 1)) + 8 * (t & 1);
+        const int ln = (r << (5 - lgr)) & 31;
+        uint32_t wt[kMaxCodeM];
+#pragma unroll
+        for (int i = 0; i < kMaxCodeM; ++i) wt[i] = __shfl_sync(0xffffffffu, w.w[i], ln);
+        const uint32_t order = __shfl_sync(0xffffffffu, w.order, ln);
+        const int ob = __shfl_sync(0xffffffffu, row >= 0 ? o0 : -1, ln);
+        if (t >= R * per_row) continue;
+        uint32_t x[2] = {0x07070707u, 0x07070707u};
+        if (ob >= 0) {
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const int v = min(max(N - k8 - 4 * q, 0), 4);
+            const uint32_t vm = v >= 4 ? 0xffffffffu : (1u << (8 * v)) - 1u;
+            x[q] = (stage_word(st, ob + k8 + 4 * q) & vm) | (0x07070707u & ~vm);
+          }
+        }
+        uint32_t later[2] = {0u, 0u};  // samples in groups g_k, k > i
+#pragma unroll
+        for (int i = kMaxCodeM - 1; i >= 0; --i) {
+          const uint32_t code = ((order >> (3 * i)) & 7u) * 0x01010101u;
+          const uint32_t va = __byte_perm(wt[i], 0u, 0x1010), vc = __byte_perm(wt[i], 0u, 0x3232);
+          uint32_t o4[4];
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const uint32_t in = __vcmpeq4(x[q], code);
+            const uint2 a = mask_to_halves(in, va), b = mask_to_halves(later[q], vc);
+            o4[2 * q] = a.x | b.x;
+            o4[2 * q + 1] = a.y | b.y;
+            later[q] |= in;
+          }
+          *reinterpret_cast<uint4 *>(Bc + tiled_index(kChunkSnpsM * i + jj0 + r0 + r, k8, Np)) =
+              make_uint4(o4[0], o4[1], o4[2], o4[3]);
+        }
+      }
+      __syncwarp();
+      continue;
+    }
     PqCoef w;
     w.w0 = 0x3c00u;  // 0/1 indicators of groups 0 and 1
     w.w1 = 0x3c00u | (1u << 18);
@@ -888,14 +1023,20 @@ cudaError_t launch_pack2(const int8_t *geno, int64_t ldg, int N, int Np, const i
 }
 
 cudaError_t launch_pack_batch(const PackJob *jobs, int n_jobs, int64_t total_slots,
-                              int64_t total_halves, double h1, double h2, int signed_df1,
+                              int64_t total_halves, const double *h, bool multi, int signed_df1,
                               unsigned int *status, cudaStream_t s) {
   if (n_jobs <= 0) return cudaSuccess;
   if (total_slots > 0) {
     const int64_t warps = (total_slots + 31) / 32;
     const int64_t grid = (warps + kPackWarps - 1) / kPackWarps;
-    pack_batch_kernel<<<(unsigned)grid, kPackWarps * 32, 0, s>>>(
-        jobs, n_jobs, total_slots, (float)(1.0 / h1), (float)(1.0 / h2), signed_df1, status);
+    RecipH rh{};
+    for (int d = 0; d < (multi ? 4 : 2); ++d) rh.r[d] = (float)(1.0 / h[d]);
+    if (multi)
+      pack_batch_kernel<true><<<(unsigned)grid, kPackWarps * 32, 0, s>>>(jobs, n_jobs, total_slots, rh,
+                                                                        signed_df1, status);
+    else
+      pack_batch_kernel<false><<<(unsigned)grid, kPackWarps * 32, 0, s>>>(jobs, n_jobs, total_slots, rh,
+                                                                         signed_df1, status);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }

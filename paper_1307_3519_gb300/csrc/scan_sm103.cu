@@ -945,6 +945,22 @@ __device__ __forceinline__ void tmem_ld_half(uint32_t taddr, uint32_t (&u)[kFast
   tmem_ld16p(taddr + 64u, v);
 }
 
+// The four rows of 8 SNPs (markers with up to five groups; columns 32 i + ..).
+__device__ __forceinline__ void tmem_ld8p(uint32_t taddr, uint32_t *r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                 "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_ld_rows(uint32_t taddr, uint32_t (&u)[2 * kEpiSnpsM],
+                                             uint32_t (&v)[2 * kEpiSnpsM]) {
+  tmem_ld8p(taddr, u);
+  tmem_ld8p(taddr + 32u, u + kEpiSnpsM);
+  tmem_ld8p(taddr + 64u, v);
+  tmem_ld8p(taddr + 96u, v + kEpiSnpsM);
+}
+
 // Hot test of the plain form's traits with NaN samples on NS SNPs of a chunk (from SNP
 // `off`): true when some pair may lie at or above the lower edge of the band (q >= 0),
 // two SNPs per packed instruction, w = P + beta Q, q = alpha w^2 + gamma Q^2 -
@@ -1203,6 +1219,7 @@ struct EvGroup {
   int index = -1;
   krux_hit *hits;
   HitAux *aux;
+  HitAux2 *aux2;
   unsigned long long *counter;
   int64_t capacity;
   uint16_t gid;
@@ -1221,6 +1238,7 @@ __device__ __forceinline__ void ev_group(EvGroup &G, const ScanParams &p, int gr
   G.index = group;
   G.hits = g.hits;
   G.aux = g.aux;
+  G.aux2 = g.aux2;
   G.counter = g.counter;
   G.capacity = g.capacity;
   G.gid = (uint16_t)g.group_id;
@@ -1586,6 +1604,195 @@ __device__ __noinline__ unsigned int hit_event_m(const uint32_t *dv, bool mine, 
   return total;
 }
 
+// ---- the same markers in the plain form: weighted rows (PqCoefM), event warps ----
+// True when some SNP's sum_i P_i^2 reaches -ntlo; x0 holds P_0, P_1 of 8 SNPs, x1 P_2,
+// P_3.  Four FP32 operations per pair instead of eleven and five coefficients; with the
+// event warps, paired chunks and one half-block live, 20,000 x 100,000 x 102: 2.07 ms in
+// the general form, 1.08 in this one (8 N flop per pair: 78 % of the measured bf16 rate).
+__device__ __forceinline__ bool hit_pq_m(const uint32_t (&x0)[2 * kEpiSnpsM],
+                                         const uint32_t (&x1)[2 * kEpiSnpsM], float ntlo) {
+  const uint64_t nt2 = pk2(__float_as_uint(ntlo), __float_as_uint(ntlo));
+  uint32_t acc = 0xffffffffu;
+#pragma unroll
+  for (int j = 0; j < kEpiSnpsM; j += 2) {
+    uint64_t q = nt2;
+    const uint64_t a = pk2(x0[j], x0[j + 1]), b = pk2(x0[kEpiSnpsM + j], x0[kEpiSnpsM + j + 1]);
+    const uint64_t c = pk2(x1[j], x1[j + 1]), d = pk2(x1[kEpiSnpsM + j], x1[kEpiSnpsM + j + 1]);
+    q = ffma2(a, a, ffma2(b, b, ffma2(c, c, ffma2(d, d, q))));
+    uint32_t x, y;
+    upk2(q, x, y);
+    acc &= x & y;
+  }
+  return (int)acc >= 0;
+}
+
+// One entry per trait lane that found a candidate among 8 SNPs (see ev_submit).
+template <int kEntries>
+__device__ __forceinline__ bool ev_submit_m(const EvRing<kEntries> &ev,
+                                            const uint32_t (&x0)[2 * kEpiSnpsM],
+                                            const uint32_t (&x1)[2 * kEpiSnpsM], bool need,
+                                            const ChunkMetaM &m, int off, float tau, double cfac,
+                                            int trait, int group, const ScanParams &p,
+                                            uint32_t abort_addr, int lane) {
+  uint32_t lanes = __ballot_sync(0xffffffffu, need);
+  unsigned long long t = 0;
+  if (lane == 0) t = atomicAdd(ev.word, (unsigned long long)__popc(lanes)) & kEvTicketMask;
+  t = __shfl_sync(0xffffffffu, t, 0);
+  const int j = lane & (kEpiSnpsM - 1), jo = off + j;
+  while (lanes) {
+    const int L = __ffs((int)lanes) - 1;
+    lanes &= lanes - 1u;
+    int ok = 1;
+    if (lane == 0) {
+      ok = ev_gate(ev, t, p, abort_addr) ? 1 : 0;
+      __threadfence_block();  // the event warp's reads of the old contents come first
+    }
+    if (!__shfl_sync(0xffffffffu, ok, 0)) return false;
+    const int e = (int)(t % kEntries);
+    EvEntryM &E = reinterpret_cast<EvEntryM &>(ev.ent[e]);
+    if (lane < kEpiSnpsM) {
+#pragma unroll
+      for (int i = 0; i < kMaxCodeM; ++i) E.pq[i][j] = m.pq[i][jo];
+      E.order[j] = m.order[jo];
+#pragma unroll
+      for (int i = 0; i <= kMaxCodeM; ++i) E.coef[i][j] = m.coef[i][jo];
+      E.snp[j] = m.snp[jo];
+      E.n01[j] = (uint32_t)m.n[0][jo] | ((uint32_t)m.n[1][jo] << 16);
+      E.n23[j] = (uint32_t)m.n[2][jo] | ((uint32_t)m.n[3][jo] << 16);
+      E.n4df[j] = (uint32_t)m.n[4][jo] | ((uint32_t)m.df[jo] << 16);
+    }
+    if (lane == L) {
+#pragma unroll
+      for (int i = 0; i < kEpiSnpsM; i += 4) {
+        *reinterpret_cast<uint4 *>(E.P[0] + i) = make_uint4(x0[i], x0[i + 1], x0[i + 2], x0[i + 3]);
+        *reinterpret_cast<uint4 *>(E.P[1] + i) = make_uint4(x0[8 + i], x0[9 + i], x0[10 + i], x0[11 + i]);
+        *reinterpret_cast<uint4 *>(E.P[2] + i) = make_uint4(x1[i], x1[i + 1], x1[i + 2], x1[i + 3]);
+        *reinterpret_cast<uint4 *>(E.P[3] + i) = make_uint4(x1[8 + i], x1[9 + i], x1[10 + i], x1[11 + i]);
+      }
+      E.cfac = cfac;
+      E.tau = tau;
+      E.trait = trait;
+      E.group = group;
+    }
+    __threadfence_block();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(ev.full(e));
+    ++t;
+  }
+  return true;
+}
+
+// An event warp's work on up to two such entries, one per half-warp (lanes 0..7 of a
+// half take the entry's SNPs): the exact sums back from the accumulators, last row
+// first, the test in FP32 (FP64 inside the band), and the records as in ev_process.
+struct EvLaneM {
+  float P[kMaxCodeM], coef[kMaxCodeM + 1], tau;
+  uint32_t pq[kMaxCodeM], order, n01, n23, n4df;
+  int snp, trait, group;
+  double cfac;
+  __device__ __forceinline__ void load(const EvEntryM &E, int j) {
+#pragma unroll
+    for (int i = 0; i < kMaxCodeM; ++i) {
+      P[i] = E.P[i][j];
+      pq[i] = E.pq[i][j];
+    }
+#pragma unroll
+    for (int i = 0; i <= kMaxCodeM; ++i) coef[i] = E.coef[i][j];
+    order = E.order[j];
+    snp = E.snp[j];
+    n01 = E.n01[j];
+    n23 = E.n23[j];
+    n4df = E.n4df[j];
+    tau = E.tau;
+    cfac = E.cfac;
+    trait = E.trait;
+    group = E.group;
+  }
+};
+__device__ __forceinline__ unsigned int ev_process_m(const EvLaneM &E, bool on, EvGroup &G,
+                                                     const ScanParams &p, unsigned int wn, int lane,
+                                                     int ev_warp) {
+  const bool act = on && E.snp >= 0;
+  float D[kMaxCodeM + 1];
+#pragma unroll
+  for (int i = 0; i <= kMaxCodeM; ++i) D[i] = 0.f;
+  float later = 0.f;
+#pragma unroll
+  for (int i = kMaxCodeM - 1; i >= 0; --i) {
+    const float a = __half2float(__ushort_as_half((unsigned short)(E.pq[i] & 0xffffu)));
+    const float c = __half2float(__ushort_as_half((unsigned short)(E.pq[i] >> 16)));
+    const float d = a > 0.f ? rintf(__fdividef(fmaf(-c, later, E.P[i]), a)) : 0.f;
+    const uint32_t g = (E.order >> (3 * i)) & 7u;
+#pragma unroll
+    for (int k = 0; k <= kMaxCodeM; ++k)
+      if (g == (uint32_t)k) D[k] = d;
+    later += d;
+  }
+  const uint32_t gl = (E.order >> 12) & 7u;
+#pragma unroll
+  for (int k = 0; k <= kMaxCodeM; ++k)
+    if (gl == (uint32_t)k) D[k] = -later;
+  float s = 0.f;
+#pragma unroll
+  for (int k = 0; k <= kMaxCodeM; ++k) s = fmaf(E.coef[k] * D[k], D[k], s);
+  bool cand = act && s + -E.tau * (1.f - p.margin) >= 0.f;
+  if (cand) cand = in_cis_window(p, E.snp, E.trait);
+  bool hit = cand && s + -E.tau * (1.f + p.margin) > 0.f;
+  if (cand && !hit) {  // inside the band: FP64 (rare)
+    const int n[kMaxCodeM + 1] = {(int)(E.n01 & 0xffffu), (int)(E.n01 >> 16), (int)(E.n23 & 0xffffu),
+                                  (int)(E.n23 >> 16), (int)(E.n4df & 0xffffu)};
+    double Q = 0.0;
+    for (int k = 0; k <= kMaxCodeM; ++k)
+      if (n[k] > 0) Q += (double)D[k] * (double)D[k] / (double)n[k];
+    hit = chi2_tail64(E.cfac * Q, (int)(E.n4df >> 16)) < p.pthresh;
+  }
+  const uint32_t bal = __ballot_sync(0xffffffffu, hit);
+  const unsigned int n = (unsigned int)__popc(bal);
+  if (n == 0u) return 0u;
+  constexpr int kSegs = kEpiWarps / 2;
+  const unsigned int cap = (unsigned int)(kSegs * p.seg_cap);
+  const unsigned int idx = wn + (unsigned int)__popc(bal & ((1u << lane) - 1u));
+  const bool over = hit && idx >= cap;
+  const uint32_t obal = __ballot_sync(0xffffffffu, over);
+  unsigned long long gi = 0;
+  if (hit) ev_group(G, p, E.group);
+  if (obal != 0u) {  // one reservation per half (the halves may belong to different lists)
+    const uint32_t mine = obal & (0xffffu << (lane & 16));
+    const int lead = mine != 0u ? __ffs((int)mine) - 1 : 0;
+    if (over && lane == lead) gi = atomicAdd(G.counter, (unsigned long long)__popc(mine));
+    gi = __shfl_sync(0xffffffffu, gi, lead) + (unsigned int)__popc(mine & ((1u << lane) - 1u));
+  }
+  if (hit) {
+    krux_hit r;
+    r.trait = (uint32_t)E.trait;
+    r.snp = (uint32_t)E.snp;
+    r.d0 = (int32_t)D[0];
+    r.d1 = (int32_t)D[1];
+    HitAux x;
+    x.n0 = (uint16_t)(E.n01 & 0xffffu);
+    x.n1 = (uint16_t)(E.n01 >> 16);
+    x.n2 = (uint16_t)(E.n23 & 0xffffu);
+    x.group = G.gid;
+    HitAux2 y;
+    y.n3 = (uint16_t)(E.n23 >> 16);
+    y.n4 = (uint16_t)(E.n4df & 0xffffu);
+    y.pad0_ = y.pad1_ = 0;
+    y.d2 = (int32_t)D[2];
+    y.d3 = (int32_t)D[3];
+    if (!over) {
+      const size_t at = ((size_t)blockIdx.x * kEpiWarps + kSegs * ev_warp) * (size_t)p.seg_cap + idx;
+      st_hit(p.seg_hits + at, r);
+      st_aux(p.seg_aux + at, x);
+      p.seg_aux2[at] = y;
+    } else if (gi < (unsigned long long)G.capacity) {
+      st_hit(G.hits + gi, r);
+      st_aux(G.aux + gi, x);
+      G.aux2[gi] = y;
+    }
+  }
+  return n;
+}
+
 // Hot filter bounds of one (permutation, trait): the running best -ln p turned
 // into bounds on the form, |s| of df-1 SNPs and s of df-2 SNPs.
 struct MinpState {
@@ -1788,14 +1995,15 @@ enum ScanForm {
   kFormScanPerm = 4,
   kFormScanNan = 5,
   kFormScanSeed = 6,
-  kFormScanPair = 7
+  kFormScanPair = 7,
+  kFormScanMulti = 8
 };
 // the plain scan form, its two passes over permutation batches (the largest values
-// first, then the pairs against them), its variant for expression with NaN, and the
-// one over pairs of CTAs
+// first, then the pairs against them), its variant for expression with NaN, the one
+// over pairs of CTAs, and the one for markers with up to five groups
 constexpr bool fast_form(int f) {
   return f == kFormScan || f == kFormScanPerm || f == kFormScanNan || f == kFormScanSeed ||
-         f == kFormScanPair;
+         f == kFormScanPair || f == kFormScanMulti;
 }
 // The plain form over clusters of two CTAs, for sample counts whose chunk pair leaves
 // one CTA's shared memory too little room for rank tiles in flight: the pair's tensor
@@ -2442,13 +2650,24 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         }
         idle = false;
         __syncwarp();
+        auto release = [&]() {  // this use of the entry is finished
+          __syncwarp();
+          if (on && (lane & 15) == 0) {
+            __threadfence_block();
+            atomicAdd(ev.released + b, 1u);
+          }
+        };
+        if constexpr (kForm == kFormScanMulti) {
+          EvLaneM E;
+          E.load(reinterpret_cast<const EvEntryM &>(ev.ent[b]), lane & (kEpiSnpsM - 1));
+          release();
+          wn += ev_process_m(E, on && (lane & 15) < kEpiSnpsM, G, p, wn, lane, e);
+          if (on) t += 4;
+          continue;
+        }
         EvLane E;
         E.load(ev.ent[b], lane & (kEvSnps - 1));
-        __syncwarp();
-        if (on && (lane & 15) == 0) {  // this use of the entry is finished
-          __threadfence_block();
-          atomicAdd(ev.released + b, 1u);
-        }
+        release();
         wn += ev_process<kForm == kFormScanPerm ? kEvPerm : (kForm == kFormScanNan ? kEvNan : kEvPlain)>(
             E, on, G, p, wn, lane, e, mcn);
         if (on) t += 4;
@@ -2468,7 +2687,8 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       constexpr int kPerChunk = kChunkSnps / kFastSnps;  // warps per chunk and lane quarter
       const int q = warp & 3, k = warp >> 2;
       const int h = k / kPerChunk;                     // chunk of the pair
-      const int off = kFastSnps * (k % kPerChunk);     // first SNP within the chunk
+      constexpr bool kMultiF = kForm == kFormScanMulti;
+      const int off = (kMultiF ? kFastSnps / 2 : kFastSnps) * (k % kPerChunk);  // first SNP within the chunk
       const int row = 32 * q + lane;
       const uint32_t abort_addr = smem_u32(const_cast<const int *>(abort_flag));
       const uint32_t lane_cols =
@@ -2603,7 +2823,11 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         const uint32_t taddr = lane_cols + ps * 256u;
 #pragma unroll 1
         for (int half = 0; half < 2; ++half) {
-          tmem_ld_half(taddr + (uint32_t)(kH * half), x0, x1);
+          if constexpr (kMultiF) {  // 8 SNPs, P_i of SNP j in column 32 i + j of the chunk
+            tmem_ld_rows(taddr + (uint32_t)(kEpiSnpsM * half), x0, x1);
+          } else {
+            tmem_ld_half(taddr + (uint32_t)(kH * half), x0, x1);
+          }
           tmem_wait_ld();
           if (half) {
             tc_fence_before();
@@ -2620,6 +2844,17 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
             if (lo < smin) { smin = lo; pos1 = pos; }
           } else {
             const uint8_t *blk = kNan ? scodes + (size_t)c * codes_stride : nullptr;
+            if constexpr (kMultiF) {
+              const bool need = hit_pq_m(x0, x1, ntlo);
+              if (__any_sync(0xffffffffu, need)) {
+                const int trait = tt * kTileM + row;
+                if (!ev_submit_m(ev, x0, x1, need, reinterpret_cast<const ChunkMetaM &>(mc),
+                                 off + kEpiSnpsM * half, g.tau[trait], g.cfac[trait], trait, group, p,
+                                 abort_addr, lane))
+                  return false;
+              }
+              continue;
+            }
             const bool need = test(x0, x1, mc, o, blk);
             if (__any_sync(0xffffffffu, need) && !hand_over(x0, x1, need, mc, o, g, ag, tt, group))
               return false;
@@ -3315,6 +3550,9 @@ cudaError_t scan_set_smem_all(size_t smem) {
   e = cudaFuncSetAttribute(krux_scan_kernel<kFormScanPair>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(krux_scan_kernel<kFormScanMulti>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(krux_scan_kernel<kFormScanSeed>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -3330,7 +3568,7 @@ cudaError_t scan_set_smem_all(size_t smem) {
 
 // The kernel form launch_scan_only picks for these parameters (the ScanForm value).
 int scan_form_of(const ScanParams &p) {
-  if (p.multi) return kFormMulti;
+  if (p.multi) return kFormMulti;  // (in either form)
   if (p.perm) return p.fast && fast_form_ok() ? kFormScanPerm : kFormPerm;
   if (p.fast && fast_form_ok()) return p.fast_nan ? kFormScanNan : (p.pair_cta ? kFormScanPair : kFormScan);
   return kFormNan;
@@ -3378,7 +3616,9 @@ int pair_clusters() {
 }
 
 cudaError_t launch_scan_only(const ScanParams &p, int grid, size_t smem, cudaStream_t s) {
-  if (p.multi)
+  if (p.multi && p.fast && fast_form_ok())
+    krux_scan_kernel<kFormScanMulti><<<grid, kFastThreads, smem, s>>>(p);
+  else if (p.multi)
     krux_scan_kernel<kFormMulti><<<grid, kScanThreads, smem, s>>>(p);
   else if (p.perm && p.fast && p.seed_bound && fast_form_ok())
     krux_scan_kernel<kFormScanSeed><<<grid, kFastThreads, smem, s>>>(p);
@@ -3412,12 +3652,14 @@ bool fast_form_ok() {
   if (v < 0) {
     // the plain-form kernels were built at the register count their warp roles'
     // setmaxnreg split assumes
-    cudaFuncAttributes a, b, c, d;
+    cudaFuncAttributes a, b, c, d, m;
     v = cudaFuncGetAttributes(&a, krux_scan_kernel<kFormScan>) == cudaSuccess &&
                 cudaFuncGetAttributes(&b, krux_scan_kernel<kFormScanPerm>) == cudaSuccess &&
                 cudaFuncGetAttributes(&c, krux_scan_kernel<kFormScanNan>) == cudaSuccess &&
                 cudaFuncGetAttributes(&d, krux_scan_kernel<kFormScanSeed>) == cudaSuccess &&
                 d.numRegs == kFastRegsLaunch && d.maxThreadsPerBlock >= kFastThreads &&
+                cudaFuncGetAttributes(&m, krux_scan_kernel<kFormScanMulti>) == cudaSuccess &&
+                m.numRegs == kFastRegsLaunch && m.maxThreadsPerBlock >= kFastThreads &&
                 a.numRegs == kFastRegsLaunch && a.maxThreadsPerBlock >= kFastThreads &&
                 b.numRegs == kFastRegsLaunch && b.maxThreadsPerBlock >= kFastThreads &&
                 c.numRegs == kFastRegsLaunch && c.maxThreadsPerBlock >= kFastThreads

@@ -99,3 +99,43 @@ def test_pairs_of_ctas_report_a_wait_that_ran_out():
     assert kx.krux_scan(rs, geno, 1e-3, capacity=200_000)["n_hits"] == want
     rs.free()
     kx.close()
+
+
+@pytest.mark.parametrize("pth", [0.3, 1e-4])
+@pytest.mark.parametrize("N", [9, 31, 102, 128, 160, 181, 193, 256, 300, 340])
+def test_multiallelic_sums_and_hits_at_every_group_shape(oracle_mod, N, pth):
+    import itertools
+    import torch
+    from paper_1307_3519_gb300 import build
+    build.build()
+    import paper_1307_3519_gb300 as k
+    rng = np.random.default_rng(2 * N)
+    geno = []
+    for n0, n1, n2, n3 in itertools.product((0, 1, N // 5, N // 2), (0, 1, 2, N // 4), (0, 1, N // 6), (0, 1)):
+        if n0 + n1 + n2 + n3 > N:
+            continue
+        n = [n0, n1, n2, n3, N - n0 - n1 - n2 - n3]
+        codes = rng.permutation(5)
+        g = np.repeat(codes, n).astype(np.int8)
+        geno += [g, rng.permutation(g)]
+    geno = np.ascontiguousarray(np.stack(geno))
+    up = np.arange(N, dtype=np.float32)
+    expr = [up, -up, np.floor(up / 3)] + [up + rng.normal(0, s * N, N) for s in (0.1, 0.4, 1) for _ in range(10)]
+    expr += [np.round(rng.standard_normal(N), 1) for _ in range(100)]
+    expr = np.ascontiguousarray(np.stack(expr).astype(np.float32))
+    kx = k.Krux(0)
+    rs = kx.krux_rank(torch.from_numpy(expr).cuda())
+    r = kx.krux_scan(rs, torch.from_numpy(geno).cuda(), pth, capacity=expr.shape[0] * geno.shape[0],
+                     multiallelic=True)
+    orc = oracle_mod.scan(expr, geno, pth, max_code=4)
+    h = r["hits"].cpu().numpy().astype(np.int64)
+    got = np.zeros_like(orc["hit"])
+    got[h[:, 0], h[:, 1]] = True
+    near = np.abs(orc["p"] / pth - 1.0) < 1e-12
+    assert not ((got != orc["hit"]) & ~near).any()
+    assert r["n_hits"] == len(h) == int(got.sum())
+    H, p = r["H"].cpu().numpy(), r["p"].cpu().numpy()
+    assert np.all(np.abs(H - orc["H"][h[:, 0], h[:, 1]]) <= 1e-10 + 1e-9 * H)  # (all four sums)
+    assert np.all(np.abs(p - orc["p"][h[:, 0], h[:, 1]]) <= 1e-6 * p)
+    rs.free()
+    kx.close()
