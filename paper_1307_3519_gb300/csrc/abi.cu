@@ -204,6 +204,7 @@ struct krux_ctx {
       list, gemm_out, bucket_ranks, permA, minpkey, seg, permNan, aux2, param, paramOut, packjobs,
       host_in, host_out,  // krux_scan_host: device copies of the inputs, device hit list
       groups2, items2, packjobs2, cfacptr2,  // launch tables of a second launch in the same call
+      densecol,  // dense output: per-SNP table of the FP64 pass
       cistab,  // cis scans: their groups, for the planning on the device
       mcand,  // plain-form permutation batches: pairs for the deferred FP64 pass
       pattern, dlist;  // device-side missing-pattern grouping: scratch, SNP lists
@@ -669,7 +670,7 @@ void krux_destroy(krux_ctx *ctx) {
                     &ctx->list, &ctx->gemm_out, &ctx->bucket_ranks, &ctx->permA, &ctx->minpkey, &ctx->seg,
                     &ctx->permNan, &ctx->aux2, &ctx->param, &ctx->paramOut, &ctx->packjobs,
                     &ctx->host_in, &ctx->host_out, &ctx->groups2, &ctx->items2, &ctx->packjobs2,
-                    &ctx->cfacptr2, &ctx->mcand, &ctx->cistab, &ctx->pattern, &ctx->dlist};
+                    &ctx->cfacptr2, &ctx->mcand, &ctx->cistab, &ctx->densecol, &ctx->pattern, &ctx->dlist};
   for (DevBuf *b : bufs) b->release();
   ctx->list_host.release();
   for (auto &pb : ctx->pool) cudaFree(pb.second);
@@ -1289,7 +1290,7 @@ krux_status materialise(krux_ctx *ctx, CallPlan &cp, cudaStream_t s) {
   cp.rerank_djobs = djobs;
   cp.rerank_drops = ddrop;
   cp.rerank_tiled = cp.slots.size() == 1 && ctx->tune_layout != 0 &&
-                    cp.groups[0].dense_H == nullptr;
+                    (cp.groups[0].dense_H == nullptr || !cp.groups[0].rs->has_nan);
   KRUX_CUDA(ctx, launch_rerank_buckets(djobs, jobs.data(), ddrop, (int)nb, cp.rerank_tiled, s));
   if (ctx->profiling) ctx->prof.launches += 1;
   // runs of buckets of the same rank set: one A map each
@@ -1332,6 +1333,7 @@ struct FusedLaunch {
   int signed_coef = 0;
   bool fast_nan = false;  // the plain form's NaN variant (coefficient sets in the codes)
   int64_t cis_tiles = 0;  // cis scans: B tiles of all groups
+  int64_t max_chunks = 0; // dense output: chunks of the largest group
   std::vector<int64_t> boff, moff, coff;
   int layout = 1;
   double hm[4] = {0.0, 0.0, 0.0, 0.0};  // markers with codes 0..4: h_d for d = 1..4
@@ -1391,7 +1393,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     for (int d = 1; d <= 4; ++d) fl.hm[d - 1] = h_dfk(o->pthresh, d);
   else
     fl.hm[0] = fl.h1, fl.hm[1] = fl.h2;
-  bool fast_shape = layout == 1 && o->dense_H == nullptr &&
+  bool fast_shape = layout == 1 &&
                     (cp.param.model == 1 ? pq_range_linear(cp.param.rl)
                                          : pq_range_ok(fl.h1, cp.multi ? fl.hm[3] : fl.h2)) &&
                     fast_form_ok();
@@ -1401,6 +1403,8 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
                (g.nan_cnt == nullptr || 128 * g.rs->nan_traits_over <= g.rs->T);
     any_nan = any_nan || g.nan_cnt != nullptr;
   }
+  // (dense output of expression with NaN: the general form, with exact sizes per pair)
+  fast_nan = fast_nan && o->dense_H == nullptr;
   fast_nan = fast_nan && any_nan;
   fast_shape = fast_shape && (!any_nan || fast_nan);
   fl.fast_nan = fast_nan;
@@ -1416,7 +1420,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     ctx->tune_nA = tnA;
     ctx->tune_ka = tka;
     // pairs of CTAs take complete data without permutations
-    const bool pairs = fast_shape && !fast_nan && fl.signed_coef == 0 && !cp.cis.on && !cp.multi && tnc == 0 && tnA == 0 &&
+    const bool pairs = fast_shape && !fast_nan && fl.signed_coef == 0 && !cp.cis.on && !cp.multi && o->dense_H == nullptr && tnc == 0 && tnA == 0 &&
                        pair_cta_wanted(kpad);
     const bool ok = pick_launch_shape(ctx, kpad, codes_k, sh, fast_shape ? kPlainExtra : 0, pairs);
     ctx->tune_nc = s_nc;
@@ -1635,10 +1639,9 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     p.n_items_dev = ctx->status.as<int32_t>() + 10;  // (cleared with the status words)
   }
   // the plain scan form: 32-byte swizzle, every group's chunks paired and its K
-  // in one rank stage (or one pair resident and its K in blocks), no dense output, at
-  // most three groups per marker
+  // in one rank stage (or one pair resident and its K in blocks)
   {
-    bool fast = layout == 1 && (!p.has_nan || fast_nan) && !p.dense &&
+    bool fast = layout == 1 && (!p.has_nan || fast_nan) &&
                 (!p.signed_coef || p.perm);
     for (const GroupDesc &d : descs) fast = fast && d.pair == 1 && (d.nkb == 1 || d.nc == 2);
     p.fast = fast && fast_shape ? 1 : 0;
@@ -1698,7 +1701,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
       j.Np = g.rs->Np;
       j.allow_missing = g.allow_missing;
       j.coef_nan = j.codes != nullptr && fast_nan ? 1 : 0;
-      j.pq_bits = p.fast ? pq_bits(g.rs->N) : 0;
+      j.pq_bits = !p.fast ? 0 : (p.dense ? -1 : pq_bits(g.rs->N));
       j.linear = cp.param.model == 1 ? 1 : 0;
       j.rl = (float)cp.param.rl;
       slots += nch * csn;
@@ -1711,6 +1714,12 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     KRUX_CUDA(ctx, cudaMemcpyAsync(t_packjobs.p, jobs.data(), sizeof(PackJob) * ng,
                                    cudaMemcpyHostToDevice, s));
     fl.packjobs = t_packjobs.as<PackJob>();
+  }
+  if (p.fast && p.dense) {
+    KRUX_CUDA(ctx, ctx->densecol.ensure((size_t)cp.groups[0].dense_ld * sizeof(DenseCol)));
+    KRUX_CUDA(ctx, dense_prepare());
+    fl.max_chunks = 0;
+    for (const GroupDesc &d : descs) fl.max_chunks = std::max<int64_t>(fl.max_chunks, d.nchunks);
   }
   if (p.fast && p.perm && !cp.perm.seed && fl.grid > 0) {
     // each event warp's list for the deferred FP64 pass: about three times the
@@ -1808,6 +1817,15 @@ krux_status enqueue_fused(krux_ctx *ctx, CallPlan &cp, const FusedLaunch &fl, cu
   ev_record(ctx, 7, s);  // the scan kernel alone: events 7 .. 4
   if (fl.grid > 0) KRUX_CUDA(ctx, launch_scan_only(fl.p, fl.grid, fl.smem, s));
   ev_record(ctx, 4, s);
+  if (fl.p.fast && fl.p.dense) {
+    const ScanGroupIn &g = cp.groups[0];
+    const OutSlot &os = cp.slots[0];
+    KRUX_CUDA(ctx, launch_dense_finish(fl.p.groups, ng, fl.max_chunks, fl.cfacptr, g.rs->T, g.dense_ld,
+                                       g.dense_snp0, g.dense_ld, g.dense_H, g.dense_p,
+                                       ctx->densecol.as<DenseCol>(), fl.p.pthresh, os.hits, os.aux,
+                                       os.capacity, ctx->counters.as<unsigned long long>(),
+                                       ctx->sm_count, s));
+  }
   unsigned long long *totals = ctx->counters.as<unsigned long long>() + nslots;
   if (fl.staged) {
     KRUX_CUDA(ctx, launch_seg_compact(fl.p.seg_hits, fl.p.seg_aux, fl.p.seg_aux2, fl.p.seg_cnt,
@@ -1868,6 +1886,7 @@ int fused_launches(const CallPlan &cp, const FusedLaunch &fl) {
   for (auto &os : cp.slots) n += (os.capacity > 0 && cp.param.model < 0) ? 1 : 0;
   if (cp.param.model >= 0) n += 1;
   if (cp.cis.on) n += 2;
+  if (fl.p.fast && fl.p.dense) n += 2;
   if (cp.perm.on) {
     // the permuted stack (and NaN lists) unless a seed pass built them; then the
     // minimum-p read-out, or after a plain-form seed pass its exact decisions

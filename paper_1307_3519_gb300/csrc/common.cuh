@@ -289,8 +289,8 @@ struct PackJob {
   int32_t N, Np, allow_missing;
   int32_t coef_nan;         // 1: codes holds the plain form's coefficient blocks (kCoefNanBytes
                             // per chunk) instead of 2-bit codes
-  int32_t pq_bits;          // > 0: weighted rows of the plain forms (their significant bits);
-                            // 0: 0/1 indicators of groups 0 and 1
+  int32_t pq_bits;          // plain forms' layout: > 0 weighted rows (their significant bits),
+                            // < 0 0/1 indicators of groups 0 and 1; 0: indicators, row-major
   int32_t linear;           // dosage regression (parametric comparison): its coefficients,
   float rl;                 // rl (2 S_0 + S_1)^2 / S_gg
 };
@@ -458,7 +458,27 @@ struct CisGroup {
   int32_t group;
 };
 
+// A column (SNP) of a dense output: with sizes n_i (1 for an empty group, whose D_i is
+// 0), sum_i D_i^2 / n_i = (a D_0^2 + b D_1^2 + c D_2^2) / den, whole numbers below 2^50.
+struct alignas(16) DenseCol {
+  double den, rcp;          // n_0 n_1 n_2 and its reciprocal
+  uint32_t a, b, c;         // n_1 n_2, n_0 n_2, n_0 n_1
+  uint16_t n0, n1, n2;      // sizes as they are
+  uint8_t df;
+  uint8_t pad_;
+  int32_t group, snp;
+};
+
 // ---- launch wrappers (defined in the .cu files) -----------------------------
+// Dense output of a plain-form launch: dense_H holds every pair's D_0, D_1 (two int32);
+// they become FP64 H and p, and the hits (p < pthresh) are appended to the list.
+cudaError_t launch_dense_finish(const GroupDesc *groups, int n_groups, int64_t max_chunks,
+                                const double *const *cfac_by_group, int T, int64_t cols,
+                                int64_t snp0, int64_t ld, double *H, double *p, DenseCol *col,
+                                double pthresh, krux_hit *hits, HitAux *aux, int64_t capacity,
+                                unsigned long long *counter, int sm_count, cudaStream_t s);
+// Its tables (once per device; not during a graph capture).
+cudaError_t dense_prepare();
 // Work items of a cis scan: every B tile of the groups (n_tiles in all) against the
 // trait tiles its window reaches, appended to items / n_items (zero at launch); tiles
 // that reach no trait get none.  Coordinates out of order set kDevUnsorted.

@@ -790,8 +790,8 @@ pack_batch_kernel(const PackJob *__restrict__ jobs, int n_jobs, int64_t total_sl
     // is walked atom by atom, so that consecutive lanes fill consecutive rows' bytes
     for (int t0 = 0; t0 < R * per_row; t0 += 32) {
       const int t = t0 + lane;
-      const int r = bits > 0 ? (t >> 1) & (R - 1) : (int)(((uint32_t)t * inv_row) >> 16);
-      const int k8 = bits > 0 ? 16 * (t >> (lgr + 1)) + 8 * (t & 1) : 8 * (t - r * per_row);
+      const int r = bits != 0 ? (t >> 1) & (R - 1) : (int)(((uint32_t)t * inv_row) >> 16);
+      const int k8 = bits != 0 ? 16 * (t >> (lgr + 1)) + 8 * (t & 1) : 8 * (t - r * per_row);
       const int ln = (r << (5 - lgr)) & 31;
       const uint32_t w0 = __shfl_sync(0xffffffffu, w.w0, ln), w1 = __shfl_sync(0xffffffffu, w.w1, ln);
       const int ob = __shfl_sync(0xffffffffu, row >= 0 ? o0 : -1, ln);
@@ -816,8 +816,8 @@ pack_batch_kernel(const PackJob *__restrict__ jobs, int n_jobs, int64_t total_sl
       const uint2 p2 = mask_to_halves(ha, va), p3 = mask_to_halves(hb, vb);
       const uint2 q0 = mask_to_halves(lb, vg), q1 = mask_to_halves(hb, vg);
       const int rp = jj0 + r0 + r, rq = kChunkSnps + rp;  // rows of the chunk
-      const int64_t ap = bits > 0 ? tiled_index(rp, k8, Np) : (int64_t)rp * Np + k8;
-      const int64_t aq = bits > 0 ? tiled_index(rq, k8, Np) : (int64_t)rq * Np + k8;
+      const int64_t ap = bits != 0 ? tiled_index(rp, k8, Np) : (int64_t)rp * Np + k8;
+      const int64_t aq = bits != 0 ? tiled_index(rq, k8, Np) : (int64_t)rq * Np + k8;
       *reinterpret_cast<uint4 *>(Bc + ap) = make_uint4(p0.x | p1.x, p0.y | p1.y, p2.x | p3.x, p2.y | p3.y);
       *reinterpret_cast<uint4 *>(Bc + aq) = make_uint4(q0.x, q0.y, q1.x, q1.y);
     }

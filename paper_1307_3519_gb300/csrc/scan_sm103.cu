@@ -1996,14 +1996,16 @@ enum ScanForm {
   kFormScanNan = 5,
   kFormScanSeed = 6,
   kFormScanPair = 7,
-  kFormScanMulti = 8
+  kFormScanMulti = 8,
+  kFormScanDense = 9
 };
 // the plain scan form, its two passes over permutation batches (the largest values
 // first, then the pairs against them), its variant for expression with NaN, the one
-// over pairs of CTAs, and the one for markers with up to five groups
+// over pairs of CTAs, the one for markers with up to five groups, and the dense one,
+// which writes every pair's rank sums (indicator rows) for the FP64 pass after it
 constexpr bool fast_form(int f) {
   return f == kFormScan || f == kFormScanPerm || f == kFormScanNan || f == kFormScanSeed ||
-         f == kFormScanPair || f == kFormScanMulti;
+         f == kFormScanPair || f == kFormScanMulti || f == kFormScanDense;
 }
 // The plain form over clusters of two CTAs, for sample counts whose chunk pair leaves
 // one CTA's shared memory too little room for rank tiles in flight: the pair's tensor
@@ -2844,6 +2846,20 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
             if (lo < smin) { smin = lo; pos1 = pos; }
           } else {
             const uint8_t *blk = kNan ? scodes + (size_t)c * codes_stride : nullptr;
+            if constexpr (kForm == kFormScanDense) {
+              const int trait = tt * kTileM + row;
+              if (trait < g.T) {
+                int2 *out = reinterpret_cast<int2 *>(g.dense_H + (int64_t)trait * g.dense_ld) - g.dense_snp0;
+#pragma unroll
+                for (int j = 0; j < kH; ++j) {
+                  const int snp = mc.snp[o + j];
+                  if (snp >= 0)
+                    out[snp] = make_int2(__float2int_rn(__uint_as_float(x0[j])),
+                                         __float2int_rn(__uint_as_float(x1[j])));
+                }
+              }
+              continue;
+            }
             if constexpr (kMultiF) {
               const bool need = hit_pq_m(x0, x1, ntlo);
               if (__any_sync(0xffffffffu, need)) {
@@ -3553,6 +3569,9 @@ cudaError_t scan_set_smem_all(size_t smem) {
   e = cudaFuncSetAttribute(krux_scan_kernel<kFormScanMulti>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(krux_scan_kernel<kFormScanDense>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(krux_scan_kernel<kFormScanSeed>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -3569,6 +3588,7 @@ cudaError_t scan_set_smem_all(size_t smem) {
 // The kernel form launch_scan_only picks for these parameters (the ScanForm value).
 int scan_form_of(const ScanParams &p) {
   if (p.multi) return kFormMulti;  // (in either form)
+  if (p.dense) return kFormNan;    // (in either form)
   if (p.perm) return p.fast && fast_form_ok() ? kFormScanPerm : kFormPerm;
   if (p.fast && fast_form_ok()) return p.fast_nan ? kFormScanNan : (p.pair_cta ? kFormScanPair : kFormScan);
   return kFormNan;
@@ -3616,7 +3636,9 @@ int pair_clusters() {
 }
 
 cudaError_t launch_scan_only(const ScanParams &p, int grid, size_t smem, cudaStream_t s) {
-  if (p.multi && p.fast && fast_form_ok())
+  if (p.dense && p.fast && fast_form_ok())
+    krux_scan_kernel<kFormScanDense><<<grid, kFastThreads, smem, s>>>(p);
+  else if (p.multi && p.fast && fast_form_ok())
     krux_scan_kernel<kFormScanMulti><<<grid, kFastThreads, smem, s>>>(p);
   else if (p.multi)
     krux_scan_kernel<kFormMulti><<<grid, kScanThreads, smem, s>>>(p);
@@ -3652,7 +3674,7 @@ bool fast_form_ok() {
   if (v < 0) {
     // the plain-form kernels were built at the register count their warp roles'
     // setmaxnreg split assumes
-    cudaFuncAttributes a, b, c, d, m;
+    cudaFuncAttributes a, b, c, d, m, n;
     v = cudaFuncGetAttributes(&a, krux_scan_kernel<kFormScan>) == cudaSuccess &&
                 cudaFuncGetAttributes(&b, krux_scan_kernel<kFormScanPerm>) == cudaSuccess &&
                 cudaFuncGetAttributes(&c, krux_scan_kernel<kFormScanNan>) == cudaSuccess &&
@@ -3660,6 +3682,8 @@ bool fast_form_ok() {
                 d.numRegs == kFastRegsLaunch && d.maxThreadsPerBlock >= kFastThreads &&
                 cudaFuncGetAttributes(&m, krux_scan_kernel<kFormScanMulti>) == cudaSuccess &&
                 m.numRegs == kFastRegsLaunch && m.maxThreadsPerBlock >= kFastThreads &&
+                cudaFuncGetAttributes(&n, krux_scan_kernel<kFormScanDense>) == cudaSuccess &&
+                n.numRegs == kFastRegsLaunch && n.maxThreadsPerBlock >= kFastThreads &&
                 a.numRegs == kFastRegsLaunch && a.maxThreadsPerBlock >= kFastThreads &&
                 b.numRegs == kFastRegsLaunch && b.maxThreadsPerBlock >= kFastThreads &&
                 c.numRegs == kFastRegsLaunch && c.maxThreadsPerBlock >= kFastThreads
