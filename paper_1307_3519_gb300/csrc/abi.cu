@@ -745,11 +745,7 @@ krux_status krux_rank(krux_ctx *ctx, const float *expr, int T, int N, int64_t ld
     return st;
   }
   ev_record(ctx, 0, s);
-  // (the rows past T of the last tile stay zero in both layouts)
-  const size_t tile0 = (size_t)(T / kTileM) * kTileM * rs->Np, tail = (size_t)rs->rows_pad * rs->Np - tile0;
-  cudaError_t e = tail ? cudaMemsetAsync(rs->dev.A + tile0, 0, tail * 2, s) : cudaSuccess;
-  if (e == cudaSuccess && tail) e = cudaMemsetAsync(rs->dev.At + tile0, 0, tail * 2, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(rs->dev.tile_nan, 0, (size_t)rs->n_ttiles * 4, s);
+  cudaError_t e = cudaMemsetAsync(rs->dev.tile_nan, 0, (size_t)rs->n_ttiles * 4, s);
   if (e == cudaSuccess) e = launch_rank(expr, T, N, ld, rs->Np, rs->rows_pad, rs->dev, s);
   ev_record(ctx, 1, s);
   uint32_t any_nan = 0;
@@ -770,7 +766,7 @@ krux_status krux_rank(krux_ctx *ctx, const float *expr, int T, int N, int64_t ld
   if (ctx->profiling) {
     ctx->prof = krux_profile{};
     ctx->prof.ms_rank = ev_ms(ctx, 0, 1);
-    ctx->prof.launches = 2;  // the rank transform and the padding-row constants
+    ctx->prof.launches = 1;
   }
   *out = rs;
   return KRUX_OK;
@@ -2111,7 +2107,7 @@ extern "C" krux_status krux_scan_host(krux_ctx *ctx, const float *expr, int T, i
   }
   if (ctx->profiling) {
     ctx->prof.ms_rank = ms_rank;
-    ctx->prof.launches += 2;  // the rank transform's two kernels
+    ctx->prof.launches += 1;  // the rank transform
   }
   const int64_t k = direct ? 0 : std::min<int64_t>(*n_hits, cap);
   if (k > 0) {
