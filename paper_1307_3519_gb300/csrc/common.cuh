@@ -71,15 +71,14 @@ struct EvEntry {
   int32_t snp[kEvSnps];                         // output SNP index
   uint32_t n01[kEvSnps];                        // N_0 | N_1 << 16
   uint32_t n2df[kEvSnps];                       // N_2 | df << 16
-  double cfac;                                  // 3 / (K(K+1)C) of the trait
-  float tau;                                    // its fast-test bound
-  int32_t trait;                                // its trait row
+  float tau;                                    // the trait's fast-test bound
+  int32_t trait;                                // its row
   int32_t group;
   int32_t ag;                                   // rank-matrix group (> 0: a permutation)
   float b1, b2;                                 // permutation: the classes' largest decided values
   uint32_t id1, id2;                            // and the identities of the pairs that have them
   int32_t nan;                                  // plain form with NaN: the trait's NaN samples
-  int32_t pad_;
+  int32_t pad_[3];
 };
 static_assert(sizeof(EvEntry) % 16 == 0, "event entries keep 16-byte alignment");
 // shared memory of the ring: alignment slack, entries, a full barrier and a
@@ -234,11 +233,10 @@ struct EvEntryM {
   int32_t snp[kEpiSnpsM];
   uint32_t n01[kEpiSnpsM], n23[kEpiSnpsM], n4df[kEpiSnpsM];
   uint32_t pad_[2 * kEpiSnpsM];
-  double cfac;
   float tau;
   int32_t trait, group;
 };
-static_assert(offsetof(EvEntryM, cfac) == offsetof(EvEntry, cfac) &&
+static_assert(offsetof(EvEntryM, tau) == offsetof(EvEntry, tau) &&
                   offsetof(EvEntryM, group) == offsetof(EvEntry, group) &&
                   sizeof(EvEntryM) <= sizeof(EvEntry),
               "event entries share their slots");

@@ -1114,7 +1114,7 @@ struct EvRing {
 };
 constexpr unsigned long long kEvTicketMask = (1ull << 40) - 1ull;
 
-// Bounded wait of lane 0 until the entry of ticket t is free for its use t /
+// Bounded wait of a lane until the entry of ticket t is free for its use t /
 // kEntries; false on timeout or abort.
 template <int kEntries>
 __device__ __forceinline__ bool ev_gate(const EvRing<kEntries> &ev, unsigned long long t,
@@ -1138,72 +1138,80 @@ __device__ __forceinline__ bool ev_gate(const EvRing<kEntries> &ev, unsigned lon
   return true;
 }
 
-// An epilogue warp hands the traits of a half-block whose hot test found a
-// candidate to the event warps: one entry per such trait lane (tickets claimed
-// together), each with that lane's kEvSnps accumulator pairs and constants and the
-// SNPs' metadata (written by lanes 0..kEvSnps-1).  False if a wait gave up.
+// An epilogue warp hands the traits of a half-block whose hot test found a candidate to
+// the event warps: one entry per such trait lane (tickets claimed together), each with
+// that lane's accumulators and constants (`own`, by the lane) and the SNPs' metadata
+// (`meta`, by a half-warp per entry).  Each lane waits for its own entry to be free, and
+// all of the warp's entries are filled between one pair of fences (a lap of the ring at
+// most: no entry waits for another of the same lap).  One entry after the other, each
+// with its own wait, fences and arrival: 20,000 x 100,000 x 102 with 76,000 isolated
+// hits 643 us, now 628; 16 x 20,000 x 200,000 permutations 24.9 -> 23.9 ms in the
+// main launch.  False if a wait gave up.
+template <int kEntries, class Own, class Meta>
+__device__ __forceinline__ bool ev_fill(const EvRing<kEntries> &ev, bool need, const ScanParams &p,
+                                        uint32_t abort_addr, int lane, Own own, Meta meta) {
+  const uint32_t lanes = __ballot_sync(0xffffffffu, need);
+  const int n = __popc(lanes), rank = __popc(lanes & ((1u << lane) - 1u));
+  unsigned long long t = 0;
+  if (lane == 0) t = atomicAdd(ev.word, (unsigned long long)n) & kEvTicketMask;
+  t = __shfl_sync(0xffffffffu, t, 0);
+  for (int lap = 0; lap < n; lap += kEntries) {
+    const bool mine = need && rank >= lap && rank < lap + kEntries;
+    const int e = (int)((t + (unsigned long long)rank) % kEntries);
+    if (!__all_sync(0xffffffffu, !mine || ev_gate(ev, t + (unsigned long long)rank, p, abort_addr)))
+      return false;
+    __threadfence_block();  // the event warps' reads of the old contents come first
+    __syncwarp();
+    if (mine) own(ev.ent[e]);
+    for (int i = lap + (lane >> 4); i < min(n, lap + kEntries); i += 2)
+      meta(ev.ent[(int)((t + (unsigned long long)i) % kEntries)]);
+    __threadfence_block();
+    __syncwarp();
+    if (mine) mbar_arrive(ev.full(e));
+  }
+  return true;
+}
 template <int kEntries>
 __device__ __forceinline__ bool ev_submit(const EvRing<kEntries> &ev, const uint32_t (&u)[kEvSnps],
                                           const uint32_t (&v)[kEvSnps], bool need,
-                                          const ChunkMeta &m, int off, float tau, double cfac,
+                                          const ChunkMeta &m, int off, float tau,
                                           int trait, int group, int ag, float b1, float b2,
                                           uint32_t id1, uint32_t id2, int nan, const ScanParams &p,
                                           uint32_t abort_addr, int lane) {
-  uint32_t lanes = __ballot_sync(0xffffffffu, need);
-  unsigned long long t = 0;
-  if (lane == 0) t = atomicAdd(ev.word, (unsigned long long)__popc(lanes)) & kEvTicketMask;
-  t = __shfl_sync(0xffffffffu, t, 0);
-  // this lane's SNP metadata (lanes 0..kEvSnps-1), written into every entry
-  const int jo = off + (lane & (kEvSnps - 1));
+  const int j = lane & (kEvSnps - 1), jo = off + j;
   const float al = m.alpha[jo], be = m.beta[jo], ga = m.gamma[jo];
   const int32_t sn = m.snp[jo];
   const uint32_t n01 = (uint32_t)m.n[0][jo] | ((uint32_t)m.n[1][jo] << 16);
   const uint32_t n2df = (uint32_t)m.n[2][jo] | ((uint32_t)m.df[jo] << 16);
   const uint32_t w0 = m.pq0[jo], w1 = m.pq1[jo];
-  while (lanes) {
-    const int L = __ffs((int)lanes) - 1;
-    lanes &= lanes - 1u;
-    int ok = 1;
-    if (lane == 0) {
-      ok = ev_gate(ev, t, p, abort_addr) ? 1 : 0;
-      __threadfence_block();  // the event warp's reads of the old contents come first
-    }
-    if (!__shfl_sync(0xffffffffu, ok, 0)) return false;
-    const int e = (int)(t % kEntries);
-    EvEntry &E = ev.ent[e];
-    if (lane < kEvSnps) {
-      E.alpha[lane] = al;
-      E.beta[lane] = be;
-      E.gamma[lane] = ga;
-      E.snp[lane] = sn;
-      E.n01[lane] = n01;
-      E.n2df[lane] = n2df;
-      E.pq0[lane] = w0;
-      E.pq1[lane] = w1;
-    }
-    if (lane == L) {
+  return ev_fill(
+      ev, need, p, abort_addr, lane,
+      [&](EvEntry &E) {
 #pragma unroll
-      for (int j = 0; j < kEvSnps; j += 4) {
-        *reinterpret_cast<uint4 *>(E.u + j) = make_uint4(u[j], u[j + 1], u[j + 2], u[j + 3]);
-        *reinterpret_cast<uint4 *>(E.v + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-      }
-      E.cfac = cfac;
-      E.tau = tau;
-      E.trait = trait;
-      E.group = group;
-      E.ag = ag;
-      E.b1 = b1;
-      E.b2 = b2;
-      E.id1 = id1;
-      E.id2 = id2;
-      E.nan = nan;
-    }
-    __threadfence_block();
-    __syncwarp();
-    if (lane == 0) mbar_arrive(ev.full(e));
-    ++t;
-  }
-  return true;
+        for (int i = 0; i < kEvSnps; i += 4) {
+          *reinterpret_cast<uint4 *>(E.u + i) = make_uint4(u[i], u[i + 1], u[i + 2], u[i + 3]);
+          *reinterpret_cast<uint4 *>(E.v + i) = make_uint4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+        }
+        E.tau = tau;
+        E.trait = trait;
+        E.group = group;
+        E.ag = ag;
+        E.b1 = b1;
+        E.b2 = b2;
+        E.id1 = id1;
+        E.id2 = id2;
+        E.nan = nan;
+      },
+      [&](EvEntry &E) {
+        E.alpha[j] = al;
+        E.beta[j] = be;
+        E.gamma[j] = ga;
+        E.snp[j] = sn;
+        E.n01[j] = n01;
+        E.n2df[j] = n2df;
+        E.pq0[j] = w0;
+        E.pq1[j] = w1;
+      });
 }
 
 // Group fields an event warp needs, cached across entries.
@@ -1261,7 +1269,6 @@ struct EvLane {
   float P, Q, al, be, ga, tau, b1, b2;
   uint32_t w0, w1, n01, n2df, id1, id2;
   int snp, trait, group, ag, nan;
-  double cfac;
   __device__ __forceinline__ void load(const EvEntry &E, int j) {
     P = E.u[j];
     Q = E.v[j];
@@ -1274,7 +1281,6 @@ struct EvLane {
     n01 = E.n01[j];
     n2df = E.n2df[j];
     tau = E.tau;
-    cfac = E.cfac;
     trait = E.trait;
     group = E.group;
     ag = E.ag;
@@ -1343,10 +1349,11 @@ __device__ __forceinline__ void ev_minp(const EvLane &E, EvGroup &G, const ScanP
     mcn += n;
   } else if (need) {  // full: decide here
     const int df = (int)(E.n2df >> 16);
+    const double cfac = p.groups[E.group].cfac[E.trait];
     double key = -1.0;
-    if (df > 0 && E.cfac > 0.0)
+    if (df > 0 && cfac > 0.0)
       key = key64_of(kw_H64((int)u, (int)v, (int)(E.n01 & 0xffffu), (int)(E.n01 >> 16),
-                            (int)(E.n2df & 0xffffu), E.cfac),
+                            (int)(E.n2df & 0xffffu), cfac),
                      df);
     if (band && key > -log(p.pthresh))
       atomicAdd(p.fdr_hist + (int64_t)E.ag * p.fdr_bins + fdr_bin(key, p.fdr_l0, p.fdr_w, p.fdr_bins),
@@ -1437,7 +1444,7 @@ __device__ __forceinline__ unsigned int ev_process(EvLane &E, bool on, EvGroup &
   bool hit = cand && (param || s + -E.tau * (1.f + p.margin) >= 0.f);
   if (cand && !hit)  // inside the band: FP64 (rare)
     hit = decide64_inl(u, v, (int)(E.n01 & 0xffffu), (int)(E.n01 >> 16), (int)(E.n2df & 0xffffu),
-                       (int)(E.n2df >> 16), E.cfac, p.pthresh);
+                       (int)(E.n2df >> 16), p.groups[E.group].cfac[E.trait], p.pthresh);
   const uint32_t bal = __ballot_sync(0xffffffffu, hit);
   const unsigned int n = (unsigned int)__popc(bal);
   if (n == 0u) return 0u;
@@ -1626,60 +1633,45 @@ __device__ __forceinline__ bool hit_pq_m(const uint32_t (&x0)[2 * kEpiSnpsM],
   return (int)acc >= 0;
 }
 
-// One entry per trait lane that found a candidate among 8 SNPs (see ev_submit).
+// One entry per trait lane that found a candidate among 8 SNPs (see ev_fill).
 template <int kEntries>
 __device__ __forceinline__ bool ev_submit_m(const EvRing<kEntries> &ev,
                                             const uint32_t (&x0)[2 * kEpiSnpsM],
                                             const uint32_t (&x1)[2 * kEpiSnpsM], bool need,
-                                            const ChunkMetaM &m, int off, float tau, double cfac,
+                                            const ChunkMetaM &m, int off, float tau,
                                             int trait, int group, const ScanParams &p,
                                             uint32_t abort_addr, int lane) {
-  uint32_t lanes = __ballot_sync(0xffffffffu, need);
-  unsigned long long t = 0;
-  if (lane == 0) t = atomicAdd(ev.word, (unsigned long long)__popc(lanes)) & kEvTicketMask;
-  t = __shfl_sync(0xffffffffu, t, 0);
   const int j = lane & (kEpiSnpsM - 1), jo = off + j;
-  while (lanes) {
-    const int L = __ffs((int)lanes) - 1;
-    lanes &= lanes - 1u;
-    int ok = 1;
-    if (lane == 0) {
-      ok = ev_gate(ev, t, p, abort_addr) ? 1 : 0;
-      __threadfence_block();  // the event warp's reads of the old contents come first
-    }
-    if (!__shfl_sync(0xffffffffu, ok, 0)) return false;
-    const int e = (int)(t % kEntries);
-    EvEntryM &E = reinterpret_cast<EvEntryM &>(ev.ent[e]);
-    if (lane < kEpiSnpsM) {
+  return ev_fill(
+      ev, need, p, abort_addr, lane,
+      [&](EvEntry &slot) {
+        EvEntryM &E = reinterpret_cast<EvEntryM &>(slot);
 #pragma unroll
-      for (int i = 0; i < kMaxCodeM; ++i) E.pq[i][j] = m.pq[i][jo];
-      E.order[j] = m.order[jo];
+        for (int i = 0; i < kEpiSnpsM; i += 4) {
+          *reinterpret_cast<uint4 *>(E.P[0] + i) = make_uint4(x0[i], x0[i + 1], x0[i + 2], x0[i + 3]);
+          *reinterpret_cast<uint4 *>(E.P[1] + i) = make_uint4(x0[8 + i], x0[9 + i], x0[10 + i], x0[11 + i]);
+          *reinterpret_cast<uint4 *>(E.P[2] + i) = make_uint4(x1[i], x1[i + 1], x1[i + 2], x1[i + 3]);
+          *reinterpret_cast<uint4 *>(E.P[3] + i) = make_uint4(x1[8 + i], x1[9 + i], x1[10 + i], x1[11 + i]);
+        }
+        E.tau = tau;
+        E.trait = trait;
+        E.group = group;
+      },
+      [&](EvEntry &slot) {
+        EvEntryM &E = reinterpret_cast<EvEntryM &>(slot);
+        if (lane & kEpiSnpsM) {  // the half-warp's upper lanes: what the records hold
 #pragma unroll
-      for (int i = 0; i <= kMaxCodeM; ++i) E.coef[i][j] = m.coef[i][jo];
-      E.snp[j] = m.snp[jo];
-      E.n01[j] = (uint32_t)m.n[0][jo] | ((uint32_t)m.n[1][jo] << 16);
-      E.n23[j] = (uint32_t)m.n[2][jo] | ((uint32_t)m.n[3][jo] << 16);
-      E.n4df[j] = (uint32_t)m.n[4][jo] | ((uint32_t)m.df[jo] << 16);
-    }
-    if (lane == L) {
+          for (int i = 0; i <= kMaxCodeM; ++i) E.coef[i][j] = m.coef[i][jo];
+          E.snp[j] = m.snp[jo];
+        } else {
 #pragma unroll
-      for (int i = 0; i < kEpiSnpsM; i += 4) {
-        *reinterpret_cast<uint4 *>(E.P[0] + i) = make_uint4(x0[i], x0[i + 1], x0[i + 2], x0[i + 3]);
-        *reinterpret_cast<uint4 *>(E.P[1] + i) = make_uint4(x0[8 + i], x0[9 + i], x0[10 + i], x0[11 + i]);
-        *reinterpret_cast<uint4 *>(E.P[2] + i) = make_uint4(x1[i], x1[i + 1], x1[i + 2], x1[i + 3]);
-        *reinterpret_cast<uint4 *>(E.P[3] + i) = make_uint4(x1[8 + i], x1[9 + i], x1[10 + i], x1[11 + i]);
-      }
-      E.cfac = cfac;
-      E.tau = tau;
-      E.trait = trait;
-      E.group = group;
-    }
-    __threadfence_block();
-    __syncwarp();
-    if (lane == 0) mbar_arrive(ev.full(e));
-    ++t;
-  }
-  return true;
+          for (int i = 0; i < kMaxCodeM; ++i) E.pq[i][j] = m.pq[i][jo];
+          E.order[j] = m.order[jo];
+          E.n01[j] = (uint32_t)m.n[0][jo] | ((uint32_t)m.n[1][jo] << 16);
+          E.n23[j] = (uint32_t)m.n[2][jo] | ((uint32_t)m.n[3][jo] << 16);
+          E.n4df[j] = (uint32_t)m.n[4][jo] | ((uint32_t)m.df[jo] << 16);
+        }
+      });
 }
 
 // An event warp's work on up to two such entries, one per half-warp (lanes 0..7 of a
@@ -1689,7 +1681,6 @@ struct EvLaneM {
   float P[kMaxCodeM], coef[kMaxCodeM + 1], tau;
   uint32_t pq[kMaxCodeM], order, n01, n23, n4df;
   int snp, trait, group;
-  double cfac;
   __device__ __forceinline__ void load(const EvEntryM &E, int j) {
 #pragma unroll
     for (int i = 0; i < kMaxCodeM; ++i) {
@@ -1704,7 +1695,6 @@ struct EvLaneM {
     n23 = E.n23[j];
     n4df = E.n4df[j];
     tau = E.tau;
-    cfac = E.cfac;
     trait = E.trait;
     group = E.group;
   }
@@ -1744,7 +1734,7 @@ __device__ __forceinline__ unsigned int ev_process_m(const EvLaneM &E, bool on, 
     double Q = 0.0;
     for (int k = 0; k <= kMaxCodeM; ++k)
       if (n[k] > 0) Q += (double)D[k] * (double)D[k] / (double)n[k];
-    hit = chi2_tail64(E.cfac * Q, (int)(E.n4df >> 16)) < p.pthresh;
+    hit = chi2_tail64(p.groups[E.group].cfac[E.trait] * Q, (int)(E.n4df >> 16)) < p.pthresh;
   }
   const uint32_t bal = __ballot_sync(0xffffffffu, hit);
   const unsigned int n = (unsigned int)__popc(bal);
@@ -2717,6 +2707,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       int nsw = 1;
       // the hot test's bounds of the step: -tau (1 - margin), or the classes' bounds
       float ntlo = 0.f, bnd1 = 0.f, bnd2 = 0.f;
+      float tau_s = 0.f;  // the lane's tau
       // seed pass: this lane's largest df-2 value and df-1 |value| in the step and
       // the 16-SNP blocks (positions in the group's SNP order) that hold them
       float smax = 0.f, smin = 0.f;
@@ -2790,8 +2781,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
                            const ChunkMeta &mc, int o, const GroupDesc &g, int ag, int tt,
                            int group) -> bool {
         const int trait = tt * kTileM + row;
-        const float tau = g.tau[trait];
-        const double cfac = g.cfac[trait];
+        const float tau = kTwo ? g.tau[trait] : tau_s;
         bool real = need;
         float mx1 = 0.f, mx2 = 0.f;
         uint32_t id1 = 0u, id2 = 0u;
@@ -2806,7 +2796,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
             if (!__any_sync(0xffffffffu, real)) return true;
           }
         }
-        return ev_submit(ev, x0, x1, real, mc, o, tau, cfac, trait, group, ag, mx1, mx2, id1, id2,
+        return ev_submit(ev, x0, x1, real, mc, o, tau, trait, group, ag, mx1, mx2, id1, id2,
                          kNan ? nsw >> 9 : 0, p, abort_addr, lane);
       };
       // one accumulator pair: wait for it, load and test this warp's two halves one
@@ -2865,7 +2855,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
               if (__any_sync(0xffffffffu, need)) {
                 const int trait = tt * kTileM + row;
                 if (!ev_submit_m(ev, x0, x1, need, reinterpret_cast<const ChunkMetaM &>(mc),
-                                 off + kEpiSnpsM * half, g.tau[trait], g.cfac[trait], trait, group, p,
+                                 off + kEpiSnpsM * half, tau_s, trait, group, p,
                                  abort_addr, lane))
                   return false;
               }
@@ -2927,6 +2917,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
             tau_n = g_tau[tt * kTileM];  // (past the last step: a row that exists, unused)
           }
           ntlo = -tau * (1.f - p.margin);
+          tau_s = tau;
           if constexpr (kNan) {
             const int nan_c = (int)nan_n;
             if (g_nan) nan_n = g_nan[tt * kTileM + row];
