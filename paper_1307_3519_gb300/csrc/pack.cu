@@ -1176,4 +1176,103 @@ cudaError_t launch_cis_items(const CisGroup *groups, int n_groups, int64_t n_til
   return cudaGetLastError();
 }
 
+// ---- SNP order of a permutation batch --------------------------------------
+// The plain permutation forms test a 16-SNP block against one bound where its SNPs are of
+// one df class, and pick a bound per SNP where they are mixed: half as many operations
+// again and a shared-memory word per SNP.  So a large batch's SNPs are packed class by
+// class, df-2 ones first, each class in its own order.  Three small launches: a class bit
+// per SNP, the bits' prefix sums, the list.
+namespace {
+
+// Bit i of words[w]: SNP 32 w + i has exactly two genotype groups.  One warp per word.
+__global__ void class_bits_kernel(const int8_t *__restrict__ geno, int64_t ldg, int N,
+                                  int64_t n_snps, uint32_t *__restrict__ words, int64_t n_words) {
+  const int lane = threadIdx.x & 31;
+  const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (w >= n_words) return;
+  const int n = (int)min((int64_t)32, n_snps - 32 * w);
+  const int8_t *g = geno + 32 * w * ldg;
+  uint32_t bits = 0u;
+#pragma unroll 4
+  for (int i = 0; i < n; ++i, g += ldg) {
+    uint32_t seen = 0u;  // genotypes 0, 1, 2
+    for (int k = lane; k < N; k += 32) seen |= 1u << (g[k] & 3);
+    seen = __reduce_or_sync(0xffffffffu, seen) & 7u;
+    bits |= (__popc(seen) == 2 ? 1u : 0u) << i;
+  }
+  if (lane == 0) words[w] = bits;
+}
+
+// base[w]: SNPs of the first w words with their bit set; base[n_words]: of all.
+__global__ void __launch_bounds__(1024)
+    class_base_kernel(const uint32_t *__restrict__ words, int64_t n_words, uint32_t *__restrict__ base) {
+  __shared__ uint32_t part[32];
+  __shared__ uint32_t carry;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) carry = 0u;
+  for (int64_t w0 = 0; w0 < n_words; w0 += 8 * 1024) {
+    // eight words a thread
+    const int64_t w = w0 + 8 * threadIdx.x;
+    uint32_t c[8], sum = 0u;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      c[i] = w + i < n_words ? (uint32_t)__popc(words[w + i]) : 0u;
+      sum += c[i];
+    }
+    uint32_t pre = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, pre, o);
+      if (lane >= o) pre += y;
+    }
+    __syncthreads();  // (part and carry of the lap before are read)
+    if (lane == 31) part[warp] = pre;
+    __syncthreads();
+    uint32_t before = carry;
+    for (int i = 0; i < warp; ++i) before += part[i];
+    uint32_t at = before + pre - sum;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      if (w + i < n_words) base[w + i] = at;
+      at += c[i];
+    }
+    __syncthreads();
+    if (threadIdx.x == 1023) carry = at;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) base[n_words] = carry;
+}
+
+__global__ void class_list_kernel(const uint32_t *__restrict__ words, const uint32_t *__restrict__ base,
+                                  int64_t n_words, int64_t snp_begin, int64_t n_snps,
+                                  int64_t *__restrict__ list) {
+  const int64_t two = n_snps - (int64_t)base[n_words];  // SNPs of the first part
+  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n_snps;
+       j += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t word = words[j >> 5], bit = 1u << (j & 31);
+    const int64_t ones = (int64_t)base[j >> 5] + __popc(word & (bit - 1u));  // set ones before j
+    list[(word & bit) ? two + ones : j - ones] = snp_begin + j;
+  }
+}
+
+}  // namespace
+
+// list, words, prefix sums
+size_t class_order_bytes(int64_t n_snps) {
+  const int64_t n_words = (n_snps + 31) / 32;
+  return (size_t)n_snps * 8 + (size_t)(2 * n_words + 1) * 4;
+}
+cudaError_t launch_class_order(const int8_t *geno, int64_t ldg, int N, int64_t snp_begin,
+                               int64_t n_snps, void *scratch, cudaStream_t s) {
+  const int64_t n_words = (n_snps + 31) / 32;
+  int64_t *list = reinterpret_cast<int64_t *>(scratch);
+  uint32_t *words = reinterpret_cast<uint32_t *>(list + n_snps), *base = words + n_words;
+  class_bits_kernel<<<(unsigned)((n_words + 7) / 8), 256, 0, s>>>(geno + snp_begin * ldg, ldg, N, n_snps,
+                                                                  words, n_words);
+  class_base_kernel<<<1, 1024, 0, s>>>(words, n_words, base);
+  class_list_kernel<<<(unsigned)std::min<int64_t>((n_snps + 255) / 256, 152 * 8), 256, 0, s>>>(
+      words, base, n_words, snp_begin, n_snps, list);
+  return cudaGetLastError();
+}
+
 }  // namespace krux

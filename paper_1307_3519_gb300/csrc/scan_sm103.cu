@@ -1055,8 +1055,21 @@ __device__ __forceinline__ bool hit_pq2(const uint32_t (&P)[NS], const uint32_t 
   return (int)(acc0 & acc1) >= 0;
 }
 
-// Seed pass of a permutation batch: the largest P^2 + Q^2 of the df-2 SNPs into smax
-// and, negated, of the df-1 SNPs into smin.
+// Seed pass of a permutation batch: the largest P^2 + Q^2 of a block of one class.
+template <int NS>
+__device__ __forceinline__ float top_pq(const uint32_t (&P)[NS], const uint32_t (&Q)[NS]) {
+  float m = 0.f;
+#pragma unroll
+  for (int j = 0; j < NS; j += 2) {
+    const uint64_t q0 = pk2(Q[j], Q[j + 1]), p0 = pk2(P[j], P[j + 1]);
+    uint32_t sa, sb;
+    upk2(ffma2(p0, p0, fmul2(q0, q0)), sa, sb);
+    m = fmax3(m, __uint_as_float(sa), __uint_as_float(sb));
+  }
+  return m;
+}
+// And of a mixed block: of the df-2 SNPs into smax and, negated, of the df-1 SNPs into
+// smin.
 template <int NS>
 __device__ __forceinline__ void range_pq(const uint32_t (&P)[NS], const uint32_t (&Q)[NS],
                                          const float *sgn, float &smax, float &smin) {
@@ -2719,8 +2732,9 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       // form spilled 268 bytes in the loop: 75.7 ms per call of 16 x 20,000 x 200,000
       // against 52.8).
       auto test = [&](const uint32_t(&x0)[kH], const uint32_t(&x1)[kH], const ChunkMeta &mc, int o,
-                      const uint8_t *blk) -> bool {
+                      const uint8_t *blk, uint32_t cls) -> bool {
         if constexpr (kTwo) {
+          if (cls == 0u || cls == 0xffffffffu) return hit_pq<kH>(x0, x1, cls ? -bnd2 : -bnd1);
           return hit_pq2<kH>(x0, x1, mc.sgn + o, bnd1, bnd2);
         } else if constexpr (kNan) {
           const int wset = (nsw >> 4) & 15, nset = (nsw & 15) - 1;
@@ -2820,6 +2834,11 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
           } else {
             tmem_ld_half(taddr + (uint32_t)(kH * half), x0, x1);
           }
+          const int o = off + kH * half;
+          // permutation batches: the classes of the block's SNPs (all ones: df 2, zero:
+          // df 1; in the order of class_order_kernel nearly every block is of one class)
+          uint32_t cls = 0u;
+          if constexpr (kTwo || kSeed) cls = __ballot_sync(0xffffffffu, mc.sgn[o + (lane & (kH - 1))] > 0.f);
           tmem_wait_ld();
           if (half) {
             tc_fence_before();
@@ -2827,11 +2846,16 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
             if constexpr (kPair) mbar_arrive_cluster_lane0(peer_addr(t_empty(ps), 0u), lane);
             else mbar_arrive_lane0(t_empty(ps), lane);
           }
-          const int o = off + kH * half;
           if constexpr (kSeed) {
             const int pos = (chunk0 + c) * kChunkSnps + o;
             float hi = 0.f, lo = 0.f;
-            range_pq<kH>(x0, x1, mc.sgn + o, hi, lo);
+            if (cls == 0u || cls == 0xffffffffu) {
+              const float top = top_pq<kH>(x0, x1);
+              if (cls) hi = top;
+              else lo = -top;
+            } else {
+              range_pq<kH>(x0, x1, mc.sgn + o, hi, lo);
+            }
             if (hi > smax) { smax = hi; pos2 = pos; }
             if (lo < smin) { smin = lo; pos1 = pos; }
           } else {
@@ -2861,7 +2885,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
               }
               continue;
             }
-            const bool need = test(x0, x1, mc, o, blk);
+            const bool need = test(x0, x1, mc, o, blk, cls);
             if (__any_sync(0xffffffffu, need) && !hand_over(x0, x1, need, mc, o, g, ag, tt, group))
               return false;
           }
@@ -3408,8 +3432,7 @@ template <int kI>
 __global__ void __launch_bounds__(256)
     seed_decide_kernel(const unsigned long long *__restrict__ rec, const __half *__restrict__ stack,
                        int rows_pad, int Np, int N, int T, int P, const int8_t *__restrict__ geno,
-                       int64_t ldg, int64_t snp_begin, int64_t n_snps,
-                       const ChunkMeta *__restrict__ meta, const double *__restrict__ cfac, double *key,
+                       int64_t ldg, int64_t n_snps, const ChunkMeta *__restrict__ meta, const double *__restrict__ cfac, double *key,
                        unsigned long long *bound) {
   const int lane = threadIdx.x & 31;
   const int64_t nrec = (int64_t)P * T * 2;
@@ -3436,10 +3459,12 @@ __global__ void __launch_bounds__(256)
         ak[t] = k < N ? (int)__half2float(stack[tiled_index(arow, k, Np)]) : 0;
       }
       const int nj = (int)min((int64_t)16, n_snps - pos0);
-      const int8_t *g = geno + (snp_begin + pos0) * ldg;
+      int snp = -1;  // of position lane
+      if (lane < nj) snp = meta[(pos0 + lane) / kChunkSnps].snp[(pos0 + lane) % kChunkSnps];
       int d0 = 0, d1 = 0;  // of SNP lane
 #pragma unroll 4
-      for (int j = 0; j < nj; ++j, g += ldg) {
+      for (int j = 0; j < nj; ++j) {
+        const int8_t *g = geno + max(__shfl_sync(0xffffffffu, snp, j), 0) * ldg;
         int a = 0, b = 0;
 #pragma unroll
         for (int t = 0; t < kI; ++t) {
@@ -3467,7 +3492,7 @@ __global__ void __launch_bounds__(256)
       if (lane < nj) {
         const ChunkMeta &m = meta[(pos0 + lane) / kChunkSnps];
         const int w = (int)((pos0 + lane) % kChunkSnps);
-        if (m.snp[w] >= 0) {
+        if (snp >= 0) {
           const float sv = kw_s((float)d0, (float)d1, m.alpha[w], m.beta[w], m.gamma[w]);
           val = fmaxf((i & 1) ? sv : -sv, 0.f);
         }
@@ -3549,7 +3574,7 @@ cudaError_t launch_minp_cands(const MinpPair *list, const unsigned int *cnt, int
 
 cudaError_t launch_seed_decide(const unsigned long long *rec, const __half *stack, int rows_pad,
                                int Np, int N, int T, int P, const int8_t *geno, int64_t ldg,
-                               int64_t snp_begin, int64_t n_snps, const ChunkMeta *meta,
+                               int64_t n_snps, const ChunkMeta *meta,
                                const double *cfac, double *key, unsigned long long *bound,
                                cudaStream_t s) {
   const int64_t warps = ((int64_t)P * T * 2 + 31) / 32;
@@ -3557,7 +3582,7 @@ cudaError_t launch_seed_decide(const unsigned long long *rec, const __half *stac
   const int64_t blocks = (warps + 7) / 8;
   const int grid = (int)(blocks < 65535 ? blocks : 65535);
   auto *kernel = N <= 128 ? seed_decide_kernel<4> : (N <= 256 ? seed_decide_kernel<8> : seed_decide_kernel<16>);
-  kernel<<<grid, 256, 0, s>>>(rec, stack, rows_pad, Np, N, T, P, geno, ldg, snp_begin, n_snps, meta, cfac,
+  kernel<<<grid, 256, 0, s>>>(rec, stack, rows_pad, Np, N, T, P, geno, ldg, n_snps, meta, cfac,
                               key, bound);
   return cudaGetLastError();
 }
