@@ -10,6 +10,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <string>
 #include <tuple>
@@ -200,15 +201,18 @@ struct krux_ctx {
   // krux_scan_host: the genotypes' copy runs on its own stream beside the rank transform
   cudaStream_t xs = nullptr;
   cudaEvent_t xev = nullptr;
-  DevBuf B, meta, codes, groups, items, status, counters, aux, cfacptr, miss_idx, miss_mask,
-      list, gemm_out, bucket_ranks, permA, minpkey, seg, permNan, aux2, param, paramOut, packjobs,
+  DevBuf B, meta, codes, status, counters, aux, cfacptr, miss_idx, miss_mask,
+      list, gemm_out, bucket_ranks, permA, minpkey, seg, permNan, aux2, param, paramOut,
       host_in, host_out,  // krux_scan_host: device copies of the inputs, device hit list
-      groups2, items2, packjobs2, cfacptr2,  // launch tables of a second launch in the same call
+      tables, tables2,  // launch tables (groups, work items, pack jobs), and of a second launch in a call
       densecol,  // dense output: per-SNP table of the FP64 pass
       clsorder,  // permutation batch: its SNPs by df class
-      cistab,  // cis scans: their groups, for the planning on the device
       mcand,  // plain-form permutation batches: pairs for the deferred FP64 pass
       pattern, dlist;  // device-side missing-pattern grouping: scratch, SNP lists
+  HostBuf back;         // read-backs land here (page-locked: no staged copy, no wait per copy)
+  HostBuf up[2];        // launch tables on their way to the device, per table set
+  bool up_busy[2] = {false, false};  // a copy out of `up` may still run, on this stream
+  cudaStream_t up_stream[2] = {nullptr, nullptr};
   HostBuf list_host;  // staging of the SNP lists
   void *blas = nullptr;
   std::vector<std::pair<size_t, void *>> pool;  // freed rank-set blocks, reused by size
@@ -666,14 +670,16 @@ krux_status krux_create(krux_ctx **out, int device) {
 void krux_destroy(krux_ctx *ctx) {
   if (!ctx) return;
   cudaSetDevice(ctx->device);
-  DevBuf *bufs[] = {&ctx->B, &ctx->meta, &ctx->codes, &ctx->groups, &ctx->items, &ctx->status,
-                    &ctx->counters, &ctx->aux, &ctx->cfacptr, &ctx->miss_idx, &ctx->miss_mask,
-                    &ctx->list, &ctx->gemm_out, &ctx->bucket_ranks, &ctx->permA, &ctx->minpkey, &ctx->seg,
-                    &ctx->permNan, &ctx->aux2, &ctx->param, &ctx->paramOut, &ctx->packjobs,
-                    &ctx->host_in, &ctx->host_out, &ctx->groups2, &ctx->items2, &ctx->packjobs2,
-                    &ctx->cfacptr2, &ctx->mcand, &ctx->cistab, &ctx->densecol, &ctx->clsorder, &ctx->pattern, &ctx->dlist};
+  DevBuf *bufs[] = {&ctx->B, &ctx->meta, &ctx->codes, &ctx->status, &ctx->counters, &ctx->aux,
+                    &ctx->cfacptr, &ctx->miss_idx, &ctx->miss_mask, &ctx->list, &ctx->gemm_out,
+                    &ctx->bucket_ranks, &ctx->permA, &ctx->minpkey, &ctx->seg, &ctx->permNan, &ctx->aux2,
+                    &ctx->param, &ctx->paramOut, &ctx->host_in, &ctx->host_out, &ctx->tables,
+                    &ctx->tables2, &ctx->densecol, &ctx->clsorder, &ctx->mcand, &ctx->pattern,
+                    &ctx->dlist};
   for (DevBuf *b : bufs) b->release();
   ctx->list_host.release();
+  ctx->back.release();
+  for (HostBuf &h : ctx->up) h.release();
   for (auto &pb : ctx->pool) cudaFree(pb.second);
   for (int i = 0; i < kEv; ++i)
     if (ctx->ev[i]) cudaEventDestroy(ctx->ev[i]);
@@ -751,12 +757,14 @@ krux_status krux_rank(krux_ctx *ctx, const float *expr, int T, int N, int64_t ld
   ev_record(ctx, 1, s);
   uint32_t any_nan = 0;
   if (e == cudaSuccess) {
-    std::vector<uint32_t> tn(rs->n_ttiles);
-    e = cudaMemcpyAsync(tn.data(), rs->dev.tile_nan, tn.size() * 4, cudaMemcpyDeviceToHost, s);
+    e = ctx->back.ensure((size_t)rs->n_ttiles * 4);
+    const uint32_t *tn = reinterpret_cast<const uint32_t *>(ctx->back.p);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(ctx->back.p, rs->dev.tile_nan, (size_t)rs->n_ttiles * 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    for (uint32_t v : tn) {
-      any_nan |= v & 0xffffu;
-      rs->nan_traits_over += (int)(v >> 16);
+    for (int i = 0; e == cudaSuccess && i < rs->n_ttiles; ++i) {
+      any_nan |= tn[i] & 0xffffu;
+      rs->nan_traits_over += (int)(tn[i] >> 16);
     }
   }
   if (e != cudaSuccess) {
@@ -803,6 +811,15 @@ krux_status krux_rankset_export(krux_ctx *ctx, const krux_rankset *rs, int16_t *
 // Missing genotypes (section "Handling missing values": one genotype matrix per
 // missing-value pattern, with the expression re-ranked without those samples).
 namespace {
+
+// Status word of the missing-code pre-pass: SNPs that carry one.
+constexpr int kMissWord = 12;
+
+// The stream has been waited for: its uploads have left the page-locked tables.
+void uploads_done(krux_ctx *ctx, cudaStream_t s) {
+  for (int t = 0; t < 2; ++t)
+    if (ctx->up_stream[t] == s) ctx->up_busy[t] = false;
+}
 
 struct Bucket {
   std::vector<int32_t> drop;   // samples removed
@@ -857,27 +874,39 @@ krux_status group_on_device(krux_ctx *ctx, int N, int64_t b, int64_t n, int64_t 
   w.offset = reinterpret_cast<int64_t *>(pb + o_off);
   w.woff = reinterpret_cast<int64_t *>(pb + o_woff);
   w.cap = cap;
-  unsigned int *cnt = ctx->counters.as<unsigned int>();
   unsigned int *status = ctx->status.as<unsigned int>();
+  unsigned int *cnt = status + kMissWord;
   const size_t mask_bytes = (size_t)std::max<int64_t>(n, 1) * (kMaxN / 8);
   uint32_t *flags = reinterpret_cast<uint32_t *>(ctx->miss_mask.as<char>() + mask_bytes);
   KRUX_CUDA(ctx, launch_pattern_group(cnt, ctx->miss_mask.as<uint64_t>(), ctx->miss_idx.as<int64_t>(),
                                       n, w, status, s));
-  unsigned int nb = 0, st = 0;
-  KRUX_CUDA(ctx, cudaMemcpyAsync(&nb, w.n_buckets, 4, cudaMemcpyDeviceToHost, s));
-  KRUX_CUDA(ctx, cudaMemcpyAsync(&st, status, 4, cudaMemcpyDeviceToHost, s));
-  KRUX_CUDA(ctx, cudaStreamSynchronize(s));
+  // the bucket count, and in the same trip the buckets themselves if they are no more
+  // than kTrip (a second one otherwise)
+  constexpr int64_t kTrip = 256;
+  int64_t nr = std::min(n, kTrip);
+  const auto read = [&](int64_t k) -> cudaError_t {
+    const size_t each = 8 + 8 + (size_t)W * 8;
+    cudaError_t e = ctx->back.ensure(64 + (size_t)k * each);
+    char *h = reinterpret_cast<char *>(ctx->back.p);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, w.n_buckets, 4, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h + 8, status, 4, cudaMemcpyDeviceToHost, s);
+    h += 64;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, w.bucket_mask, (size_t)k * W * 8, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h + k * W * 8, w.first, (size_t)k * 8, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h + k * (W + 1) * 8, w.count, (size_t)k * 4, cudaMemcpyDeviceToHost, s);
+    return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+  };
+  KRUX_CUDA(ctx, read(nr));
+  const unsigned int nb = *reinterpret_cast<const unsigned int *>(ctx->back.p);
+  const unsigned int st = reinterpret_cast<const unsigned int *>(ctx->back.p)[2];
   if (st & kDevHashCollision) {
     KRUX_CUDA(ctx, cudaMemsetAsync(status, 0, 64, s));  // the host groups instead
     return KRUX_OK;
   }
-  std::vector<unsigned int> count(nb);
-  std::vector<unsigned long long> first(nb);
-  std::vector<uint64_t> bmask((size_t)nb * W);
-  KRUX_CUDA(ctx, cudaMemcpyAsync(count.data(), w.count, (size_t)nb * 4, cudaMemcpyDeviceToHost, s));
-  KRUX_CUDA(ctx, cudaMemcpyAsync(first.data(), w.first, (size_t)nb * 8, cudaMemcpyDeviceToHost, s));
-  KRUX_CUDA(ctx, cudaMemcpyAsync(bmask.data(), w.bucket_mask, bmask.size() * 8, cudaMemcpyDeviceToHost, s));
-  KRUX_CUDA(ctx, cudaStreamSynchronize(s));
+  if ((int64_t)nb > nr) KRUX_CUDA(ctx, read(nr = nb));
+  const uint64_t *bmask = reinterpret_cast<const uint64_t *>(reinterpret_cast<char *>(ctx->back.p) + 64);
+  const unsigned long long *first = reinterpret_cast<const unsigned long long *>(bmask + nr * W);
+  const unsigned int *count = reinterpret_cast<const unsigned int *>(first + nr);
   // buckets in order of their first SNP; lists back to back, then the complete rows
   std::vector<int> order(nb);
   for (unsigned int i = 0; i < nb; ++i) order[i] = (int)i;
@@ -895,7 +924,7 @@ krux_status group_on_device(krux_ctx *ctx, int N, int64_t b, int64_t n, int64_t 
   buckets.clear();
   for (int id : order) {
     Bucket bk;
-    const uint64_t *key = bmask.data() + (size_t)id * W;
+    const uint64_t *key = bmask + (size_t)id * W;
     for (int k = 0; k < N; ++k)
       if ((key[k / 64] >> (k % 64)) & 1ull) bk.drop.push_back(k);
     bk.dev_off = dl.base + offset[id];
@@ -910,29 +939,31 @@ krux_status group_on_device(krux_ctx *ctx, int N, int64_t b, int64_t n, int64_t 
 
 // Finds SNPs of rows [b, b+n) that carry a -1, groups them by their exact
 // missing-sample set, and lists the complete rows.  `bad` reports codes outside
-// {-1,0,1,2}.  Synchronises the stream.
+// {-1,0,1,2}.  Synchronises the stream, after `meanwhile` has run beside the pre-pass
+// (it must leave the status words and the stream's earlier work alone).
 krux_status find_missing(krux_ctx *ctx, const int8_t *geno, int64_t ldg, int N, int64_t b,
                          int64_t n, cudaStream_t s, std::vector<Bucket> &buckets,
                          std::vector<int64_t> &complete, bool &bad, int max_code,
-                         DevLists *dl = nullptr) {
+                         DevLists *dl = nullptr, const std::function<void()> &meanwhile = {}) {
   KRUX_CUDA(ctx, ctx->status.ensure(64));
-  KRUX_CUDA(ctx, ctx->counters.ensure(64));
+  KRUX_CUDA(ctx, ctx->back.ensure(64));
   KRUX_CUDA(ctx, ctx->miss_idx.ensure((size_t)std::max<int64_t>(n, 1) * 8));
   // the masks, then one flag bit per SNP for the flat pre-pass
   const size_t mask_bytes = (size_t)std::max<int64_t>(n, 1) * (kMaxN / 8);
   KRUX_CUDA(ctx, ctx->miss_mask.ensure(mask_bytes + (size_t)(n + 31) / 32 * 4 + 256));
   KRUX_CUDA(ctx, cudaMemsetAsync(ctx->status.p, 0, 64, s));
-  KRUX_CUDA(ctx, cudaMemsetAsync(ctx->counters.p, 0, 64, s));
-  unsigned int *cnt = ctx->counters.as<unsigned int>();
+  unsigned int *cnt = ctx->status.as<unsigned int>() + kMissWord;
   uint32_t *flags = reinterpret_cast<uint32_t *>(ctx->miss_mask.as<char>() + mask_bytes);
   KRUX_CUDA(ctx, launch_missing_scan(geno, ldg, N, b, n, max_code, cnt, ctx->miss_idx.as<int64_t>(),
                                      ctx->miss_mask.as<uint64_t>(), ctx->status.as<unsigned int>(),
                                      flags, s));
   if (ctx->profiling) ctx->prof.launches += ldg == N ? 2 : 1;
-  unsigned int m32 = 0, st = 0;
-  KRUX_CUDA(ctx, cudaMemcpyAsync(&m32, cnt, 4, cudaMemcpyDeviceToHost, s));
-  KRUX_CUDA(ctx, cudaMemcpyAsync(&st, ctx->status.p, 4, cudaMemcpyDeviceToHost, s));
+  KRUX_CUDA(ctx, cudaMemcpyAsync(ctx->back.p, ctx->status.p, 64, cudaMemcpyDeviceToHost, s));
+  if (meanwhile) meanwhile();
   KRUX_CUDA(ctx, cudaStreamSynchronize(s));
+  uploads_done(ctx, s);
+  const unsigned int st = *reinterpret_cast<const unsigned int *>(ctx->back.p);
+  const unsigned int m32 = reinterpret_cast<const unsigned int *>(ctx->back.p)[kMissWord];
   bad = (st & kDevBadCode) != 0;
   buckets.clear();
   complete.clear();
@@ -1118,28 +1149,15 @@ size_t bucket_bytes(const krux_rankset *rs) {
 // Groups for one rank set against SNP rows [b, e) of geno: complete SNPs as one
 // group, and one group per missing-sample pattern (section "Handling missing
 // values").  A / n_agroups give the (possibly permutation-stacked) rank matrices.
+// `ahead` is called with the group that complete genotypes would make, while the device
+// looks for missing ones.
 krux_status plan_groups(krux_ctx *ctx, CallPlan &cp, const krux_rankset *rs, const int8_t *geno,
                         int64_t ldg, int64_t b, int64_t e, const __half *A, int n_agroups,
                         int slot, double *dense_H, double *dense_p, double *minp_key,
-                        cudaStream_t s) {
+                        cudaStream_t s,
+                        const std::function<void(const ScanGroupIn &)> &ahead = {}) {
   const int64_t n = e - b;
   if (n <= 0) return KRUX_OK;
-  std::vector<Bucket> buckets;
-  std::vector<int64_t> complete;
-  bool bad = false;
-  DevLists dl;
-  if ((int64_t)(ctx->dlist.n / 8) >= cp.dlist_used + n) dl.base = cp.dlist_used;
-  krux_status st = find_missing(ctx, geno, ldg, rs->N, b, n, s, buckets, complete, bad,
-                                cp.multi ? kMaxCodeM : 2, &dl);
-  if (st != KRUX_OK) return st;
-  if (dl.base >= 0 && !buckets.empty()) cp.dlist_used += n;
-  if (bad)
-    return fail(ctx, KRUX_EINVAL, cp.multi ? "genotype code outside {-1, 0..4}"
-                                           : "genotype code outside {-1,0,1,2}");
-  if (cp.multi && rs->has_nan)
-    return fail(ctx, KRUX_EUNSUPPORTED, "markers with more than three groups need complete expression");
-  if (!buckets.empty() && n_agroups > 1)
-    return fail(ctx, KRUX_EUNSUPPORTED, "permutation scan with missing genotypes");
   ScanGroupIn g0;
   g0.rs = rs;
   g0.A = A ? A : rs->dev.A;
@@ -1160,12 +1178,32 @@ krux_status plan_groups(krux_ctx *ctx, CallPlan &cp, const krux_rankset *rs, con
   g0.dense_ld = n;
   g0.dense_snp0 = b;
   g0.minp_key = minp_key;
+  g0.snp_begin = b;
+  g0.n_snps = n;
+  std::function<void()> meanwhile;
+  if (ahead && !(cp.multi && rs->has_nan)) meanwhile = [&] { ahead(g0); };
+  std::vector<Bucket> buckets;
+  std::vector<int64_t> complete;
+  bool bad = false;
+  DevLists dl;
+  if ((int64_t)(ctx->dlist.n / 8) >= cp.dlist_used + n) dl.base = cp.dlist_used;
+  krux_status st = find_missing(ctx, geno, ldg, rs->N, b, n, s, buckets, complete, bad,
+                                cp.multi ? kMaxCodeM : 2, &dl, meanwhile);
+  if (st != KRUX_OK) return st;
+  if (dl.base >= 0 && !buckets.empty()) cp.dlist_used += n;
+  if (bad)
+    return fail(ctx, KRUX_EINVAL, cp.multi ? "genotype code outside {-1, 0..4}"
+                                           : "genotype code outside {-1,0,1,2}");
+  if (cp.multi && rs->has_nan)
+    return fail(ctx, KRUX_EUNSUPPORTED, "markers with more than three groups need complete expression");
+  if (!buckets.empty() && n_agroups > 1)
+    return fail(ctx, KRUX_EUNSUPPORTED, "permutation scan with missing genotypes");
   if (buckets.empty()) {
-    g0.snp_begin = b;
-    g0.n_snps = n;
     cp.groups.push_back(g0);
     return KRUX_OK;
   }
+  g0.snp_begin = 0;
+  g0.n_snps = 0;
   if (dl.base >= 0 && dl.complete_count > 0) {  // device lists
     g0.snp_list = ctx->dlist.as<int64_t>() + dl.complete_off;
     g0.n_snps = dl.complete_count;
@@ -1340,6 +1378,7 @@ struct FusedLaunch {
   int n_pack_jobs = 0;
   int64_t pack_slots = 0, pack_halves = 0;
   const PackJob *packjobs = nullptr;        // this launch's tables (device)
+  const CisGroup *cistab = nullptr;         // cis scans: their groups, planned on the device
   const double *const *cfacptr = nullptr;
 };
 
@@ -1350,10 +1389,6 @@ struct FusedLaunch {
 // plan is made again that way when the plain form's NaN variant does not fit).
 krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, FusedLaunch &fl,
                           cudaStream_t s, int tables = 0, bool allow_fast_nan = true) {
-  DevBuf &t_groups = tables ? ctx->groups2 : ctx->groups;
-  DevBuf &t_items = tables ? ctx->items2 : ctx->items;
-  DevBuf &t_packjobs = tables ? ctx->packjobs2 : ctx->packjobs;
-  DevBuf &t_cfacptr = tables ? ctx->cfacptr2 : ctx->cfacptr;
   fl.h1 = cp.param.model == 0 ? cp.param.h1 : h_df1(o->pthresh);
   fl.h2 = cp.param.model == 0 ? cp.param.h2 : h_df2(o->pthresh);
   const int ng = (int)cp.groups.size();
@@ -1571,32 +1606,15 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
       n_items += (size_t)plans[i].n_btiles;
     }
     fl.cis_tiles = (int64_t)n_items;
-    KRUX_CUDA(ctx, ctx->cistab.ensure(sizeof(CisGroup) * ng));
-    KRUX_CUDA(ctx, cudaMemcpyAsync(ctx->cistab.p, cis.data(), sizeof(CisGroup) * ng,
-                                   cudaMemcpyHostToDevice, s));
   } else {
     items = make_items(plans, workers);
     n_items = items.size();
   }
-  KRUX_CUDA(ctx, t_groups.ensure(sizeof(GroupDesc) * ng));
-  KRUX_CUDA(ctx, t_items.ensure(sizeof(WorkItem) * std::max<size_t>(n_items, 1)));
-  // pageable uploads: staged before the calls return, so the host vectors may go
-  KRUX_CUDA(ctx, cudaMemcpyAsync(t_groups.p, descs.data(), sizeof(GroupDesc) * ng,
-                                 cudaMemcpyHostToDevice, s));
-  if (!items.empty())
-    KRUX_CUDA(ctx, cudaMemcpyAsync(t_items.p, items.data(), sizeof(WorkItem) * items.size(),
-                                   cudaMemcpyHostToDevice, s));
   std::vector<const double *> cf(ng);
   for (int i = 0; i < ng; ++i) cf[i] = cp.groups[i].cfac;
-  KRUX_CUDA(ctx, t_cfacptr.ensure(sizeof(double *) * ng));
-  KRUX_CUDA(ctx, cudaMemcpyAsync(t_cfacptr.p, cf.data(), sizeof(double *) * ng,
-                                 cudaMemcpyHostToDevice, s));
-  fl.cfacptr = t_cfacptr.as<const double *>();
   KRUX_CUDA(ctx, finalize_prepare());
   ScanParams &p = fl.p;
   p = ScanParams{};
-  p.groups = t_groups.as<GroupDesc>();
-  p.items = t_items.as<WorkItem>();
   p.n_items = (int32_t)n_items;
   // the item counters sit behind the status words, one for each launch of a call
   // (cleared with them before the first)
@@ -1673,6 +1691,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   if (fast_nan && !p.fast)  // the coefficient sets need the plain form: plan again
     return prepare_fused(ctx, cp, o, fl, s, tables, false);
   p.fast_nan = fast_nan ? 1 : 0;
+  std::vector<PackJob> jobs;
   fl.batched_pack = p.fast || (!cp.multi && cp.param.model != 1);
   if (fl.batched_pack) {
     // a permutation batch's SNPs by df class: 16 x 20,000 x 200,000 46.4 -> 45.2 ms (the seed
@@ -1681,7 +1700,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     fl.class_order = p.fast && p.perm && ng == 1 && !cp.cis.on && cp.groups[0].snp_list == nullptr &&
                      (int64_t)cp.perm.P * cp.perm.rs->rows_pad * cp.groups[0].n_snps >= (int64_t)1 << 30;
     if (fl.class_order) KRUX_CUDA(ctx, ctx->clsorder.ensure(class_order_bytes(cp.groups[0].n_snps)));
-    std::vector<PackJob> jobs(ng);
+    jobs.resize(ng);
     int64_t slots = 0, halves = 0;
     for (int i = 0; i < ng; ++i) {
       const ScanGroupIn &g = cp.groups[i];
@@ -1714,10 +1733,6 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     fl.n_pack_jobs = ng;
     fl.pack_slots = slots;
     fl.pack_halves = halves;
-    KRUX_CUDA(ctx, t_packjobs.ensure(sizeof(PackJob) * ng));
-    KRUX_CUDA(ctx, cudaMemcpyAsync(t_packjobs.p, jobs.data(), sizeof(PackJob) * ng,
-                                   cudaMemcpyHostToDevice, s));
-    fl.packjobs = t_packjobs.as<PackJob>();
   }
   if (p.fast && p.dense) {
     KRUX_CUDA(ctx, ctx->densecol.ensure((size_t)cp.groups[0].dense_ld * sizeof(DenseCol)));
@@ -1739,6 +1754,44 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   const std::string why = validate_plan(p, descs, fl.smem);
   if (!why.empty()) return fail(ctx, KRUX_EUNSUPPORTED, "%s", why.c_str());
   if (fl.grid > 0) KRUX_CUDA(ctx, scan_set_smem(fl.smem));
+  // the launch's tables: one device buffer, one copy (the work items last, those of a
+  // cis scan are made on the device)
+  size_t bytes = 0;
+  const auto place = [&](size_t n) {
+    const size_t at = bytes;
+    bytes += (n + 255) / 256 * 256;
+    return at;
+  };
+  const size_t o_groups = place(sizeof(GroupDesc) * ng), o_cf = place(sizeof(double *) * ng);
+  const size_t o_jobs = place(sizeof(PackJob) * jobs.size()), o_cis = place(sizeof(CisGroup) * cis.size());
+  const size_t o_items = bytes;
+  const size_t sent = o_items + sizeof(WorkItem) * items.size();
+  DevBuf &tab = tables ? ctx->tables2 : ctx->tables;
+  KRUX_CUDA(ctx, tab.ensure(o_items + sizeof(WorkItem) * std::max<size_t>(n_items, 1)));
+  // page-locked, unless an earlier upload may still be reading them (several parts of
+  // one call): a pageable copy is staged before its call returns
+  std::vector<char> pageable;
+  char *src = nullptr;
+  if (!ctx->up_busy[tables] && ctx->up[tables].ensure(sent) == cudaSuccess) {
+    src = reinterpret_cast<char *>(ctx->up[tables].p);
+    ctx->up_busy[tables] = true;
+    ctx->up_stream[tables] = s;
+  } else {
+    pageable.resize(sent);
+    src = pageable.data();
+  }
+  std::memcpy(src + o_groups, descs.data(), sizeof(GroupDesc) * ng);
+  std::memcpy(src + o_cf, cf.data(), sizeof(double *) * ng);
+  if (!jobs.empty()) std::memcpy(src + o_jobs, jobs.data(), sizeof(PackJob) * jobs.size());
+  if (!cis.empty()) std::memcpy(src + o_cis, cis.data(), sizeof(CisGroup) * cis.size());
+  if (!items.empty()) std::memcpy(src + o_items, items.data(), sizeof(WorkItem) * items.size());
+  KRUX_CUDA(ctx, cudaMemcpyAsync(tab.p, src, sent, cudaMemcpyHostToDevice, s));
+  char *dev = tab.as<char>();
+  p.groups = reinterpret_cast<GroupDesc *>(dev + o_groups);
+  p.items = reinterpret_cast<WorkItem *>(dev + o_items);
+  fl.cfacptr = reinterpret_cast<const double *const *>(dev + o_cf);
+  fl.packjobs = reinterpret_cast<PackJob *>(dev + o_jobs);
+  fl.cistab = reinterpret_cast<CisGroup *>(dev + o_cis);
   return KRUX_OK;
 }
 
@@ -1751,7 +1804,7 @@ krux_status enqueue_fused(krux_ctx *ctx, CallPlan &cp, const FusedLaunch &fl, cu
   if (cp.fdr_hist)
     KRUX_CUDA(ctx, cudaMemsetAsync(cp.fdr_hist, 0, (size_t)cp.fdr_rows * cp.fdr_bins * 8, s));
   if (cp.cis.on)
-    KRUX_CUDA(ctx, launch_cis_items(ng ? ctx->cistab.as<CisGroup>() : nullptr, ng, fl.cis_tiles,
+    KRUX_CUDA(ctx, launch_cis_items(ng ? fl.cistab : nullptr, ng, fl.cis_tiles,
                                     cp.cis.snp_pos, cp.cis.S, cp.cis.trait_pos, cp.cis.T,
                                     cp.cis.window, const_cast<WorkItem *>(fl.p.items),
                                     ctx->status.as<int32_t>() + 10, ctx->status.as<unsigned int>(), s));
@@ -1920,13 +1973,19 @@ krux_status finish_fused(krux_ctx *ctx, CallPlan &cp, const FusedLaunch &fl, cud
                          std::vector<unsigned long long> &counts) {
   const int nslots = fl.nslots;
   counts.assign(nslots, 0);
-  unsigned int hst[2] = {0, 0};
-  if (!cp.groups.empty() || cp.cis.on) {
-    KRUX_CUDA(ctx, cudaMemcpyAsync(counts.data(), ctx->counters.as<unsigned long long>() + nslots,
-                                   (size_t)nslots * 8, cudaMemcpyDeviceToHost, s));
+  const bool any = !cp.groups.empty() || cp.cis.on;
+  KRUX_CUDA(ctx, ctx->back.ensure((size_t)nslots * 8 + 64));
+  unsigned int *hst = reinterpret_cast<unsigned int *>(ctx->back.p);
+  hst[0] = hst[1] = 0u;
+  if (any) {
     KRUX_CUDA(ctx, cudaMemcpyAsync(hst, ctx->status.p, 8, cudaMemcpyDeviceToHost, s));
+    KRUX_CUDA(ctx, cudaMemcpyAsync(reinterpret_cast<char *>(ctx->back.p) + 64,
+                                   ctx->counters.as<unsigned long long>() + nslots,
+                                   (size_t)nslots * 8, cudaMemcpyDeviceToHost, s));
   }
   KRUX_CUDA(ctx, cudaStreamSynchronize(s));
+  uploads_done(ctx, s);
+  if (any) std::memcpy(counts.data(), reinterpret_cast<char *>(ctx->back.p) + 64, (size_t)nslots * 8);
   if (ctx->profiling && !cp.groups.empty()) {
     ctx->prof.ms_pack = ev_ms(ctx, 2, 3);
     ctx->prof.ms_scan = ev_ms(ctx, 7, 4);
@@ -2014,13 +2073,27 @@ extern "C" krux_status krux_scan(krux_ctx *ctx, const krux_rankset *rs, const in
   CallPlan cp;
   cp.multi = (opts->flags & KRUX_FLAG_MULTIALLELIC) != 0;
   cp.slots.push_back(OutSlot{hits, hit_H, hit_p, opts->hit_capacity, ctx->aux.as<HitAux>()});
+  // planned as for complete genotypes while the device looks for missing ones
+  CallPlan whole = cp;
+  FusedLaunch fl;
+  krux_status ready = KRUX_EUNSUPPORTED;
+  const auto ahead = [&](const ScanGroupIn &g) {
+    whole.groups.push_back(g);
+    const std::string err = ctx->err;
+    ready = prepare_fused(ctx, whole, opts, fl, s);
+    if (ready != KRUX_OK) ctx->err = err;  // (what counts is the plan that is launched)
+  };
   st = plan_groups(ctx, cp, rs, geno, ldg, b, e, nullptr, 1, 0, opts->dense_H, opts->dense_p,
-                   nullptr, s);
-  if (st != KRUX_OK) return st;
-  st = materialise(ctx, cp, s);
+                   nullptr, s, ahead);
   if (st != KRUX_OK) return st;
   std::vector<unsigned long long> counts;
-  st = run_fused(ctx, cp, opts, s, counts);
+  if (ready == KRUX_OK && cp.bucket_jobs.empty()) {
+    st = enqueue_fused(ctx, whole, fl, s);
+    if (st == KRUX_OK) st = finish_fused(ctx, whole, fl, s, counts);
+  } else {
+    st = materialise(ctx, cp, s);
+    if (st == KRUX_OK) st = run_fused(ctx, cp, opts, s, counts);
+  }
   if (st != KRUX_OK) return st;
   *n_hits = (int64_t)counts[0];
   if (*n_hits > opts->hit_capacity)
@@ -2163,12 +2236,26 @@ extern "C" krux_status krux_scan_cis(krux_ctx *ctx, const krux_rankset *rs, cons
   KRUX_CUDA(ctx, ctx->aux.ensure((size_t)std::max<int64_t>(opts->hit_capacity, 1) * sizeof(HitAux)));
   cp.slots.push_back(OutSlot{hits, hit_H, hit_p, opts->hit_capacity, ctx->aux.as<HitAux>()});
   KRUX_CUDA(ctx, ctx->dlist.ensure((size_t)std::max<int64_t>(e - b, 1) * 8));
-  st = plan_groups(ctx, cp, rs, geno, ldg, b, e, nullptr, 1, 0, nullptr, nullptr, nullptr, s);
-  if (st != KRUX_OK) return st;
-  st = materialise(ctx, cp, s);
+  // planned as for complete genotypes while the device looks for missing ones
+  CallPlan whole = cp;
+  FusedLaunch fl;
+  krux_status ready = KRUX_EUNSUPPORTED;
+  const auto ahead = [&](const ScanGroupIn &g) {
+    whole.groups.push_back(g);
+    const std::string err = ctx->err;
+    ready = prepare_fused(ctx, whole, opts, fl, s);
+    if (ready != KRUX_OK) ctx->err = err;  // (what counts is the plan that is launched)
+  };
+  st = plan_groups(ctx, cp, rs, geno, ldg, b, e, nullptr, 1, 0, nullptr, nullptr, nullptr, s, ahead);
   if (st != KRUX_OK) return st;
   std::vector<unsigned long long> counts;
-  st = run_fused(ctx, cp, opts, s, counts);
+  if (ready == KRUX_OK && cp.bucket_jobs.empty()) {
+    st = enqueue_fused(ctx, whole, fl, s);
+    if (st == KRUX_OK) st = finish_fused(ctx, whole, fl, s, counts);
+  } else {
+    st = materialise(ctx, cp, s);
+    if (st == KRUX_OK) st = run_fused(ctx, cp, opts, s, counts);
+  }
   if (st != KRUX_OK) return st;
   *n_hits = (int64_t)counts[0];
   if (*n_hits > opts->hit_capacity)
@@ -2679,6 +2766,7 @@ krux_status graph_capture(krux_ctx *ctx, krux_graph *g) {
                              cudaHostAllocDefault));
   std::memset(g->host, 0, (size_t)(nslots + 1) * 8);
   KRUX_CUDA(w, cudaStreamSynchronize(g->cs));
+  uploads_done(w, g->cs);
   KRUX_CUDA(w, cudaStreamBeginCapture(g->cs, cudaStreamCaptureModeThreadLocal));
   if (g->with_seed) st = enqueue_fused(w, g->seed_cp, g->seed_fl, g->cs);
   if (st == KRUX_OK) st = enqueue_fused(w, g->cp, g->fl, g->cs);
