@@ -1134,13 +1134,11 @@ struct CallPlan {
   double fdr_l0 = 0.0, fdr_w = 1.0;
 };
 
-// Device bytes of one bucket's re-ranked set apart from A (tie sums, K, tau, cfac);
+// Device bytes of one bucket's re-ranked set apart from A (tau, cfac);
 // the A matrices of a call's buckets lie back to back before these.
 size_t bucket_bytes(const krux_rankset *rs) {
   size_t off = 0;
   auto take = [&](size_t b) { off += (b + 255) / 256 * 256; };
-  take((size_t)rs->T * 8);
-  take((size_t)rs->T * 4);
   take((size_t)rs->rows_pad * 4);
   take((size_t)rs->rows_pad * 8);
   return off;
@@ -1294,8 +1292,6 @@ krux_status materialise(krux_ctx *ctx, CallPlan &cp, cudaStream_t s) {
       return r;
     };
     bs.dev.A = reinterpret_cast<__half *>(base + aoff[i]);
-    bs.dev.tie = (int64_t *)take((size_t)rs->T * 8);
-    bs.dev.K = (int32_t *)take((size_t)rs->T * 4);
     bs.dev.tau = (float *)take((size_t)rs->rows_pad * 4);
     bs.dev.cfac = (double *)take((size_t)rs->rows_pad * 8);
     // dropping samples with a missing genotype leaves the NaN samples as they are
@@ -1305,8 +1301,6 @@ krux_status materialise(krux_ctx *ctx, CallPlan &cp, cudaStream_t s) {
     RerankJob &j = jobs[i];
     j.base = rs->dev;
     j.A = bs.dev.A;
-    j.tie = bs.dev.tie;
-    j.K = bs.dev.K;
     j.tau = bs.dev.tau;
     j.cfac = bs.dev.cfac;
     j.T = rs->T;

@@ -263,8 +263,6 @@ struct RankDev {
 struct RerankJob {
   RankDev base;             // lo, eq, K and nan_cnt are read
   __half *A;                // [rows_pad][Np] (padding rows written as 0), in either layout
-  int64_t *tie;             // [T]
-  int32_t *K;               // [T]
   float *tau;               // [rows_pad]
   double *cfac;             // [rows_pad]
   int32_t T, N, Np, rows_pad;

@@ -309,14 +309,19 @@ cudaError_t launch_permute_rows(const __half *A, __half *out, int rows_pad, int 
 // so lo' = lo - #{q dropped, present, lo_q < lo_k} and
 // eq' = eq - #{q dropped, present, lo_q == lo_k}.
 //
-// One warp per trait row and kRerankChunk buckets of a run (buckets of one base
-// rank set; grid.y = chunk of buckets): the row's lo and eq are read once, into
-// registers (lane l owns samples 4l..4l+3 of every 128) and into the warp's
-// shared-memory copy (where the dropped samples' values are looked up), the
-// chunk's job fields are staged in shared memory, then each bucket costs a pass
-// over the registers, one 8-byte store per lane and 128 samples, and an integer
-// reduction of the tie sum.  Lane b keeps bucket b's K and tie sum and turns them
-// into the FP64 constants at the end, all buckets of the chunk at once.
+// With K' the present samples left, the centred rank 2 lo' + eq' - K' is the old one less
+// sum_q sign(lo_k - lo_q) over the dropped present samples q: small integers, exact in
+// FP16, so a bucket costs four packed operations per two samples and dropped sample.
+//
+// One warp per trait row and kRerankChunk buckets of a run (buckets of one base rank set;
+// grid.y = chunk of buckets): the row's lo and centred ranks are read once, into
+// registers (lane l owns samples 4l..4l+3 of every 128), lo also into the warp's
+// shared-memory copy (where the dropped samples' values are looked up); the chunk's job
+// fields are staged in shared memory.  Lane b counts bucket b's K at the start and turns
+// it and the tie sum (zero for a row without ties, whose tie pass is left out) into the
+// FP64 constants at the end, all buckets of the chunk at once.  Issue-bound: 200 buckets
+// of 5,000 x 102 took 282 us with lo, eq and the tie sum updated as 32-bit integers and
+// four conversions per lane, now 136 (229 MB written).
 namespace krux {
 namespace {
 constexpr int kRerankWarps = 8;
@@ -325,8 +330,6 @@ constexpr int kRerankDrops = 1024;          // drop-list entries staged per bloc
 
 struct RerankOut {  // a bucket's outputs and drop list, staged per block
   __half *A;
-  int64_t *tie;
-  int32_t *K;
   float *tau;
   double *cfac;
   int32_t drop_off, n_drop;
@@ -337,7 +340,7 @@ template <int kPasses>
 __global__ void __launch_bounds__(kRerankWarps * 32, kPasses == 1 ? 5 : (kPasses == 2 ? 2 : 1))
 rerank_kernel(const RerankJob *__restrict__ jobs, int n_jobs_all, const int32_t *__restrict__ drops,
               int tiled) {
-  __shared__ uint32_t srow[kRerankWarps][kMaxN];  // lo | eq << 16 of the warp's row
+  __shared__ uint32_t srow[kRerankWarps][kMaxN];  // lo of the warp's row as FP16, twice; ~0: absent
   __shared__ RerankOut sj[kRerankChunk];
   __shared__ int32_t sdrop[kRerankDrops];          // the chunk's drop lists, when they fit
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -345,7 +348,7 @@ rerank_kernel(const RerankJob *__restrict__ jobs, int n_jobs_all, const int32_t 
   const int n_jobs = min(kRerankChunk, n_jobs_all - jbase);
   if (threadIdx.x < n_jobs) {
     const RerankJob &J = jobs[jbase + threadIdx.x];
-    sj[threadIdx.x] = RerankOut{J.A, J.tie, J.K, J.tau, J.cfac, J.drop_off, J.n_drop};
+    sj[threadIdx.x] = RerankOut{J.A, J.tau, J.cfac, J.drop_off, J.n_drop};
   }
   __syncthreads();
   // the chunk's drop lists lie back to back in `drops`
@@ -373,76 +376,94 @@ rerank_kernel(const RerankJob *__restrict__ jobs, int n_jobs_all, const int32_t 
   }
   const uint16_t *lo = J0.base.lo + (int64_t)t * N;
   const uint16_t *eq = J0.base.eq + (int64_t)t * N;
-  for (int k = lane; k < N; k += 32) srow[warp][k] = (uint32_t)lo[k] | ((uint32_t)eq[k] << 16);
-  uint32_t own[kPasses][4];
+  const int K0 = J0.base.K[t];
+  const auto dup = [](int x) {
+    const uint32_t h = (uint32_t)__half_as_ushort(__int2half_rn(x));
+    return h | (h << 16);
+  };
+  for (int k = lane; k < N; k += 32) srow[warp][k] = eq[k] > 0 ? dup(lo[k]) : 0xffffffffu;
+  __half2 av[kPasses][2], lv[kPasses][2];  // the samples' centred ranks and lo
+  uint32_t pm[kPasses][2];                 // 0xffff where the sample is present
+  bool ties = false;
 #pragma unroll
   for (int ps = 0; ps < kPasses; ++ps)
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int k = 128 * ps + 4 * lane + i;
-      own[ps][i] = k < N ? (uint32_t)lo[k] | ((uint32_t)eq[k] << 16) : 0u;
+    for (int h = 0; h < 2; ++h) {
+      int a[2], l[2];
+      pm[ps][h] = 0u;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int k = 128 * ps + 4 * lane + 2 * h + i;
+        const int e = k < N ? (int)eq[k] : 0;
+        l[i] = e > 0 ? (int)lo[k] : 0;
+        a[i] = e > 0 ? 2 * l[i] + e - K0 : 0;
+        if (e > 0) pm[ps][h] |= 0xffffu << (16 * i);
+        ties = ties || e > 1;
+      }
+      av[ps][h] = __halves2half2(__int2half_rn(a[0]), __int2half_rn(a[1]));
+      lv[ps][h] = __halves2half2(__int2half_rn(l[0]), __int2half_rn(l[1]));
     }
+  ties = __any_sync(0xffffffffu, ties);
   __syncwarp();
-  const int K0 = J0.base.K[t];
-  int myK = 0, mytie = 0;  // bucket lane's, for the constants
+  int myK = K0, mytie = 0;  // bucket lane's, for the constants
+  if (lane < n_jobs) {
+    const int32_t *dl = staged ? sdrop + (sj[lane].drop_off - d0) : drops + sj[lane].drop_off;
+    for (int d = 0; d < sj[lane].n_drop; ++d) myK -= srow[warp][dl[d]] != 0xffffffffu;
+  }
+  const __half2 one = __float2half2_rn(1.f), minus = __float2half2_rn(-1.f);
+  const int64_t at0 = tiled ? tiled_index(t, 4 * lane, Np) : (int64_t)t * Np + 4 * lane;
+  const int64_t step = tiled ? 8 * 2048 : 128;  // 128 samples on
   for (int j = 0; j < n_jobs; ++j) {
     const RerankOut &J = sj[j];
     const int n_drop = J.n_drop;
     const int32_t *dl = staged ? sdrop + (J.drop_off - d0) : drops + J.drop_off;
-    int Kdrop = 0;  // dropped samples with a value
-    for (int d = 0; d < n_drop; ++d) Kdrop += (srow[warp][dl[d]] >> 16) > 0u;
-    const int K = K0 - Kdrop;
-    int tie = 0;
+    __half2 x[kPasses][2];
+    uint32_t m[kPasses][2];
 #pragma unroll
-    for (int ps = 0; ps < kPasses; ++ps) {
-      const int k0 = 128 * ps + 4 * lane;
-      int lk[4], l[4], e[4];
-      bool present[4];
+    for (int ps = 0; ps < kPasses; ++ps)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        lk[i] = (int)(own[ps][i] & 0xffffu);
-        l[i] = lk[i];
-        e[i] = (int)(own[ps][i] >> 16);
-        present[i] = e[i] > 0;
+      for (int h = 0; h < 2; ++h) {
+        x[ps][h] = av[ps][h];
+        m[ps][h] = pm[ps][h];
       }
-      for (int d = 0; d < n_drop; ++d) {
-        const int q = dl[d];
-        const uint32_t w = srow[warp][q];
-        const int lq = (int)(w & 0xffffu);
-        const bool qp = (w >> 16) > 0u;  // the dropped sample has a value
+    for (int d = 0; d < n_drop; ++d) {
+      const int q = dl[d];
+      const uint32_t w = srow[warp][q];
+      if (w == 0xffffffffu) continue;  // (the dropped sample has no value)
+      const __half2 lq = *reinterpret_cast<const __half2 *>(&w);
+#pragma unroll
+      for (int ps = 0; ps < kPasses; ++ps) {
+        const unsigned int r = (unsigned int)(q - 128 * ps - 4 * lane);
+        const uint32_t left = (r & 1u) ? 0x0000ffffu : 0xffff0000u;
+        if (r < 2u) m[ps][0] &= left;
+        if ((r & ~1u) == 2u) m[ps][1] &= left;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          x[ps][h] = __hsub2(x[ps][h], __hmin2(__hmax2(__hsub2(lv[ps][h], lq), minus), one));
+      }
+    }
+#pragma unroll
+    for (int ps = 0; ps < kPasses; ++ps)
+      if (128 * ps + 4 * lane < Np) {
+        uint2 v;
+        v.x = *reinterpret_cast<const uint32_t *>(&x[ps][0]) & m[ps][0];
+        v.y = *reinterpret_cast<const uint32_t *>(&x[ps][1]) & m[ps][1];
+        *reinterpret_cast<uint2 *>(J.A + at0 + ps * step) = v;
+      }
+    if (ties) {  // sum over the samples left of eq'^2 - 1
+      int tie = 0;
+#pragma unroll
+      for (int ps = 0; ps < kPasses; ++ps)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          present[i] = present[i] && q != k0 + i;
-          l[i] -= qp && lq < lk[i];
-          e[i] -= qp && lq == lk[i];
+          const int k = 128 * ps + 4 * lane + i;
+          if (!((m[ps][i >> 1] >> (16 * (i & 1))) & 1u)) continue;
+          int e = (int)eq[k];
+          for (int d = 0; e > 1 && d < n_drop; ++d) e -= srow[warp][dl[d]] == srow[warp][k];
+          tie += e * e - 1;
         }
-      }
-      int a[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        a[i] = 0;
-        if (present[i]) {
-          tie += e[i] * e[i] - 1;
-          a[i] = 2 * l[i] + e[i] - K;
-        }
-      }
-      if (k0 < Np) {
-        const __half2 h01 = __halves2half2(__int2half_rn(a[0]), __int2half_rn(a[1]));
-        const __half2 h23 = __halves2half2(__int2half_rn(a[2]), __int2half_rn(a[3]));
-        uint2 v;
-        v.x = *reinterpret_cast<const uint32_t *>(&h01);
-        v.y = *reinterpret_cast<const uint32_t *>(&h23);
-        *reinterpret_cast<uint2 *>(J.A + (tiled ? tiled_index(t, k0, Np) : (int64_t)t * Np + k0)) = v;
-      }
-    }
-    tie = (int)__reduce_add_sync(0xffffffffu, (unsigned)tie);
-    if (lane == 0) {
-      J.tie[t] = tie;
-      J.K[t] = K;
-    }
-    if (lane == j) {
-      myK = K;
-      mytie = tie;
+      tie = (int)__reduce_add_sync(0xffffffffu, (unsigned)tie);
+      if (lane == j) mytie = tie;
     }
   }
   if (lane < n_jobs) {  // the chunk's FP64 constants, one bucket per lane
