@@ -455,9 +455,9 @@ struct CisGroup {
 };
 
 // A column (SNP) of a dense output: with sizes n_i (1 for an empty group, whose D_i is
-// 0), sum_i D_i^2 / n_i = (a D_0^2 + b D_1^2 + c D_2^2) / den, whole numbers below 2^50.
+// 0), sum_i D_i^2 / n_i = (a D_0^2 + b D_1^2 + c D_2^2) / (n_0 n_1 n_2), whole numbers below 2^50.
 struct alignas(16) DenseCol {
-  double den, rcp;          // n_0 n_1 n_2 and its reciprocal
+  double rcp, rcp_lo;       // 1 / (n_0 n_1 n_2) in two parts
   uint32_t a, b, c;         // n_1 n_2, n_0 n_2, n_0 n_1
   uint16_t n0, n1, n2;      // sizes as they are
   uint8_t df;

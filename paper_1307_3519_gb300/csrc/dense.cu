@@ -3,13 +3,15 @@
 // "P-value calculation").
 //
 // FP64 issues at a 64th of the FP32 rate on this part, so the pass is bound by its FP64
-// operations: the statistic's numerator is formed in integers (DenseCol), exp and erfc
-// from tables and short polynomials (table reduction of the exponential as in Tang,
-// "Table-driven implementation of the exponential function", 1989; erfc(sqrt x) as
-// exp(-x) erfcx(sqrt x) with piecewise polynomials of erfcx), about 16 FP64 operations
-// for df 2 and 34 for df 1.  With three FP64 divisions and the library's exp and erfc in
-// the scan's epilogue, 1,000 x 20,003 x 102 took 4.35 ms; this pass takes 1.07 ms (FP64 issue)
-// after 0.23 ms for the rank sums.
+// operations, counted per warp: the statistic's numerator is formed in integers
+// (DenseCol), exp and erfc come from tables and short polynomials (table reduction of the
+// exponential as in Tang, "Table-driven implementation of the exponential function", 1989;
+// erfc(sqrt x) as exp(-x) erfcx(sqrt x) with piecewise polynomials of erfcx), comparisons
+// and conversions are done on the bits, and a block takes its columns by df class, so that
+// a warp runs one of the two tails: about 13 FP64 operations for df 2 and 31 for df 1.
+// With three FP64 divisions and the library's exp and erfc in the scan's epilogue, 1,000 x
+// 20,003 x 102 took 4.35 ms; a pass of 16 and 34 operations with both classes in every
+// warp 1.04 ms, this one 0.66, after 0.23 ms for the rank sums.
 #include <cmath>
 #include <atomic>
 
@@ -18,8 +20,9 @@
 namespace krux {
 
 namespace {
-constexpr int kExpTab = 128;                 // 2^(-j / 128), high and low parts
-constexpr int kErfInts = 128, kErfDeg = 8;   // erfcx on [0, 6.4), intervals of 1/20
+constexpr int kExpBits = 12, kExpTab = 1 << kExpBits;  // 2^(-j / 4096), high and low parts
+constexpr int kErfInts = 512, kErfDeg = 6;   // erfcx on [0, 6.4), intervals of 1/80
+constexpr int kDenseThreads = 512;           // and columns of a block's window
 __device__ double c_exp[2 * kExpTab];
 __device__ double c_erfcx[kErfInts * (kErfDeg + 1)];
 
@@ -28,36 +31,47 @@ struct DenseTables {
   double f[kErfInts * (kErfDeg + 1)];
 };
 
-// exp(-x), 0 <= x <= 700: x = k ln2 / 128 + r, |r| <= ln2 / 256, and exp(-r) - 1 to r^5
-// (the next term is below 6e-19); tab holds 2^(-j/128) as high and low parts.
+// A normal positive double as FP32 (truncated), and back (exact), on the bits: FP64's
+// conversions issue as slowly as its arithmetic.
+__device__ __forceinline__ float f32_of(double x) {
+  return __uint_as_float((((uint32_t)__double2hiint(x) - 0x38000000u) << 3) |
+                         ((uint32_t)__double2loint(x) >> 29));
+}
+__device__ __forceinline__ double f64_of(float x) {
+  const uint32_t b = __float_as_uint(x);
+  return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
+
+// exp(-x), 0 <= x <= 700: x = k ln2 / 4096 + r, |r| <= ln2 / 8192, and exp(-r) - 1 to r^3
+// (the next term is below 3e-18); tab holds 2^(-j/4096) as high and low parts.
 __device__ __forceinline__ double exp_neg(double x, const double *tab) {
   const double kMagic = 6755399441055744.0;  // 1.5 * 2^52: rounds to whole numbers
-  const double t = fma(x, 184.66496523378730914, kMagic);  // 128 / ln 2
+  const double t = fma(x, 5909.278887481194, kMagic);  // 4096 / ln 2
   const double kd = t - kMagic;
   const int k = __double2loint(t);
-  // ln2 / 128 in two parts, the first with 32 trailing zero bits
-  double r = fma(-kd, 0x1.62e42fefap-8, x);
-  r = fma(-kd, 0x1.cf79abc9e3b3ap-47, r);
-  double q = fma(r, -1.0 / 120.0, 1.0 / 24.0);
-  q = fma(r, q, -1.0 / 6.0);
-  q = fma(r, q, 0.5);
+  // ln2 / 4096 in two parts, the first of 30 bits (k has at most 23)
+  double r = fma(-kd, 0x1.62e42fe8p-13, x);
+  r = fma(-kd, 0x1.e8e7bcd5e4f1ep-43, r);
+  double q = fma(r, -1.0 / 6.0, 0.5);
   q = fma(r, q, -1.0);
   q *= r;
   const double2 T = *reinterpret_cast<const double2 *>(tab + 2 * (k & (kExpTab - 1)));
   const double y = T.x + fma(T.x, q, T.y);
-  return __hiloint2double(__double2hiint(y) - ((k >> 7) << 20), __double2loint(y));
+  return __hiloint2double(__double2hiint(y) - ((k >> kExpBits) << 20), __double2loint(y));
 }
 
 // erfc(sqrt x) = exp(-x) erfcx(sqrt x), x > 0.
 __device__ __forceinline__ double erfc_sqrt(double x, const double *etab, const double *ftab) {
-  if (!(x < 40.0) || x < 1e-30) return erfc(sqrt(x));
+  const int hi = __double2hiint(x);
+  if (hi >= 0x40440000 || hi < 0x39c00000) return erfc(sqrt(x));  // x >= 40, x < 2^-99
   // sqrt by two Newton steps from the FP32 reciprocal root
-  const double y = (double)rsqrtf((float)x), hy = 0.5 * y;
+  const float yf = rsqrtf(f32_of(x));
+  const double y = f64_of(yf), hy = f64_of(0.5f * yf);
   double z = x * y;
   z = fma(fma(-z, z, x), hy, z);
   z = fma(fma(-z, z, x), hy, z);
-  const int i = (int)((float)z * 20.0f);  // (the next interval's edge may fall in this one)
-  const double w = fma((double)(2 * i + 1), -0.025, z);
+  const int i = (int)(f32_of(z) * 80.0f);  // (the next interval's edge may fall in this one)
+  const double w = fma(f64_of((float)(2 * i + 1)), -0.00625, z);
   const double *c = ftab + i * (kErfDeg + 1);
   double f = c[kErfDeg];
 #pragma unroll
@@ -84,74 +98,95 @@ __global__ void dense_cols_kernel(const GroupDesc *__restrict__ groups, int g0, 
   c.a = p1 * p2;
   c.b = p0 * p2;
   c.c = p0 * p1;
-  c.den = (double)c.a * (double)p0;
-  c.rcp = 1.0 / c.den;
+  const double den = (double)c.a * (double)p0;
+  c.rcp = 1.0 / den;
+  c.rcp_lo = fma(-den, c.rcp, 1.0) * c.rcp;
   c.group = g0 + (int)blockIdx.y;
   c.snp = m.snp[jj];
   col[m.snp[jj] - snp0] = c;
 }
 
-// One thread per column and run of traits.
-__global__ void __launch_bounds__(256)
+// Work items: a window of kDenseThreads columns and a run of traits each, dealt to the
+// blocks in turn; one thread per column, df-1 columns last.
+__global__ void __launch_bounds__(kDenseThreads, 2)
 dense_finish_kernel(const DenseCol *__restrict__ col, const double *const *__restrict__ cfac_by_group,
-                    int T, int per_block, int64_t cols, int64_t ld, double *__restrict__ H,
-                    double *__restrict__ P, double pthresh, krux_hit *__restrict__ hits,
-                    HitAux *__restrict__ aux, int64_t capacity, unsigned long long *counter) {
-  __shared__ __align__(16) double etab[2 * kExpTab];
-  __shared__ double ftab[kErfInts * (kErfDeg + 1)];
+                    int T, int per_item, int64_t windows, int64_t n_items, int64_t cols, int64_t ld,
+                    double *__restrict__ H, double *__restrict__ P, double pthresh,
+                    krux_hit *__restrict__ hits, HitAux *__restrict__ aux, int64_t capacity,
+                    unsigned long long *counter) {
+  extern __shared__ __align__(16) double tables[];
+  __shared__ int ones[kDenseThreads / 32];
+  __shared__ uint16_t order[kDenseThreads];
+  double *etab = tables, *ftab = tables + 2 * kExpTab;
   for (int i = threadIdx.x; i < 2 * kExpTab; i += blockDim.x) etab[i] = c_exp[i];
   for (int i = threadIdx.x; i < kErfInts * (kErfDeg + 1); i += blockDim.x) ftab[i] = c_erfcx[i];
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const bool live = j < cols;
-  DenseCol c{};
-  if (live) c = col[j];
-  const double *cfac = cfac_by_group[c.group];
-  const int t0 = blockIdx.y * per_block, t1 = min(t0 + per_block, T);
-  for (int t = t0; t < t1; ++t) {
-    const int64_t o = (int64_t)t * ld + j;
-    int2 d = make_int2(0, 0);
-    if (live) d = *reinterpret_cast<const int2 *>(H + o);
-    const double cf = cfac[t];
-    double h = 0.0, p = 1.0;
-    if (c.df > 0 && cf > 0.0) {
-      const unsigned long long d0 = (unsigned long long)((long long)d.x * d.x);
-      const unsigned long long d1 = (unsigned long long)((long long)d.y * d.y);
-      const int e = d.x + d.y;
-      const unsigned long long d2 = (unsigned long long)((long long)e * e);
-      const unsigned long long num = d0 * c.a + d1 * c.b + d2 * c.c;  // < 2^50
-      const double nd = __longlong_as_double((long long)(num | 0x4330000000000000ull)) - 4503599627370496.0;
-      double q = nd * c.rcp;  // the quotient, corrected to its last place
-      q = fma(fma(-q, c.den, nd), c.rcp, q);
-      h = cf * q;
-      const double x = 0.5 * h;
-      if (c.df == 1) p = h > 0.0 ? erfc_sqrt(x, etab, ftab) : 1.0;
-      else p = x < 700.0 ? exp_neg(x, etab) : exp(-x);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long pbits = __double_as_longlong(pthresh);  // (positive doubles order as integers)
+  for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
+    const int64_t j0 = item % windows * kDenseThreads;
+    const bool one = j0 + threadIdx.x < cols && col[j0 + threadIdx.x].df == 1;
+    const uint32_t bal1 = __ballot_sync(0xffffffffu, one);
+    __syncthreads();  // (tables written; the order of the item before read)
+    if (lane == 0) ones[warp] = __popc(bal1);
+    __syncthreads();
+    int before = 0, total = 0;
+    for (int w = 0; w < kDenseThreads / 32; ++w) {
+      before += w < warp ? ones[w] : 0;
+      total += ones[w];
     }
-    if (live) {
-      H[o] = h;
-      P[o] = p;
-    }
-    const bool hit = live && p < pthresh;
-    const uint32_t bal = __ballot_sync(0xffffffffu, hit);
-    if (bal == 0u) continue;
-    unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(counter, (unsigned long long)__popc(bal));
-    base = __shfl_sync(0xffffffffu, base, 0) + (unsigned int)__popc(bal & ((1u << lane) - 1u));
-    if (hit && base < (unsigned long long)capacity) {
-      krux_hit r;
-      r.trait = (uint32_t)t;
-      r.snp = (uint32_t)c.snp;
-      r.d0 = d.x;
-      r.d1 = d.y;
-      st_hit(hits + base, r);
-      HitAux a;
-      a.n0 = c.n0;
-      a.n1 = c.n1;
-      a.n2 = c.n2;
-      a.group = (uint16_t)c.group;
-      st_aux(aux + base, a);
+    before += __popc(bal1 & ((1u << lane) - 1u));
+    order[one ? kDenseThreads - total + before : (int)threadIdx.x - before] = (uint16_t)threadIdx.x;
+    __syncthreads();
+    const int64_t j = j0 + order[threadIdx.x];
+    const bool live = j < cols;
+    DenseCol c{};
+    if (live) c = col[j];
+    const double *cfac = cfac_by_group[c.group];
+    const int t0 = (int)(item / windows) * per_item, t1 = min(t0 + per_item, T);
+    for (int t = t0; t < t1; ++t) {
+      const int64_t o = (int64_t)t * ld + j;
+      int2 d = make_int2(0, 0);
+      if (live) d = *reinterpret_cast<const int2 *>(H + o);
+      const double cf = cfac[t];
+      double h = 0.0, p = 1.0;
+      if (c.df > 0 && __double_as_longlong(cf) > 0) {
+        const unsigned long long d0 = (unsigned long long)((long long)d.x * d.x);
+        const unsigned long long d1 = (unsigned long long)((long long)d.y * d.y);
+        const int e = d.x + d.y;
+        const unsigned long long d2 = (unsigned long long)((long long)e * e);
+        const unsigned long long num = d0 * c.a + d1 * c.b + d2 * c.c;  // < 2^50
+        const double nd = __longlong_as_double((long long)(num | 0x4330000000000000ull)) - 4503599627370496.0;
+        h = cf * fma(nd, c.rcp, nd * c.rcp_lo);  // (the quotient to its last place)
+        const int hh = __double2hiint(h);
+        const bool some = hh >= 0x00200000;  // else 0
+        const double x = some ? __hiloint2double(hh - 0x00100000, __double2loint(h)) : 0.0;  // h / 2
+        if (c.df == 1) p = some ? erfc_sqrt(x, etab, ftab) : 1.0;
+        else p = hh < 0x4095e000 ? exp_neg(x, etab) : exp(-x);  // (h < 1400)
+      }
+      if (live) {
+        H[o] = h;
+        P[o] = p;
+      }
+      const bool hit = live && __double_as_longlong(p) < pbits;
+      const uint32_t bal = __ballot_sync(0xffffffffu, hit);
+      if (bal == 0u) continue;
+      unsigned long long base = 0;
+      if (lane == 0) base = atomicAdd(counter, (unsigned long long)__popc(bal));
+      base = __shfl_sync(0xffffffffu, base, 0) + (unsigned int)__popc(bal & ((1u << lane) - 1u));
+      if (hit && base < (unsigned long long)capacity) {
+        krux_hit r;
+        r.trait = (uint32_t)t;
+        r.snp = (uint32_t)c.snp;
+        r.d0 = d.x;
+        r.d1 = d.y;
+        st_hit(hits + base, r);
+        HitAux a;
+        a.n0 = c.n0;
+        a.n1 = c.n1;
+        a.n2 = c.n2;
+        a.group = (uint16_t)c.group;
+        st_aux(aux + base, a);
+      }
     }
   }
 }
@@ -162,14 +197,21 @@ dense_finish_kernel(const DenseCol *__restrict__ col, const double *const *__res
 void erfcx_poly(long double mid, long double h, double *out) {
   constexpr int n = kErfDeg + 4;
   const long double pi = 3.14159265358979323846264338327950288L;
+  static const struct Cosines {
+    long double c[n][n];  // of i (j + 1/2) pi / n
+    explicit Cosines(long double pi) {
+      for (int i = 0; i < n; ++i)
+        for (int j = 0; j < n; ++j) c[i][j] = std::cos(pi * i * (j + 0.5L) / n);
+    }
+  } cosines(pi);
   long double f[n], cheb[n];
   for (int j = 0; j < n; ++j) {
-    const long double z = mid + h * std::cos(pi * (j + 0.5L) / n);
+    const long double z = mid + h * cosines.c[1][j];
     f[j] = std::exp(z * z) * std::erfc(z);
   }
   for (int i = 0; i < n; ++i) {
     long double c = 0.0L;
-    for (int j = 0; j < n; ++j) c += f[j] * std::cos(pi * i * (j + 0.5L) / n);
+    for (int j = 0; j < n; ++j) c += f[j] * cosines.c[i][j];
     cheb[i] = c * (i ? 2.0L : 1.0L) / n;
   }
   // powers of the Chebyshev polynomials up to the kept degree
@@ -195,7 +237,7 @@ const DenseTables &dense_tables() {
       x.e[2 * j] = (double)v;
       x.e[2 * j + 1] = (double)(v - (long double)x.e[2 * j]);
     }
-    for (int i = 0; i < kErfInts; ++i) erfcx_poly((2 * i + 1) * 0.025L, 0.0251L, x.f + i * (kErfDeg + 1));
+    for (int i = 0; i < kErfInts; ++i) erfcx_poly((2 * i + 1) * 0.00625L, 0.006275L, x.f + i * (kErfDeg + 1));
     return x;
   }();
   return t;
@@ -213,6 +255,9 @@ cudaError_t dense_prepare() {
   const DenseTables &t = dense_tables();
   e = cudaMemcpyToSymbol(c_exp, t.e, sizeof t.e);
   if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_erfcx, t.f, sizeof t.f);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(dense_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(DenseTables));
   if (e == cudaSuccess && dev < 64) uploaded.fetch_or(1ull << dev, std::memory_order_acq_rel);
   return e;
 }
@@ -231,15 +276,15 @@ cudaError_t launch_dense_finish(const GroupDesc *groups, int n_groups, int64_t m
                     (unsigned)(n_groups - g0 < 65535 ? n_groups - g0 : 65535));
     dense_cols_kernel<<<grid, 256, 0, s>>>(groups, g0, snp0, col);
   }
-  // runs of traits: enough blocks for two full waves, at least 8 traits each
-  const int64_t cb = (cols + 255) / 256;
-  int64_t runs = (int64_t)sm_count * 16 / cb + 1;
+  // two blocks per SM; runs of traits such that each has eight items, at least 8 traits each
+  const int64_t windows = (cols + kDenseThreads - 1) / kDenseThreads;
+  int64_t runs = (int64_t)sm_count * 16 / windows + 1;
   if (runs > (T + 7) / 8) runs = (T + 7) / 8;
-  if (runs > 65535) runs = 65535;
   const int per = (int)((T + runs - 1) / runs);
-  const dim3 grid((unsigned)cb, (unsigned)((T + per - 1) / per));
-  dense_finish_kernel<<<grid, 256, 0, s>>>(col, cfac_by_group, T, per, cols, ld, H, p, pthresh, hits,
-                                           aux, capacity, counter);
+  const int64_t items = windows * ((T + per - 1) / per);
+  const int grid = (int)(items < 2 * sm_count ? items : 2 * sm_count);
+  dense_finish_kernel<<<grid, kDenseThreads, sizeof(DenseTables), s>>>(
+      col, cfac_by_group, T, per, windows, items, cols, ld, H, p, pthresh, hits, aux, capacity, counter);
   return cudaGetLastError();
 }
 
