@@ -2820,14 +2820,17 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       // half's test the loop held 64 of them and spilled (N = 128, 15,000 x 200,000:
       // 0.898 against 0.875 ms; the permutation form's main launch of 16 x 20,000 x
       // 200,000: 30.9 against 25.1 ms); the four warps of a scheduler cover each
-      // other's loads.
+      // other's loads.  The two halves are spelt out (20,000 x 200,000: N = 24 845 -> 753 us,
+      // 48 864 -> 829, 102 1067 -> 1052, 256 2295 -> 2201; 176 to 224, bound by the tensor
+      // cores, 0.6 to 1 % longer; 16 permutations 45.3 -> 44.2 ms), but for the NaN form,
+      // whose two tests make the code long (missing values 1.15 -> 1.18 ms).
       auto pair_slot = [&](uint32_t ps, uint32_t phase, const ChunkMeta &mc, int c, int chunk0,
                            const GroupDesc &g, int ag, int tt, int group) -> bool {
         if (!wait_warp(t_full(ps), phase, p, abort_addr, 7)) return false;
         tc_fence_after();
         uint32_t x0[kH], x1[kH];
         const uint32_t taddr = lane_cols + ps * 256u;
-#pragma unroll 1
+#pragma unroll(kNan ? 1 : 2)
         for (int half = 0; half < 2; ++half) {
           if constexpr (kMultiF) {  // 8 SNPs, P_i of SNP j in column 32 i + j of the chunk
             tmem_ld_rows(taddr + (uint32_t)(kEpiSnpsM * half), x0, x1);
