@@ -1311,7 +1311,7 @@ struct EvLane {
 // their FP64 -ln p, and raise the trait's class bounds (largest df-1 |s| and df-2 s of
 // the pairs listed, less the margin: a later pair of the class below them cannot beat
 // those pairs).  With the FDR histogram on, every pair at or above the band is listed.
-__device__ __forceinline__ void ev_minp(const EvLane &E, EvGroup &G, const ScanParams &p, int lane,
+__device__ __forceinline__ void ev_minp(EvLane &E, EvGroup &G, const ScanParams &p, int lane,
                                         bool on, float s, float u, float v, unsigned int &mcn,
                                         int ev_warp) {
   const bool valid = on && E.snp >= 0;
@@ -1321,6 +1321,15 @@ __device__ __forceinline__ void ev_minp(const EvLane &E, EvGroup &G, const ScanP
   // decided already
   const float keep = 1.f - p.margin;
   const uint32_t pid = pair_id((int)u, (int)v);
+  if (p.fdr_hist != nullptr && on) {
+    ev_group(G, p, E.group);
+    const uint4 bb = __ldcg(reinterpret_cast<const uint4 *>(G.minp_bound) +
+                            (int64_t)(E.ag - 1) * G.rows + E.trait);
+    E.b1 = fmaxf(__uint_as_float(bb.y), 1e-30f);
+    E.id1 = bb.x;
+    E.b2 = fmaxf(__uint_as_float(bb.w), 1e-30f);
+    E.id2 = bb.z;
+  }
   bool cand = valid && ((s > E.b2 * keep && !(s == E.b2 && pid == E.id2)) ||
                         (-s > E.b1 * keep && !(-s == E.b1 && pid == E.id1)));
   // within a class the key grows with the value: only the entry's largest value
@@ -2795,12 +2804,16 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
                            const ChunkMeta &mc, int o, const GroupDesc &g, int ag, int tt,
                            int group) -> bool {
         const int trait = tt * kTileM + row;
-        const float tau = kTwo ? g.tau[trait] : tau_s;
+        const float tau = tau_s;
         bool real = need;
         float mx1 = 0.f, mx2 = 0.f;
         uint32_t id1 = 0u, id2 = 0u;
         if constexpr (kTwo) {
-          if (ag > 0) {
+          // (with the FDR histogram on, nearly every candidate is a pair of its band: all go
+          // to the event warps, which read the class words themselves.  Read and filtered
+          // here, a round trip to L2 with the accumulator slot held, 16 x 20,000 x 200,000
+          // took 44.1 ms, now 40.5)
+          if (ag > 0 && p.fdr_hist == nullptr) {
             const uint4 bb = class_words(g, ag, trait);
             mx1 = fmaxf(__uint_as_float(bb.y), kBoundMin);
             id1 = bb.x;
