@@ -16,6 +16,7 @@
 #include <atomic>
 
 #include "common.cuh"
+#include "fp64_tables.cuh"
 
 namespace krux {
 
@@ -42,24 +43,6 @@ __device__ __forceinline__ double f64_of(float x) {
   return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
 }
 
-// exp(-x), 0 <= x <= 700: x = k ln2 / 4096 + r, |r| <= ln2 / 8192, and exp(-r) - 1 to r^3
-// (the next term is below 3e-18); tab holds 2^(-j/4096) as high and low parts.
-__device__ __forceinline__ double exp_neg(double x, const double *tab) {
-  const double kMagic = 6755399441055744.0;  // 1.5 * 2^52: rounds to whole numbers
-  const double t = fma(x, 5909.278887481194, kMagic);  // 4096 / ln 2
-  const double kd = t - kMagic;
-  const int k = __double2loint(t);
-  // ln2 / 4096 in two parts, the first of 30 bits (k has at most 23)
-  double r = fma(-kd, 0x1.62e42fe8p-13, x);
-  r = fma(-kd, 0x1.e8e7bcd5e4f1ep-43, r);
-  double q = fma(r, -1.0 / 6.0, 0.5);
-  q = fma(r, q, -1.0);
-  q *= r;
-  const double2 T = *reinterpret_cast<const double2 *>(tab + 2 * (k & (kExpTab - 1)));
-  const double y = T.x + fma(T.x, q, T.y);
-  return __hiloint2double(__double2hiint(y) - ((k >> kExpBits) << 20), __double2loint(y));
-}
-
 // erfc(sqrt x) = exp(-x) erfcx(sqrt x), x > 0.
 __device__ __forceinline__ double erfc_sqrt(double x, const double *etab, const double *ftab) {
   const int hi = __double2hiint(x);
@@ -76,7 +59,7 @@ __device__ __forceinline__ double erfc_sqrt(double x, const double *etab, const 
   double f = c[kErfDeg];
 #pragma unroll
   for (int j = kErfDeg - 1; j >= 0; --j) f = fma(f, w, c[j]);
-  return exp_neg(x, etab) * f;
+  return exp_neg<kExpBits>(x, etab) * f;
 }
 
 // One thread per packed slot: its column's entry.
@@ -161,7 +144,7 @@ dense_finish_kernel(const DenseCol *__restrict__ col, const double *const *__res
         const bool some = hh >= 0x00200000;  // else 0
         const double x = some ? __hiloint2double(hh - 0x00100000, __double2loint(h)) : 0.0;  // h / 2
         if (c.df == 1) p = some ? erfc_sqrt(x, etab, ftab) : 1.0;
-        else p = hh < 0x4095e000 ? exp_neg(x, etab) : exp(-x);  // (h < 1400)
+        else p = hh < 0x4095e000 ? exp_neg<kExpBits>(x, etab) : exp(-x);  // (h < 1400)
       }
       if (live) {
         H[o] = h;
@@ -232,11 +215,7 @@ void erfcx_poly(long double mid, long double h, double *out) {
 const DenseTables &dense_tables() {
   static const DenseTables t = [] {
     DenseTables x;
-    for (int j = 0; j < kExpTab; ++j) {
-      const long double v = std::exp2(-(long double)j / kExpTab);
-      x.e[2 * j] = (double)v;
-      x.e[2 * j + 1] = (double)(v - (long double)x.e[2 * j]);
-    }
+    fill_exp_table<kExpBits>(x.e);
     for (int i = 0; i < kErfInts; ++i) erfcx_poly((2 * i + 1) * 0.00625L, 0.006275L, x.f + i * (kErfDeg + 1));
     return x;
   }();

@@ -11,12 +11,74 @@
 // Every pair at or above the lower edge of a wide band is kept as a provisional
 // hit; this file's finalisation recomputes each one from the caller's FP32 values
 // (exact group sums, FP64 after them) and keeps those with p < P_c.
+#include <atomic>
+
 #include "common.cuh"
+#include "fp64_tables.cuh"
 #include "param_tails.cuh"
 
 namespace krux {
 
 namespace {
+
+// The continued fraction of I_x(a, 1/2) on [0, kTabMax]: a polynomial of degree kTabDeg
+// in t = (x - middle) / half width on each of kTabInts equal intervals, from the
+// Chebyshev interpolation there (the nearest singularity, x = 1, lies at least eleven
+// interval widths away: the terms left out are below 1e-16).  One warp per interval; a =
+// (N - 2) / 2 is the only one a call needs (two genotype groups, or the regression).
+constexpr int kTabInts = 128, kTabDeg = 9;
+constexpr double kTabMax = 0.92;
+__global__ void cf_table_kernel(double a, double *__restrict__ table) {
+  const int i = threadIdx.x & 31, interval = blockIdx.x;
+  const double h = 0.5 * kTabMax / kTabInts, mid = (2 * interval + 1) * h;
+  constexpr int n = kTabDeg + 1;
+  const double f = i < n ? ibeta_cf(a, 0.5, mid + h * cospi((i + 0.5) / n)) : 0.0;
+  double c = 0.0;  // lane i: the coefficient of T_i
+  for (int j = 0; j < n; ++j) c += __shfl_sync(0xffffffffu, f, j) * cospi(i * (j + 0.5) / n);
+  c *= (i ? 2.0 : 1.0) / n;
+  // powers of t: lane i gathers row i of the Chebyshev polynomials' coefficients
+  double t0 = i == 0 ? 1.0 : 0.0, t1 = i == 1 ? 1.0 : 0.0, p = 0.0;
+  for (int k = 0; k < n; ++k) {
+    p += __shfl_sync(0xffffffffu, c, k) * t0;
+    const double up = __shfl_up_sync(0xffffffffu, t1, 1);
+    const double t2 = (i ? 2.0 * up : 0.0) - t0;
+    t0 = t1;
+    t1 = t2;
+  }
+  if (i < n) table[interval * n + i] = p;
+}
+
+// The polynomial at x, 0 < x < kTabMax.
+__device__ __forceinline__ double cf_of(double x, const double *__restrict__ table) {
+  const int i = min((int)((float)x * (float)(kTabInts / kTabMax)), kTabInts - 1);
+  const double t = fma(x, 2.0 * kTabInts / kTabMax, -(double)(2 * i + 1));
+  const double *c = table + i * (kTabDeg + 1);
+  double f = c[kTabDeg];
+#pragma unroll
+  for (int k = kTabDeg - 1; k >= 0; --k) f = fma(f, t, c[k]);
+  return f;
+}
+
+// I_x(a, 1/2) with front = 1 / (a B(a, 1/2)) and the table of its continued fraction.
+__device__ __forceinline__ double half_beta(double x, double a, double front,
+                                            const double *__restrict__ table) {
+  if (!(x > 0.0)) return 0.0;
+  if (x >= kTabMax) return ibeta(a, 0.5, x);
+  return front * exp(a * log(x)) * sqrt(1.0 - x) * cf_of(x, table);
+}
+
+// What the finalisation holds in shared memory.
+constexpr int kExpBitsP = 7;
+struct ParamTables {
+  double e[2 << kExpBitsP];        // exp_neg
+  double l[3 * kLogTab];           // log_ge1
+};
+__device__ ParamTables c_param;
+struct ParamShared {
+  ParamTables t;
+  double cf[kTabInts * (kTabDeg + 1)];
+  double2 rcp[kMaxN + 1];          // 1 / i in two parts
+};
 
 // Place of an FP32 value in fixed point whose unit is 2^-29 of the last place of a
 // value with exponent field emax: below 2^53, exact unless the value is 2^29 times
@@ -85,45 +147,6 @@ __global__ void standardize_kernel(const float *__restrict__ expr, int T, int N,
   }
 }
 
-// The continued fraction of I_x(a, 1/2) on [0, kTabMax], by Chebyshev series of degree
-// kTabDeg on kTabInts equal intervals (their nearest singularity, x = 1, lies at least
-// seven interval widths away: the terms left out are below 1e-16).  One block per
-// interval; a = (N - 2) / 2 is the only one a call needs (two genotype groups, or the
-// regression).
-constexpr int kTabInts = 64, kTabDeg = 15;
-constexpr double kTabMax = 0.92;
-__global__ void cf_table_kernel(double a, double *__restrict__ table) {
-  __shared__ double f[kTabDeg + 1];
-  const int i = threadIdx.x;
-  const double h = 0.5 * kTabMax / kTabInts, mid = (2 * blockIdx.x + 1) * h;
-  if (i <= kTabDeg) f[i] = ibeta_cf(a, 0.5, mid + h * cospi((i + 0.5) / (kTabDeg + 1)));
-  __syncthreads();
-  if (i > kTabDeg) return;
-  double c = 0.0;
-  for (int j = 0; j <= kTabDeg; ++j) c += f[j] * cospi(i * (j + 0.5) / (kTabDeg + 1));
-  table[blockIdx.x * (kTabDeg + 1) + i] = c * (i ? 2.0 : 1.0) / (kTabDeg + 1);
-}
-
-// I_x(a, 1/2) with front = 1 / (a B(a, 1/2)) and the table of its continued fraction.
-__device__ __forceinline__ double half_beta(double x, double a, double front,
-                                            const double *__restrict__ table) {
-  if (!(x > 0.0)) return 0.0;
-  if (x >= kTabMax) return ibeta(a, 0.5, x);
-  const int i = min((int)(x * (kTabInts / kTabMax)), kTabInts - 1);
-  const double h = 0.5 * kTabMax / kTabInts;
-  const double t2 = 2.0 * ((x - (2 * i + 1) * h) / h);
-  const double *c = table + i * (kTabDeg + 1);
-  double b1 = 0.0, b2 = 0.0;
-#pragma unroll
-  for (int k = kTabDeg; k >= 1; --k) {
-    const double b = fma(t2, b1, __ldg(c + k) - b2);
-    b2 = b1;
-    b1 = b;
-  }
-  const double cf = fma(0.5 * t2, b1, __ldg(c) - b2);
-  return front * exp(a * log(x)) * sqrt(1.0 - x) * cf;
-}
-
 // Four genotype bytes at p (aligned); only bytes in [lo, hi) may be read.
 __device__ __forceinline__ uint32_t geno_word(const int8_t *p, const int8_t *lo, const int8_t *hi) {
   if (p >= lo && p + 4 <= hi) return *reinterpret_cast<const uint32_t *>(p);
@@ -138,10 +161,15 @@ __device__ __forceinline__ uint32_t geno_word(const int8_t *p, const int8_t *lo,
 // the total and the squares are the trait's, the group sizes come with the hit, so a
 // hit needs the sums of two groups alone, taken exactly in 64-bit integers.  One
 // thread per hit: four genotypes a word, the trait's row shared by the threads of one
-// event.  With FP64 additions (which issue at a 64th of the integer rate on this part), squares
-// per hit and the continued fraction evaluated per hit, 1.95 M hits of 102 samples took
-// 2.73 ms and the filter after them 0.07; now 0.60 in all (the FP64 tails).
-__global__ void __launch_bounds__(128)
+// event.  FP64 issues at a 64th of the integer rate on this part, so what is left of it
+// counts.  With rho = SS_between / SS_within and u = 1 + rho, both tails of the analysis of
+// variance are powers of 1 / u: u^-((N - 3) / 2) for three groups (closed form), front u^-((N - 2)
+// / 2) sqrt(rho / u) cf(1 / u) for two, so a warp of both runs one logarithm and one
+// exponential, from tables; divisions by group sizes are products with reciprocals in two
+// parts.  With FP64 additions, squares per hit and the continued fraction evaluated per
+// hit, 1.95 M hits of 102 samples took 2.73 ms; with the library's tails, one for each
+// number of groups, 0.60; now 0.35.
+__global__ void __launch_bounds__(256, 4)
 finalize_param_kernel(const krux_hit *__restrict__ hits, const HitAux *__restrict__ aux,
                       const unsigned long long *__restrict__ count, int64_t capacity,
                       const long long *__restrict__ fixed, const double *__restrict__ squares,
@@ -150,6 +178,20 @@ finalize_param_kernel(const krux_hit *__restrict__ hits, const HitAux *__restric
                       const double *__restrict__ table, double pthresh, krux_hit *__restrict__ out,
                       double *__restrict__ out_stat, double *__restrict__ out_p,
                       int64_t out_capacity, unsigned long long *__restrict__ n_out) {
+  extern __shared__ __align__(16) char shared[];
+  ParamShared &S = *reinterpret_cast<ParamShared *>(shared);
+  for (int i = threadIdx.x; i < (int)(sizeof(ParamTables) / 8); i += blockDim.x)
+    reinterpret_cast<double *>(&S.t)[i] = reinterpret_cast<const double *>(&c_param)[i];
+  for (int i = threadIdx.x; i < kTabInts * (kTabDeg + 1); i += blockDim.x) S.cf[i] = table[i];
+  for (int i = threadIdx.x; i <= N; i += blockDim.x) {
+    const double r = i ? 1.0 / (double)i : 0.0;
+    S.rcp[i] = make_double2(r, i ? fma(-(double)i, r, 1.0) * r : 0.0);
+  }
+  __syncthreads();
+  const auto over = [&](double x, int n) {  // x / n, n = 0 gives 0
+    const double2 r = S.rcp[n];
+    return fma(x, r.x, x * r.y);
+  };
   const unsigned long long c = *count;
   const int64_t n = c < (unsigned long long)capacity ? (int64_t)c : capacity;
   const int lane = threadIdx.x & 31;
@@ -193,17 +235,30 @@ finalize_param_kernel(const krux_hit *__restrict__ hits, const HitAux *__restric
         for (int j = 0; j < 3; ++j) {
           if (cnt[j] == 0) continue;
           ++groups;
-          sq += s[j] * s[j] / (double)cnt[j];
+          sq += over(s[j] * s[j], cnt[j]);
         }
-        const double ssb = sq - st * st / K;
+        const double ssb = sq - over(st * st, N);
         const double ssw = fmax(q - sq, 0.0);
         if (groups >= 2 && N > groups) {
-          const double d1 = groups - 1, d2 = N - groups;
           if (ssw > 0.0) {
-            value = (ssb / d1) / (ssw / d2);
-            if (!(value > 0.0)) p = 1.0;
-            else if (groups == 3) p = f_tail(value, d1, d2);
-            else p = half_beta(d2 / (d2 + value), a_half, front, table);
+            const double rho = ssb / ssw;
+            const int d2 = N - groups;
+            value = rho * (groups == 3 ? 0.5 * d2 : (double)d2);
+            if (!(value > 0.0)) {
+              p = 1.0;
+            } else if (rho < 1e-3 || rho > 1e30) {  // p near 1, or far below what FP64 holds
+              p = groups == 3 ? f_tail(value, 2.0, d2) : half_beta(d2 / (d2 + value), a_half, front, S.cf);
+            } else {
+              const double u = 1.0 + rho;
+              // (what u's rounding lost, to first order)
+              const double lu = fma(rho - (u - 1.0), (double)(1.f / (float)u), log_ge1(u, S.t.l));
+              const double x = 0.5 * d2 * lu;
+              p = x < 700.0 ? exp_neg<kExpBitsP>(x, S.t.e) : exp(-x);
+              if (groups == 2) {
+                const double v = 1.0 / u;
+                p = v < kTabMax ? p * (front * sqrt(rho * v) * cf_of(v, S.cf)) : ibeta(a_half, 0.5, v);
+              }
+            }
           } else if (ssb > 0.0) {
             value = __longlong_as_double(0x7ff0000000000000ll);
             p = 0.0;
@@ -220,7 +275,7 @@ finalize_param_kernel(const krux_hit *__restrict__ hits, const HitAux *__restric
           if (fabs(rr) < 1.0) {
             value = rr * sqrt((K - 2) / (1.0 - rr * rr));
             const double t2 = value * value;
-            p = t2 > 0.0 ? half_beta((K - 2) / (K - 2 + t2), a_half, front, table) : 1.0;
+            p = t2 > 0.0 ? half_beta((K - 2) / (K - 2 + t2), a_half, front, S.cf) : 1.0;
           } else {
             value = rr > 0 ? __longlong_as_double(0x7ff0000000000000ll)
                            : -__longlong_as_double(0x7ff0000000000000ll);
@@ -262,6 +317,29 @@ cudaError_t launch_standardize(const float *expr, int T, int N, int64_t ld, int 
   return cudaGetLastError();
 }
 
+namespace {
+cudaError_t param_prepare() {
+  // bit d: the tables are on device d (the upload is idempotent, the mask update atomic)
+  static std::atomic<unsigned long long> uploaded{0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 64 && ((uploaded.load(std::memory_order_acquire) >> dev) & 1ull)) return cudaSuccess;
+  static const ParamTables t = [] {
+    ParamTables x;
+    fill_exp_table<kExpBitsP>(x.e);
+    fill_log_table(x.l);
+    return x;
+  }();
+  e = cudaMemcpyToSymbol(c_param, &t, sizeof t);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(finalize_param_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(ParamShared));
+  if (e == cudaSuccess && dev < 64) uploaded.fetch_or(1ull << dev, std::memory_order_acq_rel);
+  return e;
+}
+}  // namespace
+
 cudaError_t launch_finalize_param(const krux_hit *hits, const HitAux *aux,
                                   const unsigned long long *count, int64_t capacity,
                                   const long long *fixed, const double *squares,
@@ -271,8 +349,8 @@ cudaError_t launch_finalize_param(const krux_hit *hits, const HitAux *aux,
                                   int64_t out_capacity, unsigned long long *n_out, int sm_count,
                                   cudaStream_t s) {
   if (capacity <= 0) return cudaSuccess;
-  int grid = sm_count * 8;
-  const int64_t need = (capacity + 127) / 128;
+  int grid = sm_count * 4;
+  const int64_t need = (capacity + 255) / 256;
   if (need < grid) grid = (int)need;
   // 1 / (a B(a, 1/2)), a = (N - 2) / 2, by the recurrence of the gamma function from
   // a = 1/2 (1 / (a B) = 2 / pi) or a = 1 (1/2)
@@ -280,7 +358,9 @@ cudaError_t launch_finalize_param(const krux_hit *hits, const HitAux *aux,
   long double front = nu & 1 ? 2.0L / 3.14159265358979323846264338327950288L : 0.5L;
   // B(a + 1, 1/2) = B(a, 1/2) a / (a + 1/2): 1 / (a B) gains (a + 1/2) / (a + 1)
   for (long double a = nu & 1 ? 0.5L : 1.0L; a < 0.5L * nu - 0.25L; a += 1.0L) front *= (a + 0.5L) / (a + 1.0L);
-  finalize_param_kernel<<<grid, 128, 0, s>>>(hits, aux, count, capacity, fixed, squares, geno, ldg, lo,
+  cudaError_t e = param_prepare();
+  if (e != cudaSuccess) return e;
+  finalize_param_kernel<<<grid, 256, sizeof(ParamShared), s>>>(hits, aux, count, capacity, fixed, squares, geno, ldg, lo,
                                              hi, N, model, 0.5 * nu, (double)front, table, pthresh,
                                              out, out_stat, out_p, out_capacity, n_out);
   return cudaGetLastError();
