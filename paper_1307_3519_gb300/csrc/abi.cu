@@ -33,8 +33,9 @@ cudaError_t launch_pack_linear(const int8_t *geno, int64_t ldg, int N, int Np, i
 size_t param_table_bytes();
 cudaError_t launch_standardize(const float *expr, int T, int N, int64_t ld, int Np, __half *A,
                                __half *At, long long *fixed, double *squares, float *tau,
-                               double *cfac, uint16_t *nan_cnt, double *table,
-                               unsigned int *status, cudaStream_t s);
+                               double *cfac, uint16_t *nan_cnt, unsigned int *status,
+                               cudaStream_t s);
+cudaError_t launch_param_table(int N, double *table, cudaStream_t s);
 cudaError_t launch_finalize_param(const krux_hit *hits, const HitAux *aux,
                                   const unsigned long long *count, int64_t capacity,
                                   const long long *fixed, const double *squares,
@@ -2323,7 +2324,7 @@ extern "C" krux_status krux_scan_parametric(krux_ctx *ctx, const float *expr, in
   KRUX_CUDA(ctx, cudaMemsetAsync(ctx->status.p, 0, 64, s));
   ev_record(ctx, 0, s);
   KRUX_CUDA(ctx, launch_standardize(expr, T, N, ld, rs.Np, rs.dev.A, rs.dev.At, fixed, squares,
-                                    rs.dev.tau, rs.dev.cfac, rs.dev.nan_cnt, table,
+                                    rs.dev.tau, rs.dev.cfac, rs.dev.nan_cnt,
                                     ctx->status.as<unsigned int>(), s));
   KRUX_CUDA(ctx, launch_pad_traits(T, rs.rows_pad, rs.dev.tau, rs.dev.cfac, rs.dev.nan_cnt, s));
   ev_record(ctx, 1, s);
@@ -2331,6 +2332,7 @@ extern "C" krux_status krux_scan_parametric(krux_ctx *ctx, const float *expr, in
   KRUX_CUDA(ctx, cudaMemcpyAsync(&hst, ctx->status.p, 4, cudaMemcpyDeviceToHost, s));
   KRUX_CUDA(ctx, cudaStreamSynchronize(s));
   if (hst & kDevBadCode) return fail(ctx, KRUX_EINVAL, "parametric scans take expression without NaN");
+  KRUX_CUDA(ctx, launch_param_table(N, table, s));
   // bounds of the fused test
   CallPlan cp;
   cp.param.model = model;

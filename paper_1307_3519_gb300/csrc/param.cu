@@ -98,8 +98,7 @@ __device__ __forceinline__ long long to_fixed(float x, int emax) {
 // the standardised FP16 row of A (0 in the padding columns, in both layouts), and the
 // constants the scan reads (bound 1, no NaN).  A NaN sets kDevBadCode.  The mean comes
 // from the exact integer sum; only the squares need FP64, two operations a value (with
-// the mean, deviations and scale in FP64, 20,000 x 102: 257 us against 104, both with the
-// table of the tail).
+// the mean, deviations and scale in FP64, 20,000 x 102: some 200 us against 38).
 __global__ void standardize_kernel(const float *__restrict__ expr, int T, int N, int64_t ld, int Np,
                                    __half *__restrict__ A, __half *__restrict__ At,
                                    long long *__restrict__ fixed, double *__restrict__ squares,
@@ -306,13 +305,19 @@ size_t param_table_bytes() { return kTabInts * (kTabDeg + 1) * sizeof(double); }
 
 cudaError_t launch_standardize(const float *expr, int T, int N, int64_t ld, int Np, __half *A,
                                __half *At, long long *fixed, double *squares, float *tau,
-                               double *cfac, uint16_t *nan_cnt, double *table,
-                               unsigned int *status, cudaStream_t s) {
+                               double *cfac, uint16_t *nan_cnt, unsigned int *status,
+                               cudaStream_t s) {
   if (T <= 0) return cudaSuccess;
   const int warps_per_block = 8;
   const int grid = (T + warps_per_block - 1) / warps_per_block;
   standardize_kernel<<<grid, warps_per_block * 32, 0, s>>>(expr, T, N, ld, Np, A, At, fixed, squares,
                                                            tau, cfac, nan_cnt, status);
+  return cudaGetLastError();
+}
+
+// The finalisation's table of a call: some 60 us of serial FP64 chains, queued where the
+// host computes the call's bounds.
+cudaError_t launch_param_table(int N, double *table, cudaStream_t s) {
   cf_table_kernel<<<kTabInts, 32, 0, s>>>(0.5 * (N - 2), table);
   return cudaGetLastError();
 }
