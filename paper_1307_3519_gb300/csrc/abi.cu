@@ -466,13 +466,16 @@ struct GroupPlan {
 // read), a range holds at most kRangeBytes of them and the ranges come one after the
 // other, each over all B tiles, so that the CTAs running at one time stream the same
 // part; with every range in flight at once the batch of 16 x 20,000 x 200,000 took 2 to
-// 4 % longer (85.3 against 81.5 ms when measured).
+// 4 % longer (85.3 against 81.5 ms when measured).  Not so (`together` off) in the general
+// permutation form, whose CTAs raise the minima of the rows they share as they go: all of
+// them on the same rows at once meet too many candidates that the others have beaten (4 x
+// 20,000 x 20,000: 15.0 against 5.0 ms).
 //
 // Several groups (cohorts, missing-value patterns) differ in the cost of a B tile by
 // up to a factor of ten: each is cut into ranges of about the same cost, and the
 // items are taken longest first (5,000 x 100,000 x 102 with 196 missing patterns and
 // 1 % NaN: the scan 1.03 -> 0.58 ms, with two event entries per event warp).
-std::vector<WorkItem> make_items(const std::vector<GroupPlan> &gp, int grid) {
+std::vector<WorkItem> make_items(const std::vector<GroupPlan> &gp, int grid, bool together = true) {
   constexpr int64_t kRangeBytes = 16 << 20;
   std::vector<WorkItem> items;
   auto cut = [&](size_t gi, int64_t b, int64_t k, int64_t s) {
@@ -488,7 +491,7 @@ std::vector<WorkItem> make_items(const std::vector<GroupPlan> &gp, int grid) {
     const GroupPlan &g = gp[0];
     const int64_t L = g.steps - g.step_lo;
     const int64_t min_split =
-        std::max<int64_t>(1, (L * kTileM * g.d.Np * 2 + kRangeBytes - 1) / kRangeBytes);
+        together ? std::max<int64_t>(1, (L * kTileM * g.d.Np * 2 + kRangeBytes - 1) / kRangeBytes) : 1;
     int64_t split = std::max<int64_t>(1, std::min(min_split, L));
     double best = 1e300;
     for (int64_t s = split; s <= std::max<int64_t>(32, min_split + 4) && s <= L; ++s) {
@@ -1402,7 +1405,16 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   } else {
     // a shape picked by krux_autotune for this width, if there is one
     auto it = ctx->tuned.find(round_up(kpad0, 16));
-    if (it != ctx->tuned.end()) {
+    // (it was timed on scans of complete data.  One without a plain form, which inputs
+    // full of hits can make the fastest there, is left to such scans and to expression
+    // with NaN: 4 permutations of 20,000 x 20,000 with 0.9 % hits, 12.9 ms with the shape
+    // picked for the scan, 2.0 in the plain form)
+    bool nan = false;
+    for (auto &g : cp.groups) nan = nan || g.nan_cnt != nullptr;
+    const bool scan = !cp.multi && !cp.cis.on && cp.param.model < 0 && fl.signed_coef == 0 &&
+                      o->dense_H == nullptr;
+    if (it != ctx->tuned.end() &&
+        (scan || nan || (it->second[0] != 0 && it->second[1] > 0 && it->second[1] % 2 == 0))) {
       lay = it->second[0];
       tnc = it->second[1];
       tnA = it->second[2];
@@ -1602,7 +1614,9 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     }
     fl.cis_tiles = (int64_t)n_items;
   } else {
-    items = make_items(plans, workers);
+    bool pairs = fast_shape;  // (as p.fast below)
+    for (const GroupDesc &d : descs) pairs = pairs && d.pair == 1 && (d.nkb == 1 || d.nc == 2);
+    items = make_items(plans, workers, pairs || fl.signed_coef == 0);
     n_items = items.size();
   }
   std::vector<const double *> cf(ng);
@@ -1854,18 +1868,14 @@ krux_status enqueue_fused(krux_ctx *ctx, CallPlan &cp, const FusedLaunch &fl, cu
     const krux_rankset *rs = g.rs;
     __half *B = reinterpret_cast<__half *>(ctx->B.as<char>() + fl.boff[i]);
     ChunkMeta *meta = ctx->meta.as<ChunkMeta>() + fl.moff[i];
-    uint64_t *codes = g.nan_cnt ? ctx->codes.as<uint64_t>() + fl.coff[i] : nullptr;
+    // (the regression, or markers with up to five groups, in a general form)
     if (cp.param.model == 1)
       KRUX_CUDA(ctx, launch_pack_linear(g.geno, g.ldg, rs->N, rs->Np, g.snp_begin, g.n_snps,
                                         cp.param.rl, B, meta, status, s));
-    else if (cp.multi)
+    else
       KRUX_CUDA(ctx, launch_pack_multi(g.geno, g.ldg, rs->N, rs->Np, g.snp_list, g.snp_begin,
                                        g.n_snps, fl.hm, g.allow_missing, B,
                                        reinterpret_cast<ChunkMetaM *>(meta), status, s));
-    else
-      KRUX_CUDA(ctx, launch_pack2(g.geno, g.ldg, rs->N, rs->Np, g.snp_list, g.snp_begin, g.n_snps,
-                                  0, fl.h1, fl.h2, g.allow_missing, fl.signed_coef, B, meta, codes,
-                                  status, s));
   }
   ev_record(ctx, 3, s);
   if (fl.p.mc_cnt)
@@ -1939,7 +1949,7 @@ int fused_launches(const CallPlan &cp, const FusedLaunch &fl) {
   if (fl.batched_pack)
     n += cp.perm.packed ? 0 : (fl.pack_slots > 0 ? 1 : 0) + (fl.pack_halves > 0 ? 1 : 0);
   else
-    for (auto &g : cp.groups) n += g.nan_cnt ? 2 : 1;
+    n += (int)cp.groups.size();
   for (auto &os : cp.slots) n += (os.capacity > 0 && cp.param.model < 0) ? 1 : 0;
   if (cp.param.model >= 0) n += 1;
   if (cp.cis.on) n += 2;

@@ -16,7 +16,7 @@ namespace krux {
 // ---- fixed tile geometry ---------------------------------------------------
 constexpr int kTileM = 128;        // traits per MMA tile = TMEM lanes
 constexpr int kChunkSnps = 64;     // SNPs per chunk
-constexpr int kChunkRows = 128;    // B rows per chunk: [I_0 of 64 SNPs | I_1 of 64 SNPs]
+constexpr int kChunkRows = 128;    // B rows per chunk: two of each of 64 SNPs (see pack.cu)
 constexpr int kMaxN = 512;         // samples: centred 2*rank fits FP16 exactly below 2048
 constexpr int kAtomK = 64;         // K elements per 128-byte swizzle atom (fp16)
 constexpr int kTmemSlots = 4;      // accumulator ring: 4 x 128 fp32 columns = all of TMEM
@@ -25,11 +25,11 @@ constexpr int kEpiSnps = 16;       // SNPs of a chunk each epilogue warp evaluat
 constexpr int kProducerWarp = 16;  // TMA producer
 constexpr int kMmaWarp = 17;       // tcgen05.mma issuer, owns the TMEM allocation
 constexpr int kScanThreads = 576;
-// The plain scan form (complete data, chunks paired into N = 256 MMAs): each of
-// its epilogue warps owns kFastSnps SNPs of one chunk of every accumulator pair
-// for one TMEM lane quarter (32 traits); after them come the producer, the MMA
-// issuer and two idle warps that complete their warpgroup, whose registers go to
-// the epilogue warps (setmaxnreg: both splits use all registers of the launch).
+// The plain scan forms (chunks paired into N = 256 MMAs): each of their epilogue warps
+// owns kFastSnps SNPs of one chunk of every accumulator pair for one TMEM lane quarter
+// (32 traits); after them come the producer, the MMA issuer and two event warps, whose
+// warpgroup gives registers to the epilogue warps (setmaxnreg: both splits use all
+// registers of the launch).
 constexpr int kFastSnps = 32;
 constexpr int kFastEpiWarps = 4 * (2 * kChunkSnps / kFastSnps);  // 16
 constexpr int kFastThreads = 32 * (kFastEpiWarps + 4);
@@ -44,10 +44,10 @@ static_assert(4 * (kFastRegsLaunch - kFastRegsLow) >= kFastEpiWarps * (kFastRegs
               "the epilogue's extra registers must come from the producer warpgroup");
 
 
-// Hit events of the plain scan form are handed to the two idle warps of the
-// producer warpgroup through a ring of shared-memory entries: an epilogue warp
+// Hit events of the plain scan forms are handed to two warps of the producer's
+// warpgroup through a ring of shared-memory entries: an epilogue warp
 // whose half-block (kEvSnps SNPs x 32 traits) has a candidate writes, for each
-// trait lane that found one, an entry with that trait's kEvSnps centred sums and
+// trait lane that found one, an entry with that trait's kEvSnps accumulator pairs and
 // constants and the SNPs' metadata, and goes on; an event warp classifies the
 // entry's pairs (FP64 inside the band) and appends the hit records.
 constexpr int kEvSnps = kFastSnps / 2;  // 16
@@ -87,9 +87,8 @@ static_assert(sizeof(EvEntry) % 16 == 0, "event entries keep 16-byte alignment")
 constexpr size_t ev_region(int entries) { return 128 + entries * (sizeof(EvEntry) + 8 + 4) + 8; }
 // Per-step trait constants staged in shared memory by the producer (one entry per
 // 128-trait tile step): tau f32 [128] @0, 3/(K(K+1)C) f64 [128] @512, starting
-// -ln p key f64 [128] @1536 (permutation batches), NaN count u16 [128] @2560; the
-// two-sided plain form stages instead the classes' decided values with their pair
-// identities, u64 [128][2] @1536 (it has no NaN).
+// -ln p key f64 [128] @1536 (permutation batches), NaN count u16 [128] @2560.  General
+// forms only.
 constexpr int kTcDepth = 4;
 constexpr int kItemDepth = 4;  // work items the producer may announce ahead
 constexpr int kTcBytes = 3584;
@@ -426,10 +425,11 @@ struct ScanParams {
   MinpPair *mc_list = nullptr;
   unsigned int *mc_cnt = nullptr;
   int32_t mc_cap = 0;
-  // the plain scan form applies: 32-byte swizzle, every group's chunks paired, no
-  // dense output, no cis window, no provisional hits (permutation batches take its
-  // two-sided variant; NaN in the expression its variant with coefficient sets,
-  // fast_nan = 1, when at most one trait in 128 has more than kNanCMax NaN samples)
+  // 1: a plain form (640 threads, event warps): the 32-byte swizzle layout, every group's
+  // chunks paired, room for the event ring.  Permutation batches take its seed and
+  // two-class variants, five-group markers, dense output and pairs of CTAs their own, NaN
+  // in the expression the variant with coefficient sets (fast_nan = 1, when at most one
+  // trait in 128 has more than kNanCMax NaN samples)
   int32_t fast = 0;
   int32_t fast_nan = 0;
   // 1: over pairs of CTAs (steps are pairs of trait tiles, each CTA holds one chunk)

@@ -2,10 +2,10 @@
 // statistic by matrix multiplication": the index matrices I_i(m,k) = [G(m,k) = i]
 // and the group sizes N_i(m) = sum_k I_i(m,k)).
 //
-// Only I_0 and I_1 are materialised: with centred ranks the three rank sums
-// satisfy D_0 + D_1 + D_2 = 0, so D_2 follows from the other two.  The packed
-// operand is FP16 0/1 in chunks of 64 SNPs: chunk c holds rows [0,64) = I_0 and
-// rows [64,128) = I_1 of SNPs 64c .. 64c+63, each row Np samples long.
+// Two rows per SNP are enough: with centred ranks the three rank sums satisfy D_0 + D_1 +
+// D_2 = 0.  The packed operand is FP16 in chunks of 64 SNPs of 128 rows.  For the general
+// forms rows [0,64) are I_0 and [64,128) I_1, each Np samples long; for the plain forms
+// they are the weighted rows P and Q (PqCoef), in tiles (tiled_index).
 #include <algorithm>
 
 #include "common.cuh"

@@ -1,22 +1,27 @@
 // scan_sm103.cu -- fused Kruskal-Wallis scan for sm_103a (tcgen05 + TMA + TMEM).
 //
 // For a tile of 128 traits and a chunk of 64 SNPs the tensor cores contract the
-// centred rank matrix A (traits x samples, FP16 integers) with the packed
-// indicator rows [I_0 | I_1] of the chunk (Eq. 4: S_i = R I_i^T, here in centred
-// form D_i = 2 S_i - N_i (K+1)), accumulating exact FP32 integers in TMEM.  The
-// epilogue never writes the rank sums to memory: it evaluates Eq. 2 in centred
-// form, H = 3/(K(K+1)C) sum_i D_i^2/N_i with D_2 = -D_0 - D_1 and the tie factor
-// C (section "Handling tied data"), compares it with the chi-square threshold of
-// the SNP's degrees of freedom (section "P-value calculation and empirical FDR
-// correction"), decides pairs within a relative margin of the threshold in
-// FP64, and appends hits with one atomic per warp.
+// centred rank matrix A (traits x samples, FP16 integers) with the packed genotype rows
+// of the chunk (Eq. 4: S_i = R I_i^T, here in centred form D_i = 2 S_i - N_i (K+1)),
+// accumulating exactly in FP32 in TMEM.  The epilogue never writes the rank sums to
+// memory (but for a dense output): it compares Eq. 2 in centred form, H = 3/(K(K+1)C)
+// sum_i D_i^2/N_i with D_2 = -D_0 - D_1 and the tie factor C (section "Handling tied
+// data"), with the chi-square threshold of the SNP's degrees of freedom (section
+// "P-value calculation and empirical FDR correction"); pairs within a relative margin
+// of the threshold are decided in FP64.
 //
-// Roles (576 threads, one CTA per SM, persistent over work items):
-//   warps 0-15: epilogue; warp w reads TMEM lanes 32*(w%4).. (traits) and the
-//               16 SNPs 16*(w/4).. of each 64-SNP chunk
-//   warp 16   : TMA producer (A tiles stream through nA stages; a B tile of nc
-//               chunks stays resident while all trait tiles pass)
-//   warp 17   : TMEM allocator and tcgen05.mma issuer (one thread)
+// Plain forms (kFormScan*; 640 threads, one CTA per SM, persistent over work items taken
+// from a common counter), on weighted genotype rows (ChunkMeta) in the tensor cores' own
+// tile layout (tiled_index):
+//   warps 0-15 : epilogue; warp 4k + q reads TMEM lanes 32q.. (traits) and 32 SNPs of a
+//                chunk of each accumulator pair, and tests P^2 + Q^2 against the bound
+//   warp 16    : producer (rank tiles stream through nA stages by bulk copies; a B tile
+//                of nc chunks stays resident while all trait tiles pass)
+//   warp 17    : TMEM allocator and tcgen05.mma issuer (one thread; with kFormScanPair
+//                over a cluster of two CTAs, cta_group::2)
+//   warps 18-19: event warps (candidates to exact sums, decisions and hit records)
+// General forms (kFormMulti, kFormPerm, kFormNan; 576 threads): 0/1 indicator rows by TMA
+// boxes, warps 0-15 test and append their hits themselves, 16 SNPs each.
 // Every mbarrier wait is bounded: on timeout the kernel raises an error bit,
 // drains its own asynchronous copies and MMAs, frees TMEM and returns.
 #include <atomic>
