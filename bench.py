@@ -55,19 +55,17 @@ WORKLOAD = ("paper-scale fused scan: N=102 samples, T=20000 traits, S=500000 SNP
 #            -k regex:krux_scan_kernel -s 1 -c 1 python bench.py --scan-only --traits 20000
 #            --snps 100000 --data paper --tile 1,4,2,0 --reps 2
 #            (warp instructions x 32 lanes / pairs = lane issue slots per pair)
-# Measured on the kernel below: 241.71 MB read + 74.28 MB written per 500k-SNP launch;
-# 676.60 M warp instructions (567.48 M on the FMA-heavy, FMA-lite and ALU pipes) per
+# Measured on the kernel below: 246.86 MB read + 72.80 MB written per 500k-SNP launch;
+# 372.91 M warp instructions (301.91 M on the FMA-heavy, FMA-lite and ALU pipes) per
 # 100k-SNP launch of 2x10^9 pairs.
-SCAN_TRAFFIC = {"blob": "bcf763037070c5d9692f0da6d0549752132f2260", "bytes": 315.98e6}
-SCAN_ISSUE = {"blob": "bcf763037070c5d9692f0da6d0549752132f2260", "slots_per_pair": 10.83,
-              "fp32_int_slots_per_pair": 9.08,
+SCAN_TRAFFIC = {"blob": "44ab1f5c3b5b0a62351e839dd9e6aea5da6e501d", "bytes": 319.67e6}
+SCAN_ISSUE = {"blob": "44ab1f5c3b5b0a62351e839dd9e6aea5da6e501d", "slots_per_pair": 5.97,
+              "fp32_int_slots_per_pair": 4.83,
               "workload": "planted 20000 x 100000 x 102 (0.19% of pairs are hits)"}
-# Epilogue issue slots per pair by the operation count of the fused test: one add
-# for D_2, three multiplies by 1/n_i, one multiply and two fused multiply-adds for
-# Q, one select of the threshold by df, one compare/branch, plus the amortised
-# TMEM load: about 10 lane slots.  The epilogue bound is SMs x 128 lanes x SM clock
-# / 10 pairs per second.
-EPILOGUE_SLOTS_PER_PAIR = 10.0
+# Epilogue issue slots per pair by the operation count of the fused test P^2 + Q^2 >=
+# bound: two fused multiply-adds, half a sign accumulation and the TMEM load's eighth,
+# 2.6 lane slots.  The epilogue bound is SMs x 128 lanes x SM clock / 2.6 pairs per second.
+EPILOGUE_SLOTS_PER_PAIR = 2.6
 
 
 def kernel_blob():
@@ -556,7 +554,7 @@ def extra_workloads(kx, flush, stream, pk, sms, mhz, steps=5, warmup=3):
                       "per_cohort": per,
                       "what": "8 x krux_rank + one krux_scan_grouped launch; per-cohort rows: the "
                               "cohort scanned alone, frac against its slower bound (4 N_c flop "
-                              "per pair on the tensor pipe, 10 issue slots per pair)"}
+                              "per pair on the tensor pipe, 2.6 issue slots per pair)"}
     del cin, d
     torch.cuda.empty_cache()
     return out
