@@ -48,8 +48,9 @@ inline void fill_exp_table(double *tab) {
 // m's 512th of [1, 2), r = m inv - 1 (|r| < 2^-9), and log1p(r) to r^5 (the next term is
 // below 1e-17).  tab holds inv, -log(inv) to 40 bits below the point and the rest of it,
 // for each 512th; the first has inv = 1.
+// The result comes with what its rounding left out, in `low`.
 constexpr int kLogTab = 512;
-__device__ __forceinline__ double log_ge1(double u, const double *tab) {
+__device__ __forceinline__ double log_ge1(double u, const double *tab, double &low) {
   const int hi = __double2hiint(u);
   const double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(u));
   const double *T = tab + 3 * ((hi >> 11) & (kLogTab - 1));
@@ -61,7 +62,10 @@ __device__ __forceinline__ double log_ge1(double u, const double *tab) {
   // e as FP64 on the bits (2^52 + e, less 2^52), ln 2 to 40 bits below the point and the rest
   const double e = __hiloint2double(0x43300000, (hi >> 20) - 1023) - 4503599627370496.0;
   const double high = fma(e, 0x1.62e42fefa2p-1, T[1]);
-  return high + (q + fma(e, 0x1.9ef35793c7673p-41, T[2]));
+  const double rest = q + fma(e, 0x1.9ef35793c7673p-41, T[2]);
+  const double l = high + rest;
+  low = (high - l) + rest;  // (high is 0 or the larger of the two)
+  return l;
 }
 inline void fill_log_table(double *tab) {
   for (int i = 0; i < kLogTab; ++i) {

@@ -249,10 +249,15 @@ finalize_param_kernel(const krux_hit *__restrict__ hits, const HitAux *__restric
               p = groups == 3 ? f_tail(value, 2.0, d2) : half_beta(d2 / (d2 + value), a_half, front, S.cf);
             } else {
               const double u = 1.0 + rho;
-              // (what u's rounding lost, to first order)
-              const double lu = fma(rho - (u - 1.0), (double)(1.f / (float)u), log_ge1(u, S.t.l));
-              const double x = 0.5 * d2 * lu;
+              // log(1 + rho) in two parts (what u's rounding lost, to first order), and its
+              // multiple as well: the exponent is large, p keeps its last places (from its
+              // statistic to 2e-15, without this and with the library's functions 8e-15)
+              double low;
+              const double lu = log_ge1(u, S.t.l, low), a = 0.5 * d2, x = a * lu;
+              low = fma(rho - (u - 1.0), (double)(1.f / (float)u), low);
+              low = fma(a, low, fma(a, lu, -x));
               p = x < 700.0 ? exp_neg<kExpBitsP>(x, S.t.e) : exp(-x);
+              p = fma(-p, low, p);
               if (groups == 2) {
                 const double v = 1.0 / u;
                 p = v < kTabMax ? p * (front * sqrt(rho * v) * cf_of(v, S.cf)) : ibeta(a_half, 0.5, v);
