@@ -2100,6 +2100,9 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
   // counter when there is one, so that CTAs whose items hold many hits, or short
   // ones, take fewer or more of them) and the other roles follow through it.
   volatile int *item_ring = reinterpret_cast<volatile int *>(tmem_holder + 4);
+  // Plain forms: rank tiles the producer has asked for, the event warps' sign that the
+  // CTA moves on while no entry comes (a launch may run for any time without one).
+  volatile uint32_t *progress = tmem_holder + 2;
   struct ItemPos {
     uint32_t e = 0, phase = 0;
   };
@@ -2148,6 +2151,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       mbar_init(it_empty(e), 1 + R::kEpi);
     }
     *abort_flag = 0;
+    *progress = 0u;
     if constexpr (fast_form(kForm)) {
       for (int e = 0; e < kEv; ++e) {
         mbar_init(ev.full(e), 1);
@@ -2190,6 +2194,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       uint32_t a_stage = 0, a_phase = 0, b_bits = 0;
       uint32_t a_used = 0, a_last = 0, b_used = 0, b_last = 0;
       uint32_t tc_e = 0, tc_phase = 0, tc_used = 0, tc_last = 0;
+      uint32_t tiles = 0;  // rank tiles asked for
       ItemPos ip;
       // (the two CTAs of a pair take the same items, in fixed turns)
       for (int it = kPair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;;
@@ -2278,6 +2283,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
                 tma_load_pair(sA + (uint32_t)a_stage * a_tile_bytes,
                               na == atoms_per_block ? &g->tmA : &g->tmB, 0, y + 32 * a0,
                               peer_addr(a_full(a_stage), 0u));
+                *progress = ++tiles;
                 if (++a_stage == (uint32_t)nA) {
                   a_stage = 0;
                   a_phase ^= 1u;
@@ -2293,6 +2299,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
               mbar_expect_tx(a_full(a_stage), (uint32_t)na * 4096u);
               bulk_load(sA + (uint32_t)a_stage * a_tile_bytes, tile + a0 * 2048, (uint32_t)na * 4096u,
                         a_full(a_stage));
+              *progress = ++tiles;
               a_used |= 1u << a_stage;
               a_last = (a_last & ~(1u << a_stage)) | (a_phase << a_stage);
               if (++a_stage == (uint32_t)nA) {
@@ -2636,7 +2643,9 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       unsigned long long t = (unsigned long long)(2 * e + half);
       bool idle = false;
       long long t0 = 0;
-      while (true) {
+      uint32_t seen = 0;
+      // (the seed pass and the dense form submit nothing)
+      while (kForm != kFormScanSeed && kForm != kFormScanDense) {
         const int b = (int)(t % kEv);
         // the halves' first lanes look whether their ticket is filled, or no more can come
         int got = 0;
@@ -2653,10 +2662,15 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         const bool on = got == 1;
         if (!__any_sync(0xffffffffu, on)) {
           if (__all_sync(0xffffffffu, got == 2)) break;
+          // idle for as long as the CTA works on items without a candidate.  Every other
+          // wait of the CTA gives up by itself, so the end of the epilogue warps always
+          // comes; this limit, counted from the producer's last rank tile, is a last resort
           const long long now = clock64();
-          if (!idle) t0 = now;
+          const uint32_t at = *progress;
+          if (!idle || at != seen) t0 = now;
           idle = true;
-          if (now - t0 > p.timeout_cycles) {
+          seen = at;
+          if (__any_sync(0xffffffffu, ((now - t0) >> 1) > p.timeout_cycles)) {
             if (lane == 0) {
               *abort_flag = 1;
               atomicOr(p.status, kDevTimeout);
