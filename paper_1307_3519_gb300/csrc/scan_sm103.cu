@@ -180,7 +180,7 @@ __device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, const S
 
 // Wait used while shutting down: ignores the abort flag (copies and MMAs already
 // issued must land before the CTA can release its shared memory and TMEM) and
-// gives up only after a fixed bound of about two seconds.
+// gives up only after a fixed bound of about two seconds (reported as 32 + where).
 // (inline: it is also reached by warps that have given registers away with
 // setmaxnreg, which must call no function compiled for more registers)
 __device__ __forceinline__ void wait_drain(uint32_t bar, uint32_t parity, unsigned int *status,
@@ -189,7 +189,7 @@ __device__ __forceinline__ void wait_drain(uint32_t bar, uint32_t parity, unsign
   while (!mbar_try_wait(bar, parity)) {
     if (clock64() - t0 > 4000000000LL) {
       atomicOr(status, kDevTimeout);
-      atomicMax(status + 1, where);
+      atomicMax(status + 1, 32u + where);
       return;
     }
   }
@@ -256,11 +256,6 @@ __device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
       "h"((uint16_t)3)
       : "memory");
 }
-// arrives on this CTA's barrier only
-__device__ __forceinline__ void tc_commit_own(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
-}
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -271,6 +266,14 @@ __device__ __forceinline__ uint32_t peer_addr(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
+}
+__device__ __forceinline__ void st_cluster(uint32_t cluster_addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
+}
+// Counts bytes as arrived that no copy will bring.
+__device__ __forceinline__ void mbar_complete_tx(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes)
+               : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr)
@@ -2127,6 +2130,19 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
 
   constexpr bool kPair = pair_form(kForm);
   const uint32_t rank = kPair ? cluster_rank() : 0u;  // 0: issues the MMAs
+  // Pairs of CTAs: what a CTA has asked for when its roles have ended, own and (after the
+  // first cluster barrier of the shutdown) the other's, in the place of the trait
+  // constants' barriers.
+  struct PairNote {
+    uint32_t loads;        // rank tiles (K blocks of them) asked for, in the order both CTAs share
+    uint32_t stage_atoms;  // atoms of the last one in each stage, 4 bits each
+    uint32_t chunks;       // genotype chunks asked for
+    uint32_t announced;    // of the second CTA's chunks, those announced to the first
+    uint32_t aborted;
+  };
+  static_assert(2 * sizeof(PairNote) <= 2 * kTcDepth * sizeof(uint64_t), "notes of a pair");
+  volatile PairNote *note =
+      reinterpret_cast<volatile PairNote *>(bars + 2 * nA + 2 * nc + 2 * kTmemSlots + 1);
   if (threadIdx.x == 0) {
     for (int s = 0; s < nA; ++s) {
       mbar_init(a_full(s), 1);
@@ -2142,7 +2158,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       mbar_init(t_empty(s), kPair ? 2 * R::kEpi : R::kEpi);
     }
     mbar_init(drain, 1);
-    for (int e = 0; e < kTcDepth; ++e) {
+    for (int e = 0; e < kTcDepth && !fast_form(kForm); ++e) {
       mbar_init(tc_full(e), 1);
       mbar_init(tc_empty(e), R::kEpi);
     }
@@ -2195,6 +2211,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       uint32_t a_used = 0, a_last = 0, b_used = 0, b_last = 0;
       uint32_t tc_e = 0, tc_phase = 0, tc_used = 0, tc_last = 0;
       uint32_t tiles = 0;  // rank tiles asked for
+      uint32_t stage_atoms = 0, chunks = 0;  // (PairNote)
       ItemPos ip;
       // (the two CTAs of a pair take the same items, in fixed turns)
       for (int it = kPair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;;
@@ -2230,8 +2247,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
             bulk_load(sB, g->Bt + (int64_t)(chunk + (int)rank) * kChunkRows * g->Np, b_tx, b_full(0));
           bulk_load(smem_u32(smeta), g->meta + chunk, (uint32_t)nc_item * (uint32_t)sizeof(ChunkMeta),
                     b_full(0));
-          b_used |= 1u;
-          b_last = ph;
+          ++chunks;
           b_bits ^= 1u;
         }
         for (int c = 0; c < nc_item && !kPair; ++c) {
@@ -2275,14 +2291,11 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
               for (int a0 = 0; a0 < n_atoms; a0 += atoms_per_block) {
                 if (!wait_bar(a_empty(a_stage), a_phase ^ 1u, wc, 2)) goto producer_done;
                 const int na = min(atoms_per_block, n_atoms - a0);
-                if (rank == 0u) {
-                  mbar_expect_tx(a_full(a_stage), (uint32_t)na * 8192u);
-                  a_used |= 1u << a_stage;
-                  a_last = (a_last & ~(1u << a_stage)) | (a_phase << a_stage);
-                }
+                if (rank == 0u) mbar_expect_tx(a_full(a_stage), (uint32_t)na * 8192u);
                 tma_load_pair(sA + (uint32_t)a_stage * a_tile_bytes,
                               na == atoms_per_block ? &g->tmA : &g->tmB, 0, y + 32 * a0,
                               peer_addr(a_full(a_stage), 0u));
+                stage_atoms = (stage_atoms & ~(15u << (4 * a_stage))) | ((uint32_t)na << (4 * a_stage));
                 *progress = ++tiles;
                 if (++a_stage == (uint32_t)nA) {
                   a_stage = 0;
@@ -2356,9 +2369,12 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       }
     producer_done:
       // let every copy this thread issued land before the CTA can exit (a pair of CTAs
-      // counts them together: without a timeout every copy was waited for by the MMAs,
-      // after one the pause before the exit stands in)
-      if (kPair && *abort_flag) a_used = b_used = 0u;
+      // counts them together and drains them after both producers have ended, see below)
+      if constexpr (kPair) {
+        note[0].loads = tiles;
+        note[0].stage_atoms = stage_atoms;
+        note[0].chunks = chunks;
+      }
       for (int s = 0; s < nA; ++s)
         if ((a_used >> s) & 1u) wait_drain(a_full(s), (a_last >> s) & 1u, p.status, 10);
       for (int c = 0; c < nc; ++c)
@@ -2371,6 +2387,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFastRegsLow) : "memory");
     if (lane == 0) {
       uint32_t a_stage = 0, a_phase = 0, b_bits = 0, ps = 0, ps_phase = 0;
+      uint32_t announced = 0;
       ItemPos ip;
       while (true) {
         if (!wait_bar(it_full(ip.e), ip.phase, wc, 19)) goto pair_done;
@@ -2386,6 +2403,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
           // announce this CTA's chunk to the issuing one
           if (!wait_bar(b_full(0), b_bits, wc, 4)) goto pair_done;
           mbar_arrive_cluster(peer_addr(b_full(0), 0u));
+          ++announced;
         } else {
           if (!wait_bar_cluster(b_full(0), b_bits, wc, 4)) goto pair_done;
           for (int step = w.step_begin; step < w.step_end; ++step) {
@@ -2416,8 +2434,11 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
         b_bits ^= 1u;
       }
     pair_done:
-      if (rank == 0u) {  // all issued MMAs must finish before TMEM is released
-        tc_commit_own(drain);
+      note[0].announced = announced;
+      if (rank == 0u) {
+        // all issued MMAs must finish before TMEM is released (and their commits have
+        // arrived at the second CTA before it ends: it waits for this one below)
+        tc_commit_pair(drain);
         wait_drain(drain, 0, p.status, 12);
       }
     }
@@ -3303,15 +3324,46 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
 
   __syncthreads();
   if constexpr (kPair) {
-    // The other CTA may still read this one's shared memory.  After a wait that gave up
-    // (a launch that ends in KRUX_ETIMEOUT) rank tiles of the second CTA may be under
-    // way that nothing counts any more: they land well within this pause.
-    if (*abort_flag) {
-      const long long t0 = clock64();
-      while (clock64() - t0 < 400000) __nanosleep(1000);
+    // Both CTAs' roles have ended, and each tells the other what it has asked for.
+    if (threadIdx.x == 0) {
+      note[0].aborted = (uint32_t)*abort_flag;
+      const uint32_t to = peer_addr(smem_u32(const_cast<PairNote *>(note + 1)), rank ^ 1u);
+      st_cluster(to + offsetof(PairNote, loads), note[0].loads);
+      st_cluster(to + offsetof(PairNote, stage_atoms), note[0].stage_atoms);
+      st_cluster(to + offsetof(PairNote, chunks), note[0].chunks);
+      st_cluster(to + offsetof(PairNote, announced), note[0].announced);
+      st_cluster(to + offsetof(PairNote, aborted), note[0].aborted);
     }
     cluster_sync();
+    // Without a wait that gave up, the MMAs waited for every copy.  After one the CTAs may
+    // have stopped at different tiles, at most nA apart (tile i is asked for when the MMAs
+    // have read tile i - nA, which takes both halves), and the first CTA's barriers lack
+    // what the one behind never asked for: those bytes are counted as arrived where the
+    // first CTA expects both halves, and the second CTA's half alone is expected where it
+    // had not armed the barrier yet.  Then every copy can be waited for.
+    if (note[0].aborted | note[1].aborted) {
+      if (threadIdx.x == 0) {
+        const uint32_t chunks = note[0].chunks;
+        if (rank == 0u) {
+          const uint32_t n0 = note[0].loads, n1 = note[1].loads, most = max(n0, n1);
+          const uint32_t atoms = n0 > n1 ? note[0].stage_atoms : note[1].stage_atoms;
+          for (uint32_t i = min(n0, n1); i < most; ++i) {
+            const uint32_t st = i % (uint32_t)nA, half = ((atoms >> (4 * st)) & 15u) * 4096u;
+            if (n0 > n1) mbar_complete_tx(a_full(st), half);
+            else mbar_expect_tx(a_full(st), half);
+          }
+          for (uint32_t i = most > (uint32_t)nA ? most - (uint32_t)nA : 0u; i < most; ++i)
+            wait_drain(a_full(i % (uint32_t)nA), (i / (uint32_t)nA) & 1u, p.status, 10);
+          // (a chunk that the second CTA has not announced: its arrival is made here)
+          if (chunks > note[1].announced) mbar_arrive(b_full(0));
+        }
+        if (chunks > 0u) wait_drain(b_full(0), (chunks - 1u) & 1u, p.status, 11);
+      }
+      cluster_sync();  // the second CTA's copies are counted in the first one's memory
+    }
     if (warp == R::kMma) {
+      if (rank != 0u && lane == 0) wait_drain(drain, 0, p.status, 12);
+      __syncwarp();
       tc_fence_after();
       asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
     }

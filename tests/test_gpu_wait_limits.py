@@ -41,3 +41,35 @@ def test_a_launch_may_take_longer_than_a_wait(kind, T, S, N):
     got = call()
     assert bool((torch.as_tensor(got) == torch.as_tensor(want)).all())
     kx.close()
+
+
+@pytest.mark.parametrize("limit", [1, 1000, 3000, 10_000, 30_000])
+@pytest.mark.parametrize("N", [257, 300, 400, 512])  # one to three K blocks, a shorter last one
+def test_pairs_of_ctas_drain_what_they_asked_for(N, limit):
+    """After a wait that gave up, the two CTAs of a pair may have stopped at different
+    tiles: the launch ends with KRUX_ETIMEOUT without any drain giving up too (sites from
+    32 on), and the next call is right."""
+    import re
+    import torch
+    from paper_1307_3519_gb300 import build
+    build.build()
+    import paper_1307_3519_gb300 as k
+    g = torch.Generator(device="cuda").manual_seed(N)
+    geno = torch.randint(0, 3, (20_000, N), generator=g, device="cuda", dtype=torch.int8)
+    expr = torch.randn((2300, N), generator=g, device="cuda")
+    kx = k.Krux(0)
+    rs = kx.krux_rank(expr)
+    want = kx.krux_scan(rs, geno, 1e-3, capacity=200_000)["n_hits"]
+    for _ in range(3):
+        kx.set_wait_limit(limit)
+        try:
+            assert kx.krux_scan(rs, geno, 1e-3, capacity=200_000)["n_hits"] == want
+        except k.KruxError as e:
+            assert e.status == k.KRUX_ETIMEOUT
+            assert int(re.search(r"site (\d+)", str(e)).group(1)) < 32
+        else:
+            assert limit > 1
+        kx.set_wait_limit(0)
+        assert kx.krux_scan(rs, geno, 1e-3, capacity=200_000)["n_hits"] == want
+    rs.free()
+    kx.close()
