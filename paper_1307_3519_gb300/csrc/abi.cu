@@ -31,6 +31,7 @@ cudaError_t launch_pack_linear(const int8_t *geno, int64_t ldg, int N, int Np, i
                                int64_t n_snps, double rl, __half *B, ChunkMeta *meta,
                                unsigned int *status, cudaStream_t s);
 size_t param_table_bytes();
+cudaError_t param_prepare(cudaStream_t s);
 cudaError_t launch_standardize(const float *expr, int T, int N, int64_t ld, int Np, __half *A,
                                __half *At, long long *fixed, double *squares, float *tau,
                                double *cfac, uint16_t *nan_cnt, unsigned int *status,
@@ -1621,7 +1622,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   }
   std::vector<const double *> cf(ng);
   for (int i = 0; i < ng; ++i) cf[i] = cp.groups[i].cfac;
-  KRUX_CUDA(ctx, finalize_prepare());
+  KRUX_CUDA(ctx, finalize_prepare(s));
   ScanParams &p = fl.p;
   p = ScanParams{};
   p.n_items = (int32_t)n_items;
@@ -1745,7 +1746,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   }
   if (p.fast && p.dense) {
     KRUX_CUDA(ctx, ctx->densecol.ensure((size_t)cp.groups[0].dense_ld * sizeof(DenseCol)));
-    KRUX_CUDA(ctx, dense_prepare());
+    KRUX_CUDA(ctx, dense_prepare(s));
     fl.max_chunks = 0;
     for (const GroupDesc &d : descs) fl.max_chunks = std::max<int64_t>(fl.max_chunks, d.nchunks);
   }
@@ -2332,6 +2333,7 @@ extern "C" krux_status krux_scan_parametric(krux_ctx *ctx, const float *expr, in
   double *squares = reinterpret_cast<double *>(pb + oSq), *table = reinterpret_cast<double *>(pb + oTab);
   KRUX_CUDA(ctx, ctx->status.ensure(64));
   KRUX_CUDA(ctx, cudaMemsetAsync(ctx->status.p, 0, 64, s));
+  KRUX_CUDA(ctx, param_prepare(s));
   ev_record(ctx, 0, s);
   KRUX_CUDA(ctx, launch_standardize(expr, T, N, ld, rs.Np, rs.dev.A, rs.dev.At, fixed, squares,
                                     rs.dev.tau, rs.dev.cfac, rs.dev.nan_cnt,

@@ -7,6 +7,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
+#include <atomic>
 #include <stdint.h>
 
 #include "../../include/krux.h"
@@ -466,6 +467,22 @@ struct alignas(16) DenseCol {
 };
 
 // ---- launch wrappers (defined in the .cu files) -----------------------------
+// A table's upload, once per device (bit d of `done`): upload(s) queues its copies on the
+// call's own stream, and they are waited for before the bit is set, so that whoever reads
+// the table after this, on any stream and thread, reads all of it.  (A copy from pageable
+// memory on the default stream returns when its source is staged, and a non-blocking
+// stream is not ordered after it.)
+template <class Upload>
+inline cudaError_t once_per_device(std::atomic<unsigned long long> &done, cudaStream_t s, Upload upload) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 64 && ((done.load(std::memory_order_acquire) >> dev) & 1ull)) return cudaSuccess;
+  e = upload(s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e == cudaSuccess && dev < 64) done.fetch_or(1ull << dev, std::memory_order_acq_rel);
+  return e;
+}
 // Dense output of a plain-form launch: dense_H holds every pair's D_0, D_1 (two int32);
 // they become FP64 H and p, and the hits (p < pthresh) are appended to the list.
 cudaError_t launch_dense_finish(const GroupDesc *groups, int n_groups, int64_t max_chunks,
@@ -474,7 +491,7 @@ cudaError_t launch_dense_finish(const GroupDesc *groups, int n_groups, int64_t m
                                 double pthresh, krux_hit *hits, HitAux *aux, int64_t capacity,
                                 unsigned long long *counter, int sm_count, cudaStream_t s);
 // Its tables (once per device; not during a graph capture).
-cudaError_t dense_prepare();
+cudaError_t dense_prepare(cudaStream_t s);
 // Work items of a cis scan: every B tile of the groups (n_tiles in all) against the
 // trait tiles its window reaches, appended to items / n_items (zero at launch); tiles
 // that reach no trait get none.  Coordinates out of order set kDevUnsorted.
@@ -547,7 +564,7 @@ cudaError_t launch_pad_traits(int T, int rows_pad, float *tau, double *cfac, uin
                               cudaStream_t s);
 // Uploads the 1/n table the finalisation uses (once per device; not during a
 // graph capture).
-cudaError_t finalize_prepare();
+cudaError_t finalize_prepare(cudaStream_t s);
 // Finalisation of min(*count, capacity) hits, the count read on the device;
 // aux2 is non-null for markers with more than three groups.  pthresh: the hits'
 // threshold P_c (a reported p at or above it is taken again in full FP64).

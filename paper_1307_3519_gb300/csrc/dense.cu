@@ -224,21 +224,18 @@ const DenseTables &dense_tables() {
 
 }  // namespace
 
-cudaError_t dense_prepare() {
-  // bit d: the tables are on device d (the upload is idempotent, the mask update atomic)
+cudaError_t dense_prepare(cudaStream_t s) {
   static std::atomic<unsigned long long> uploaded{0};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 64 && ((uploaded.load(std::memory_order_acquire) >> dev) & 1ull)) return cudaSuccess;
-  const DenseTables &t = dense_tables();
-  e = cudaMemcpyToSymbol(c_exp, t.e, sizeof t.e);
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_erfcx, t.f, sizeof t.f);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(dense_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(DenseTables));
-  if (e == cudaSuccess && dev < 64) uploaded.fetch_or(1ull << dev, std::memory_order_acq_rel);
-  return e;
+  return once_per_device(uploaded, s, [](cudaStream_t s) {
+    const DenseTables &t = dense_tables();
+    cudaError_t e = cudaMemcpyToSymbolAsync(c_exp, t.e, sizeof t.e, 0, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+      e = cudaMemcpyToSymbolAsync(c_erfcx, t.f, sizeof t.f, 0, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(dense_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)sizeof(DenseTables));
+    return e;
+  });
 }
 
 cudaError_t launch_dense_finish(const GroupDesc *groups, int n_groups, int64_t max_chunks,

@@ -327,28 +327,22 @@ cudaError_t launch_param_table(int N, double *table, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-namespace {
-cudaError_t param_prepare() {
-  // bit d: the tables are on device d (the upload is idempotent, the mask update atomic)
+cudaError_t param_prepare(cudaStream_t s) {
   static std::atomic<unsigned long long> uploaded{0};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 64 && ((uploaded.load(std::memory_order_acquire) >> dev) & 1ull)) return cudaSuccess;
-  static const ParamTables t = [] {
-    ParamTables x;
-    fill_exp_table<kExpBitsP>(x.e);
-    fill_log_table(x.l);
-    return x;
-  }();
-  e = cudaMemcpyToSymbol(c_param, &t, sizeof t);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(finalize_param_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(ParamShared));
-  if (e == cudaSuccess && dev < 64) uploaded.fetch_or(1ull << dev, std::memory_order_acq_rel);
-  return e;
+  return once_per_device(uploaded, s, [](cudaStream_t s) {
+    static const ParamTables t = [] {
+      ParamTables x;
+      fill_exp_table<kExpBitsP>(x.e);
+      fill_log_table(x.l);
+      return x;
+    }();
+    cudaError_t e = cudaMemcpyToSymbolAsync(c_param, &t, sizeof t, 0, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(finalize_param_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)sizeof(ParamShared));
+    return e;
+  });
 }
-}  // namespace
 
 cudaError_t launch_finalize_param(const krux_hit *hits, const HitAux *aux,
                                   const unsigned long long *count, int64_t capacity,
@@ -368,8 +362,6 @@ cudaError_t launch_finalize_param(const krux_hit *hits, const HitAux *aux,
   long double front = nu & 1 ? 2.0L / 3.14159265358979323846264338327950288L : 0.5L;
   // B(a + 1, 1/2) = B(a, 1/2) a / (a + 1/2): 1 / (a B) gains (a + 1/2) / (a + 1)
   for (long double a = nu & 1 ? 0.5L : 1.0L; a < 0.5L * nu - 0.25L; a += 1.0L) front *= (a + 0.5L) / (a + 1.0L);
-  cudaError_t e = param_prepare();
-  if (e != cudaSuccess) return e;
   finalize_param_kernel<<<grid, 256, sizeof(ParamShared), s>>>(hits, aux, count, capacity, fixed, squares, geno, ldg, lo,
                                              hi, N, model, 0.5 * nu, (double)front, table, pthresh,
                                              out, out_stat, out_p, out_capacity, n_out);

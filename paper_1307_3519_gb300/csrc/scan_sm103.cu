@@ -3872,21 +3872,18 @@ cudaError_t launch_scan(const ScanParams &p, int grid, size_t smem, cudaStream_t
   return launch_scan_only(p, grid, smem, s);
 }
 
-cudaError_t finalize_prepare() {
-  // bit d: the table is on device d (callers on several host threads may race
-  // to upload it; the upload is idempotent, the mask update atomic)
+cudaError_t finalize_prepare(cudaStream_t s) {
   static std::atomic<unsigned long long> uploaded{0};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 64 && ((uploaded.load(std::memory_order_acquire) >> dev) & 1ull)) return cudaSuccess;
-  double t[kMaxN + 1];
-  t[0] = 0.0;  // empty groups have D_i = 0 and contribute nothing
-  for (int k = 1; k <= kMaxN; ++k) t[k] = 1.0 / (double)k;
-  e = cudaMemcpyToSymbol(c_rcp, t, sizeof t);
-  if (e != cudaSuccess) return e;
-  if (dev < 64) uploaded.fetch_or(1ull << dev, std::memory_order_acq_rel);
-  return cudaSuccess;
+  return once_per_device(uploaded, s, [](cudaStream_t s) {
+    static const struct Reciprocals {
+      double t[kMaxN + 1];
+      Reciprocals() {
+        t[0] = 0.0;  // empty groups have D_i = 0 and contribute nothing
+        for (int k = 1; k <= kMaxN; ++k) t[k] = 1.0 / (double)k;
+      }
+    } rcp;
+    return cudaMemcpyToSymbolAsync(c_rcp, rcp.t, sizeof rcp.t, 0, cudaMemcpyHostToDevice, s);
+  });
 }
 
 cudaError_t launch_finalize(const krux_hit *hits, const HitAux *aux, int64_t n,
@@ -3894,7 +3891,7 @@ cudaError_t launch_finalize(const krux_hit *hits, const HitAux *aux, int64_t n,
                             cudaStream_t s, unsigned long long *fdr_hist, int fdr_bins,
                             double fdr_l0, double fdr_w, double pthresh) {
   if (n <= 0) return cudaSuccess;
-  cudaError_t e = finalize_prepare();
+  cudaError_t e = finalize_prepare(s);
   if (e != cudaSuccess) return e;
   int grid = (int)((n + 255) / 256);
   if (grid > 152 * 8) grid = 152 * 8;
