@@ -282,9 +282,11 @@ struct LaunchShape {
   bool pair_cta = false;  // for the plain form over pairs of CTAs: one chunk in each
 };
 constexpr size_t kSmemLimit = 232448;
-// Shared memory of the plain forms beyond the general one's: the hit-event ring, less
-// what they do without.
-constexpr size_t kPlainExtra = ev_region(kEvEntries) - kFastSaved;
+// Shared memory of the plain forms with nc chunks beyond the general one's: the hit-event
+// ring and the weights' part of the metadata, less what they do without.
+constexpr size_t plain_extra(int nc) {
+  return ev_region(kEvEntries) - kFastSaved + nc * (sizeof(ChunkMeta) - kMetaGeneral);
+}
 constexpr size_t kPairSaved = ev_region(kEvEntries) - ev_region(kEvEntriesPair);
 
 size_t shape_overhead(int nA, int codes_k) {
@@ -298,10 +300,9 @@ size_t shape_overhead(int nA, int codes_k) {
 // against 1.68, N = 256 2.00 against 1.75, N = 320 3.10 against 2.07).
 bool pair_cta_wanted(int kpad) { return kpad >= 240 && pair_clusters() > 0; }
 
-// reserve: shared memory kept free for the plain form's hit-event ring (0 when
-// the call cannot take that form).
+// plain: the call can take a plain form, whose extra shared memory is kept free.
 bool pick_launch_shape(const krux_ctx *ctx, int kpad, int codes_k, LaunchShape &sh,
-                       size_t reserve = 0, bool pair_cta = false) {
+                       bool plain = false, bool pair_cta = false) {
   const size_t chunk = (size_t)256 * kpad;
   if (ctx->tune_nc > 0) {  // explicit shape (tests, autotuner)
     sh.ka = ctx->tune_ka > 0 ? ctx->tune_ka : kpad;
@@ -311,12 +312,12 @@ bool pick_launch_shape(const krux_ctx *ctx, int kpad, int codes_k, LaunchShape &
     if (sh.ka % 64 != 0 && sh.ka != kpad) return false;
     return shape_overhead(sh.nA, codes_k) + (size_t)sh.nA * 256 * sh.ka + sh.b_region <= kSmemLimit;
   }
-  if (reserve > 0) {
+  if (plain) {
     // the plain form: whole K per stage and an even number of chunks
     int best = 0;
     sh.plain = true;
     for (int a = 3; a >= 2; --a) {
-      const size_t used = shape_overhead(a, codes_k) + (size_t)a * chunk + reserve;
+      const size_t used = shape_overhead(a, codes_k) + (size_t)a * chunk + plain_extra(kTmemSlots);
       if (used >= kSmemLimit) continue;
       const int ncf = (int)std::min<size_t>(kTmemSlots, (kSmemLimit - used) / chunk) & ~1;
       if (ncf > best) {
@@ -331,7 +332,7 @@ bool pick_launch_shape(const krux_ctx *ctx, int kpad, int codes_k, LaunchShape &
     // equal blocks that leave three stages, four in a pair of CTAs, whose second CTA's
     // operands are announced a little later
     const int held = pair_cta ? 1 : 2;
-    const size_t fixed = scan_smem_bytes2(2, 8, 0, 0, std::max(codes_k, 16)) + held * chunk + reserve -
+    const size_t fixed = scan_smem_bytes2(2, 8, 0, 0, std::max(codes_k, 16)) + held * chunk + plain_extra(2) -
                          (pair_cta ? kPairSaved : 0);
     const int atoms = kpad / 16;
     for (int blocks = pair_cta ? 1 : 2; fixed < kSmemLimit && blocks <= atoms; ++blocks) {
@@ -379,11 +380,11 @@ int plain_form_fits(const krux_ctx *ctx, int Np, bool pairs) {
   if (ctx->tune_layout == 0) return 0;
   const int kpad = round_up(Np, 16);
   LaunchShape sh;
-  if (!pick_launch_shape(ctx, kpad, 0, sh, kPlainExtra, pairs && pair_cta_wanted(kpad))) return 0;
+  if (!pick_launch_shape(ctx, kpad, 0, sh, true, pairs && pair_cta_wanted(kpad))) return 0;
   if (sh.pair_cta) return 1;
   const int nc = (int)(sh.b_region / (256 * kpad));
   if (nc < 2 || nc % 2 != 0 ||
-      shape_overhead(sh.nA, 0) + (size_t)sh.nA * 256 * sh.ka + sh.b_region + kPlainExtra > kSmemLimit)
+      shape_overhead(sh.nA, 0) + (size_t)sh.nA * 256 * sh.ka + sh.b_region + plain_extra(kTmemSlots) > kSmemLimit)
     return 0;
   return sh.ka == kpad ? 2 : (sh.plain ? 1 : 0);
 }
@@ -1463,7 +1464,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     // pairs of CTAs take complete data without permutations
     const bool pairs = fast_shape && !fast_nan && fl.signed_coef == 0 && !cp.cis.on && !cp.multi && o->dense_H == nullptr && tnc == 0 && tnA == 0 &&
                        pair_cta_wanted(kpad);
-    const bool ok = pick_launch_shape(ctx, kpad, codes_k, sh, fast_shape ? kPlainExtra : 0, pairs);
+    const bool ok = pick_launch_shape(ctx, kpad, codes_k, sh, fast_shape, pairs);
     ctx->tune_nc = s_nc;
     ctx->tune_nA = s_nA;
     ctx->tune_ka = s_ka;
@@ -1693,7 +1694,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   }
   fl.smem = scan_smem_bytes2(nc_max, sh.nA, (size_t)p.a_tile_bytes, (size_t)p.b_region, p.kpad);
   if (p.fast) {  // the plain scan form also holds its ring of hit-event buffers
-    const size_t with_ring = fl.smem + kPlainExtra - (sh.pair_cta ? kPairSaved : 0);
+    const size_t with_ring = fl.smem + plain_extra(nc_max) - (sh.pair_cta ? kPairSaved : 0);
     if (with_ring <= kSmemLimit) fl.smem = with_ring;
     else p.fast = 0;
   }
@@ -3068,7 +3069,7 @@ extern "C" krux_status krux_debug_plan(int N, int with_nan, int layout, int nc, 
   if (plain && lay != 1) return KRUX_EUNSUPPORTED;
   const int codes_k = with_nan == 1 ? Np : (with_nan == 3 ? kCoefNanRows : 0);
   LaunchShape sh;
-  if (!pick_launch_shape(&tmp, kpad, codes_k, sh, plain ? kPlainExtra : 0)) return KRUX_EUNSUPPORTED;
+  if (!pick_launch_shape(&tmp, kpad, codes_k, sh, plain)) return KRUX_EUNSUPPORTED;
   GroupDesc d;
   std::memset(&d, 0, sizeof d);
   d.Np = Np;
@@ -3087,7 +3088,7 @@ extern "C" krux_status krux_debug_plan(int N, int with_nan, int layout, int nc, 
   p.b_region = sh.b_region;
   p.layout = lay;
   const size_t smem = scan_smem_bytes2(p.nc, p.nA, (size_t)p.a_tile_bytes, (size_t)p.b_region, p.kpad) +
-                     (plain ? kPlainExtra : 0);
+                     (plain ? plain_extra(p.nc) : 0);
   out[0] = sh.ka;
   out[1] = sh.nA;
   out[2] = sh.b_region;

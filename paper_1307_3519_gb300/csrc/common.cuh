@@ -166,6 +166,13 @@ struct ChunkMetaM {               // the same shared-memory slot as ChunkMeta
   uint8_t pad_[2304 - 640 - 128 - 320 - 32 - 512 - 128];
 };
 static_assert(sizeof(ChunkMetaM) == sizeof(ChunkMeta), "ChunkMetaM must fill a ChunkMeta slot");
+// The general forms read none of the plain forms' weights and keep only what lies before
+// them in shared memory.  (With whole entries there they lost a resident chunk or a rank
+// stage: complete data of 145 to 160, 257 to 272, 289 to 304 and 321 to 336 samples, NaN data
+// of 97 to 112, 257 to 272, 289 to 304 and 481 to 496.)
+constexpr size_t kMetaGeneral = offsetof(ChunkMeta, pq0);
+static_assert(kMetaGeneral == 1536 && offsetof(ChunkMetaM, pq) <= kMetaGeneral,
+              "the general forms' part of a chunk's metadata");
 
 // Side record of a hit, written next to the public krux_hit record and used by the
 // FP64 finalisation: the pair's group sizes and the group (cohort / bucket) index.

@@ -2062,9 +2062,12 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
   const uint32_t a_tile_bytes = (uint32_t)p.a_tile_bytes;
   const uint32_t sA = base;
   const uint32_t sB = base + (uint32_t)p.nA * a_tile_bytes;
-  ChunkMeta *smeta =
-      reinterpret_cast<ChunkMeta *>(sbase + (size_t)p.nA * a_tile_bytes + (size_t)p.b_region);
-  uint8_t *scodes = reinterpret_cast<uint8_t *>(smeta + p.nc);
+  constexpr uint32_t kMeta = fast_form(kForm) ? sizeof(ChunkMeta) : kMetaGeneral;
+  uint8_t *smeta = sbase + (size_t)p.nA * a_tile_bytes + (size_t)p.b_region;
+  const auto meta_of = [&](int c) -> const ChunkMeta & {
+    return *reinterpret_cast<const ChunkMeta *>(smeta + (uint32_t)c * kMeta);
+  };
+  uint8_t *scodes = smeta + (uint32_t)p.nc * kMeta;
   const uint32_t codes_stride = (uint32_t)p.kpad * 16u;
   uint8_t *stc = scodes + (size_t)p.nc * codes_stride;  // trait-constant ring
   // permutation form: per trait row, the min-p filter bounds of the current step
@@ -2242,11 +2245,10 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
           if (!wait_bar(b_empty(0), ph ^ 1u, wc, 1)) goto producer_done;
           const int chunk = w.btile * 2;
           const bool own = (int)rank < nc_item;
-          mbar_expect_tx(b_full(0), (own ? b_tx : 0u) + (uint32_t)nc_item * (uint32_t)sizeof(ChunkMeta));
+          mbar_expect_tx(b_full(0), (own ? b_tx : 0u) + (uint32_t)nc_item * kMeta);
           if (own)
             bulk_load(sB, g->Bt + (int64_t)(chunk + (int)rank) * kChunkRows * g->Np, b_tx, b_full(0));
-          bulk_load(smem_u32(smeta), g->meta + chunk, (uint32_t)nc_item * (uint32_t)sizeof(ChunkMeta),
-                    b_full(0));
+          bulk_load(smem_u32(smeta), g->meta + chunk, (uint32_t)nc_item * kMeta, b_full(0));
           ++chunks;
           b_bits ^= 1u;
         }
@@ -2254,7 +2256,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
           const uint32_t ph = (b_bits >> c) & 1u;
           if (!wait_bar(b_empty(c), ph ^ 1u, wc, 1)) goto producer_done;
           const int chunk = w.btile * ncg + c;
-          mbar_expect_tx(b_full(c), b_tx + (uint32_t)sizeof(ChunkMeta) + codes_bytes);
+          mbar_expect_tx(b_full(c), b_tx + kMeta + codes_bytes);
           // paired groups interleave chunks 2j, 2j+1 per K atom: [atom][chunk of pair][128 rows]
           const uint32_t bbase = g->pair ? sB + (uint32_t)(c >> 1) * 2u * b_stride + (uint32_t)(c & 1) * abytes
                                          : sB + (uint32_t)c * b_stride;
@@ -2268,7 +2270,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
               tma_load_2d(bbase + (uint32_t)a * astep, &g->tmB, a * ak, g->b_row0 + chunk * kChunkRows,
                           b_full(c));
           }
-          bulk_load(smem_u32(smeta + c), g->meta + chunk, (uint32_t)sizeof(ChunkMeta), b_full(c));
+          bulk_load(smem_u32(smeta) + (uint32_t)c * kMeta, g->meta + chunk, kMeta, b_full(c));
           if (codes_bytes)
             bulk_load(smem_u32(scodes + (size_t)c * codes_stride), g->codes + (size_t)chunk * g->codes_k * 2,
                       codes_bytes, b_full(c));
@@ -3054,7 +3056,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
           pos1 = 0;
           for (int c = h; c - h < nc_item; c += 2) {
             if (c < nc_item) {
-              if (!pair_slot(ps, ps_phase, smeta[c], c, chunk0, g, ag0, tt0, w.group))
+              if (!pair_slot(ps, ps_phase, meta_of(c), c, chunk0, g, ag0, tt0, w.group))
                 goto epi_done_scan;
             } else {  // an odd last chunk leaves warps 8-15 idle: release only
               if (!wait_warp(t_full(ps), ps_phase, p, abort_addr, 7)) goto epi_done_scan;
@@ -3199,7 +3201,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
               slot = 0;
               slot_phase ^= 1u;
             }
-            const ChunkMetaM &mm = *reinterpret_cast<const ChunkMetaM *>(&smeta[c]);
+            const ChunkMetaM &mm = reinterpret_cast<const ChunkMetaM &>(meta_of(c));
             const bool need = hit_fast_m(dd, mm, h, et.ntlo);
             if (__any_sync(0xffffffffu, need)) {
               uint32_t dv[kMaxCodeM * kEpiSnpsM];
@@ -3226,7 +3228,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
             }
             const uint64_t *codes =
                 g.codes ? reinterpret_cast<const uint64_t *>(scodes + (size_t)c * codes_stride) : nullptr;
-            const ChunkMeta &mc = smeta[c];
+            const ChunkMeta &mc = meta_of(c);
             bool need;
             if (minp_mode && seed_pass) {
               // seed pass: only the range of the values (traits with NaN sit out)
@@ -3704,7 +3706,7 @@ size_t scan_smem_bytes(int nc, int nA, int kpad) {
 }
 
 size_t scan_smem_bytes2(int nc, int nA, size_t a_tile_bytes, size_t b_region, int codes_k) {
-  return 1024 + (size_t)nA * a_tile_bytes + b_region + (size_t)nc * sizeof(ChunkMeta) +
+  return 1024 + (size_t)nA * a_tile_bytes + b_region + (size_t)nc * kMetaGeneral +
          (size_t)nc * codes_k * 16 + (size_t)kTcDepth * kTcBytes + 16 * (size_t)kTileM +
          8 * (size_t)(2 * nA + 2 * nc + 2 * kTmemSlots + 1 + 2 * kTcDepth + 2 * kItemDepth) + 32;
 }
