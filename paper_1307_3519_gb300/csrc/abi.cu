@@ -477,7 +477,14 @@ struct GroupPlan {
 // up to a factor of ten: each is cut into ranges of about the same cost, and the
 // items are taken longest first (5,000 x 100,000 x 102 with 196 missing patterns and
 // 1 % NaN: the scan 1.03 -> 0.58 ms, with two event entries per event warp).
-std::vector<WorkItem> make_items(const std::vector<GroupPlan> &gp, int grid, bool together = true) {
+//
+// `fine` (dense output of the general form, whose FP64 work a pair takes by its trait and
+// SNP makes steps of very uneven length): at least eight items per CTA.  With the few items
+// that fill whole waves, taken from the counter as CTAs come free, 1,000 x 20,003 x 102 in LD
+// blocks with 1 % NaN took 4.6 ms in fixed turns, 5.0 from the counter, now 3.2
+// (2,500 x 30,000 18.8 -> 10.5, independent SNPs 12.1 -> 9.9).
+std::vector<WorkItem> make_items(const std::vector<GroupPlan> &gp, int grid, bool together = true,
+                                 bool fine = false) {
   constexpr int64_t kRangeBytes = 16 << 20;
   std::vector<WorkItem> items;
   auto cut = [&](size_t gi, int64_t b, int64_t k, int64_t s) {
@@ -504,6 +511,7 @@ std::vector<WorkItem> make_items(const std::vector<GroupPlan> &gp, int grid, boo
         split = s;
       }
     }
+    if (fine) split = std::min(L, std::max(split, (8 * (int64_t)grid + g.n_btiles - 1) / g.n_btiles));
     for (int64_t i = 0; i < split * g.n_btiles; ++i) {
       if (min_split > 1) cut(0, i % g.n_btiles, i / g.n_btiles, split);
       else cut(0, i / split, i % split, split);
@@ -1618,7 +1626,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   } else {
     bool pairs = fast_shape;  // (as p.fast below)
     for (const GroupDesc &d : descs) pairs = pairs && d.pair == 1 && (d.nkb == 1 || d.nc == 2);
-    items = make_items(plans, workers, pairs || fl.signed_coef == 0);
+    items = make_items(plans, workers, pairs || fl.signed_coef == 0, o->dense_H != nullptr && !pairs);
     n_items = items.size();
   }
   std::vector<const double *> cf(ng);
