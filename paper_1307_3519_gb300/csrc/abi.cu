@@ -1472,7 +1472,17 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
     // pairs of CTAs take complete data without permutations
     const bool pairs = fast_shape && !fast_nan && fl.signed_coef == 0 && !cp.cis.on && !cp.multi && o->dense_H == nullptr && tnc == 0 && tnA == 0 &&
                        pair_cta_wanted(kpad);
-    const bool ok = pick_launch_shape(ctx, kpad, codes_k, sh, fast_shape, pairs);
+    bool ok = pick_launch_shape(ctx, kpad, codes_k, sh, fast_shape, pairs);
+    // Permutation batches contract twice in the plain form, once in the general one, which
+    // has the longer K blocks where the plain form's fall below 48 samples (from 321 on): 8 x
+    // 4,000 x 20,000 independent SNPs, N = 320 2.72 ms against 2.93 in the general form, N = 336
+    // 3.25 against 3.02, N = 360 4.72 against 3.93.  (In LD blocks N = 336 3.15 against 4.19, N =
+    // 360 4.65 against 4.90; the data of a call are not known when it is planned.)
+    if (ok && fast_shape && fl.signed_coef && tnc == 0 && sh.ka != kpad && sh.ka < 48) {
+      fast_shape = false;
+      sh = LaunchShape{};
+      ok = pick_launch_shape(ctx, kpad, codes_k, sh);
+    }
     ctx->tune_nc = s_nc;
     ctx->tune_nA = s_nA;
     ctx->tune_ka = s_ka;
