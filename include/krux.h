@@ -89,11 +89,12 @@ typedef struct {
   int32_t launches;     /* kernels the last call launched */
   int32_t scan_grid;    /* CTAs of the fused scan launch */
   int64_t pairs;        /* SNP x trait pairs the last call tested */
-  int32_t scan_form;    /* kernel form of the fused scan launch: 0 plain, 1 markers with up to
-                           five groups, 2 permutation batch, 3 general (dense, cis, NaN
-                           beyond the plain form's coefficient sets), 4 plain permutation
-                           batch, 5 plain with NaN expression, 7 plain over pairs of CTAs
-                           (large sample counts) */
+  int32_t scan_form;    /* kernel form of the (last) fused scan launch.  Plain forms: 0 complete
+                           data (cis and parametric scans too), 4 permutation batch, 5 NaN
+                           expression, 7 over pairs of CTAs (240 samples and more), 8 markers
+                           with up to five groups, 9 dense output.  General forms, where no
+                           plain one fits or pays: 1 markers with up to five groups, 2
+                           permutation batch, 3 everything else */
   int32_t reserved_;
 } krux_profile;
 

@@ -3761,11 +3761,12 @@ cudaError_t scan_set_smem_all(size_t smem) {
 
 // The kernel form launch_scan_only picks for these parameters (the ScanForm value).
 int scan_form_of(const ScanParams &p) {
-  if (p.multi) return kFormMulti;  // (in either form)
-  if (p.dense) return kFormNan;    // (in either form)
-  if (p.perm) return p.fast && fast_form_ok() ? kFormScanPerm : kFormPerm;
-  if (p.fast && fast_form_ok()) return p.fast_nan ? kFormScanNan : (p.pair_cta ? kFormScanPair : kFormScan);
-  return kFormNan;
+  const bool plain = p.fast && fast_form_ok();
+  if (p.dense && plain) return kFormScanDense;
+  if (p.multi) return plain ? kFormScanMulti : kFormMulti;
+  if (p.perm) return !plain ? kFormPerm : (p.seed_bound ? kFormScanSeed : kFormScanPerm);
+  if (!plain) return kFormNan;
+  return p.fast_nan ? kFormScanNan : (p.pair_cta ? kFormScanPair : kFormScan);
 }
 
 // Launch of the pair form: clusters of two CTAs.
@@ -3810,31 +3811,24 @@ int pair_clusters() {
 }
 
 cudaError_t launch_scan_only(const ScanParams &p, int grid, size_t smem, cudaStream_t s) {
-  if (p.dense && p.fast && fast_form_ok())
-    krux_scan_kernel<kFormScanDense><<<grid, kFastThreads, smem, s>>>(p);
-  else if (p.multi && p.fast && fast_form_ok())
-    krux_scan_kernel<kFormScanMulti><<<grid, kFastThreads, smem, s>>>(p);
-  else if (p.multi)
-    krux_scan_kernel<kFormMulti><<<grid, kScanThreads, smem, s>>>(p);
-  else if (p.perm && p.fast && p.seed_bound && fast_form_ok())
-    krux_scan_kernel<kFormScanSeed><<<grid, kFastThreads, smem, s>>>(p);
-  else if (p.perm && p.fast && fast_form_ok())
-    krux_scan_kernel<kFormScanPerm><<<grid, kFastThreads, smem, s>>>(p);
-  else if (p.perm)
-    krux_scan_kernel<kFormPerm><<<grid, kScanThreads, smem, s>>>(p);
-  else if (p.fast && p.fast_nan && fast_form_ok())
-    krux_scan_kernel<kFormScanNan><<<grid, kFastThreads, smem, s>>>(p);
-  else if (p.fast && p.pair_cta && fast_form_ok()) {
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute attr{};
-    pair_config(cfg, attr, grid, smem, s);
-    return cudaLaunchKernelEx(&cfg, krux_scan_kernel<kFormScanPair>, p);
-  } else if (p.fast && fast_form_ok())
-    krux_scan_kernel<kFormScan><<<grid, kFastThreads, smem, s>>>(p);
-  else
-    // the general form: traits with NaN, dense output, cis window, provisional
-    // hits, unpaired chunks
-    krux_scan_kernel<kFormNan><<<grid, kScanThreads, smem, s>>>(p);
+  switch (scan_form_of(p)) {
+    case kFormScan: krux_scan_kernel<kFormScan><<<grid, kFastThreads, smem, s>>>(p); break;
+    case kFormScanNan: krux_scan_kernel<kFormScanNan><<<grid, kFastThreads, smem, s>>>(p); break;
+    case kFormScanDense: krux_scan_kernel<kFormScanDense><<<grid, kFastThreads, smem, s>>>(p); break;
+    case kFormScanMulti: krux_scan_kernel<kFormScanMulti><<<grid, kFastThreads, smem, s>>>(p); break;
+    case kFormScanSeed: krux_scan_kernel<kFormScanSeed><<<grid, kFastThreads, smem, s>>>(p); break;
+    case kFormScanPerm: krux_scan_kernel<kFormScanPerm><<<grid, kFastThreads, smem, s>>>(p); break;
+    case kFormScanPair: {
+      cudaLaunchConfig_t cfg{};
+      cudaLaunchAttribute attr{};
+      pair_config(cfg, attr, grid, smem, s);
+      return cudaLaunchKernelEx(&cfg, krux_scan_kernel<kFormScanPair>, p);
+    }
+    case kFormMulti: krux_scan_kernel<kFormMulti><<<grid, kScanThreads, smem, s>>>(p); break;
+    case kFormPerm: krux_scan_kernel<kFormPerm><<<grid, kScanThreads, smem, s>>>(p); break;
+    default:  // NaN beyond the coefficient sets, and whatever fits no plain form
+      krux_scan_kernel<kFormNan><<<grid, kScanThreads, smem, s>>>(p);
+  }
   return cudaGetLastError();
 }
 

@@ -45,3 +45,30 @@ def test_wide_permutation_batches(kx, oracle_mod, N, form):
     want = oracle_mod.perm_minp(expr, geno, perms)
     assert np.all(np.abs(r["minp"].cpu().numpy() - want) <= 1e-6 * want)
     rs.free()
+
+
+@pytest.mark.parametrize("N,scan,dense,multi,cis,anova,nan", [
+    (60, 0, 9, 8, 0, 0, 5), (102, 0, 9, 8, 0, 0, 5), (224, 0, 9, 8, 0, 0, 5), (240, 7, 9, 8, 0, 7, 5),
+    (336, 7, 9, 8, 0, 7, 5), (368, 7, 9, 8, 0, 7, 3), (369, 7, 3, 1, 3, 7, 3), (512, 7, 3, 1, 3, 7, 3)])
+def test_the_profile_names_the_form_that_ran(kx, N, scan, dense, multi, cis, anova, nan):
+    import torch
+    expr, geno = _data(N)
+    e, g, g5 = _dev(expr), _dev(geno), _dev(_data(N, codes=5)[1])
+    rs = kx.krux_rank(e)
+    T, S = 200, 700
+    got = []
+    for call in (lambda: kx.krux_scan(rs, g, 1e-4, T * S),
+                 lambda: kx.krux_scan(rs, g, 1e-4, T * S, dense=True),
+                 lambda: kx.krux_scan(rs, g5, 1e-4, T * S, multiallelic=True),
+                 lambda: kx.krux_scan_cis(rs, g, torch.arange(S, device="cuda"), torch.arange(T, device="cuda"),
+                                          300, 1e-4, T * S),
+                 lambda: kx.krux_scan_parametric(e, g, "anova", 1e-4, T * S)):
+        call()
+        got.append(kx.profile()["scan_form"])
+    e[3, 5] = float("nan")
+    rn = kx.krux_rank(e)
+    kx.krux_scan(rn, g, 1e-4, T * S)
+    got.append(kx.profile()["scan_form"])
+    assert got == [scan, dense, multi, cis, anova, nan]
+    rs.free()
+    rn.free()
