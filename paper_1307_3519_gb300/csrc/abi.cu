@@ -1390,6 +1390,24 @@ struct FusedLaunch {
   const double *const *cfacptr = nullptr;
 };
 
+// Whether a call's hits, about P_c of its pairs where nothing is associated, are few
+// enough for the plain form of its kind.  Two event warps per CTA write them there, all
+// sixteen epilogue warps in the general form, which pays from some 0.2 % of independent SNPs on
+// (scan kernel, plain against general, us; in brackets SNPs in LD blocks, whose hits come
+// together):
+//   cis, 10,000 x 40,000 x 102         P_c = 1e-3 621 (259) against 843 (729), 2e-3 1,316
+//                                      (337) against 1,071 (938), 1e-2 6,743 (1,022) against 1,593 (1,714)
+//   ANOVA, the same                    1e-3 602 (210) against 598 (440), 2e-3 1,136 (262)
+//                                      against 720 (509), 1e-2 4,758 (872) against 933 (739)
+//   five groups, the same              3e-3 1,288 against 1,796, 5e-3 2,180 against 2,260, 1e-2
+//                                      4,416 against 2,896
+// (Scans and permutations of biallelic markers have no such line: they have always been
+// in the plain form.)
+bool few_hits(const CallPlan &cp, double pthresh) {
+  if (cp.multi) return pthresh <= 4e-3;
+  return !(cp.cis.on || cp.param.model >= 0) || pthresh <= 1.5e-3;
+}
+
 // tables = 1 puts this launch's tables (group descriptors, work items, pack jobs,
 // tie-factor pointers) in the context's second set, so that two prepared launches
 // can be enqueued back to back without a host synchronisation between them.
@@ -1446,7 +1464,7 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   bool fast_shape = layout == 1 &&
                     (cp.param.model == 1 ? pq_range_linear(cp.param.rl)
                                          : pq_range_ok(fl.h1, cp.multi ? fl.hm[3] : fl.h2)) &&
-                    fast_form_ok();
+                    fast_form_ok() && few_hits(cp, o->pthresh);
   bool any_nan = false, fast_nan = allow_fast_nan && fast_shape;
   for (auto &g : cp.groups) {
     fast_nan = fast_nan && g.minp_key == nullptr &&
@@ -2468,7 +2486,7 @@ extern "C" krux_status krux_scan_grouped(krux_ctx *ctx, krux_cohort *cohorts, in
   constexpr int kParts = 3;
   std::vector<int> plain(n_cohorts, 2);
   for (const ScanGroupIn &g : cp.groups)
-    plain[g.out_slot] = g.nan_cnt || g.bucket >= 0
+    plain[g.out_slot] = g.nan_cnt || g.bucket >= 0 || !few_hits(cp, opts->pthresh)
                             ? 0
                             : std::min(plain[g.out_slot], plain_form_fits(ctx, g.rs->Np, !cp.multi));
   CallPlan parts[kParts];

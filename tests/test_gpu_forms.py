@@ -72,3 +72,39 @@ def test_the_profile_names_the_form_that_ran(kx, N, scan, dense, multi, cis, ano
     assert got == [scan, dense, multi, cis, anova, nan]
     rs.free()
     rn.free()
+
+
+@pytest.mark.parametrize("kind,pth,form", [("cis", 1.5e-3, 0), ("cis", 1.6e-3, 3), ("cis", 0.2, 3),
+                                           ("anova", 1.5e-3, 0), ("anova", 1.6e-3, 3), ("anova", 0.2, 3),
+                                           ("linear", 1.5e-3, 0), ("linear", 1.6e-3, 3), ("linear", 0.2, 3),
+                                           ("multi", 4e-3, 8), ("multi", 4.1e-3, 1), ("multi", 0.2, 1),
+                                           ("scan", 0.2, 0)])
+def test_calls_with_many_hits(kx, oracle_mod, kind, pth, form):
+    """cis, parametric and five-group scans leave the plain form where P_c lets through more
+    hits than its event warps write in time."""
+    import torch
+    T, S, N = 200, 700, 102
+    expr, geno = _data(N, codes=5 if kind == "multi" else 3)
+    e, g = _dev(expr), _dev(geno)
+    rs = kx.krux_rank(e)
+    if kind in ("anova", "linear"):
+        r = kx.krux_scan_parametric(e, g, kind, pth, T * S)
+        orc = oracle_mod.parametric_scan(expr, geno, pth, kind)
+        want = orc["hit"]
+    else:
+        orc = oracle_mod.scan(expr, geno, pth, max_code=4 if kind == "multi" else 2)
+        want = orc["hit"]
+        if kind == "cis":
+            r = kx.krux_scan_cis(rs, g, torch.arange(S, device="cuda"), torch.arange(T, device="cuda"), 150, pth, T * S)
+            want = want & (np.abs(np.arange(S)[None, :] - np.arange(T)[:, None]) <= 150)
+        else:
+            r = kx.krux_scan(rs, g, pth, T * S, multiallelic=kind == "multi")
+    assert kx.profile()["scan_form"] == form
+    h = r["hits"].cpu().numpy().astype(np.int64)
+    got = np.zeros_like(want)
+    got[h[:, 0], h[:, 1]] = True
+    near = np.abs(orc["p"] / pth - 1.0) < 1e-9
+    assert not ((got != want) & ~near).any() and r["n_hits"] == len(h) == int(got.sum())
+    p = r["p"].cpu().numpy()
+    assert np.all(np.abs(p - orc["p"][h[:, 0], h[:, 1]]) <= 1e-6 * p)
+    rs.free()
