@@ -954,11 +954,13 @@ krux_status group_on_device(krux_ctx *ctx, int N, int64_t b, int64_t n, int64_t 
 // Finds SNPs of rows [b, b+n) that carry a -1, groups them by their exact
 // missing-sample set, and lists the complete rows.  `bad` reports codes outside
 // {-1,0,1,2}.  Synchronises the stream, after `meanwhile` has run beside the pre-pass
-// (it must leave the status words and the stream's earlier work alone).
+// (it must leave the status words and the stream's earlier work alone).  `beside` queues
+// other checks that report in the status words; *word is what they and the pre-pass set.
 krux_status find_missing(krux_ctx *ctx, const int8_t *geno, int64_t ldg, int N, int64_t b,
                          int64_t n, cudaStream_t s, std::vector<Bucket> &buckets,
                          std::vector<int64_t> &complete, bool &bad, int max_code,
-                         DevLists *dl = nullptr, const std::function<void()> &meanwhile = {}) {
+                         DevLists *dl = nullptr, const std::function<void()> &meanwhile = {},
+                         const std::function<cudaError_t()> &beside = {}, unsigned int *word = nullptr) {
   KRUX_CUDA(ctx, ctx->status.ensure(64));
   KRUX_CUDA(ctx, ctx->back.ensure(64));
   KRUX_CUDA(ctx, ctx->miss_idx.ensure((size_t)std::max<int64_t>(n, 1) * 8));
@@ -972,6 +974,7 @@ krux_status find_missing(krux_ctx *ctx, const int8_t *geno, int64_t ldg, int N, 
                                      ctx->miss_mask.as<uint64_t>(), ctx->status.as<unsigned int>(),
                                      flags, s));
   if (ctx->profiling) ctx->prof.launches += ldg == N ? 2 : 1;
+  if (beside) KRUX_CUDA(ctx, beside());
   KRUX_CUDA(ctx, cudaMemcpyAsync(ctx->back.p, ctx->status.p, 64, cudaMemcpyDeviceToHost, s));
   if (meanwhile) meanwhile();
   KRUX_CUDA(ctx, cudaStreamSynchronize(s));
@@ -979,6 +982,7 @@ krux_status find_missing(krux_ctx *ctx, const int8_t *geno, int64_t ldg, int N, 
   const unsigned int st = *reinterpret_cast<const unsigned int *>(ctx->back.p);
   const unsigned int m32 = reinterpret_cast<const unsigned int *>(ctx->back.p)[kMissWord];
   bad = (st & kDevBadCode) != 0;
+  if (word) *word = st;
   buckets.clear();
   complete.clear();
   if (bad || m32 == 0) return KRUX_OK;
@@ -1199,9 +1203,20 @@ krux_status plan_groups(krux_ctx *ctx, CallPlan &cp, const krux_rankset *rs, con
   bool bad = false;
   DevLists dl;
   if ((int64_t)(ctx->dlist.n / 8) >= cp.dlist_used + n) dl.base = cp.dlist_used;
+  // the order of a cis scan's coordinates is read with the missing codes, before anything
+  // of the call is launched
+  std::function<cudaError_t()> beside;
+  if (cp.cis.on)
+    beside = [&] {
+      return launch_cis_order(cp.cis.snp_pos, cp.cis.S, cp.cis.trait_pos, cp.cis.T,
+                              ctx->status.as<unsigned int>(), s);
+    };
+  unsigned int word = 0;
   krux_status st = find_missing(ctx, geno, ldg, rs->N, b, n, s, buckets, complete, bad,
-                                cp.multi ? kMaxCodeM : 2, &dl, meanwhile);
+                                cp.multi ? kMaxCodeM : 2, &dl, meanwhile, beside, &word);
   if (st != KRUX_OK) return st;
+  if (ctx->profiling && cp.cis.on) ctx->prof.launches += 1;
+  if (word & kDevUnsorted) return fail(ctx, KRUX_EINVAL, "cis coordinates must be nondecreasing");
   if (dl.base >= 0 && !buckets.empty()) cp.dlist_used += n;
   if (bad)
     return fail(ctx, KRUX_EINVAL, cp.multi ? "genotype code outside {-1, 0..4}"
@@ -1850,11 +1865,13 @@ krux_status enqueue_fused(krux_ctx *ctx, CallPlan &cp, const FusedLaunch &fl, cu
     KRUX_CUDA(ctx, cudaMemsetAsync(ctx->status.p, 0, 64, s));
   if (cp.fdr_hist)
     KRUX_CUDA(ctx, cudaMemsetAsync(cp.fdr_hist, 0, (size_t)cp.fdr_rows * cp.fdr_bins * 8, s));
-  if (cp.cis.on)
-    KRUX_CUDA(ctx, launch_cis_items(ng ? fl.cistab : nullptr, ng, fl.cis_tiles,
-                                    cp.cis.snp_pos, cp.cis.S, cp.cis.trait_pos, cp.cis.T,
-                                    cp.cis.window, const_cast<WorkItem *>(fl.p.items),
-                                    ctx->status.as<int32_t>() + 10, ctx->status.as<unsigned int>(), s));
+  if (cp.cis.on && ng > 0)
+    KRUX_CUDA(ctx, launch_cis_items(fl.cistab, ng, fl.cis_tiles, cp.cis.snp_pos, cp.cis.trait_pos,
+                                    cp.cis.T, cp.cis.window, const_cast<WorkItem *>(fl.p.items),
+                                    ctx->status.as<int32_t>() + 10, s));
+  if (cp.cis.on && ng == 0)  // (an empty range of SNPs: the pre-pass has not run)
+    KRUX_CUDA(ctx, launch_cis_order(cp.cis.snp_pos, cp.cis.S, cp.cis.trait_pos, cp.cis.T,
+                                    ctx->status.as<unsigned int>(), s));
   if (ng == 0) {  // nothing to scan: a permutation batch still reports min p = 1
     if (cp.perm.on) {
       KRUX_CUDA(ctx, cudaMemsetAsync(ctx->minpkey.p, 0,
@@ -1990,7 +2007,7 @@ int fused_launches(const CallPlan &cp, const FusedLaunch &fl) {
     n += (int)cp.groups.size();
   for (auto &os : cp.slots) n += (os.capacity > 0 && cp.param.model < 0) ? 1 : 0;
   if (cp.param.model >= 0) n += 1;
-  if (cp.cis.on) n += 2;
+  if (cp.cis.on) n += 1;
   if (fl.p.fast && fl.p.dense) n += 2;
   if (cp.perm.on) {
     // the permuted stack (and NaN lists) unless a seed pass built them; then the

@@ -501,10 +501,12 @@ cudaError_t launch_dense_finish(const GroupDesc *groups, int n_groups, int64_t m
 cudaError_t dense_prepare(cudaStream_t s);
 // Work items of a cis scan: every B tile of the groups (n_tiles in all) against the
 // trait tiles its window reaches, appended to items / n_items (zero at launch); tiles
-// that reach no trait get none.  Coordinates out of order set kDevUnsorted.
+// that reach no trait get none.
 cudaError_t launch_cis_items(const CisGroup *groups, int n_groups, int64_t n_tiles,
-                             const int64_t *snp_pos, int64_t S, const int64_t *trait_pos, int T,
-                             int64_t window, WorkItem *items, int32_t *n_items,
+                             const int64_t *snp_pos, const int64_t *trait_pos, int T,
+                             int64_t window, WorkItem *items, int32_t *n_items, cudaStream_t s);
+// Coordinates out of order set kDevUnsorted.
+cudaError_t launch_cis_order(const int64_t *snp_pos, int64_t S, const int64_t *trait_pos, int T,
                              unsigned int *status, cudaStream_t s);
 cudaError_t launch_rank(const float *expr, int T, int N, int64_t ld, int Np, int rows_pad,
                         const RankDev &r, cudaStream_t s);

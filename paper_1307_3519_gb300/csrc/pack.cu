@@ -1162,14 +1162,18 @@ __global__ void cis_items_kernel(const CisGroup *__restrict__ groups, int n_grou
 }
 }  // namespace
 
-cudaError_t launch_cis_items(const CisGroup *groups, int n_groups, int64_t n_tiles,
-                             const int64_t *snp_pos, int64_t S, const int64_t *trait_pos, int T,
-                             int64_t window, WorkItem *items, int32_t *n_items,
+cudaError_t launch_cis_order(const int64_t *snp_pos, int64_t S, const int64_t *trait_pos, int T,
                              unsigned int *status, cudaStream_t s) {
   const int64_t most = S > T ? S : T;
   if (most > 1)
     order_kernel<<<(unsigned)std::min<int64_t>((most + 255) / 256, 152 * 8), 256, 0, s>>>(
         snp_pos, S, trait_pos, T, status);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_cis_items(const CisGroup *groups, int n_groups, int64_t n_tiles,
+                             const int64_t *snp_pos, const int64_t *trait_pos, int T,
+                             int64_t window, WorkItem *items, int32_t *n_items, cudaStream_t s) {
   if (n_tiles > 0)
     cis_items_kernel<<<(unsigned)((n_tiles + 7) / 8), 256, 0, s>>>(groups, n_groups, n_tiles, snp_pos,
                                                                    trait_pos, T, window, items, n_items);
