@@ -368,7 +368,8 @@ void krux_graph_destroy(krux_graph *g);
  * would use, after the same shared-memory plan check every launch passes.
  * with_nan: 0 complete data, 1 NaN expression in the general form (2-bit codes),
  * 2 the plain form on complete data (with its hit-event ring), 3 the plain form's
- * NaN variant (coefficient sets).  out[7] = {samples per rank stage, rank stages,
+ * NaN variant (coefficient sets), these two with the whole K per rank stage; 5 and 6 the
+ * same with K blocks too, 7 the plain form over pairs of CTAs.  out[7] = {samples per rank stage, rank stages,
  * B region bytes, resident chunks, K blocks per step, B chunk stride,
  * shared-memory bytes}.  Returns KRUX_OK, KRUX_EUNSUPPORTED if no sound plan of
  * that kind exists, KRUX_EINVAL for arguments out of range. */

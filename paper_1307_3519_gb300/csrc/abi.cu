@@ -421,7 +421,8 @@ std::string validate_plan(const ScanParams &p, const std::vector<GroupDesc> &g, 
     if (d.nc < 1 || d.nc > p.nc) return bad("group chunk count");
     if (d.b_stride % 4096 || (int64_t)(p.pair_cta ? 1 : d.nc) * d.b_stride > p.b_region)
       return bad("group B chunks");
-    if (p.pair_cta && (d.nc != 2 || d.n_agroups > 1 || p.next != nullptr)) return bad("pairs of CTAs");
+    if (p.pair_cta && (d.nc != 2 || d.n_agroups > 1 || p.next != nullptr || p.nA > 8 || p.ka > 128))
+      return bad("pairs of CTAs");
     if (d.b_stride < 256 * d.n_atoms * atom) return bad("group B stride");
     if ((int64_t)d.nkb * p.ka < (int64_t)d.n_atoms * atom || d.nkb < 1) return bad("group K blocks");
     if (d.nkb > 1 && d.nc * 2 > kTmemSlots) return bad("TMEM slots for K blocks");
@@ -3116,13 +3117,15 @@ extern "C" krux_status krux_debug_plan(int N, int with_nan, int layout, int nc, 
   const int kpad = round_up(Np, atom);
   // with_nan: 0 complete data, 1 the general form's 2-bit codes, 2 the plain form
   // (complete data, room for its hit-event ring), 3 the plain form's NaN variant
-  // (its coefficient sets in place of the codes)
-  if (with_nan < 0 || with_nan > 3) return KRUX_EINVAL;
-  const bool plain = with_nan >= 2;
+  // (its coefficient sets in place of the codes), both with the whole K per rank stage; 5
+  // and 6 the same with K blocks too, 7 the plain form over pairs of CTAs
+  if (with_nan < 0 || with_nan > 7 || with_nan == 4) return KRUX_EINVAL;
+  const bool plain = with_nan >= 2, blocks = with_nan >= 5, pairs = with_nan == 7;
   if (plain && lay != 1) return KRUX_EUNSUPPORTED;
-  const int codes_k = with_nan == 1 ? Np : (with_nan == 3 ? kCoefNanRows : 0);
+  const int codes_k = with_nan == 1 ? Np : (with_nan == 3 || with_nan == 6 ? kCoefNanRows : 0);
   LaunchShape sh;
-  if (!pick_launch_shape(&tmp, kpad, codes_k, sh, plain)) return KRUX_EUNSUPPORTED;
+  if (!pick_launch_shape(&tmp, kpad, codes_k, sh, plain, pairs)) return KRUX_EUNSUPPORTED;
+  if (pairs && !sh.pair_cta) return KRUX_EUNSUPPORTED;
   GroupDesc d;
   std::memset(&d, 0, sizeof d);
   d.Np = Np;
@@ -3130,8 +3133,9 @@ extern "C" krux_status krux_debug_plan(int N, int with_nan, int layout, int nc, 
   d.codes = codes_k ? reinterpret_cast<const uint64_t *>(16) : nullptr;
   d.codes_k = codes_k;
   group_shape(sh, kpad, atom, d);
-  // the plain forms: the whole K per rank stage, chunk pairs
-  if (plain && (sh.ka != kpad || d.pair != 1 || d.nkb != 1)) return KRUX_EUNSUPPORTED;
+  // the plain forms: chunk pairs, the whole K per rank stage or one pair and K blocks
+  if (plain && (d.pair != 1 || (d.nkb > 1 && d.nc != 2))) return KRUX_EUNSUPPORTED;
+  if (plain && !blocks && (sh.ka != kpad || d.nkb != 1)) return KRUX_EUNSUPPORTED;
   ScanParams p{};
   p.nc = d.nc;
   p.nA = sh.nA;
@@ -3140,8 +3144,9 @@ extern "C" krux_status krux_debug_plan(int N, int with_nan, int layout, int nc, 
   p.a_tile_bytes = 256 * sh.ka;
   p.b_region = sh.b_region;
   p.layout = lay;
+  p.pair_cta = pairs ? 1 : 0;
   const size_t smem = scan_smem_bytes2(p.nc, p.nA, (size_t)p.a_tile_bytes, (size_t)p.b_region, p.kpad) +
-                     (plain ? plain_extra(p.nc) : 0);
+                     (plain ? plain_extra(p.nc) : 0) - (pairs ? kPairSaved : 0);
   out[0] = sh.ka;
   out[1] = sh.nA;
   out[2] = sh.b_region;
