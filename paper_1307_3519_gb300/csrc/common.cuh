@@ -217,6 +217,23 @@ __device__ __forceinline__ HitAux ld_aux(const HitAux *src) {
   return a;
 }
 
+// ---- the decision of a pair -------------------------------------------------
+// H and p in FP64 from the exact centred sums and group sizes: what every form decides
+// p < P_c on where its own arithmetic leaves a doubt.
+__device__ __forceinline__ double kw_H64(int u, int v, int n0, int n1, int n2, double cfac) {
+  const double D0 = (double)u, D1 = (double)v, D2 = -(double)(u + v);
+  double Q = 0.0;
+  if (n0 > 0) Q += D0 * D0 / (double)n0;
+  if (n1 > 0) Q += D1 * D1 / (double)n1;
+  if (n2 > 0) Q += D2 * D2 / (double)n2;
+  return cfac * Q;
+}
+__device__ __forceinline__ double kw_p64(double H, int df) {
+  if (df == 1) return erfc(sqrt(0.5 * H));
+  if (df == 2) return exp(-0.5 * H);
+  return 1.0;
+}
+
 // ---- the plain forms' operand layout ---------------------------------------
 // Their rank and genotype operands lie in global memory as the tiles that the tensor
 // cores read: per 128 rows, atoms of 16 samples, each [128 rows][32 bytes] with the

@@ -62,6 +62,12 @@ __device__ __forceinline__ double erfc_sqrt(double x, const double *etab, const 
   return exp_neg<kExpBits>(x, etab) * f;
 }
 
+// p within some 1e-12 of P_c: as the other forms decide it (they may differ in the last
+// places, and P_c may be a p of the data).
+__device__ __noinline__ double p_at_threshold(int d0, int d1, int n0, int n1, int n2, int df, double cf) {
+  return kw_p64(kw_H64(d0, d1, n0, n1, n2, cf), df);
+}
+
 // One thread per packed slot: its column's entry.
 __global__ void dense_cols_kernel(const GroupDesc *__restrict__ groups, int g0, int64_t snp0,
                                   DenseCol *__restrict__ col) {
@@ -145,6 +151,8 @@ dense_finish_kernel(const DenseCol *__restrict__ col, const double *const *__res
         const double x = some ? __hiloint2double(hh - 0x00100000, __double2loint(h)) : 0.0;  // h / 2
         if (c.df == 1) p = some ? erfc_sqrt(x, etab, ftab) : 1.0;
         else p = hh < 0x4095e000 ? exp_neg<kExpBits>(x, etab) : exp(-x);  // (h < 1400)
+        if ((unsigned long long)(__double_as_longlong(p) - pbits + 4096) < 8192ull)
+          p = p_at_threshold(d.x, d.y, c.n0, c.n1, c.n2, c.df, cf);
       }
       if (live) {
         H[o] = h;

@@ -401,12 +401,6 @@ __device__ __forceinline__ double chi2_tail64(double H, int df) {
   return exp(-x) * (1.0 + x);
 }
 
-// p-value of the pair in FP64 from the exact centred sums and group sizes.
-__device__ __forceinline__ double kw_p64(double H, int df) {
-  if (df == 1) return erfc(sqrt(0.5 * H));
-  if (df == 2) return exp(-0.5 * H);
-  return 1.0;
-}
 // The reported p of a hit (df 1, 2; the decisions use kw_p64): exp(-x), x = H/2, as
 // 2^-k 2^-f with k = floor(x log2 e) and f the fraction, both from FP64, and 2^-f
 // from exp2f; for df = 1, erfc(z) = exp(-z^2) erfcx(z), z = sqrt(x), with erfcx in
@@ -422,14 +416,6 @@ __device__ __forceinline__ double kw_p_report(double H, int df) {
   double e = (double)exp2f(-(float)(t - k)) * two_mk;
   if (df == 1) e *= (double)erfcxf(sqrtf((float)x));
   return e;
-}
-__device__ __forceinline__ double kw_H64(int u, int v, int n0, int n1, int n2, double cfac) {
-  const double D0 = (double)u, D1 = (double)v, D2 = -(double)(u + v);
-  double Q = 0.0;
-  if (n0 > 0) Q += D0 * D0 / (double)n0;
-  if (n1 > 0) Q += D1 * D1 / (double)n1;
-  if (n2 > 0) Q += D2 * D2 / (double)n2;
-  return cfac * Q;
 }
 
 struct EpiTrait {

@@ -59,3 +59,29 @@ def test_dense_values_and_hits(oracle_mod, N, S, missing):
         assert np.array_equal(h[:, 2], orc["d"][h[:, 0], h[:, 1], 0])
     rs.free()
     kx.close()
+
+
+@pytest.mark.parametrize("N", [40, 102, 200])
+def test_hits_at_a_threshold_of_the_data(N):
+    """P_c that is a p of the data, or next to one: the dense form lists the hits that the
+    plain scan lists, and its p values say the same."""
+    import torch
+    from paper_1307_3519_gb300 import build
+    build.build()
+    import paper_1307_3519_gb300 as k
+    T, S = 60, 600
+    rng = np.random.default_rng(N)
+    geno = rng.integers(0, 3, (S, N)).astype(np.int8)
+    geno[::4] = np.minimum(geno[::4], 1)
+    geno, expr = _dev(geno), _dev(rng.standard_normal((T, N)).astype(np.float32))
+    kx = k.Krux(0)
+    rs = kx.krux_rank(expr)
+    p = kx.krux_scan(rs, geno, 0.3, T * S, dense=True)["dense_p"].cpu().numpy().ravel()
+    for v in rng.choice(p[p < 0.2], 100, replace=False):
+        for pth in (float(v), float(np.nextafter(v, 1)), float(np.nextafter(v, 0))):
+            d = kx.krux_scan(rs, geno, pth, T * S, dense=True)
+            s = kx.krux_scan(rs, geno, pth, T * S)
+            key = lambda r: (r["hits"][:, 0].long() * S + r["hits"][:, 1].long()).sort().values
+            assert torch.equal(key(d), key(s)) and int((d["dense_p"] < pth).sum()) == d["n_hits"]
+    rs.free()
+    kx.close()
