@@ -330,7 +330,12 @@ bool pick_launch_shape(const krux_ctx *ctx, int kpad, int codes_k, LaunchShape &
     if (best >= 2) return true;
     // or one resident pair (in one CTA, or a chunk in each of two) and K in the fewest
     // equal blocks that leave three stages, four in a pair of CTAs, whose second CTA's
-    // operands are announced a little later
+    // operands are announced a little later.  In one CTA the blocks shrink to 16 samples, and
+    // the form still pays for all but permutation batches (prepare_fused); whole calls, plain
+    // against general, us: dense 1,000 x 20,003 N = 336 920 against 3,220, N = 368 950 against
+    // 3,220; cis 20,000 x 100,000, a wide window, 834 against 1,317 and 1,250 against 1,345; five
+    // groups 10,000 x 50,000 1,695 against 2,856 and 2,679 against 2,920; NaN 5,000 x 50,000 N =
+    // 336 835 against 1,351, N = 352, the last that fits, 875 against 1,363
     const int held = pair_cta ? 1 : 2;
     const size_t fixed = scan_smem_bytes2(2, 8, 0, 0, std::max(codes_k, 16)) + held * chunk + plain_extra(2) -
                          (pair_cta ? kPairSaved : 0);

@@ -574,13 +574,13 @@ cudaError_t launch_minp_cands(const MinpPair *list, const unsigned int *cnt, int
                               const double *cfac, int rows_pad, double pthresh, double *key,
                               unsigned long long *fdr_hist, int fdr_bins, double fdr_l0,
                               double fdr_w, cudaStream_t s);
-// After a plain-form seed pass: decides, per (permutation, trait, class), the pair
-// with the seed's largest value exactly (see seed_decide_kernel).
 // A permutation batch's SNP order by df class (list of n_snps rows; scratch: see
 // class_order_bytes).
 size_t class_order_bytes(int64_t n_snps);
 cudaError_t launch_class_order(const int8_t *geno, int64_t ldg, int N, int64_t snp_begin,
                                int64_t n_snps, void *scratch, cudaStream_t s);
+// After a plain-form seed pass: decides, per (permutation, trait, class), the pair
+// with the seed's largest value exactly (see seed_decide_kernel).
 cudaError_t launch_seed_decide(const unsigned long long *rec, const __half *stack, int rows_pad,
                                int Np, int N, int T, int P, const int8_t *geno, int64_t ldg,
                                int64_t n_snps, const ChunkMeta *meta,

@@ -184,7 +184,6 @@ extern "C" krux_status krux_scan_noalloc(const float *expr, int T, int N, int64_
 
   // the previous call's data stays in the array: clear what must start at zero
   NA_CUDA(cudaMemsetAsync(sc + kOffCnt, 0, 64, s));
-  NA_CUDA(cudaMemsetAsync(r.A, 0, (size_t)rows_pad * Np * 2, s));
   NA_CUDA(cudaMemsetAsync(r.tile_nan, 0, (size_t)n_ttiles * 4, s));
   const double *cf = r.cfac;
   NA_CUDA(cudaMemcpyAsync(cfacptr, &cf, sizeof cf, cudaMemcpyHostToDevice, s));

@@ -71,7 +71,7 @@ __device__ __forceinline__ void warp_sort(uint32_t (&v)[E], int lane) {
 
 // E values per lane (32 E >= N).  The O(N^2) count of smaller and equal values that this
 // replaces took 884 us for 15,000 x 500, 163 for 15,000 x 200 and 69 for 20,000 x 102;
-// the network and the searches 100, 38 and 27.  The block's last warps write the FP64 constants of
+// the network and the searches 100, 38 and 27.  The block's first warp writes the FP64 constants of
 // its rows together (FP64 issue is slow on this part); rows past T are padding: zero
 // ranks, never a hit.
 template <int E>

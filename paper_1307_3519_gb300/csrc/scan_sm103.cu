@@ -1988,11 +1988,12 @@ __device__ __noinline__ double minp_step_best(MinpLead *L, double cfac) {
   return best;
 }
 
-// Kernel forms: the plain scan, markers with up to five genotype groups (32-SNP
-// chunks, ChunkMetaM), the permutation scan (groups with a min-p key), and the
-// plain scan of rank sets with NaN (exact group sizes in the hot test); the
-// producer and MMA warps are the same in all four.  Separate forms keep the
-// state of one out of the registers of the others.
+// Kernel forms.  General ones: markers with up to five genotype groups (kFormMulti: 32-SNP
+// chunks, ChunkMetaM), permutation batches (kFormPerm: groups with a min-p key), and
+// everything else (kFormNan: exact group sizes of traits with NaN in the hot test); the
+// others are plain (fast_form).  The producer's and the MMA warp's code is shared, but for the
+// pairs of CTAs' own issuer.  Separate forms keep the state of one out of the registers of
+// the others.
 enum ScanForm {
   kFormScan = 0,
   kFormMulti = 1,
@@ -2027,7 +2028,7 @@ constexpr bool fast_form(int f) {
 constexpr bool pair_form(int f) { return f == kFormScanPair; }
 
 // Warp roles of a kernel form: the epilogue warps first, then the producer and
-// the MMA issuer (the plain scan form also has two idle warps after them).
+// the MMA issuer (in the plain forms two event warps after them).
 template <int kForm>
 struct ScanRoles {
   static constexpr int kEpi = fast_form(kForm) ? kFastEpiWarps : kEpiWarps;
@@ -2189,7 +2190,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
   tc_fence_after();
   const uint32_t tmem_base = *tmem_holder;
   const WaitCtl wc{abort_flag, p.status, p.timeout_cycles};
-  // plain scan form: the registers of the producer warpgroup (warps 8-11) go to
+  // plain scan form: the registers of the producer warpgroup (warps 16-19) go to
   // the epilogue warps; each role's code sits under its own setmaxnreg
 
   if (warp == R::kProducer) {
@@ -2434,7 +2435,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
   } else if (warp == R::kMma && fast_form(kForm)) {
     // MMA issuer of the plain scan form: one N = 256 MMA chain per chunk pair (N =
     // 128 for an odd last chunk) into accumulator pair `ps` (TMEM columns ps *
-    // 256 ..), released by the 8 epilogue warps as soon as they have loaded it
+    // 256 ..), released by the 16 epilogue warps as soon as they have loaded it
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFastRegsLow) : "memory");
     if (lane == 0) {
       uint32_t a_stage = 0, a_phase = 0, b_bits = 0, ps = 0, ps_phase = 0;
@@ -2638,9 +2639,9 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
     __syncwarp();
   } else if constexpr (fast_form(kForm)) {
     // epilogue warps of the plain scan form: warp 4k + q owns lane quarter q of
-    // kFastSnps SNPs of one chunk of every accumulator pair; it loads their D_0 and
-    // D_1 with one wait, releases the pair at once, then runs the hot test (and,
-    // when a lane has a candidate, the hit event) on the registers
+    // kFastSnps SNPs of one chunk of every accumulator pair; it loads and tests them in
+    // two halves, releases the pair after the second load, and hands a half-block with a
+    // candidate to the event warps
     if (warp >= R::kEpi) {  // the two event warps of the producer warpgroup
       asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFastRegsLow) : "memory");
       const int e = warp - (R::kMma + 1);
@@ -2735,7 +2736,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       const uint32_t abort_addr = smem_u32(const_cast<const int *>(abort_flag));
       const uint32_t lane_cols =
           tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(128 * h + off);
-      uint32_t ps = 0, ps_phase = 0, b_bits = 0, tc_e = 0, tc_phase = 0;
+      uint32_t ps = 0, ps_phase = 0, b_bits = 0;
       constexpr int kH = kFastSnps / 2;
       // permutation batches: per class (df 1, df 2) a pair may pass when its value
       // exceeds the largest decided one of the lane's trait, staged for the step, less
@@ -2880,7 +2881,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
           }
           const int o = off + kH * half;
           // permutation batches: the classes of the block's SNPs (all ones: df 2, zero:
-          // df 1; in the order of class_order_kernel nearly every block is of one class)
+          // df 1; in the order of launch_class_order nearly every block is of one class)
           uint32_t cls = 0u;
           if constexpr (kTwo || kSeed) cls = __ballot_sync(0xffffffffu, mc.sgn[o + (lane & (kH - 1))] > 0.f);
           tmem_wait_ld();

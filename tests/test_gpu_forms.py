@@ -108,3 +108,29 @@ def test_calls_with_many_hits(kx, oracle_mod, kind, pth, form):
     p = r["p"].cpu().numpy()
     assert np.all(np.abs(p - orc["p"][h[:, 0], h[:, 1]]) <= 1e-6 * p)
     rs.free()
+
+
+@pytest.mark.parametrize("missing", [False, True])
+@pytest.mark.parametrize("N", [176, 193, 240, 257, 305, 321, 337, 352])  # whole K, K blocks of 128 to 16 samples
+def test_nan_expression_at_wide_shapes(kx, oracle_mod, N, missing):
+    import synth
+    T, S, pth = 200, 700, 0.02
+    rng = np.random.default_rng(N)
+    expr, geno = _data(N)
+    geno[::5] = np.minimum(geno[::5], 1)
+    geno[::7, 1:] = np.where(rng.random((100, N - 1)) < 0.02, 2, 0)  # small groups that NaN samples may empty
+    if missing:
+        synth.add_missing_genotypes(rng, geno, n_patterns=9)
+    for t in range(T):  # up to the last coefficient set's count, one trait beyond it
+        expr[t, rng.choice(N, 11 if t == 40 else t % 7, replace=False)] = np.nan
+    rs = kx.krux_rank(_dev(expr))
+    r = kx.krux_scan(rs, _dev(geno), pth, capacity=T * S)
+    assert kx.profile()["scan_form"] == 5
+    orc = oracle_mod.scan(expr, geno, pth)
+    h = r["hits"].cpu().numpy().astype(np.int64)
+    got = np.zeros_like(orc["hit"])
+    got[h[:, 0], h[:, 1]] = True
+    near = np.abs(orc["p"] / pth - 1.0) < 1e-12
+    assert not ((got != orc["hit"]) & ~near).any() and r["n_hits"] == len(h) == int(got.sum())
+    assert np.array_equal(h[:, 2], orc["d"][h[:, 0], h[:, 1], 0])
+    rs.free()
