@@ -122,7 +122,7 @@ struct ChunkMeta {
   uint8_t pad_[64];
   uint32_t pq0[kChunkSnps];     // plain forms: A0 | A1 << 16 (FP16 bits)
   uint32_t pq1[kChunkSnps];     // G (FP16 bits) | code of group a << 16 | code of group b << 18
-  float sgn[kChunkSnps];        // permutation batches: -1 for a df-1 SNP, else 1
+  float sgn[kChunkSnps];        // permutation batches: -1 for a df-1 SNP, 1 for a df-2 one, else 0
 };
 static_assert(sizeof(ChunkMeta) == 2304, "ChunkMeta must be 2304 bytes");
 

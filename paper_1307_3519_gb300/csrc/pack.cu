@@ -781,7 +781,8 @@ pack_batch_kernel(const PackJob *__restrict__ jobs, int n_jobs, int64_t total_sl
       if (bits > 0) {
         m.pq0[jj] = w.w0;
         m.pq1[jj] = w.w1;
-        m.sgn[jj] = signed_df1 && (n0 > 0) + (n1 > 0) + (n2 > 0) == 2 ? -1.f : 1.f;
+        const int groups = row < 0 || excl ? 0 : (n0 > 0) + (n1 > 0) + (n2 > 0);
+        m.sgn[jj] = groups < 2 ? 0.f : (signed_df1 && groups == 2 ? -1.f : 1.f);
         if (J.coef_nan)
           write_coef_nan(reinterpret_cast<uint8_t *>(J.codes) + c * kCoefNanBytes, jj, w, rh1, rh2);
       }
