@@ -3532,27 +3532,30 @@ __global__ void minp_cands_kernel(const MinpPair *__restrict__ list, const unsig
 // empirical FDR correction") is folded into the key, and its value becomes the class's
 // largest decided value.
 //
-// A warp works on 32 records in turn, its lanes on the samples (whole genotype rows),
+// A warp works on `per` records in turn, its lanes on the samples (whole genotype rows),
 // then lane j on the block's SNP j, and keeps each record's winner in a lane of its own:
-// the FP64 part, the slowest unit of this chip, runs once for the 32 of them.  With one
+// the FP64 part, the slowest unit of this chip, runs once for all of them.  With one
 // record per warp, FP64 on a single lane and a rank loaded again for each SNP, 16 x
-// 20,000 permuted traits took 2.82 ms, now 0.90.  kI: the samples of a lane.
+// 20,000 permuted traits took 2.82 ms, with 32 0.90.  kI: the samples of a lane.
+// A batch too small to give every SM 16 warps of 32 records takes fewer in a warp, whose
+// records are a chain of dependent loads (whole calls: 3 x 2,000 x 10,000, N = 102 527 -> 414
+// us, N = 300 1,140 -> 563; 3 x 128 x 500, N = 200 447 -> 289).
 template <int kI>
 __global__ void __launch_bounds__(256)
     seed_decide_kernel(const unsigned long long *__restrict__ rec, const __half *__restrict__ stack,
                        int rows_pad, int Np, int N, int T, int P, const int8_t *__restrict__ geno,
                        int64_t ldg, int64_t n_snps, const ChunkMeta *__restrict__ meta, const double *__restrict__ cfac, double *key,
-                       unsigned long long *bound) {
+                       unsigned long long *bound, int per) {
   const int lane = threadIdx.x & 31;
   const int64_t nrec = (int64_t)P * T * 2;
   const bool packed = N <= 360;  // both sums (at most K^2 / 4) fit 16 bits
-  for (int64_t r0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * 32; r0 < nrec;
-       r0 += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t r0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * per; r0 < nrec;
+       r0 += (int64_t)gridDim.x * (blockDim.x >> 5) * per) {
     float best = 0.f;  // of record r0 + lane
     int bu = 0, bv = 0;
     int64_t bpos = -1;
     const unsigned long long mine =
-        r0 + lane < nrec ? rec[2 * ((r0 + lane) / 2 / T * rows_pad + (r0 + lane) / 2 % T) + (lane & 1)] : 0ull;
+        lane < per && r0 + lane < nrec ? rec[2 * ((r0 + lane) / 2 / T * rows_pad + (r0 + lane) / 2 % T) + (lane & 1)] : 0ull;
     uint32_t todo = __ballot_sync(0xffffffffu, mine != 0ull);
     while (todo) {
       const int i = __ffs((int)todo) - 1;
@@ -3686,13 +3689,19 @@ cudaError_t launch_seed_decide(const unsigned long long *rec, const __half *stac
                                int64_t n_snps, const ChunkMeta *meta,
                                const double *cfac, double *key, unsigned long long *bound,
                                cudaStream_t s) {
-  const int64_t warps = ((int64_t)P * T * 2 + 31) / 32;
-  if (warps <= 0) return cudaSuccess;
-  const int64_t blocks = (warps + 7) / 8;
+  const int64_t records = (int64_t)P * T * 2;
+  if (records <= 0) return cudaSuccess;
+  int per = 32;  // records of a warp (even: a lane's class is its parity)
+  while (per > 2 && records < (int64_t)per * 152 * 48) per >>= 1;
+  const int64_t blocks = ((records + per - 1) / per + 7) / 8;
   const int grid = (int)(blocks < 65535 ? blocks : 65535);
-  auto *kernel = N <= 128 ? seed_decide_kernel<4> : (N <= 256 ? seed_decide_kernel<8> : seed_decide_kernel<16>);
+  auto *kernel = N <= 128   ? seed_decide_kernel<4>
+                 : N <= 192 ? seed_decide_kernel<6>
+                 : N <= 256 ? seed_decide_kernel<8>
+                 : N <= 320 ? seed_decide_kernel<10>
+                            : seed_decide_kernel<16>;
   kernel<<<grid, 256, 0, s>>>(rec, stack, rows_pad, Np, N, T, P, geno, ldg, n_snps, meta, cfac,
-                              key, bound);
+                              key, bound, per);
   return cudaGetLastError();
 }
 
