@@ -2750,6 +2750,7 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
       constexpr bool kNan = kForm == kFormScanNan;
       constexpr bool kSeed = kForm == kFormScanSeed;
       constexpr float kBoundMin = 1e-30f, kBoundMax = 1e30f;
+      constexpr int kMany = 8;
       // expression with NaN: the bound of this lane's trait is coefficient set
       // nset - 1 of the chunk's block (0: the chunk metadata's exact coefficients;
       // -1: more NaN samples than any set covers, every pair goes to the exact
@@ -2845,8 +2846,10 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
           // (with the FDR histogram on, nearly every candidate is a pair of its band: all go
           // to the event warps, which read the class words themselves.  Read and filtered
           // here, a round trip to L2 with the accumulator slot held, 16 x 20,000 x 200,000
-          // took 44.1 ms, now 40.5)
-          if (ag > 0 && p.fdr_hist == nullptr) {
+          // took 44.1 ms, now 40.5.  Not so where more than kMany traits of the warp have one: those
+          // are values that repeat, as in the only block of a small batch, and most are copies of
+          // the decided pair: 3 x 128 x 16 x 300 286 -> 255 us)
+          if (ag > 0 && (p.fdr_hist == nullptr || __popc(__ballot_sync(0xffffffffu, need)) > kMany)) {
             const uint4 bb = class_words(g, ag, trait);
             mx1 = fmaxf(__uint_as_float(bb.y), kBoundMin);
             id1 = bb.x;
