@@ -1133,6 +1133,7 @@ struct CallPlan {
     bool pre_done = false;       // the stacking was queued already (before a seed pass)
     bool packed = false;         // and so was the packing (a seed pass over the same SNPs)
     bool seed = false;           // min-p seed pass: permuted agroups only, no hits, no FDR
+    bool fdr = false;            // the batch counts its FDR histogram (in its main launch)
   } perm;
   bool multi = false;  // markers with codes 0..4 (chunks of kChunkSnpsM SNPs)
   struct Param {  // parametric comparison: fused test bounds and the FP64 decision
@@ -1422,11 +1423,19 @@ struct FusedLaunch {
 //                                      against 720 (509), 1e-2 4,758 (872) against 933 (739)
 //   five groups, the same              3e-3 1,288 against 1,796, 5e-3 2,180 against 2,260, 1e-2
 //                                      4,416 against 2,896
-// (Scans and permutations of biallelic markers have no such line: they have always been
-// in the plain form.)
-bool few_hits(const CallPlan &cp, double pthresh) {
+//   scan, N = 300, 6,000 x 20,000      (whole calls) 2e-3 0.88 (0.67) of the general form's time,
+//                                      3e-3 1.12 (0.67), 1e-2 2.54 (0.89), 5e-2 9.2 (1.8)
+//   NaN, N = 300, the same             3e-3 0.94 (0.40), 5e-3 1.17 (0.43), 5e-2 3.3 (0.89)
+//   3 permutations, N = 300,           4e-3 0.92 (0.58), 1e-2 1.10 (0.63), 5e-2 1.98 (0.84); with
+//   2,000 x 10,000                     FDR counts 1e-2 0.53 (0.18), 5e-2 1.16 (0.25)
+// (the last three alike from 180 samples on).  Up to 176 samples, with NaN 160, these have no
+// line: there the plain form is the only one that a call takes by itself, it is ahead in LD
+// blocks, the usual input, up to some 2 % of hits, and krux_autotune times both on the data.
+bool few_hits(const CallPlan &cp, double pthresh, int Np, bool nan) {
   if (cp.multi) return pthresh <= 4e-3;
-  return !(cp.cis.on || cp.param.model >= 0) || pthresh <= 1.5e-3;
+  if (cp.cis.on || cp.param.model >= 0) return pthresh <= 1.5e-3;
+  if (cp.perm.on) return Np <= 176 || pthresh <= (cp.perm.fdr ? 3e-2 : 7e-3);
+  return nan ? Np <= 160 || pthresh <= 4e-3 : Np <= 176 || pthresh <= 2.5e-3;
 }
 
 // tables = 1 puts this launch's tables (group descriptors, work items, pack jobs,
@@ -1485,13 +1494,15 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   bool fast_shape = layout == 1 &&
                     (cp.param.model == 1 ? pq_range_linear(cp.param.rl)
                                          : pq_range_ok(fl.h1, cp.multi ? fl.hm[3] : fl.h2)) &&
-                    fast_form_ok() && few_hits(cp, o->pthresh);
+                    fast_form_ok();
   bool any_nan = false, fast_nan = allow_fast_nan && fast_shape;
   for (auto &g : cp.groups) {
     fast_nan = fast_nan && g.minp_key == nullptr &&
                (g.nan_cnt == nullptr || 128 * g.rs->nan_traits_over <= g.rs->T);
     any_nan = any_nan || g.nan_cnt != nullptr;
   }
+  fast_shape = fast_shape && (o->dense_H != nullptr || few_hits(cp, o->pthresh, kpad0, any_nan));
+  fast_nan = fast_nan && fast_shape;
   // (dense output of expression with NaN: the general form, with exact sizes per pair)
   fast_nan = fast_nan && o->dense_H == nullptr;
   fast_nan = fast_nan && any_nan;
@@ -2509,7 +2520,8 @@ extern "C" krux_status krux_scan_grouped(krux_ctx *ctx, krux_cohort *cohorts, in
   constexpr int kParts = 3;
   std::vector<int> plain(n_cohorts, 2);
   for (const ScanGroupIn &g : cp.groups)
-    plain[g.out_slot] = g.nan_cnt || g.bucket >= 0 || !few_hits(cp, opts->pthresh)
+    plain[g.out_slot] = g.nan_cnt || g.bucket >= 0 ||
+                                    !few_hits(cp, opts->pthresh, g.rs->Np, false)
                             ? 0
                             : std::min(plain[g.out_slot], plain_form_fits(ctx, g.rs->Np, !cp.multi));
   CallPlan parts[kParts];
@@ -2657,6 +2669,7 @@ static krux_status plan_permute(krux_ctx *ctx, CallPlan &cp, const krux_rankset 
   cp.fdr_l0 = -std::log10(opts->pthresh);
   cp.fdr_w = fdr_bin_width;
   cp.perm.on = true;
+  cp.perm.fdr = fdr_hist != nullptr;
   cp.perm.rs = rs;
   cp.perm.perms = perms;
   cp.perm.P = P;
@@ -2736,6 +2749,7 @@ extern "C" krux_status krux_permute(krux_ctx *ctx, const krux_rankset *rs, const
   if (with_seed) {
     st = prepare_fused(ctx, seed, opts, fs, s, 1);
     if (st != KRUX_OK) return st;
+    if (fs.p.fast != fm.p.fast) return fail(ctx, KRUX_EUNSUPPORTED, "internal launch plan: seed pass");
     KRUX_CUDA(ctx, scan_set_smem(std::max(fs.smem, fm.smem)));
     st = enqueue_fused(ctx, seed, fs, s);
     if (st != KRUX_OK) return st;
@@ -2825,6 +2839,8 @@ krux_status graph_capture(krux_ctx *ctx, krux_graph *g) {
   if (g->with_seed) {
     st = prepare_fused(w, g->seed_cp, &g->opts, g->seed_fl, g->cs, 1);
     if (st != KRUX_OK) return st;
+    if (g->seed_fl.p.fast != g->fl.p.fast)
+      return fail(w, KRUX_EUNSUPPORTED, "internal launch plan: seed pass");
     KRUX_CUDA(w, scan_set_smem(std::max(g->seed_fl.smem, g->fl.smem)));
     g->cp.perm.pre_done = true;
     g->cp.perm.packed = g->seed_cp.groups[0].n_snps == g->cp.groups[0].n_snps;

@@ -34,13 +34,13 @@ def test_wide_permutation_batches(kx, oracle_mod, N, form):
     expr, geno = _data(N)
     perms = k.krux_make_perms(N, 3, N)
     rs = kx.krux_rank(_dev(expr))
-    r = kx.krux_permute(rs, _dev(geno), _dev(perms), 1e-2, capacity=200 * 700)
+    r = kx.krux_permute(rs, _dev(geno), _dev(perms), 5e-3, capacity=200 * 700)
     assert kx.profile()["scan_form"] == form
-    orc = oracle_mod.scan(expr, geno, 1e-2)
+    orc = oracle_mod.scan(expr, geno, 5e-3)
     h = r["hits"].cpu().numpy().astype(np.int64)
     got = np.zeros_like(orc["hit"])
     got[h[:, 0], h[:, 1]] = True
-    near = np.abs(orc["p"] / 1e-2 - 1.0) < 1e-12
+    near = np.abs(orc["p"] / 5e-3 - 1.0) < 1e-12
     assert not ((got != orc["hit"]) & ~near).any() and r["n_hits"] == len(h)
     want = oracle_mod.perm_minp(expr, geno, perms)
     assert np.all(np.abs(r["minp"].cpu().numpy() - want) <= 1e-6 * want)
@@ -114,7 +114,7 @@ def test_calls_with_many_hits(kx, oracle_mod, kind, pth, form):
 @pytest.mark.parametrize("N", [176, 193, 240, 257, 305, 321, 337, 352])  # whole K, K blocks of 128 to 16 samples
 def test_nan_expression_at_wide_shapes(kx, oracle_mod, N, missing):
     import synth
-    T, S, pth = 200, 700, 0.02
+    T, S, pth = 200, 700, 4e-3
     rng = np.random.default_rng(N)
     expr, geno = _data(N)
     geno[::5] = np.minimum(geno[::5], 1)
@@ -133,4 +133,33 @@ def test_nan_expression_at_wide_shapes(kx, oracle_mod, N, missing):
     near = np.abs(orc["p"] / pth - 1.0) < 1e-12
     assert not ((got != orc["hit"]) & ~near).any() and r["n_hits"] == len(h) == int(got.sum())
     assert np.array_equal(h[:, 2], orc["d"][h[:, 0], h[:, 1], 0])
+    rs.free()
+
+
+@pytest.mark.parametrize("kind,N,pth,form", [
+    ("scan", 176, 0.2, 0), ("scan", 177, 2.5e-3, 0), ("scan", 177, 2.6e-3, 3), ("scan", 300, 2.5e-3, 7),
+    ("scan", 300, 2.6e-3, 3), ("nan", 160, 0.2, 5), ("nan", 161, 4e-3, 5), ("nan", 161, 4.1e-3, 3),
+    ("nan", 300, 0.2, 3), ("dense", 300, 0.2, 9), ("permute", 176, 0.2, 4), ("permute", 300, 7e-3, 4),
+    ("permute", 300, 7.1e-3, 2), ("fdr", 177, 7.1e-3, 4), ("fdr", 300, 0.03, 4), ("fdr", 177, 0.031, 2)])
+def test_wide_calls_with_many_hits(kx, oracle_mod, kind, N, pth, form):
+    import paper_1307_3519_gb300 as k
+    T, S = 200, 700
+    expr, geno = _data(N)
+    if kind == "nan":
+        expr[::3, 4] = np.nan
+    rs, g = kx.krux_rank(_dev(expr)), _dev(geno)
+    if kind in ("permute", "fdr"):
+        perms = k.krux_make_perms(N, 3, N)
+        r = kx.krux_permute(rs, g, _dev(perms), pth, T * S, fdr_bins=9 if kind == "fdr" else 0)
+        want = oracle_mod.perm_minp(expr, geno, perms, traits=np.arange(0, T, 20))
+        assert np.all(np.abs(r["minp"].cpu().numpy()[:, ::20] - want) <= 1e-6 * want)
+    else:
+        r = kx.krux_scan(rs, g, pth, T * S, dense=kind == "dense")
+    assert kx.profile()["scan_form"] == form
+    orc = oracle_mod.scan(expr, geno, pth)
+    h = r["hits"].cpu().numpy().astype(np.int64)
+    got = np.zeros_like(orc["hit"])
+    got[h[:, 0], h[:, 1]] = True
+    near = np.abs(orc["p"] / pth - 1.0) < 1e-12
+    assert not ((got != orc["hit"]) & ~near).any() and r["n_hits"] == len(h) == int(got.sum())
     rs.free()
