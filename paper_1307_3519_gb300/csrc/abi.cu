@@ -200,7 +200,8 @@ struct krux_ctx {
   int tune_layout = -1, tune_nc = 0, tune_nA = 0, tune_ka = 0;  // 0 / -1 = automatic
   PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
   cudaEvent_t ev[kEv] = {};
-  // krux_scan_host: the genotypes' copy runs on its own stream beside the rank transform
+  // a second stream: krux_scan_host's genotype copy beside the rank transform, the table of a
+  // parametric call's tails beside its scan
   cudaStream_t xs = nullptr;
   cudaEvent_t xev = nullptr;
   DevBuf B, meta, codes, status, counters, aux, cfacptr, miss_idx, miss_mask,
@@ -1142,7 +1143,8 @@ struct CallPlan {
     double rl = 0.0;                // regression: 1 / ((K - 1) r_c^2)
     const long long *fixed = nullptr;  // the centred values in fixed point, for the recomputation
     const double *squares = nullptr;   // and their sums of squares
-    const double *table = nullptr;     // continued fraction of the tail
+    const double *table = nullptr;     // continued fraction of the tail, and when it is there
+    cudaEvent_t table_ready = nullptr;
     krux_hit *out = nullptr;        // the caller's lists
     double *out_stat = nullptr, *out_p = nullptr;
     int64_t out_capacity = 0;
@@ -1980,6 +1982,7 @@ krux_status enqueue_fused(krux_ctx *ctx, CallPlan &cp, const FusedLaunch &fl, cu
   if (cp.param.model >= 0) {  // the exact decision of the provisional hits
     const OutSlot &os = cp.slots[0];
     const ScanGroupIn &g = cp.groups[0];
+    KRUX_CUDA(ctx, cudaStreamWaitEvent(s, cp.param.table_ready, 0));
     KRUX_CUDA(ctx, launch_finalize_param(
                        os.hits, os.aux, totals, os.capacity, cp.param.fixed, cp.param.squares, g.geno,
                        g.ldg, g.geno + g.row_lo * g.ldg, g.geno + (g.row_hi - 1) * g.ldg + g.rs->N,
@@ -2179,6 +2182,15 @@ extern "C" krux_status krux_scan(krux_ctx *ctx, const krux_rankset *rs, const in
   return KRUX_OK;
 }
 
+// The context's second stream, to be used after whatever `s` holds.
+static cudaError_t second_stream(krux_ctx *ctx, cudaStream_t s) {
+  cudaError_t e = cudaSuccess;
+  if (!ctx->xs) e = cudaStreamCreateWithFlags(&ctx->xs, cudaStreamNonBlocking);
+  if (e == cudaSuccess && !ctx->xev) e = cudaEventCreateWithFlags(&ctx->xev, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventRecord(ctx->xev, s);
+  return e == cudaSuccess ? cudaStreamWaitEvent(ctx->xs, ctx->xev, 0) : e;
+}
+
 // The device address of page-locked host memory mapped into the device's address
 // space (cudaHostAlloc; cudaHostRegister with the mapped flag), else null.
 static void *mapped_device_ptr(const void *host) {
@@ -2222,12 +2234,7 @@ extern "C" krux_status krux_scan_host(krux_ctx *ctx, const float *expr, int T, i
     KRUX_CUDA(ctx, cudaMemcpy2DAsync(din, (size_t)N * 4, expr, (size_t)lde * 4, (size_t)N * 4, T,
                                      cudaMemcpyHostToDevice, s));
   if (S > 0) {  // on the context's copy stream, while `stream` ranks
-    if (!ctx->xs) {
-      KRUX_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->xs, cudaStreamNonBlocking));
-      KRUX_CUDA(ctx, cudaEventCreateWithFlags(&ctx->xev, cudaEventDisableTiming));
-    }
-    KRUX_CUDA(ctx, cudaEventRecord(ctx->xev, s));  // (after whatever `stream` holds)
-    KRUX_CUDA(ctx, cudaStreamWaitEvent(ctx->xs, ctx->xev, 0));
+    KRUX_CUDA(ctx, second_stream(ctx, s));
     if (ldg == N)
       KRUX_CUDA(ctx, cudaMemcpyAsync(din + goff, geno, gbytes, cudaMemcpyHostToDevice, ctx->xs));
     else
@@ -2405,6 +2412,12 @@ extern "C" krux_status krux_scan_parametric(krux_ctx *ctx, const float *expr, in
   KRUX_CUDA(ctx, ctx->status.ensure(64));
   KRUX_CUDA(ctx, cudaMemsetAsync(ctx->status.p, 0, 64, s));
   KRUX_CUDA(ctx, param_prepare(s));
+  // (some 60 us of serial chains on a few warps; in line with the rest, calls with few hits took
+  // longer than with every tail evaluated by itself: regression of 500 x 4,000 x 102 without a
+  // hit 228 us then, 261 with the table in line, 219 beside the scan)
+  KRUX_CUDA(ctx, second_stream(ctx, s));
+  KRUX_CUDA(ctx, launch_param_table(N, table, ctx->xs));
+  KRUX_CUDA(ctx, cudaEventRecord(ctx->xev, ctx->xs));
   ev_record(ctx, 0, s);
   KRUX_CUDA(ctx, launch_standardize(expr, T, N, ld, rs.Np, rs.dev.A, rs.dev.At, fixed, squares,
                                     rs.dev.tau, rs.dev.cfac, rs.dev.nan_cnt,
@@ -2415,7 +2428,6 @@ extern "C" krux_status krux_scan_parametric(krux_ctx *ctx, const float *expr, in
   KRUX_CUDA(ctx, cudaMemcpyAsync(&hst, ctx->status.p, 4, cudaMemcpyDeviceToHost, s));
   KRUX_CUDA(ctx, cudaStreamSynchronize(s));
   if (hst & kDevBadCode) return fail(ctx, KRUX_EINVAL, "parametric scans take expression without NaN");
-  KRUX_CUDA(ctx, launch_param_table(N, table, s));
   // bounds of the fused test
   CallPlan cp;
   cp.param.model = model;
@@ -2434,6 +2446,7 @@ extern "C" krux_status krux_scan_parametric(krux_ctx *ctx, const float *expr, in
   cp.param.fixed = fixed;
   cp.param.squares = squares;
   cp.param.table = table;
+  cp.param.table_ready = ctx->xev;
   cp.param.out = hits;
   cp.param.out_stat = hit_stat;
   cp.param.out_p = hit_p;

@@ -320,8 +320,8 @@ cudaError_t launch_standardize(const float *expr, int T, int N, int64_t ld, int 
   return cudaGetLastError();
 }
 
-// The finalisation's table of a call: some 60 us of serial FP64 chains, queued where the
-// host computes the call's bounds.
+// The finalisation's table of a call: some 60 us of serial FP64 chains, on a stream of its own
+// beside the scan.
 cudaError_t launch_param_table(int N, double *table, cudaStream_t s) {
   cf_table_kernel<<<kTabInts, 32, 0, s>>>(0.5 * (N - 2), table);
   return cudaGetLastError();
