@@ -1274,8 +1274,34 @@ krux_status plan_groups(krux_ctx *ctx, CallPlan &cp, const krux_rankset *rs, con
   return KRUX_OK;
 }
 
+// Whether a call's hits, about P_c of its pairs where nothing is associated, are few
+// enough for the plain form of its kind.  Two event warps per CTA write them there, all
+// sixteen epilogue warps in the general form, which pays from some 0.2 % of independent SNPs on
+// (scan kernel, plain against general, us; in brackets SNPs in LD blocks, whose hits come
+// together):
+//   cis, 10,000 x 40,000 x 102         P_c = 1e-3 621 (259) against 843 (729), 2e-3 1,316
+//                                      (337) against 1,071 (938), 1e-2 6,743 (1,022) against 1,593 (1,714)
+//   ANOVA, the same                    1e-3 602 (210) against 598 (440), 2e-3 1,136 (262)
+//                                      against 720 (509), 1e-2 4,758 (872) against 933 (739)
+//   five groups, the same              3e-3 1,288 against 1,796, 5e-3 2,180 against 2,260, 1e-2
+//                                      4,416 against 2,896
+//   scan, N = 300, 6,000 x 20,000      (whole calls) 2e-3 0.88 (0.67) of the general form's time,
+//                                      3e-3 1.12 (0.67), 1e-2 2.54 (0.89), 5e-2 9.2 (1.8)
+//   NaN, N = 300, the same             3e-3 0.94 (0.40), 5e-3 1.17 (0.43), 5e-2 3.3 (0.89)
+//   3 permutations, N = 300,           4e-3 0.92 (0.58), 1e-2 1.10 (0.63), 5e-2 1.98 (0.84); with
+//   2,000 x 10,000                     FDR counts 1e-2 0.53 (0.18), 5e-2 1.16 (0.25)
+// (the last three alike from 180 samples on).  Up to 176 samples, with NaN 160, these have no
+// line: there the plain form is the only one that a call takes by itself, it is ahead in LD
+// blocks, the usual input, up to some 2 % of hits, and krux_autotune times both on the data.
+bool few_hits(const CallPlan &cp, double pthresh, int Np, bool nan) {
+  if (cp.multi) return pthresh <= 4e-3;
+  if (cp.cis.on || cp.param.model >= 0) return pthresh <= 1.5e-3;
+  if (cp.perm.on) return Np <= 176 || pthresh <= (cp.perm.fdr ? 3e-2 : 7e-3);
+  return nan ? Np <= 160 || pthresh <= 4e-3 : Np <= 176 || pthresh <= 2.5e-3;
+}
+
 // Uploads SNP lists, re-ranks every bucket, and points the groups at the results.
-krux_status materialise(krux_ctx *ctx, CallPlan &cp, cudaStream_t s) {
+krux_status materialise(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, cudaStream_t s) {
   if (!cp.lists.empty()) {
     KRUX_CUDA(ctx, ctx->list.ensure(cp.lists.size() * 8));
     KRUX_CUDA(ctx, ctx->list_host.ensure(cp.lists.size() * 8));
@@ -1351,13 +1377,17 @@ krux_status materialise(krux_ctx *ctx, CallPlan &cp, cudaStream_t s) {
   int32_t *ddrop = reinterpret_cast<int32_t *>(base + drop_off);
   KRUX_CUDA(ctx, cudaMemcpyAsync(djobs, jobs.data(), nb * sizeof(RerankJob), cudaMemcpyHostToDevice, s));
   KRUX_CUDA(ctx, cudaMemcpyAsync(ddrop, drops.data(), drops.size() * 4, cudaMemcpyHostToDevice, s));
-  // most calls with buckets take the plain form: their matrices are written in its
-  // layout now, beside the host's planning, and again (enqueue_fused) if not
+  // the matrices are written in the layout of the form that the call will take, as far as can be
+  // told here (see prepare_fused), beside the host's planning, and again (enqueue_fused) if it
+  // takes the other
   cp.rerank_hjobs = jobs;
   cp.rerank_djobs = djobs;
   cp.rerank_drops = ddrop;
-  cp.rerank_tiled = cp.slots.size() == 1 && ctx->tune_layout != 0 &&
-                    (cp.groups[0].dense_H == nullptr || !cp.groups[0].rs->has_nan);
+  const krux_rankset *rs0 = cp.groups[0].rs;
+  const bool dense = cp.groups[0].dense_H != nullptr;
+  cp.rerank_tiled = cp.slots.size() == 1 && plain_form_fits(ctx, rs0->Np, false) != 0 &&
+                    (!rs0->has_nan || (!dense && 128 * rs0->nan_traits_over <= rs0->T)) &&
+                    (dense || few_hits(cp, o->pthresh, rs0->Np, rs0->has_nan));
   KRUX_CUDA(ctx, launch_rerank_buckets(djobs, jobs.data(), ddrop, (int)nb, cp.rerank_tiled, s));
   if (ctx->profiling) ctx->prof.launches += 1;
   // runs of buckets of the same rank set: one A map each
@@ -1413,32 +1443,6 @@ struct FusedLaunch {
   const CisGroup *cistab = nullptr;         // cis scans: their groups, planned on the device
   const double *const *cfacptr = nullptr;
 };
-
-// Whether a call's hits, about P_c of its pairs where nothing is associated, are few
-// enough for the plain form of its kind.  Two event warps per CTA write them there, all
-// sixteen epilogue warps in the general form, which pays from some 0.2 % of independent SNPs on
-// (scan kernel, plain against general, us; in brackets SNPs in LD blocks, whose hits come
-// together):
-//   cis, 10,000 x 40,000 x 102         P_c = 1e-3 621 (259) against 843 (729), 2e-3 1,316
-//                                      (337) against 1,071 (938), 1e-2 6,743 (1,022) against 1,593 (1,714)
-//   ANOVA, the same                    1e-3 602 (210) against 598 (440), 2e-3 1,136 (262)
-//                                      against 720 (509), 1e-2 4,758 (872) against 933 (739)
-//   five groups, the same              3e-3 1,288 against 1,796, 5e-3 2,180 against 2,260, 1e-2
-//                                      4,416 against 2,896
-//   scan, N = 300, 6,000 x 20,000      (whole calls) 2e-3 0.88 (0.67) of the general form's time,
-//                                      3e-3 1.12 (0.67), 1e-2 2.54 (0.89), 5e-2 9.2 (1.8)
-//   NaN, N = 300, the same             3e-3 0.94 (0.40), 5e-3 1.17 (0.43), 5e-2 3.3 (0.89)
-//   3 permutations, N = 300,           4e-3 0.92 (0.58), 1e-2 1.10 (0.63), 5e-2 1.98 (0.84); with
-//   2,000 x 10,000                     FDR counts 1e-2 0.53 (0.18), 5e-2 1.16 (0.25)
-// (the last three alike from 180 samples on).  Up to 176 samples, with NaN 160, these have no
-// line: there the plain form is the only one that a call takes by itself, it is ahead in LD
-// blocks, the usual input, up to some 2 % of hits, and krux_autotune times both on the data.
-bool few_hits(const CallPlan &cp, double pthresh, int Np, bool nan) {
-  if (cp.multi) return pthresh <= 4e-3;
-  if (cp.cis.on || cp.param.model >= 0) return pthresh <= 1.5e-3;
-  if (cp.perm.on) return Np <= 176 || pthresh <= (cp.perm.fdr ? 3e-2 : 7e-3);
-  return nan ? Np <= 160 || pthresh <= 4e-3 : Np <= 176 || pthresh <= 2.5e-3;
-}
 
 // tables = 1 puts this launch's tables (group descriptors, work items, pack jobs,
 // tie-factor pointers) in the context's second set, so that two prepared launches
@@ -2171,7 +2175,7 @@ extern "C" krux_status krux_scan(krux_ctx *ctx, const krux_rankset *rs, const in
     st = enqueue_fused(ctx, whole, fl, s);
     if (st == KRUX_OK) st = finish_fused(ctx, whole, fl, s, counts);
   } else {
-    st = materialise(ctx, cp, s);
+    st = materialise(ctx, cp, opts, s);
     if (st == KRUX_OK) st = run_fused(ctx, cp, opts, s, counts);
   }
   if (st != KRUX_OK) return st;
@@ -2337,7 +2341,7 @@ extern "C" krux_status krux_scan_cis(krux_ctx *ctx, const krux_rankset *rs, cons
     st = enqueue_fused(ctx, whole, fl, s);
     if (st == KRUX_OK) st = finish_fused(ctx, whole, fl, s, counts);
   } else {
-    st = materialise(ctx, cp, s);
+    st = materialise(ctx, cp, opts, s);
     if (st == KRUX_OK) st = run_fused(ctx, cp, opts, s, counts);
   }
   if (st != KRUX_OK) return st;
@@ -2463,7 +2467,7 @@ extern "C" krux_status krux_scan_parametric(krux_ctx *ctx, const float *expr, in
   if (st != KRUX_OK) return st;
   if (!cp.bucket_jobs.empty())
     return fail(ctx, KRUX_EUNSUPPORTED, "parametric scans take complete genotypes (no -1 codes)");
-  st = materialise(ctx, cp, s);
+  st = materialise(ctx, cp, opts, s);
   if (st != KRUX_OK) return st;
   std::vector<unsigned long long> counts;
   st = run_fused(ctx, cp, opts, s, counts);
@@ -2524,7 +2528,7 @@ extern "C" krux_status krux_scan_grouped(krux_ctx *ctx, krux_cohort *cohorts, in
     st = plan_groups(ctx, cp, k.rs, k.geno, k.ldg, 0, k.S, nullptr, 1, c, nullptr, nullptr, nullptr, s);
     if (st != KRUX_OK) return st;
   }
-  st = materialise(ctx, cp, s);
+  st = materialise(ctx, cp, opts, s);
   if (st != KRUX_OK) return st;
   // Cohorts whose every group can take the plain scan form run in one launch of
   // that form for each of its shapes (one launch has one shape), the others in one
@@ -2709,7 +2713,7 @@ static krux_status plan_permute(krux_ctx *ctx, CallPlan &cp, const krux_rankset 
       g.nan_ag_stride = (int64_t)lst;
     }
   }
-  return materialise(ctx, cp, s);
+  return materialise(ctx, cp, opts, s);
 }
 
 extern "C" krux_status krux_permute(krux_ctx *ctx, const krux_rankset *rs, const int8_t *geno,
@@ -2921,7 +2925,7 @@ extern "C" krux_status krux_graph_scan(krux_ctx *ctx, const krux_rankset *rs, co
   g->cp.slots.push_back(OutSlot{hits, hit_H, hit_p, opts->hit_capacity, w->aux.as<HitAux>()});
   st = plan_groups(w, g->cp, rs, geno, ldg, b, e, nullptr, 1, 0, opts->dense_H, opts->dense_p,
                    nullptr, g->cs);
-  if (st == KRUX_OK) st = materialise(w, g->cp, g->cs);
+  if (st == KRUX_OK) st = materialise(w, g->cp, opts, g->cs);
   if (st == KRUX_OK) st = graph_capture(ctx, g);
   if (st != KRUX_OK) return graph_fail(ctx, g, st);
   *out = g;
@@ -2989,7 +2993,7 @@ extern "C" krux_status krux_graph_grouped(krux_ctx *ctx, const krux_cohort *coho
     st = plan_groups(w, g->cp, k.rs, k.geno, k.ldg, 0, k.S, nullptr, 1, c, nullptr, nullptr,
                      nullptr, g->cs);
   }
-  if (st == KRUX_OK) st = materialise(w, g->cp, g->cs);
+  if (st == KRUX_OK) st = materialise(w, g->cp, opts, g->cs);
   if (st == KRUX_OK) st = graph_capture(ctx, g);
   if (st != KRUX_OK) return graph_fail(ctx, g, st);
   *out = g;
