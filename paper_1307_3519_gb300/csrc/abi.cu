@@ -485,8 +485,10 @@ struct GroupPlan {
 // items are taken longest first (5,000 x 100,000 x 102 with 196 missing patterns and
 // 1 % NaN: the scan 1.03 -> 0.58 ms, with two event entries per event warp).
 //
-// `fine` (dense output of the general form, whose FP64 work a pair takes by its trait and
-// SNP makes steps of very uneven length): at least eight items per CTA.  With the few items
+// `fine` (the general forms' dense output and several groups, whose work a pair takes by its
+// trait and SNP, FP64 or the counting of NaN samples, makes steps of very uneven length): at
+// least eight items per CTA, four with several groups (half the SNPs in 300 patterns, 30 % NaN,
+// 3,000 x 20,000 x 102 4.9 ms with one, 4.5 with four; one tile of traits with NaN 0.66 and 0.67).  With the few items
 // that fill whole waves, taken from the counter as CTAs come free, 1,000 x 20,003 x 102 in LD
 // blocks with 1 % NaN took 4.6 ms in fixed turns, 5.0 from the counter, now 3.2
 // (2,500 x 30,000 18.8 -> 10.5, independent SNPs 12.1 -> 9.9).
@@ -534,7 +536,7 @@ std::vector<WorkItem> make_items(const std::vector<GroupPlan> &gp, int grid, boo
     total += (double)(g.steps - g.step_lo) * g.n_btiles * step_cost(g.d, std::min(g.d.nc, g.d.nchunks));
   std::vector<int64_t> split(gp.size(), 1), best_split;
   double best = 1e300;
-  for (int m = 1; m <= 32; ++m) {
+  for (int m = fine ? 4 : 1; m <= 32; ++m) {
     const double target = total / ((double)grid * m);
     double longest = 0.0, extra = 0.0;
     for (size_t i = 0; i < gp.size(); ++i) {
@@ -1692,7 +1694,8 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
   } else {
     bool pairs = fast_shape;  // (as p.fast below)
     for (const GroupDesc &d : descs) pairs = pairs && d.pair == 1 && (d.nkb == 1 || d.nc == 2);
-    items = make_items(plans, workers, pairs || fl.signed_coef == 0, o->dense_H != nullptr && !pairs);
+    items = make_items(plans, workers, pairs || fl.signed_coef == 0,
+                       (o->dense_H != nullptr || ng > 1) && !pairs);
     n_items = items.size();
   }
   std::vector<const double *> cf(ng);

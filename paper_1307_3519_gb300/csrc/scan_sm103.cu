@@ -2359,6 +2359,10 @@ __global__ void __launch_bounds__(ScanRoles<kForm>::kThreads, 1)
             }
           }
         }
+        // The general forms' steps differ in length by up to a factor of ten (traits with many
+        // NaN samples): the next item is taken when this one's first chunk is free, which its
+        // copies wait for anyway, and not by a CTA that still has most of this one to do
+        if (p.next && !wait_bar(b_empty(0), (b_bits & 1u) ^ 1u, wc, 1)) goto producer_done;
       }
     producer_done:
       // let every copy this thread issued land before the CTA can exit (a pair of CTAs
