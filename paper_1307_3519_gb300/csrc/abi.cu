@@ -1532,11 +1532,12 @@ krux_status prepare_fused(krux_ctx *ctx, CallPlan &cp, const krux_opts *o, Fused
                        pair_cta_wanted(kpad);
     bool ok = pick_launch_shape(ctx, kpad, codes_k, sh, fast_shape, pairs);
     // Permutation batches contract twice in the plain form, once in the general one, which
-    // has the longer K blocks where the plain form's fall below 48 samples (from 321 on): 8 x
-    // 4,000 x 20,000 independent SNPs, N = 320 2.72 ms against 2.93 in the general form, N = 336
-    // 3.25 against 3.02, N = 360 4.72 against 3.93.  (In LD blocks N = 336 3.15 against 4.19, N =
-    // 360 4.65 against 4.90; the data of a call are not known when it is planned.)
-    if (ok && fast_shape && fl.signed_coef && tnc == 0 && sh.ka != kpad && sh.ka < 48) {
+    // has the longer K blocks where the plain form's fall to 16 samples (from 337 on): 8 x
+    // 10,000 x 50,000 independent SNPs, N = 320 10.6 ms against 13.3 in the general form, N = 336
+    // 13.7 against 13.8, N = 344 20.3 against 17.5, N = 368 22.0 against 17.6.  (In LD blocks 11.5
+    // against 18.7, 15.4 against 18.9, 21.1 against 24.5, 23.7 against 24.7; the data of a call are
+    // not known when it is planned.)
+    if (ok && fast_shape && fl.signed_coef && tnc == 0 && sh.ka != kpad && sh.ka < 32) {
       fast_shape = false;
       sh = LaunchShape{};
       ok = pick_launch_shape(ctx, kpad, codes_k, sh);

@@ -3706,6 +3706,7 @@ cudaError_t launch_seed_decide(const unsigned long long *rec, const __half *stac
                  : N <= 192 ? seed_decide_kernel<6>
                  : N <= 256 ? seed_decide_kernel<8>
                  : N <= 320 ? seed_decide_kernel<10>
+                 : N <= 384 ? seed_decide_kernel<12>
                             : seed_decide_kernel<16>;
   kernel<<<grid, 256, 0, s>>>(rec, stack, rows_pad, Np, N, T, P, geno, ldg, n_snps, meta, cfac,
                               key, bound, per);

@@ -27,9 +27,9 @@ def _data(N, T=200, S=700, codes=3):
     return rng.standard_normal((T, N)).astype(np.float32), rng.integers(0, codes, (S, N)).astype(np.int8)
 
 
-@pytest.mark.parametrize("N,form", [(102, 4), (304, 4), (320, 4), (321, 2), (336, 2), (368, 2), (400, 2)])
+@pytest.mark.parametrize("N,form", [(102, 4), (304, 4), (320, 4), (321, 4), (336, 4), (337, 2), (368, 2), (400, 2)])
 def test_wide_permutation_batches(kx, oracle_mod, N, form):
-    """The plain form up to the width where its K blocks hold 48 samples."""
+    """The plain form up to the width where its K blocks hold 32 samples."""
     import paper_1307_3519_gb300 as k
     expr, geno = _data(N)
     perms = k.krux_make_perms(N, 3, N)
