@@ -55,12 +55,12 @@ WORKLOAD = ("paper-scale fused scan: N=102 samples, T=20000 traits, S=500000 SNP
 #            -k regex:krux_scan_kernel -s 1 -c 1 python bench.py --scan-only --traits 20000
 #            --snps 100000 --data paper --tile 1,4,2,0 --reps 2
 #            (warp instructions x 32 lanes / pairs = lane issue slots per pair)
-# Measured on the kernel below: 247.63 MB read + 72.87 MB written per 500k-SNP launch;
-# 372.91 M warp instructions (301.91 M on the FMA-heavy, FMA-lite and ALU pipes) per
+# Measured on the kernel below: 246.87 MB read + 72.91 MB written per 500k-SNP launch;
+# 376.79 M warp instructions (303.88 M on the FMA-heavy, FMA-lite and ALU pipes) per
 # 100k-SNP launch of 2x10^9 pairs.
-SCAN_TRAFFIC = {"blob": "ff4c48a68e669ecba582a513645022214655270e", "bytes": 320.50e6}
-SCAN_ISSUE = {"blob": "ff4c48a68e669ecba582a513645022214655270e", "slots_per_pair": 5.97,
-              "fp32_int_slots_per_pair": 4.83,
+SCAN_TRAFFIC = {"blob": "e2ec363f0749ce45399dd2fb7eedf0112c3aa3ff", "bytes": 319.78e6}
+SCAN_ISSUE = {"blob": "e2ec363f0749ce45399dd2fb7eedf0112c3aa3ff", "slots_per_pair": 6.03,
+              "fp32_int_slots_per_pair": 4.86,
               "workload": "planted 20000 x 100000 x 102 (0.19% of pairs are hits)"}
 # Epilogue issue slots per pair by the operation count of the fused test P^2 + Q^2 >=
 # bound: two fused multiply-adds, half a sign accumulation and the TMEM load's eighth,

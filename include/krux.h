@@ -91,7 +91,7 @@ typedef struct {
   int64_t pairs;        /* SNP x trait pairs the last call tested */
   int32_t scan_form;    /* kernel form of the (last) fused scan launch.  Plain forms: 0 complete
                            data (cis and parametric scans too), 4 permutation batch, 5 NaN
-                           expression, 7 over pairs of CTAs (240 samples and more), 8 markers
+                           expression, 7 over pairs of CTAs (225 samples and more), 8 markers
                            with up to five groups, 9 dense output.  General forms, where no
                            plain one fits or pays: 1 markers with up to five groups, 2
                            permutation batch, 3 everything else */
