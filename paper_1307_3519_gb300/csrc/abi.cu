@@ -2425,6 +2425,12 @@ extern "C" krux_status krux_scan_parametric(krux_ctx *ctx, const float *expr, in
   // hit 228 us then, 261 with the table in line, 219 beside the scan)
   KRUX_CUDA(ctx, second_stream(ctx, s));
   KRUX_CUDA(ctx, launch_param_table(N, table, ctx->xs));
+  // a call that ends early (refused inputs, no SNPs) leaves no table under way, which the next
+  // call on another layout of the same buffer would find written into its values
+  struct Settle {
+    cudaStream_t xs;
+    ~Settle() { cudaStreamSynchronize(xs); }
+  } settle{ctx->xs};
   KRUX_CUDA(ctx, cudaEventRecord(ctx->xev, ctx->xs));
   ev_record(ctx, 0, s);
   KRUX_CUDA(ctx, launch_standardize(expr, T, N, ld, rs.Np, rs.dev.A, rs.dev.At, fixed, squares,
